@@ -2,25 +2,116 @@
 // sequence with potential size n draws n next tokens as independent trials from ONE logits row; equal draws are
 // grouped afterwards with ss_dedup_paths on (sequence, token) pairs.
 //
-// One block per sequence.  The cost is the fp64 exponentials (the token decision is taken in fp64 so that it agrees
-// with a plain fp64 CPU evaluation except for draws within ~1e-15 of a boundary), so they are evaluated once per
-// logit where possible:
-//   1. maximum                                   (fp32, exact; the row then stays in L2)
-//   2. running sum of exp((logit_v - max) / T) in chunks of 4096 tokens (fp64, block scan): only the cumulative sum
-//      at the end of every chunk is kept; the last one is the normaliser Z
-//   3. every draw finds its chunk by binary search over those sums; the chunks that hold a draw (one or two for a
-//      typical potential size) are evaluated again, now keeping the whole CDF in shared memory, and the draw finds
-//      its token by binary search there.
-// Bound by the fp64 pipe, not by memory: about one fp64 exponential per logit instead of two.
+// The token decision is taken in fp64 (so that it agrees with a plain fp64 CPU evaluation except for draws within
+// ~1e-15 of a boundary), one exponential per logit.  A row is split over the 16 warps of a block, or of a CLUSTER of
+// 2, 4 or 8 blocks when there are too few rows to give every SM one: each warp has one contiguous slice, and the slice sums
+// meet in (distributed) shared memory.  Nothing is read twice but the 512 tokens around each draw.
+//   1. every warp sums 2^(logit_v * c), c = log2(e) / temperature, over its slice in segments of 512 tokens and keeps
+//      the running sum at every segment's end (shared memory)
+//   2. the slice sums are written to every block of the cluster
+//   3. each of the row's warps takes a share of its draws: it finds the slice that holds u * Z from the slice sums, the
+//      segment from the running sums of the slice's owner, evaluates the segment again with a warp scan, and writes the
+//      token
+// A block that handles several rows takes step 1 of the next row before step 3 of the current one, between the two halves
+// of a split barrier, so that neither the barrier nor a draw is waited for; the warps that draw change from row to row.
+// There is no pass for the maximum: fp64 holds 2^(logit * c) itself for rows whose largest exponent lies in
+// [kLowTop, kHighTop], which every ordinary row does; a row outside (or a temperature outside [1e-3, 1e6]) is summed again
+// relative to its maximum with the library's exp.
+//
+// The exponential (after Tang, "Table-driven implementation of the exponential function in IEEE floating-point
+// arithmetic", ACM TOMS 15, 1989): K = the integer nearest to 128 * x from ONE fp32 FMA (it only has to be near), r =
+// 128 * x - K exactly by one fp64 FMA, 2^(K/128) from a table of 128 entries and an integer addition to the exponent,
+// 2^(r/128) by a polynomial of degree 4 (interpolated at Chebyshev nodes, relative error below 1.7e-16 for |r| <= 0.505).
+// 8 fp64 instructions with the summation; the table is copied 16 times so that every lane reads its own bank pair.
+// Bound: issue slots.  An fp64 instruction holds two, so 32 logits take ~30 clocks of a sub-partition, 120 us for
+// 922 x 151936 logits (the loop alone, measured; 4 bytes a logit from HBM would take 85).  Measured, the call: 922 rows
+// 582 -> 186 us, 16 rows 91 -> 18 us, against one block of 1024 threads per row with a pass for the maximum, CUDA's exp
+// and a block-wide scan for every 4096 tokens.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 
 namespace ss {
 namespace sample {
 
-constexpr int kThreads = 1024;
-constexpr int kPerThread = 4;
-constexpr int kChunk = kThreads * kPerThread;
-constexpr int kMaxChunks = 512;                              // vocabularies of up to 2 M tokens
+namespace cg = cooperative_groups;
+
+constexpr int kThreads = 512;                                 // one block per SM (128 registers a thread)
+constexpr int kWarps = kThreads / 32;
+constexpr int kSeg = 512;                                     // tokens per segment: 16 per lane, 4 x 128 bits
+constexpr int kMaxSegs = 32;                                  // per slice
+constexpr int kMaxVocab = 2097152;
+constexpr int kTable = 128;
+constexpr float kLowTop = -200.f, kHighTop = 900.f;           // exponent range of a row's largest term
+constexpr float kLowest = -1020.f;                            // smaller exponents count as this one (2^-820 of the sum)
+constexpr double kTiny = 1e-300;                              // above 2^-1020: what a masked token counts for
+
+struct Args {
+  const float* logits;
+  const int64_t* draw_offsets;
+  const float* uniforms;
+  int32_t* tokens_out;
+  int64_t* seq_out;
+  int n_seq, row0, vocab;
+  int slice;                   // tokens per warp, a multiple of kSeg / 2
+  double inv_temperature;
+  double ck;                   // kTable * log2(e) / temperature
+  float ckf, lowest;           // lowest: the logit whose exponent is kLowest
+  bool fast;                   // the temperature allows the table path
+};
+
+template <int CL>
+struct Sums {                          // of one row
+  double seg_end[kWarps][kMaxSegs];    // own slices: sum up to the end of each segment
+  double slice_sum[CL * kWarps];       // the whole row's, written by the cluster's blocks
+  float slice_max[CL * kWarps];
+};
+template <int CL>
+struct Shared {
+  double table[kTable * 16];
+  Sums<CL> sums[4];                    // rows in turn (a warp may be two rows ahead of one that reads its running sums);
+};                                     // [3]: a row outside the table path's range
+
+// 2^(l * c) for -1021 < l * c < 1021 (see the head of the file); `bank` = table + (lane & 15)
+__device__ __forceinline__ double exp2_table(float l, const Args& A, const double* bank) {
+  constexpr float kRound = 12582912.f;                        // 1.5 * 2^23: the sum's low bits are the nearest integer
+  constexpr double a1 = 0.005415212348124257, a2 = 1.466226238764014e-05, a3 = 2.6466431340771855e-08,
+                   a4 = 3.5830331985890313e-11;
+  const int bits = __float_as_int(fmaf(l, A.ckf, kRound));    // 0x4b400000 + K
+  const double K = __hiloint2double(0x43300000, bits) - (4503599627370496.0 + 1262485504.0);   // 2^52 + bits - (2^52 + 0x4b400000)
+  const double r = fma(static_cast<double>(l), A.ck, -K);
+  const double t0 = bank[(bits & (kTable - 1)) * 16];
+  // K / 128 into the exponent field: the table has K % 128 taken off again, and the bits of 0x4b400000 that the shift
+  // keeps are zero
+  const double t = __hiloint2double(__double2hiint(t0) + (bits << 13), __double2loint(t0));
+  double q = fma(a4, r, a3);
+  q = fma(q, r, a2);
+  q = fma(q, r, a1);
+  return fma(t * r, q, t);
+}
+// The term relative to the row's maximum (rows outside the table path's range).  Tokens past the end (and masked ones)
+// count as 2^-1020 on the table path, exactly 0 here.
+__device__ __noinline__ double term_exact(float l, double dmax, double inv_temperature) {
+  return exp((static_cast<double>(l) - dmax) * inv_temperature);
+}
+
+// 8 logits of a lane, half of its share of a segment: tokens base + 128 j + 4 lane + x for j = 0, 1; -inf past the end.
+// VEC: rows start on 16 bytes and are whole 16-byte units.
+template <bool VEC>
+__device__ __forceinline__ void load_half(const float* __restrict__ row, int base, int vocab, int lane, float (&l)[8]) {
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const int v = base + 128 * j + 4 * lane;
+    if (VEC) {
+      const float4 f = v < vocab ? __ldg(reinterpret_cast<const float4*>(row + v))
+                                 : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+      l[4 * j] = f.x; l[4 * j + 1] = f.y; l[4 * j + 2] = f.z; l[4 * j + 3] = f.w;
+    } else {
+#pragma unroll
+      for (int x = 0; x < 4; ++x) l[4 * j + x] = v + x < vocab ? __ldg(row + v + x) : -INFINITY;
+    }
+  }
+}
 
 __device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
@@ -28,122 +119,289 @@ __device__ __forceinline__ double warp_sum_d(double v) {
   return v;
 }
 
-__global__ void __launch_bounds__(kThreads)
-branch_sample_kernel(const float* __restrict__ logits, const int64_t* __restrict__ draw_offsets,
-                     const float* __restrict__ uniforms, int vocab, double inv_temperature,
-                     int32_t* __restrict__ tokens_out, int64_t* __restrict__ seq_out) {
-  ss::grid_dependency_enter();
-  __shared__ double s_cdf[kChunk];
-  __shared__ double s_warp[32];
-  __shared__ float s_wmax[32];
-  __shared__ double s_end[kMaxChunks];                     // cumulative sum at the end of every chunk
-  __shared__ int s_need[kMaxChunks];
-  const int s = blockIdx.x;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float* row = logits + static_cast<int64_t>(s) * vocab;
-  const int64_t d0 = draw_offsets[s], d1 = draw_offsets[s + 1];
-  if (d1 <= d0) return;                                      // nothing to draw for this sequence
-
-  // ---- 1. maximum ---------------------------------------------------------------------------------------------
-  float mx = -INFINITY;
-  for (int v = tid; v < vocab; v += kThreads) mx = fmaxf(mx, row[v]);
-  mx = warp_max(mx);
-  if (lane == 0) s_wmax[warp] = mx;
-  __syncthreads();
-  mx = s_wmax[0];
+// Sum of the warp's slice of n_half half segments, the first of which is in `a`; `mx`: the largest logit of the lane.
+template <bool VEC>
+__device__ __forceinline__ double slice_sums(const float* __restrict__ row, const Args& A, const double* bank,
+                                             double* seg_end, int v0, int n_half, int lane, float (&a)[8], float& mx) {
+  double end = 0.0;
+  mx = -INFINITY;
+  float b[8];                                                  // one half in flight while the other is summed
+  auto add = [&](float (&l)[8], double& s0, double& s1) {
+    float mn = l[0];
 #pragma unroll
-  for (int w = 1; w < 32; ++w) mx = fmaxf(mx, s_wmax[w]);
-  const double dmax = static_cast<double>(mx);
-
-  // ---- 2. cumulative sums at the chunk ends; Z -----------------------------------------------------------------------
-  // inclusive CDF of chunk `base`: thread t owns tokens base + 4t .. base + 4t + 3; returns the chunk's last value and,
-  // if `keep`, leaves every value in s_cdf
-  auto chunk_cdf = [&](int base, double carry, bool keep) -> double {
-    double e[kPerThread], run = 0.0;
+    for (int x = 0; x < 8; ++x) { mx = fmaxf(mx, l[x]); mn = fminf(mn, l[x]); }
+    if (__any_sync(0xffffffffu, !(mn >= A.lowest))) {          // masked tokens, or past the end
 #pragma unroll
-    for (int x = 0; x < kPerThread; ++x) {
-      const int v = base + tid * kPerThread + x;
-      e[x] = v < vocab ? exp((static_cast<double>(row[v]) - dmax) * inv_temperature) : 0.0;
-      run += e[x];
+      for (int x = 0; x < 8; ++x) l[x] = fmaxf(l[x], A.lowest);
     }
-    double incl = run;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const double y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
+    for (int x = 0; x < 8; x += 2) {
+      s0 += exp2_table(l[x], A, bank);
+      s1 += exp2_table(l[x + 1], A, bank);
     }
-    __syncthreads();                                         // (s_warp / s_cdf of the previous chunk are no longer read)
-    if (lane == 31) s_warp[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-      double t = s_warp[lane];
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const double y = __shfl_up_sync(0xffffffffu, t, o);
-        if (lane >= o) t += y;
-      }
-      s_warp[lane] = t;
-    }
-    __syncthreads();
-    double c = carry + (warp ? s_warp[warp - 1] : 0.0) + incl - run;
-    if (keep) {
-#pragma unroll
-      for (int x = 0; x < kPerThread; ++x) {
-        c += e[x];
-        s_cdf[tid * kPerThread + x] = c;
-      }
-      __syncthreads();
-    }
-    return carry + s_warp[31];
   };
-  const int n_chunks = (vocab + kChunk - 1) / kChunk;
-  {
-    double carry = 0.0;
-    for (int k = 0; k < n_chunks; ++k) {
-      carry = chunk_cdf(k * kChunk, carry, false);
-      if (tid == 0) s_end[k] = carry;
+#pragma unroll 1
+  for (int h = 0; h < n_half; h += 2) {
+    double s0 = 0.0, s1 = 0.0;
+    const bool second = h + 1 < n_half;
+    if (second) load_half<VEC>(row, v0 + (h + 1) * (kSeg / 2), A.vocab, lane, b);
+    add(a, s0, s1);
+    if (second) {
+      if (h + 2 < n_half) load_half<VEC>(row, v0 + (h + 2) * (kSeg / 2), A.vocab, lane, a);
+      add(b, s0, s1);
     }
+    end += warp_sum_d(s0 + s1);
+    if (lane == 0) seg_end[h >> 1] = end;
+  }
+  return end;
+}
+// The same relative to the row's maximum.
+template <bool VEC>
+__device__ __noinline__ double slice_sums_exact(const float* __restrict__ row, const Args& A, double* seg_end, int v0,
+                                                int n_half, int lane, double dmax) {
+  double end = 0.0;
+  for (int h = 0; h < n_half; ++h) {
+    float l[8];
+    load_half<VEC>(row, v0 + h * (kSeg / 2), A.vocab, lane, l);
+    double sum = 0.0;
+#pragma unroll 1
+    for (int x = 0; x < 8; ++x) sum += term_exact(l[x], dmax, A.inv_temperature);
+    end += warp_sum_d(sum);
+    if (lane == 0) seg_end[h >> 1] = end;
+  }
+  return end;
+}
+
+// The slice's sum and maximum to every block of the cluster (visible there after the cluster's next barrier).
+template <int CL>
+__device__ __forceinline__ void publish(cg::cluster_group& cl, Sums<CL>& S, int slice, int lane, double sum, float mx) {
+  if (lane < CL) {
+    Sums<CL>* R = cl.map_shared_rank(&S, lane);
+    R->slice_sum[slice] = sum;
+    R->slice_max[slice] = mx;
+  }
+}
+// The two halves of the cluster's barrier (a cluster of one block: of the block's).
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// A slice's place in its row.
+struct Slice {
+  int v0, n_half;                                              // n_half: half segments
+};
+__device__ __forceinline__ Slice slice_of(const Args& A, int slice) {
+  const int64_t first = static_cast<int64_t>(slice) * A.slice;
+  const int v0 = static_cast<int>(first < A.vocab ? first : A.vocab);
+  return Slice{v0, (min(A.slice, A.vocab - v0) + kSeg / 2 - 1) / (kSeg / 2)};
+}
+
+// The token of target t, which lies in the segment [base, min(base + kSeg, end)); `before`: the sum in front of it.
+template <bool FAST, bool VEC>
+__device__ __forceinline__ int token_in_segment(const float* __restrict__ row, const Args& A, const double* bank,
+                                                double dmax, int base, int end, double before, double t, int lane) {
+  double e[4][4], run[4], incl[4];                            // terms; sums of the lane's share of a group of 128; scanned
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    float l[8];
+    load_half<VEC>(row, base + h * (kSeg / 2), end, lane, l);
+#pragma unroll
+    for (int x = 0; x < 8; ++x)
+      e[2 * h + (x >> 2)][x & 3] = FAST ? exp2_table(fmaxf(l[x], A.lowest), A, bank) : term_exact(l[x], dmax, A.inv_temperature);
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) incl[j] = run[j] = (e[j][0] + e[j][1]) + (e[j][2] + e[j][3]);
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const double y = __shfl_up_sync(0xffffffffu, incl[j], o);
+      if (lane >= o) incl[j] += y;
+    }
+  }
+  int token = -1;                                              // if rounding leaves t above everything: the last that counts
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const uint32_t some = __ballot_sync(0xffffffffu, run[j] > kTiny);
+    const uint32_t over = __ballot_sync(0xffffffffu, run[j] > kTiny && before + incl[j] > t);
+    if (some) {
+      const int f = over ? __ffs(over) - 1 : 31 - __clz(some);
+      double c = before + (incl[j] - run[j]);
+      int hit = -1, tail = 0;
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        c += e[j][x];
+        if (e[j][x] > kTiny) {
+          tail = x;
+          if (hit < 0 && c > t) hit = x;
+        }
+      }
+      token = base + 128 * j + 4 * f + __shfl_sync(0xffffffffu, hit < 0 ? tail : hit, f);
+      if (over) return token;
+    }
+    before += __shfl_sync(0xffffffffu, incl[j], 31);
+  }
+  return token < 0 ? A.vocab - 1 : token;
+}
+
+template <bool VEC>
+__device__ __noinline__ int token_in_segment_exact(const float* __restrict__ row, const Args& A, double dmax, int base, int end,
+                                                   double before, double t, int lane) {
+  return token_in_segment<false, VEC>(row, A, nullptr, dmax, base, end, before, t, lane);
+}
+
+// This warp's share of the draws of row `seq`; `at`: which of `sums` holds the row.
+template <int CL, bool VEC>
+__device__ __forceinline__ void draws(const Args& A, Sums<CL>* sums, const double* bank, int at, int64_t seq, int slice, int lane) {
+  constexpr int kSlices = CL * kWarps;
+  cg::cluster_group cl = cg::this_cluster();
+  const float* row = A.logits + seq * A.vocab;
+  const int64_t d0 = A.draw_offsets[seq], d1 = A.draw_offsets[seq + 1];
+  const int turn = static_cast<int>((slice + seq) % kSlices);
+  float mx = -INFINITY;
+  for (int i = lane; i < kSlices; i += 32) mx = fmaxf(mx, sums[at].slice_max[i]);
+  mx = warp_max(mx);
+  const double dmax = static_cast<double>(mx);
+  const float top = mx * A.ckf * (1.f / kTable);
+  const bool fast = A.fast && top >= kLowTop && top <= kHighTop;
+  if (!fast) {                                                 // again, relative to the row's maximum (the cluster agrees)
+    at = 3;
+    const Slice L = slice_of(A, slice);
+    const double sum = slice_sums_exact<VEC>(row, A, sums[at].seg_end[slice % kWarps], L.v0, L.n_half, lane, dmax);
+    publish<CL>(cl, sums[at], slice, lane, sum, mx);
+    cl.sync();
+  }
+  if (d0 + turn >= d1) return;
+  Sums<CL>& S = sums[at];
+  // Cumulative sums at the ends of the slices: the first lanes add up a block's, then the blocks in turn.  A slice ends at
+  // (start of its block) + (sum of the block's slices so far), so the ends ascend whatever the rounding.
+  double in_block = 0.0, end_b = 0.0, Z = 0.0;
+  if (lane < CL)
+    for (int w = 0; w < kWarps; ++w) in_block += S.slice_sum[lane * kWarps + w];
+#pragma unroll
+  for (int b = 0; b < CL; ++b) {
+    Z += __shfl_sync(0xffffffffu, in_block, b);
+    if (lane == b) end_b = Z;
+  }
+  for (int64_t d = d0 + turn; d < d1; d += kSlices) {
+    const double t = static_cast<double>(A.uniforms[d]) * Z;
+    int token = A.vocab - 1;                                   // the answer if t is not below the total
+    if (t == 0.0) {                                            // the first term that is not 0 at all
+      for (int v = 0; v < A.vocab; v += 32) {
+        const bool pos = v + lane < A.vocab && term_exact(row[v + lane], dmax, A.inv_temperature) > 0.0;
+        const uint32_t any = __ballot_sync(0xffffffffu, pos);
+        if (any) { token = v + __ffs(any) - 1; break; }
+      }
+    } else if (t < Z) {
+      const int b = __ffs(__ballot_sync(0xffffffffu, lane < CL && end_b > t)) - 1;
+      const double start = b ? __shfl_sync(0xffffffffu, end_b, max(b - 1, 0)) : 0.0;
+      int w = 0;
+      double in_front = 0.0;                                   // of slice w in its block
+      for (; w < kWarps - 1; ++w) {
+        const double e = in_front + S.slice_sum[b * kWarps + w];
+        if (start + e > t) break;
+        in_front = e;
+      }
+      const Slice L = slice_of(A, b * kWarps + w);
+      const double* seg_end = cl.map_shared_rank(&S, b)->seg_end[w];
+      const double before = start + in_front;
+      const int n_seg = (L.n_half + 1) >> 1;                   // at most kMaxSegs
+      const double end_s = lane < n_seg ? seg_end[lane] : 0.0;
+      const uint32_t hit = __ballot_sync(0xffffffffu, lane < n_seg && before + end_s > t);
+      const int s = hit ? __ffs(hit) - 1 : n_seg - 1;
+      if (s >= 0) {
+        const double in_slice = s ? __shfl_sync(0xffffffffu, end_s, max(s - 1, 0)) : 0.0;
+        const int base = L.v0 + s * kSeg, end = min(A.vocab, L.v0 + A.slice);
+        token = fast ? token_in_segment<true, VEC>(row, A, bank, dmax, base, end, before + in_slice, t, lane)
+                     : token_in_segment_exact<VEC>(row, A, dmax, base, end, before + in_slice, t, lane);
+      }
+    }
+    if (lane == 0) {
+      A.tokens_out[d] = token;
+      A.seq_out[d] = seq;
+    }
+  }
+}
+
+template <int CL, bool VEC>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kThreads, 1)
+branch_sample_kernel(const __grid_constant__ Args A) {
+  ss::grid_dependency_enter();
+  __shared__ Shared<CL> S;
+  cg::cluster_group cl = cg::this_cluster();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int slice = static_cast<int>(cl.block_rank()) * kWarps + warp;
+  const Slice L = slice_of(A, slice);
+  const double* bank = S.table + (lane & 15);
+  // rows with something to draw, in turn (the cluster's blocks agree)
+  auto next_row = [&](int64_t r) {
+    while (r < A.n_seq && A.draw_offsets[r + 1] <= A.draw_offsets[r]) r += gridDim.x / CL;
+    return r;
+  };
+  const int64_t row0 = A.row0 + static_cast<int64_t>(blockIdx.x / CL);   // (there are no more clusters than rows)
+  float first[8];
+  load_half<VEC>(A.logits + row0 * A.vocab, L.v0, A.vocab, lane, first);   // in flight while the table is made
+  int64_t row = next_row(row0), prev = -1;
+  if (row != row0 && row < A.n_seq) load_half<VEC>(A.logits + row * A.vocab, L.v0, A.vocab, lane, first);
+  if (tid < kTable) {
+    const double e = exp2(static_cast<double>(tid) / kTable);
+    S.table[tid * 16] = __hiloint2double(__double2hiint(e) - (tid << 13), __double2loint(e));
   }
   __syncthreads();
-  const double Z = s_end[n_chunks - 1];
+  for (int i = tid; i < kTable * 16; i += kThreads)
+    if (i & 15) S.table[i] = S.table[i & ~15];
+  cl.sync();                                                   // (the table; and every block runs before it is written to)
 
-  // ---- 3. the draws, in batches of one per thread ----------------------------------------------------------------------
-  for (int64_t db = d0; db < d1; db += kThreads) {
-    const int64_t d = db + tid;
-    const bool have = d < d1;
-    const double target = have ? static_cast<double>(uniforms[d]) * Z : 0.0;
-    int token = vocab - 1;                                   // the answer if rounding leaves the target above the total
-    int my_chunk = -1;
-    if (have && s_end[n_chunks - 1] > target) {              // first chunk whose end exceeds the target
-      int lo = 0, hi = n_chunks - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (s_end[mid] > target) hi = mid; else lo = mid + 1;
-      }
-      my_chunk = lo;
-    }
-    for (int k = tid; k < n_chunks; k += kThreads) s_need[k] = 0;
-    __syncthreads();
-    if (my_chunk >= 0) s_need[my_chunk] = 1;
-    __syncthreads();
-    for (int k = 0; k < n_chunks; ++k) {
-      if (!s_need[k]) continue;                              // (block-uniform)
-      chunk_cdf(k * kChunk, k ? s_end[k - 1] : 0.0, true);
-      if (my_chunk == k) {                                   // first index of the chunk whose CDF exceeds the target
-        int lo = 0, hi = min(kChunk, vocab - k * kChunk) - 1;
-        while (lo < hi) {
-          const int mid = (lo + hi) >> 1;
-          if (s_cdf[mid] > target) hi = mid; else lo = mid + 1;
+  int at = 0, prev_at = 0;
+  for (;;) {
+    double sum = 0.0;
+    float mx = -INFINITY;
+    const bool more = row < A.n_seq;
+    int64_t after = row;
+    if (more) {
+      const float* p = A.logits + row * A.vocab;
+      if (A.fast) {
+        sum = slice_sums<VEC>(p, A, bank, S.sums[at].seg_end[warp], L.v0, L.n_half, lane, first, mx);
+      } else {
+        for (int h = 0; h < L.n_half; ++h) {
+          load_half<VEC>(p, L.v0 + h * (kSeg / 2), A.vocab, lane, first);
+#pragma unroll
+          for (int x = 0; x < 8; ++x) mx = fmaxf(mx, first[x]);
         }
-        token = k * kChunk + lo;
       }
+      mx = warp_max(mx);
+      after = next_row(row + gridDim.x / CL);
+      if (after < A.n_seq) load_half<VEC>(A.logits + after * A.vocab, L.v0, A.vocab, lane, first);
     }
-    if (have) {
-      tokens_out[d] = token;
-      seq_out[d] = s;
+    if (prev >= 0) {
+      cluster_wait();
+      draws<CL, VEC>(A, S.sums, bank, prev_at, prev, slice, lane);
     }
-    __syncthreads();
+    if (!more) break;
+    publish<CL>(cl, S.sums[at], slice, lane, sum, mx);
+    cluster_arrive();
+    prev = row;
+    prev_at = at;
+    at = at == 2 ? 0 : at + 1;
+    row = after;
   }
+  if (CL > 1) cl.sync();                                       // (a block's running sums may still be read by another)
+}
+
+// Rows row0 .. n_seq-1, `clusters` at a time.
+template <int CL>
+static int32_t launch(Args A, bool vec, int row0, int n_seq, int clusters, cudaStream_t st) {
+  constexpr int kUnit = kSeg / 2;
+  A.slice = (A.vocab + CL * kWarps * kUnit - 1) / (CL * kWarps * kUnit) * kUnit;
+  A.row0 = row0;
+  A.n_seq = n_seq;
+  if (vec)
+    SS_LAUNCH((branch_sample_kernel<CL, true>), clusters * CL, kThreads, 0, st, A);
+  else
+    SS_LAUNCH((branch_sample_kernel<CL, false>), clusters * CL, kThreads, 0, st, A);
+  return SS_OK;
 }
 
 }  // namespace sample
@@ -153,11 +411,44 @@ extern "C" int32_t ss_branch_sample(const float* logits, const int64_t* draw_off
                                     int32_t n_seq, int32_t vocab, float temperature, int32_t* tokens_out,
                                     int64_t* seq_out, void* stream) {
   using namespace ss;
+  using namespace ss::sample;
   if (n_seq < 0 || vocab < 1 || !(temperature > 0.f)) return SS_ERR_INVALID_ARG;
-  if (vocab > sample::kChunk * sample::kMaxChunks) return SS_ERR_UNSUPPORTED;
+  if (vocab > kMaxVocab) return SS_ERR_UNSUPPORTED;
   if (n_seq == 0) return SS_OK;
   if (!logits || !draw_offsets || !uniforms || !tokens_out || !seq_out) return SS_ERR_INVALID_ARG;
-  SS_LAUNCH(sample::branch_sample_kernel, n_seq, sample::kThreads, 0, as_stream(stream), logits, draw_offsets, uniforms,
-            vocab, 1.0 / static_cast<double>(temperature), tokens_out, seq_out);
-  return SS_OK;
+  const double T = static_cast<double>(temperature), c = 1.4426950408889634 / T;
+  Args A{};
+  A.logits = logits;
+  A.draw_offsets = draw_offsets;
+  A.uniforms = uniforms;
+  A.tokens_out = tokens_out;
+  A.seq_out = seq_out;
+  A.vocab = vocab;
+  A.inv_temperature = 1.0 / T;
+  A.ck = kTable * c;
+  A.ckf = static_cast<float>(A.ck);
+  A.lowest = static_cast<float>(kLowest / c);
+  A.fast = T >= 1e-3 && T <= 1e6;
+  const bool vec = reinterpret_cast<uintptr_t>(logits) % 16 == 0 && vocab % 4 == 0;
+  cudaStream_t st = as_stream(stream);
+  const int sms = sm_count_of_current_device();
+  // Whole rounds of one row per SM, then the rows that are left over on clusters as large as they fit: a GPC of 18 SMs
+  // holds 2 clusters of 8 blocks, 4 of 4, 9 of 2 (one block per SM), and there are 8.  (Clusters for all rows: the
+  // launch and the barriers of a block that has an eighth of a row cost more than the uneven last round, 250-400 us
+  // instead of 186 for 922 rows; persistent clusters depend on all of them being placed at once.)
+  constexpr int kMaxSlice = kMaxSegs * kSeg * kWarps;           // vocabulary that one block can take (262144)
+  const int blocks_min = (vocab + kMaxSlice - 1) / kMaxSlice;   // 1 .. 8
+  auto cluster_size = [&](int rows) { return rows <= 16 ? 8 : rows <= 32 ? 4 : rows <= 72 ? 2 : 1; };
+  int whole = blocks_min > 1 ? 0 : n_seq / sms * sms;
+  if (blocks_min == 1 && cluster_size(n_seq - whole) == 1) whole = n_seq;
+  if (whole > 0) {
+    const int32_t rc = launch<1>(A, vec, 0, whole, whole < sms ? whole : sms, st);
+    if (rc != SS_OK) return rc;
+  }
+  const int rest = n_seq - whole;
+  if (rest == 0) return SS_OK;
+  const int size = cluster_size(rest) > blocks_min ? cluster_size(rest) : blocks_min;
+  if (size > 4) return launch<8>(A, vec, whole, n_seq, rest < 16 ? rest : 16, st);
+  if (size > 2) return launch<4>(A, vec, whole, n_seq, rest < 32 ? rest : 32, st);
+  return launch<2>(A, vec, whole, n_seq, rest < 72 ? rest : 72, st);
 }

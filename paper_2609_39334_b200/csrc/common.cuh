@@ -55,6 +55,8 @@ inline int current_device_slot() {
   return (dev >= 0 && dev < kDeviceSlots) ? dev : -1;
 }
 
+int sm_count_of_current_device();
+
 constexpr size_t kAlign = 256;
 inline size_t align_up(size_t x, size_t a = kAlign) { return (x + a - 1) / a * a; }
 

@@ -77,3 +77,31 @@ def test_branch_sample_vs_oracle(S, V, T, maxpot):
         r = oracle.dedup(want_tok, np.arange(len(want_tok) + 1), ctx_key=want_seq)
         assert np.array_equal(uniq, r["unique_paths"]) and np.array_equal(mult, r["multiplicity"])
         assert int(mult.sum()) == int(off[-1])
+
+
+@pytest.mark.parametrize("V", [1, 3, 127, 511, 512, 513, 32767, 32772, 65537])
+@pytest.mark.parametrize("kind", ["plain", "offset_up", "offset_down", "cold", "hot", "masked"])
+def test_branch_sample_slices_segments_and_ranges(V, kind):
+    """Vocabularies at the edges of a warp's slice and its segments, rows inside and outside the table path's range of
+    exponents, masks of -inf and of a large negative number, uniforms of exactly 0 and just below 1.  Draws are compared
+    where the oracle's distance to a boundary is above 1e-12 of the sum (both sides round at 1e-15)."""
+    rng = np.random.default_rng(V)
+    S, T = 5, {"cold": 2e-4, "hot": 3e6}.get(kind, 0.8)
+    logits = (rng.normal(size=(S, V)) * 3).astype(np.float32)
+    logits += np.float32({"offset_up": 3000.0, "offset_down": -700.0}.get(kind, 0.0))
+    if kind == "masked":
+        logits[:, : V // 3] = -np.inf
+        logits[rng.random((S, V)) < 0.2] = -1e9
+        logits[:, V - 1] = 1.0                                     # (something to draw)
+    pot = np.asarray([1, 33, 0, 70, 4])
+    off = np.concatenate([[0], np.cumsum(pot)]).astype(np.int64)
+    u = rng.random(int(off[-1])).astype(np.float32)
+    u[:40:7] = 0.0
+    u[3:60:9] = np.float32(1.0) - np.float32(2.0 ** -24)
+    tok, seq = run(logits, off, u, T)
+    want_tok, want_seq, margin = oracle.branch_sample(logits, off, u, T)
+    got = tok.cpu().numpy()
+    assert np.array_equal(seq.cpu().numpy(), want_seq)
+    sure = margin > 1e-12
+    assert np.array_equal(got[sure], want_tok[sure])
+    assert np.array_equal(got[u == 0.0], want_tok[u == 0.0])
