@@ -2,289 +2,263 @@
 // "Computation Deduplication": candidates of a step share a large part of their tokens; Section "Experimental Setup":
 // prefix KV caching and sharing).  Only whole pages are shared; every path gets a private leaf node.
 //
-// Pipeline (all on the caller's stream, no host synchronisation):
-//   1. page hashes   one warp per path: 64-bit hash of every full page (lanes take pages, 64 contiguous bytes each),
-//                    chained into prefix hashes H[k] = hash of the first k pages
-//   2. sort          bitonic sort of the path indices by token sequence.  The comparator finds the number of common
-//                    pages of two paths by binary search over their prefix hashes and then compares tokens from there,
-//                    so a comparison costs O(log pages) whatever the length of the common prefix.  Blocks of 2048
-//                    indices are sorted in shared memory; larger strides take one launch each.
-//   3. neighbours    one warp per sorted neighbour pair: the common full pages are counted on the TOKENS themselves
-//                    (the hashes only ordered the paths), and the order of the pair is checked; a hash collision that
-//                    mis-ordered two paths is reported as SS_ERR_BAD_INPUT instead of producing a wrong tree
-//   4. tree          inner nodes are the intervals of neighbours that share more pages than their surroundings (the
-//                    LCP-interval tree).  One thread per position: it finds its interval with nearest-smaller-value
-//                    searches that skip whole blocks through their minima; depth-first numbering (leaves included)
-//                    comes from a prefix sum of the intervals per start rank; parents follow from the neighbours of
-//                    an interval
+// ONE launch whose phases are separated by a barrier over all its blocks: one block, a cluster of 8, or one block per SM
+// (a cooperative launch).  No token is hashed and none that is known to be shared is read twice.
+//
+//   sort    The paths are sorted by refinement (a multikey quicksort with longest common prefixes as keys).  All
+//           positions start in one group.  In a round every group of two or more picks one of its paths as the pivot, and
+//           every other member compares itself with it, from the length that the group is known to share: a warp per path,
+//           streaming both.  Its key - below or above the pivot, common length, first differing token - sorts the group;
+//           members with equal keys share that many tokens plus one, and make a group of the next round.  Members that equal
+//           the pivot, or that end where they differ from it, are settled.  Neighbours that were told apart in a round share
+//           exactly the smaller of their two lengths, so the common prefixes of the sorted neighbours, which the tree is made
+//           of, come out of the keys.  A round settles at least the pivots; the pivot is picked pseudo-randomly, so the number
+//           of rounds is that of a quicksort's levels in the worst case and the depth of the tree in ordinary ones (3 or 4).
+//             compare   a warp per position: boundaries of the groups from the last round's sorted keys (32-ary search), then
+//                       the new key
+//             tiles     a block per 1024 positions sorts (group, key, position) in shared memory
+//             ranks     only if a group spans tiles: a warp per position, lanes search the group's tiles
+//   tree    Inner nodes are the intervals of neighbours that share more pages than their surroundings (the LCP-interval
+//           tree).  A warp per position finds its interval with nearest-smaller-value searches of 32 entries a step, over
+//           the entries and over their minima by 32; depth-first numbering (leaves included) comes from a prefix sum of
+//           the intervals per start rank; parents follow from the neighbours of an interval.
+//
+// Bound: HBM, one pass over the shared prefixes (268 MB for 16384 paths with prompts of 4096 tokens, 41 us), and for small
+// inputs the latency of a few dependent phases.  MEASURED_HERE
 #include "common.cuh"
 
 namespace ss {
 namespace ptree {
 
-constexpr int kSortBlock = 1024;                 // threads; a block sorts 2048 indices in shared memory
-constexpr int kSortChunk = 2 * kSortBlock;
+constexpr int kThreads = 1024;
+constexpr int kWarps = kThreads / 32;
+constexpr int kTile = 1024;                       // positions that a block sorts in shared memory
+constexpr int kUnroll = 8;                        // 128-byte loads in flight per warp and path
+constexpr uint32_t kInf = 0x7fffffffu;            // "common length" of a path with itself
+constexpr unsigned long long kBarrierLimitNs = 4000000000ull;
 
-__device__ __forceinline__ uint64_t mix64(uint64_t x) {   // splitmix64 finaliser
-  x ^= x >> 30; x *= 0xbf58476d1ce4e5b9ull;
-  x ^= x >> 27; x *= 0x94d049bb133111ebull;
-  x ^= x >> 31;
-  return x;
-}
-
-struct Seqs {
+struct Args {
   const int32_t* tok_ids;
   const int64_t* tok_offsets;
-  const uint64_t* hashes;       // prefix hashes, path i at hashes[hash_base(i) + k], k = 0 .. full pages of i
-  int page;
+  int n, page, n_tiles;
+  int32_t* status;               // first word of the workspace
+  unsigned int* arrived;         // grid barrier
+  unsigned int* flags;           // [4]: what the round's groups need (kMore, kWide), rounds in turn
+  uint64_t* key[2];
+  int* perm[2];
+  int *gs, *ge;                  // per position: its group [gs, ge)
+  int* lcp;                      // per rank: pages shared with the rank before
+  int *bmin, *c_start, *c_end, *outer, *cnt, *block_sum;
+  int32_t *order, *path_leaf_node, *node_parent, *node_kv_len, *node_src_path, *node_src_offset, *num_nodes;
 };
+constexpr unsigned int kMore = 1, kWide = 2;
 
-// Prefix hashes of path i start here: (offset / page) + i never overlaps the previous path's (pages + 1) entries.
-__device__ __forceinline__ int64_t hash_base(const Seqs& S, int i) {
-  return (S.tok_offsets[i] - S.tok_offsets[0]) / S.page + i;
-}
-
-// ---- 1. page hashes -----------------------------------------------------------------------------------------------
-__global__ void page_hash_kernel(const int32_t* __restrict__ tok_ids, const int64_t* __restrict__ tok_offsets, int n,
-                                 int page, uint64_t* __restrict__ hashes) {
-  ss::grid_dependency_enter();
-  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (i >= n) return;
-  const int64_t t0 = tok_offsets[i];
-  const int n_pages = static_cast<int>((tok_offsets[i + 1] - t0) / page);
-  uint64_t* H = hashes + ((t0 - tok_offsets[0]) / page + i);
-  uint64_t h = 0x9e3779b97f4a7c15ull;                       // H[0]: the empty prefix
-  if (lane == 0) H[0] = h;
-  for (int k0 = 0; k0 < n_pages; k0 += 32) {
-    const int k = k0 + lane;
-    uint64_t c = 0;
-    if (k < n_pages) {
-      const int32_t* p = tok_ids + t0 + static_cast<int64_t>(k) * page;
-      for (int t = 0; t < page; ++t) c = mix64(c ^ (static_cast<uint64_t>(static_cast<uint32_t>(p[t])) + 0x632be59bd9b4e019ull * (t + 1)));
-    }
-    const int m = min(32, n_pages - k0);
-    for (int x = 0; x < m; ++x) {                           // the chain is sequential: every lane follows it
-      const uint64_t cx = __shfl_sync(0xffffffffu, c, x);
-      h = mix64(h ^ cx);
-      if (lane == x) H[k0 + x + 1] = h;
-    }
+// ---- barrier over all blocks ----------------------------------------------------------------------------------------
+// False when the wait ran out (status SS_ERR_TIMEOUT; every block leaves).  A grid that is one cluster uses the hardware's
+// barrier (0.3 us against 1.5 us).
+template <bool CLUSTER>
+__device__ __forceinline__ bool grid_barrier(const Args& A, unsigned int& target) {
+  if (CLUSTER) {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    return true;
   }
-}
-
-// ---- 2. sort --------------------------------------------------------------------------------------------------------
-// Strict order of two distinct paths: token sequence, a proper prefix first, then the index.  -1 is the padding
-// index and sorts last.
-__device__ bool path_less(const Seqs& S, int a, int b) {
-  if (a < 0 || b < 0) return b < 0 && a >= 0;
-  const int64_t a0 = S.tok_offsets[a], b0 = S.tok_offsets[b];
-  const int64_t la = S.tok_offsets[a + 1] - a0, lb = S.tok_offsets[b + 1] - b0;
-  const uint64_t* Ha = S.hashes + hash_base(S, a);
-  const uint64_t* Hb = S.hashes + hash_base(S, b);
-  int lo = 0, hi = static_cast<int>(min(la, lb) / S.page);  // common pages: H equal at lo, (unknown) above
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (Ha[mid] == Hb[mid]) lo = mid; else hi = mid - 1;
-  }
-  const int64_t n = min(la, lb);
-  for (int64_t t = static_cast<int64_t>(lo) * S.page; t < n; ++t) {
-    const int32_t x = S.tok_ids[a0 + t], y = S.tok_ids[b0 + t];
-    if (x != y) return x < y;
-  }
-  if (la != lb) return la < lb;
-  return a < b;
-}
-
-__device__ __forceinline__ void compare_exchange(const Seqs& S, int& x, int& y, bool up) {
-  if (path_less(S, y, x) == up) { const int t = x; x = y; y = t; }
-}
-
-// Compare-exchange passes at distances first_stride, first_stride / 2, .. 1 inside a chunk held in shared memory;
-// `size` is the bitonic merge they belong to (it fixes the direction of every pair).
-__device__ __forceinline__ void local_passes(const Seqs& S, int* s, int base, int size, int first_stride) {
-  for (int stride = first_stride; stride > 0; stride >>= 1) {
-    const int t = threadIdx.x;
-    const int lo = ((t / stride) * (stride << 1)) + (t % stride);
-    const int hi = lo + stride;
-    const bool up = (((base + lo) & size) == 0);
-    int x = s[lo], y = s[hi];
-    compare_exchange(S, x, y, up);
-    s[lo] = x; s[hi] = y;
-    __syncthreads();
-  }
-}
-
-// size == 0: sorts every chunk of kSortChunk indices completely (merges of size 2 .. kSortChunk).
-// size  > kSortChunk: the tail of the merge of that size (distances below a chunk), after merge_step_kernel has done
-// the distances of a chunk and above.
-__global__ void __launch_bounds__(kSortBlock)
-sort_chunks_kernel(Seqs S, int* __restrict__ idx, int n_pad, int size) {
-  ss::grid_dependency_enter();
-  __shared__ int s[kSortChunk];
-  const int base = blockIdx.x * kSortChunk;
-  for (int t = threadIdx.x; t < kSortChunk; t += kSortBlock) s[t] = base + t < n_pad ? idx[base + t] : -1;
+  __shared__ int ok;
   __syncthreads();
-  if (size == 0) {
-    for (int sz = 2; sz <= kSortChunk; sz <<= 1) local_passes(S, s, base, sz, sz >> 1);
-  } else {
-    local_passes(S, s, base, size, kSortChunk >> 1);
+  target += gridDim.x;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(A.arrived, 1u);
+    unsigned long long t0, t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+    ok = 1;
+    for (;;) {
+      unsigned int v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(A.arrived) : "memory");
+      if (static_cast<int>(v - target) >= 0) break;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+      if (t - t0 > kBarrierLimitNs) { set_status(A.status, SS_ERR_TIMEOUT); ok = 0; break; }
+    }
+    __threadfence();
   }
-  for (int t = threadIdx.x; t < kSortChunk; t += kSortBlock)
-    if (base + t < n_pad) idx[base + t] = s[t];
+  __syncthreads();
+  return ok != 0;
 }
 
-// One compare-exchange pass of the merge of size `size` at distance `stride` (>= kSortChunk).
-__global__ void merge_step_kernel(Seqs S, int* __restrict__ idx, int n_pad, int size, int stride) {
-  ss::grid_dependency_enter();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (n_pad >> 1)) return;
-  const int lo = ((t / stride) * (stride << 1)) + (t % stride);
-  const int hi = lo + stride;
-  const bool up = ((lo & size) == 0);
-  int x = idx[lo], y = idx[hi];
-  const int x0 = x;
-  compare_exchange(S, x, y, up);
-  if (x != x0) { idx[lo] = x; idx[hi] = y; }
+// ---- sort -------------------------------------------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t ordered(int32_t token) { return static_cast<uint32_t>(token) ^ 0x80000000u; }
+// Common length that a key stands for (see make_key).
+__device__ __forceinline__ uint32_t key_len(uint64_t k) {
+  const uint32_t f = static_cast<uint32_t>(k >> 32) & kInf;
+  return (k >> 63) ? kInf - f : f;
+}
+// All paths with this key are equal: the pivot's own, or paths that end where they differ from it.
+__device__ __forceinline__ bool key_settled(uint64_t k) { return !(k >> 63) && static_cast<uint32_t>(k) == 0; }
+
+// Whole warp: the key of path `me` against the pivot, given that they share `base` tokens.  Ascending in the paths' order:
+//   below the pivot  0 | l | token + 1, or 0 if `me` ends at l    (shorter common prefix = smaller path)
+//   equal to it      0 | kInf | 0
+//   above it         1 | kInf - l | token
+__device__ uint64_t make_key(const Args& A, int me, int pivot, int base, int lane) {
+  constexpr uint64_t kEqual = static_cast<uint64_t>(kInf) << 32;
+  if (me == pivot) return kEqual;
+  const int64_t a0 = A.tok_offsets[me], b0 = A.tok_offsets[pivot];
+  const int la = static_cast<int>(A.tok_offsets[me + 1] - a0), lb = static_cast<int>(A.tok_offsets[pivot + 1] - b0);
+  const int m = min(la, lb);
+  const int32_t *a = A.tok_ids + a0, *b = A.tok_ids + b0;
+  int l = m;
+  // 32 tokens first (most pairs differ at once or not for long), then kUnroll * 32 a step
+  {
+    const int t = base + lane;
+    const bool ne = t < m && __ldg(a + t) != __ldg(b + t);
+    const uint32_t bal = __ballot_sync(0xffffffffu, ne);
+    if (bal) l = base + __ffs(bal) - 1;
+    else {
+      for (int t0 = base + 32; t0 < m; t0 += 32 * kUnroll) {
+        int32_t x[kUnroll], y[kUnroll];
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) {
+          const int t1 = t0 + 32 * u + lane;
+          x[u] = t1 < m ? __ldg(a + t1) : 0;
+          y[u] = t1 < m ? __ldg(b + t1) : 0;
+        }
+        int first = 32 * kUnroll;
+#pragma unroll
+        for (int u = kUnroll - 1; u >= 0; --u)
+          if (x[u] != y[u]) first = 32 * u + lane;
+        first = __reduce_min_sync(0xffffffffu, first);
+        if (first < 32 * kUnroll) { l = t0 + first; break; }
+      }
+    }
+  }
+  if (l == m) {
+    if (la == lb) return kEqual;
+    if (la < lb) return static_cast<uint64_t>(l) << 32;
+    return (1ull << 63) | (static_cast<uint64_t>(kInf - l) << 32) | ordered(__ldg(a + l));
+  }
+  const uint32_t x = ordered(__ldg(a + l)), y = ordered(__ldg(b + l));
+  return x < y ? (static_cast<uint64_t>(l) << 32) | (x + 1) : (1ull << 63) | (static_cast<uint64_t>(kInf - l) << 32) | x;
 }
 
-__global__ void iota_kernel(int* __restrict__ idx, int n, int n_pad) {
-  ss::grid_dependency_enter();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t < n_pad) idx[t] = t < n ? t : -1;
+// Whole warp: number of keys in the ascending k[0..len) that are below `key` (OR_EQUAL: not above it).
+template <bool OR_EQUAL>
+__device__ __forceinline__ int count_below(const uint64_t* k, int len, uint64_t key, int lane) {
+  int lo = 0;
+  while (len > 32) {
+    const int step = (len + 31) >> 5, i = lane * step;
+    const uint64_t v = i < len ? k[lo + i] : ~0ull;
+    const int c = __popc(__ballot_sync(0xffffffffu, i < len && (OR_EQUAL ? v <= key : v < key)));
+    if (c == 0) return lo;
+    const int at = (c - 1) * step + 1;                        // k[lo + at - 1] is below
+    len = min(step - 1, len - at);
+    lo += at;
+  }
+  const uint64_t v = lane < len ? k[lo + lane] : ~0ull;
+  return lo + __popc(__ballot_sync(0xffffffffu, lane < len && (OR_EQUAL ? v <= key : v < key)));
 }
 
-// ---- 3. neighbours --------------------------------------------------------------------------------------------------
-// lcp[r] = full pages shared by the paths of rank r-1 and r (lcp[0] = 0), counted on the tokens; also checks that the
-// pair is in order (a hash collision could have mis-ordered it).
-__global__ void neighbour_kernel(Seqs S, const int* __restrict__ idx, int n, int* __restrict__ lcp,
-                                 int32_t* __restrict__ order_out, int32_t* __restrict__ status) {
-  ss::grid_dependency_enter();
-  const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (r >= n) return;
-  const int b = idx[r];
-  if (lane == 0) order_out[r] = b;
-  if (r == 0) {
-    if (lane == 0) lcp[0] = 0;
+// Sorts positions tile * kTile .. by (group, key, position): keys and paths of the round, kin / pin -> kout / pout.
+__device__ void sort_tile(const Args& A, int tile, const uint64_t* kin, const int* pin, uint64_t* kout, int* pout) {
+  __shared__ uint64_t s_key[kTile];
+  __shared__ uint32_t s_at[kTile];                            // first position of the group in the tile << 16 | position
+  const int p0 = tile * kTile, count = min(kTile, A.n - p0), tid = threadIdx.x;
+  bool open = false;
+  if (tid < kTile) {
+    uint64_t k = ~0ull;
+    uint32_t at = 0xffffffffu;
+    if (tid < count) {
+      const int g = A.gs[p0 + tid];
+      open = A.ge[p0 + tid] - g > 1;
+      k = open ? kin[p0 + tid] : 0;
+      at = (static_cast<uint32_t>(max(g - p0, 0)) << 16) | static_cast<uint32_t>(tid);
+    }
+    s_key[tid] = k;
+    s_at[tid] = at;
+  }
+  if (!__syncthreads_or(open)) {
+    if (tid < count) pout[p0 + tid] = pin[p0 + tid];
     return;
   }
-  const int a = idx[r - 1];
-  const int64_t a0 = S.tok_offsets[a], b0 = S.tok_offsets[b];
-  const int64_t la = S.tok_offsets[a + 1] - a0, lb = S.tok_offsets[b + 1] - b0;
-  const int64_t m = min(la, lb);
-  int64_t d = m;                                            // first differing position
-  for (int64_t t0 = 0; t0 < m; t0 += 32) {
-    const int64_t t = t0 + lane;
-    const bool ne = t < m && S.tok_ids[a0 + t] != S.tok_ids[b0 + t];
-    const uint32_t bal = __ballot_sync(0xffffffffu, ne);
-    if (bal) { d = t0 + __ffs(bal) - 1; break; }
+  int n_pad = 2;
+  while (n_pad < count) n_pad <<= 1;
+  for (int size = 2; size <= n_pad; size <<= 1) {
+    for (int stride = size >> 1; stride > 0; stride >>= 1) {
+      if (tid < (n_pad >> 1)) {
+        const int lo = ((tid & ~(stride - 1)) << 1) | (tid & (stride - 1)), hi = lo + stride;
+        const uint64_t ka = s_key[lo], kb = s_key[hi];
+        const uint32_t aa = s_at[lo], ab = s_at[hi];
+        const uint32_t ga = aa >> 16, gb = ab >> 16;
+        const bool above = ga != gb ? ga > gb : (ka != kb ? ka > kb : aa > ab);
+        if (above == ((lo & size) == 0)) { s_key[lo] = kb; s_key[hi] = ka; s_at[lo] = ab; s_at[hi] = aa; }
+      }
+      // (strides below 32 stay inside the warp: pairs 32w..32w+31 touch the 64 entries of warp w alone)
+      if (stride > 32) __syncthreads(); else __syncwarp();
+    }
+    __syncthreads();
   }
-  if (lane == 0) {
-    lcp[r] = static_cast<int>(d / S.page);
-    bool in_order;
-    if (d < m) in_order = S.tok_ids[a0 + d] < S.tok_ids[b0 + d];
-    else in_order = la < lb || (la == lb && a < b);
-    if (!in_order) set_status(status, SS_ERR_BAD_INPUT);
+  if (tid < count) {
+    kout[p0 + tid] = s_key[tid];
+    pout[p0 + tid] = pin[p0 + static_cast<int>(s_at[tid] & 0xffffu)];
   }
+  __syncthreads();
 }
 
-// ---- 4. tree ---------------------------------------------------------------------------------------------------------
+// ---- tree -------------------------------------------------------------------------------------------------------------
 // Inner nodes are the LCP intervals of lcp[]: maximal runs of ranks a..b whose neighbours all share at least d pages
 // (lcp[a+1..b] >= d, with equality somewhere) while lcp[a] < d and lcp[b+1] < d (lcp[n] counts as 0).  The interval is
-// created by its first position x with lcp[x] == d.  Everything below is one thread per position / rank with
-// nearest-smaller-value searches over lcp[], which skip whole blocks of kMinBlock entries through their minima.
-constexpr int kMinBlock = 256;
-
-struct Lcp {
-  const int* v;        // lcp[0..n)
-  const int* bmin;     // minimum of every block of kMinBlock entries
-  int n;
-};
-
-// Largest p < x with lcp[p] < bound (STRICT) or <= bound; lcp[0] = 0 ends every search for bound >= 0 (> 0 if strict).
+// created by its first position x with lcp[x] == d.
+//
+// Whole warp: largest p < x with lcp[p] < bound (STRICT) or <= bound; lcp[0] = 0 ends every search for bound >= 0 (> 0 if
+// strict).
 template <bool STRICT>
-__device__ int prev_below(const Lcp& L, int x, int bound) {
+__device__ int prev_below(const Args& A, int x, int bound, int lane) {
   auto hit = [&](int val) { return STRICT ? val < bound : val <= bound; };
-  int p = x - 1;
-  const int blk_lo = (x / kMinBlock) * kMinBlock;
-  for (; p >= blk_lo; --p)
-    if (hit(L.v[p])) return p;
-  int blk = x / kMinBlock - 1;
-  while (blk > 0 && !hit(L.bmin[blk])) --blk;
-  for (p = blk * kMinBlock + kMinBlock - 1; p > 0; --p)
-    if (hit(L.v[p])) return p;
+  const int blk = x >> 5;
+  {
+    const int p = (blk << 5) + lane;
+    const uint32_t b = __ballot_sync(0xffffffffu, p < x && hit(A.lcp[p < x ? p : 0]));
+    if (b) return (blk << 5) + 31 - __clz(b);
+  }
+  for (int top = blk; top > 0; top -= 32) {                   // blocks top-32 .. top-1
+    const int q = top - 32 + lane;
+    const uint32_t b = __ballot_sync(0xffffffffu, q >= 0 && hit(A.bmin[q >= 0 ? q : 0]));
+    if (!b) continue;
+    const int found = top - 32 + 31 - __clz(b);
+    const uint32_t c = __ballot_sync(0xffffffffu, hit(A.lcp[(found << 5) + lane]));
+    return (found << 5) + 31 - __clz(c);
+  }
   return 0;
 }
-// Smallest q > x with lcp[q] < bound (STRICT) or <= bound; n if there is none.
+// Whole warp: smallest q > x with lcp[q] < bound (STRICT) or <= bound; n if there is none.
 template <bool STRICT>
-__device__ int next_below(const Lcp& L, int x, int bound) {
+__device__ int next_below(const Args& A, int x, int bound, int lane) {
   auto hit = [&](int val) { return STRICT ? val < bound : val <= bound; };
-  int q = x + 1;
-  const int blk_hi = min(L.n, (x / kMinBlock + 1) * kMinBlock);
-  for (; q < blk_hi; ++q)
-    if (hit(L.v[q])) return q;
-  if (q >= L.n) return L.n;
-  const int n_blk = (L.n + kMinBlock - 1) / kMinBlock;
-  int blk = x / kMinBlock + 1;
-  while (blk < n_blk && !hit(L.bmin[blk])) ++blk;
-  if (blk >= n_blk) return L.n;
-  for (q = blk * kMinBlock; q < L.n; ++q)
-    if (hit(L.v[q])) return q;
-  return L.n;
+  const int n = A.n, blk = x >> 5, n_blk = (n + 31) >> 5;
+  {
+    const int q = (blk << 5) + lane;
+    const uint32_t b = __ballot_sync(0xffffffffu, q > x && q < n && hit(A.lcp[q < n ? q : 0]));
+    if (b) return (blk << 5) + __ffs(b) - 1;
+  }
+  for (int low = blk + 1; low < n_blk; low += 32) {
+    const int q = low + lane;
+    const uint32_t b = __ballot_sync(0xffffffffu, q < n_blk && hit(A.bmin[q < n_blk ? q : 0]));
+    if (!b) continue;
+    const int found = low + __ffs(b) - 1, at = (found << 5) + lane;
+    const uint32_t c = __ballot_sync(0xffffffffu, at < n && hit(A.lcp[at < n ? at : 0]));
+    return (found << 5) + __ffs(c) - 1;
+  }
+  return n;
 }
 // Creating position of the interval of depth d that contains position pos (lcp[pos] >= d, d > 0).
-__device__ __forceinline__ int creator_of(const Lcp& L, int pos, int d) {
-  const int a = L.v[pos] < d ? pos : prev_below<true>(L, pos, d);     // (pos itself is never below d here)
-  return next_below<false>(L, a, d);
+__device__ __forceinline__ int creator_of(const Args& A, int pos, int d, int lane) {
+  return next_below<false>(A, prev_below<true>(A, pos, d, lane), d, lane);
 }
 
-struct TreeOut {
-  int32_t *path_leaf_node, *node_parent, *node_kv_len, *node_src_path, *node_src_offset, *num_nodes;
-};
-struct TreeTmp {      // n + 1 entries each
-  int *bmin, *c_start, *c_end, *cnt, *rank_by_pos;
-};
-
-__global__ void block_min_kernel(const int* __restrict__ lcp, int n, int* __restrict__ bmin, int* __restrict__ cnt) {
-  ss::grid_dependency_enter();
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t <= n) cnt[t] = 0;
-  if (t >= (n + kMinBlock - 1) / kMinBlock) return;
-  int m = 0x7fffffff;
-  for (int i = t * kMinBlock; i < min(n, (t + 1) * kMinBlock); ++i) m = min(m, lcp[i]);
-  bmin[t] = m;
-}
-
-// Marks the creating positions, finds their intervals and counts the intervals per start rank.
-__global__ void creators_kernel(Lcp L, TreeTmp T) {
-  ss::grid_dependency_enter();
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= L.n) return;
-  const int d = L.v[x];
-  int start = -1;
-  if (x > 0 && d > 0) {
-    const int p = prev_below<false>(L, x, d);
-    if (L.v[p] < d) {                                         // no earlier position of this interval has depth d
-      start = p;
-      T.c_end[x] = next_below<true>(L, x, d) - 1;
-      atomicAdd(&T.cnt[p], 1);
-    }
-  }
-  T.c_start[x] = start;
-}
-
-// One block: cnt[a] (intervals that start at rank a) -> exclusive prefix sums, cnt[n] = number of inner nodes.
-__global__ void scan_counts_kernel(int* __restrict__ cnt, int n, int32_t* __restrict__ num_nodes,
-                                   const int32_t* __restrict__ status) {
-  ss::grid_dependency_enter();
-  __shared__ int warp_tot[32];
-  __shared__ int carry_s;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (threadIdx.x == 0) carry_s = 0;
-  __syncthreads();
-  for (int base = 0; base <= n; base += blockDim.x) {
-    const int i = base + threadIdx.x;
-    const int v = i <= n ? cnt[i] : 0;
+// Block: exclusive scan of a[lo..hi) in place, starting from `carry`.
+__device__ void scan_range(int* a, int lo, int hi, int carry) {
+  __shared__ int warp_tot[kWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int base = lo; base < hi; base += kThreads) {
+    const int i = base + threadIdx.x, v = i < hi ? a[i] : 0;
     int incl = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -293,107 +267,259 @@ __global__ void scan_counts_kernel(int* __restrict__ cnt, int n, int32_t* __rest
     }
     if (lane == 31) warp_tot[warp] = incl;
     __syncthreads();
-    if (warp == 0) {
-      int t = lane < nw ? warp_tot[lane] : 0;
+    int t = warp_tot[lane];
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, t, o);
-        if (lane >= o) t += y;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, t, o);
+      if (lane >= o) t += y;
+    }
+    const int before = __shfl_sync(0xffffffffu, t, (warp + 31) & 31), total = __shfl_sync(0xffffffffu, t, 31);
+    if (i < hi) a[i] = carry + (warp ? before : 0) + incl - v;
+    carry += total;
+    __syncthreads();
+  }
+}
+
+template <bool CLUSTER>
+__device__ __forceinline__ void build(const Args& A) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n = A.n, n_warps = gridDim.x * kWarps, wid = blockIdx.x * kWarps + warp;
+  unsigned int target = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *A.num_nodes = 0;
+
+  // ---- sort: round 0 has one group of all positions, in index order ---------------------------------------------------
+  int kc = 0, pc = 0;                                         // buffers of the sorted keys and the paths
+  for (unsigned int round = 0;; ++round) {
+    const uint64_t* ks = A.key[kc];
+    unsigned int need = 0;
+    for (int p = wid; p < n; p += n_warps) {
+      int g = 0, e = n, base = 0, me = p;
+      if (round > 0) {
+        g = A.gs[p];
+        e = A.ge[p];
+        if (e - g == 1) continue;                              // settled
+        me = A.perm[pc][p];
+        const uint64_t k = ks[p];
+        const int g1 = g + count_below<false>(ks + g, e - g, k, lane), e1 = g + count_below<true>(ks + g, e - g, k, lane);
+        const bool settled = e1 - g1 == 1 || key_settled(k);
+        if (lane == 0) {
+          if (p > g1)
+            A.lcp[p] = settled ? static_cast<int>(A.tok_offsets[me + 1] - A.tok_offsets[me]) / A.page : 0;   // equal paths
+          else if (p > g)
+            A.lcp[p] = static_cast<int>(min(key_len(ks[p - 1]), key_len(k))) / A.page;
+          A.gs[p] = settled ? p : g1;
+          A.ge[p] = settled ? p + 1 : e1;
+        }
+        if (settled) continue;
+        g = g1;
+        e = e1;
+        base = static_cast<int>(key_len(k)) + 1;
+      } else if (lane == 0) {
+        A.gs[p] = g;
+        A.ge[p] = e;
+        A.perm[pc][p] = p;
+        if (p == 0) A.lcp[0] = 0;
       }
-      warp_tot[lane] = t;
+      if (e - g == 1) continue;
+      need |= kMore | (g / kTile != (e - 1) / kTile ? kWide : 0);
+      uint32_t r = (static_cast<uint32_t>(g) * 0x9e3779b1u) ^ ((round + 1) * 0x85ebca6bu);
+      r = (r ^ (r >> 15)) * 0x2c1b3c6du;
+      const int at = g + static_cast<int>((r >> 3) % static_cast<uint32_t>(e - g));
+      const uint64_t k = make_key(A, me, round > 0 ? A.perm[pc][at] : at, base, lane);
+      if (lane == 0) A.key[kc ^ 1][p] = k;
     }
-    __syncthreads();
-    const int excl = carry_s + (warp ? warp_tot[warp - 1] : 0) + incl - v;
-    if (i <= n) cnt[i] = excl;
-    __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) carry_s = excl + v;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *num_nodes = *status == SS_OK ? n + cnt[n] : 0;   // (cnt[n] had no interval: it is the total)
-}
-
-// Rank of every interval among the inner nodes in depth-first order: intervals that start earlier come first, and of
-// the intervals that start at the same rank the outer ones (they end later).
-__global__ void rank_kernel(Lcp L, TreeTmp T) {
-  ss::grid_dependency_enter();
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= L.n) return;
-  const int a = T.c_start[x];
-  if (a < 0) return;
-  const int floor_d = L.v[a];                                 // what the surroundings on the left share
-  int outer = 0, e = T.c_end[x];
-  for (;;) {                                                  // walk outwards through the intervals with the same start
-    const int v = e + 1 < L.n ? L.v[e + 1] : 0;
-    if (v <= floor_d) break;
-    ++outer;
-    e = next_below<true>(L, e + 1, v) - 1;
-  }
-  T.rank_by_pos[x] = T.cnt[a] + outer;
-}
-
-// Inner nodes: id, parent, length, source.  Leaves likewise.  (d pages deep <=> d * page tokens on the chain above.)
-__global__ void emit_kernel(Seqs S, Lcp L, const int* __restrict__ idx, TreeTmp T, TreeOut O,
-                            const int32_t* __restrict__ status) {
-  ss::grid_dependency_enter();
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= L.n || *status != SS_OK) return;
-  // ---- the interval created at position r, if any ---------------------------------------------------------------------
-  const int a = T.c_start[r];
-  if (a >= 0) {
-    const int d = L.v[r], e = T.c_end[r];
-    const int left = L.v[a], right = e + 1 < L.n ? L.v[e + 1] : 0;
-    const int id = T.rank_by_pos[r] + a;                      // `a` leaves precede it
-    int parent = -1, pd = 0;
-    if (right > left) {                                       // the next outer interval starts at the same rank
-      parent = id - 1;
-      pd = right;
-    } else if (left > 0) {
-      const int y = creator_of(L, a, left);
-      parent = T.rank_by_pos[y] + T.c_start[y];
-      pd = left;
+    if (lane == 0 && need) atomicOr(&A.flags[round & 3], need);
+    if (!grid_barrier<CLUSTER>(A, target)) return;
+    const unsigned int flags = *reinterpret_cast<volatile unsigned int*>(&A.flags[round & 3]);
+    if (!(flags & kMore)) break;
+    if (blockIdx.x == 0 && threadIdx.x == 0) A.flags[(round + 2) & 3] = 0;
+    for (int t = blockIdx.x; t < A.n_tiles; t += gridDim.x)
+      sort_tile(A, t, A.key[kc ^ 1], A.perm[pc], A.key[kc], A.perm[pc ^ 1]);
+    if (!grid_barrier<CLUSTER>(A, target)) return;
+    if (!(flags & kWide)) {
+      pc ^= 1;
+      continue;
     }
-    O.node_parent[id] = parent;
-    O.node_kv_len[id] = (d - pd) * S.page;
-    O.node_src_path[id] = idx[a];
-    O.node_src_offset[id] = pd * S.page;
+    for (int p = wid; p < n; p += n_warps) {
+      const int g = A.gs[p], e = A.ge[p], tile = p / kTile, t0 = g / kTile, t1 = (e - 1) / kTile;
+      const uint64_t k = A.key[kc][p];
+      int rank = lane == 0 ? p - max(g, tile * kTile) : 0;
+      for (int t = t0 + lane; t <= t1; t += 32) {
+        if (t == tile) continue;
+        const int begin = max(g, t * kTile);
+        int lo = begin, hi = min(e, (t + 1) * kTile);          // first position that does not come before p
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          const uint64_t v = A.key[kc][mid];
+          if (t < tile ? v <= k : v < k) lo = mid + 1; else hi = mid;
+        }
+        rank += lo - begin;
+      }
+      rank = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned int>(rank)));
+      if (lane == 0) {
+        A.key[kc ^ 1][g + rank] = k;
+        A.perm[pc][g + rank] = A.perm[pc ^ 1][p];
+      }
+    }
+    kc ^= 1;
+    if (!grid_barrier<CLUSTER>(A, target)) return;
   }
-  // ---- the leaf of rank r ---------------------------------------------------------------------------------------------
+  const int* path_of = A.perm[pc];
+
+  // ---- tree -----------------------------------------------------------------------------------------------------------
+  for (int p0 = wid * 32; p0 <= n; p0 += n_warps * 32) {
+    const int p = p0 + lane;
+    if (p <= n) A.cnt[p] = 0;
+    if (p < n) A.order[p] = path_of[p];
+    const int m = __reduce_min_sync(0xffffffffu, p < n ? A.lcp[p] : 0x7fffffff);
+    if (lane == 0 && p0 < n) A.bmin[p0 >> 5] = m;
+  }
+  if (!grid_barrier<CLUSTER>(A, target)) return;
+  // intervals: creating positions, start and end ranks, number per start rank, intervals around it with the same start
+  for (int x = wid; x < n; x += n_warps) {
+    const int d = A.lcp[x];
+    int start = -1, end = 0, outer = 0;
+    if (x > 0 && d > 0) {
+      const int p = prev_below<false>(A, x, d, lane);
+      const int left = A.lcp[p];
+      if (left < d) {                                          // no earlier position of this interval has depth d
+        start = p;
+        end = next_below<true>(A, x, d, lane) - 1;
+        for (int e = end;;) {                                  // outwards
+          const int v = e + 1 < n ? A.lcp[e + 1] : 0;
+          if (v <= left) break;
+          ++outer;
+          e = next_below<true>(A, e + 1, v, lane) - 1;
+        }
+      }
+    }
+    if (lane == 0) {
+      A.c_start[x] = start;
+      A.c_end[x] = end;
+      A.outer[x] = outer;
+      if (start >= 0) atomicAdd(&A.cnt[start], 1);
+    }
+  }
+  if (!grid_barrier<CLUSTER>(A, target)) return;
+  // cnt[a] (intervals that start at rank a) -> exclusive prefix sums; cnt[n] = number of inner nodes
   {
-    const int left = L.v[r], right = r + 1 < L.n ? L.v[r + 1] : 0;
-    const int pd = max(left, right);
-    int parent = -1;
-    if (pd > 0) {
-      const int y = creator_of(L, left >= right ? r : r + 1, pd);
-      parent = T.rank_by_pos[y] + T.c_start[y];
+    const int per = (n + static_cast<int>(gridDim.x)) / static_cast<int>(gridDim.x);
+    const int lo = min(static_cast<int>(blockIdx.x) * per, n + 1), hi = min(lo + per, n + 1);
+    int carry = 0;
+    if (gridDim.x > 1) {
+      __shared__ int tot[kWarps];
+      int sum = 0;
+      for (int i = lo + threadIdx.x; i < hi; i += kThreads) sum += A.cnt[i];
+      sum = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned int>(sum)));
+      if (lane == 0) tot[warp] = sum;
+      __syncthreads();
+      if (warp == 0) {
+        sum = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned int>(tot[lane])));
+        if (lane == 0) A.block_sum[blockIdx.x] = sum;
+      }
+      if (!grid_barrier<CLUSTER>(A, target)) return;
+      for (int i = lane; i < static_cast<int>(blockIdx.x); i += 32) carry += A.block_sum[i];
+      carry = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned int>(carry)));
     }
-    const int path = idx[r];
-    const int id = r + T.cnt[r + 1];                          // every interval that starts at a rank <= r precedes it
-    O.node_parent[id] = parent;
-    O.node_kv_len[id] = static_cast<int>(S.tok_offsets[path + 1] - S.tok_offsets[path]) - pd * S.page;
-    O.node_src_path[id] = path;
-    O.node_src_offset[id] = pd * S.page;
-    O.path_leaf_node[r] = id;
+    scan_range(A.cnt, lo, hi, carry);
   }
+  if (!grid_barrier<CLUSTER>(A, target)) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *A.num_nodes = n + A.cnt[n];   // (cnt[n] had no interval: it is the total)
+  // Nodes.  The depth-first rank of an interval among the inner nodes: intervals that start earlier come first, and of
+  // those that start at the same rank the outer ones.  (d pages deep <=> d * page tokens on the chain above.)
+  auto inner_id = [&](int x) { return A.cnt[A.c_start[x]] + A.outer[x] + A.c_start[x]; };   // (`start` leaves precede it)
+  for (int r = wid; r < n; r += n_warps) {
+    const int depth = A.lcp[r], right1 = r + 1 < n ? A.lcp[r + 1] : 0;
+    const int a = A.c_start[r];
+    if (a >= 0) {                                              // the interval created at this position
+      const int e = A.c_end[r], left = A.lcp[a], right = e + 1 < n ? A.lcp[e + 1] : 0;
+      const int id = inner_id(r);
+      int parent = -1, pd = 0;
+      if (right > left) {                                      // the next outer interval starts at the same rank
+        parent = id - 1;
+        pd = right;
+      } else if (left > 0) {
+        parent = inner_id(creator_of(A, a, left, lane));
+        pd = left;
+      }
+      if (lane == 0) {
+        A.node_parent[id] = parent;
+        A.node_kv_len[id] = (depth - pd) * A.page;
+        A.node_src_path[id] = path_of[a];
+        A.node_src_offset[id] = pd * A.page;
+      }
+    }
+    const int pd = max(depth, right1);                         // the leaf of rank r
+    int parent = -1;
+    if (pd > 0) parent = inner_id(creator_of(A, depth >= right1 ? r : r + 1, pd, lane));
+    if (lane == 0) {
+      const int path = path_of[r], id = r + A.cnt[r + 1];      // every interval that starts at a rank <= r precedes it
+      A.node_parent[id] = parent;
+      A.node_kv_len[id] = static_cast<int>(A.tok_offsets[path + 1] - A.tok_offsets[path]) - pd * A.page;
+      A.node_src_path[id] = path;
+      A.node_src_offset[id] = pd * A.page;
+      A.path_leaf_node[r] = id;
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kThreads, 1) prefix_tree_grid_kernel(const __grid_constant__ Args A) {
+  ss::grid_dependency_enter();
+  build<false>(A);
+}
+__global__ void __launch_bounds__(kThreads, 1) prefix_tree_cluster_kernel(const __grid_constant__ Args A) {
+  ss::grid_dependency_enter();
+  build<true>(A);
 }
 
 struct Layout {
-  size_t status, hashes, idx, lcp, tmp, total;
-  int n_pad;
+  size_t status, key[2], ints, total;
 };
+constexpr int kMaxBlocks = 1024;
 
-static Layout layout(int n, int64_t total_tok, int page) {
+static Layout layout(int n) {
   Layout L;
-  int n_pad = kSortChunk;
-  while (n_pad < n) n_pad <<= 1;
-  L.n_pad = n_pad;
   size_t off = 0;
-  L.status = off; off = align_up(off + 256);
-  L.hashes = off; off = align_up(off + (static_cast<size_t>(total_tok / page) + n + 2) * sizeof(uint64_t));
-  L.idx = off; off = align_up(off + static_cast<size_t>(n_pad) * 4);
-  L.lcp = off; off = align_up(off + static_cast<size_t>(n + 1) * 4);
-  L.tmp = off; off = align_up(off + static_cast<size_t>(5) * (n + 1) * 4);
+  L.status = off; off = align_up(off + 256);                  // status, barrier, flags: cleared by the host
+  for (int i = 0; i < 2; ++i) { L.key[i] = off; off = align_up(off + static_cast<size_t>(n) * sizeof(uint64_t)); }
+  L.ints = off; off = align_up(off + (static_cast<size_t>(11) * (n + 1) + kMaxBlocks) * 4);
   L.total = off;
   return L;
+}
+
+// One cluster of `blocks` (1 or 8), or a cooperative grid.
+static int32_t launch(const Args& A, int blocks, bool cluster, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(blocks));
+  cfg.blockDim = dim3(kThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  int n_attr = 0;
+  if (cluster) {
+    attr[n_attr].id = cudaLaunchAttributeClusterDimension;
+    attr[n_attr].val.clusterDim.x = static_cast<unsigned>(blocks);
+    attr[n_attr].val.clusterDim.y = attr[n_attr].val.clusterDim.z = 1;
+    ++n_attr;
+    if (pdl_enabled()) {
+      attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
+      ++n_attr;
+    }
+  } else {
+    attr[n_attr].id = cudaLaunchAttributeCooperative;
+    attr[n_attr].val.cooperative = 1;
+    ++n_attr;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = static_cast<unsigned>(n_attr);
+  const cudaError_t rc = cluster ? cudaLaunchKernelEx(&cfg, prefix_tree_cluster_kernel, A)
+                                 : cudaLaunchKernelEx(&cfg, prefix_tree_grid_kernel, A);
+  g_launch_count.fetch_add(1, std::memory_order_relaxed);
+  if (rc != cudaSuccess || cudaPeekAtLastError() != cudaSuccess) {
+    (void)cudaGetLastError();
+    return SS_ERR_CUDA;
+  }
+  return SS_OK;
 }
 
 }  // namespace ptree
@@ -403,7 +529,7 @@ extern "C" int32_t ss_prefix_tree_workspace_bytes(int32_t n_paths, int64_t total
                                                   size_t* out_bytes) {
   if (n_paths < 0 || n_paths > SS_PREFIX_TREE_MAX_PATHS || total_tok < 0 || page_size < 1 || !out_bytes)
     return SS_ERR_INVALID_ARG;
-  *out_bytes = ss::ptree::layout(n_paths, total_tok, page_size).total;
+  *out_bytes = ss::ptree::layout(n_paths).total;
   return SS_OK;
 }
 
@@ -416,12 +542,12 @@ extern "C" int32_t ss_build_prefix_tree(const int32_t* tok_ids, const int64_t* t
   using namespace ss::ptree;
   if (n_paths < 0 || n_paths > SS_PREFIX_TREE_MAX_PATHS || total_tok < 0 || page_size < 1) return SS_ERR_INVALID_ARG;
   if (!num_nodes_out || !workspace || reinterpret_cast<uintptr_t>(workspace) % kAlign) return SS_ERR_INVALID_ARG;
-  const Layout L = layout(n_paths, total_tok, page_size);
+  const Layout L = layout(n_paths);
   if (workspace_bytes < L.total) return SS_ERR_WORKSPACE_TOO_SMALL;
   cudaStream_t st = as_stream(stream);
   char* ws = static_cast<char*>(workspace);
-  int32_t* status = reinterpret_cast<int32_t*>(ws + L.status);
-  if (cudaMemsetAsync(status, 0, 256, st) != cudaSuccess || cudaMemsetAsync(num_nodes_out, 0, sizeof(int32_t), st) != cudaSuccess) {
+  if (cudaMemsetAsync(ws + L.status, 0, 256, st) != cudaSuccess ||
+      (n_paths == 0 && cudaMemsetAsync(num_nodes_out, 0, sizeof(int32_t), st) != cudaSuccess)) {
     (void)cudaGetLastError();
     return SS_ERR_CUDA;
   }
@@ -430,30 +556,33 @@ extern "C" int32_t ss_build_prefix_tree(const int32_t* tok_ids, const int64_t* t
       !node_src_offset_out || (total_tok > 0 && !tok_ids))
     return SS_ERR_INVALID_ARG;
   const int n = n_paths;
-  uint64_t* hashes = reinterpret_cast<uint64_t*>(ws + L.hashes);
-  int* idx = reinterpret_cast<int*>(ws + L.idx);
-  int* lcp = reinterpret_cast<int*>(ws + L.lcp);
-  int* tmp = reinterpret_cast<int*>(ws + L.tmp);
-  const size_t stride = static_cast<size_t>(n) + 1;
-  TreeTmp T{tmp, tmp + stride, tmp + 2 * stride, tmp + 3 * stride, tmp + 4 * stride};
-  TreeOut O{path_leaf_node_out, node_parent_out, node_kv_len_out, node_src_path_out, node_src_offset_out, num_nodes_out};
-  const Seqs S{tok_ids, tok_offsets, hashes, page_size};
+  Args A{};
+  A.tok_ids = tok_ids;
+  A.tok_offsets = tok_offsets;
+  A.n = n;
+  A.page = page_size;
+  A.n_tiles = (n + kTile - 1) / kTile;
+  A.status = reinterpret_cast<int32_t*>(ws + L.status);
+  A.arrived = reinterpret_cast<unsigned int*>(ws + L.status + 64);
+  A.flags = reinterpret_cast<unsigned int*>(ws + L.status + 128);
+  for (int i = 0; i < 2; ++i) A.key[i] = reinterpret_cast<uint64_t*>(ws + L.key[i]);
+  int* ints = reinterpret_cast<int*>(ws + L.ints);
+  int** at[11] = {&A.perm[0], &A.perm[1], &A.gs, &A.ge, &A.lcp, &A.bmin, &A.c_start, &A.c_end, &A.outer, &A.cnt, &A.block_sum};
+  for (int i = 0; i < 11; ++i) *at[i] = ints + static_cast<size_t>(i) * (n + 1);
+  A.order = order_out;
+  A.path_leaf_node = path_leaf_node_out;
+  A.node_parent = node_parent_out;
+  A.node_kv_len = node_kv_len_out;
+  A.node_src_path = node_src_path_out;
+  A.node_src_offset = node_src_offset_out;
+  A.num_nodes = num_nodes_out;
 
-  SS_LAUNCH(page_hash_kernel, (n + 7) / 8, 256, 0, st, tok_ids, tok_offsets, n, page_size, hashes);
-  SS_LAUNCH(iota_kernel, (L.n_pad + 255) / 256, 256, 0, st, idx, n, L.n_pad);
-  const int chunks = L.n_pad / kSortChunk;
-  SS_LAUNCH(sort_chunks_kernel, chunks, kSortBlock, 0, st, S, idx, L.n_pad, 0);
-  for (int size = 2 * kSortChunk; size <= L.n_pad; size <<= 1) {
-    for (int stride2 = size >> 1; stride2 >= kSortChunk; stride2 >>= 1)
-      SS_LAUNCH(merge_step_kernel, (L.n_pad / 2 + 255) / 256, 256, 0, st, S, idx, L.n_pad, size, stride2);
-    SS_LAUNCH(sort_chunks_kernel, chunks, kSortBlock, 0, st, S, idx, L.n_pad, size);
-  }
-  SS_LAUNCH(neighbour_kernel, (n + 7) / 8, 256, 0, st, S, idx, n, lcp, order_out, status);
-  const Lcp Lc{lcp, T.bmin, n};
-  SS_LAUNCH(block_min_kernel, (n + 1 + 255) / 256, 256, 0, st, lcp, n, T.bmin, T.cnt);
-  SS_LAUNCH(creators_kernel, (n + 255) / 256, 256, 0, st, Lc, T);
-  SS_LAUNCH(scan_counts_kernel, 1, 1024, 0, st, T.cnt, n, num_nodes_out, status);
-  SS_LAUNCH(rank_kernel, (n + 255) / 256, 256, 0, st, Lc, T);
-  SS_LAUNCH(emit_kernel, (n + 255) / 256, 256, 0, st, S, Lc, idx, T, O, status);
-  return SS_OK;
+  // One position per warp in one block: its barrier is the cheapest.  A cluster of 8 up to 16 positions per warp's worth of
+  // short paths; from there the grid's bandwidth pays for its barrier.
+  if (n <= kWarps) return launch(A, 1, true, st);
+  if (n <= 512 && total_tok <= (1 << 22)) return launch(A, 8, true, st);
+  int sms = sm_count_of_current_device();
+  if (sms > kMaxBlocks) sms = kMaxBlocks;
+  const int wanted = (n + kWarps - 1) / kWarps;
+  return launch(A, wanted < sms ? wanted : sms, false, st);
 }

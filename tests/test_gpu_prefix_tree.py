@@ -203,3 +203,23 @@ def test_prefix_tree_feeds_tree_attention():
     err = np.abs(got_o - o_ref[rows])
     assert err.max() <= 2e-2 and err.mean() <= 2e-3, (err.max(), err.mean())
     assert np.abs(got_l - l_ref[rows]).max() <= 1e-3
+
+
+@pytest.mark.parametrize("n", [2, 31, 32, 33, 511, 512, 513, 1023, 1025, 3000, 40000])
+def test_prefix_tree_grids_tiles_and_pivots(n):
+    """Path counts at the edges of the one-block, cluster and grid launches and of a sort tile: a caterpillar (every path
+    leaves the chain one token further on: the worst case for a fixed pivot), equal paths, negative and extreme ids."""
+    rng = np.random.default_rng(n)
+    kind = n % 3
+    long_prompt = [int(x) for x in rng.integers(0, 99, size=1000)]
+    seqs = []
+    for i in range(n):
+        if kind == 0:
+            k = int(rng.integers(0, min(n, 400)))
+            s = [7] * k + [8] + [int(x) for x in rng.integers(-2, 2, size=3)]
+        elif kind == 1:
+            s = long_prompt[:int(rng.integers(0, 300 if n > 5000 else 1000))] + [int(rng.choice([-2**31, 2**31 - 1, 0, -1]))]
+        else:
+            s = [int(x) for x in rng.integers(0, 3, size=int(rng.integers(0, 12)))]
+        seqs.append(s)
+    check(*csr(seqs), 4)
