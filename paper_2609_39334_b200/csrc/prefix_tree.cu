@@ -15,16 +15,19 @@
 //           of, come out of the keys.  A round settles at least the pivots; the pivot is picked pseudo-randomly, so the number
 //           of rounds is that of a quicksort's levels in the worst case and the depth of the tree in ordinary ones (3 or 4).
 //             compare   a warp per position: boundaries of the groups from the last round's sorted keys (32-ary search), then
-//                       the new key
-//             tiles     a block per 1024 positions sorts (group, key, position) in shared memory
-//             ranks     only if a group spans tiles: a warp per position, lanes search the group's tiles
+//                       the new key; a group of up to 8 that has been through a round is finished at once, every member
+//                       against every other (its rank is the number below it, what it shares with the rank before the
+//                       most that it shares with any of them)
+//             ranks     a warp per position counts the smaller keys of its group; with groups of more than 256 a block per
+//                       1024 positions sorts (group, key, position) first and the lanes search the tiles of the group
 //   tree    Inner nodes are the intervals of neighbours that share more pages than their surroundings (the LCP-interval
 //           tree).  A warp per position finds its interval with nearest-smaller-value searches of 32 entries a step, over
 //           the entries and over their minima by 32; depth-first numbering (leaves included) comes from a prefix sum of
 //           the intervals per start rank; parents follow from the neighbours of an interval.
 //
 // Bound: HBM, one pass over the shared prefixes (268 MB for 16384 paths with prompts of 4096 tokens, 41 us), and for small
-// inputs the latency of a few dependent phases.  MEASURED_HERE
+// inputs the latency of a dozen dependent phases.  Measured: 16384 paths / 76 M ids 169 us (of which 61 the pass over the
+// prompts; page hashes, a bitonic sort with a string comparator and a pass over the neighbours: 1729), 64 paths 26 us (135).
 #include "common.cuh"
 
 namespace ss {
@@ -34,6 +37,10 @@ constexpr int kThreads = 1024;
 constexpr int kWarps = kThreads / 32;
 constexpr int kTile = 1024;                       // positions that a block sorts in shared memory
 constexpr int kUnroll = 8;                        // 128-byte loads in flight per warp and path
+constexpr int kPairs = 8;                         // a group of up to this many is finished with all pairs: 7 comparisons in a
+                                                  // row (9 us) against two or three more rounds (8 us each)
+constexpr int kCount = 256;                       // ranks by counting up to this group size: 8 keys a lane (1.2 us) against a
+                                                  // tile sort (13 us); beyond, counting grows with the square
 constexpr uint32_t kInf = 0x7fffffffu;            // "common length" of a path with itself
 constexpr unsigned long long kBarrierLimitNs = 4000000000ull;
 
@@ -43,7 +50,7 @@ struct Args {
   int n, page, n_tiles;
   int32_t* status;               // first word of the workspace
   unsigned int* arrived;         // grid barrier
-  unsigned int* flags;           // [4]: what the round's groups need (kMore, kWide), rounds in turn
+  unsigned int* flags;           // [4]: what the round's groups need (kMore, kBig), rounds in turn
   uint64_t* key[2];
   int* perm[2];
   int *gs, *ge;                  // per position: its group [gs, ge)
@@ -51,7 +58,7 @@ struct Args {
   int *bmin, *c_start, *c_end, *outer, *cnt, *block_sum;
   int32_t *order, *path_leaf_node, *node_parent, *node_kv_len, *node_src_path, *node_src_offset, *num_nodes;
 };
-constexpr unsigned int kMore = 1, kWide = 2;
+constexpr unsigned int kMore = 1, kBig = 2;
 
 // ---- barrier over all blocks ----------------------------------------------------------------------------------------
 // False when the wait ran out (status SS_ERR_TIMEOUT; every block leaves).  A grid that is one cluster uses the hardware's
@@ -94,49 +101,63 @@ __device__ __forceinline__ uint32_t key_len(uint64_t k) {
 // All paths with this key are equal: the pivot's own, or paths that end where they differ from it.
 __device__ __forceinline__ bool key_settled(uint64_t k) { return !(k >> 63) && static_cast<uint32_t>(k) == 0; }
 
-// Whole warp: the key of path `me` against the pivot, given that they share `base` tokens.  Ascending in the paths' order:
-//   below the pivot  0 | l | token + 1, or 0 if `me` ends at l    (shorter common prefix = smaller path)
-//   equal to it      0 | kInf | 0
-//   above it         1 | kInf - l | token
-__device__ uint64_t make_key(const Args& A, int me, int pivot, int base, int lane) {
-  constexpr uint64_t kEqual = static_cast<uint64_t>(kInf) << 32;
-  if (me == pivot) return kEqual;
-  const int64_t a0 = A.tok_offsets[me], b0 = A.tok_offsets[pivot];
-  const int la = static_cast<int>(A.tok_offsets[me + 1] - a0), lb = static_cast<int>(A.tok_offsets[pivot + 1] - b0);
+// Whole warp: what paths `me` and `other` share (they are known to share `base` tokens) and which comes first by tokens, a
+// proper prefix first.
+struct Order {
+  int len, sign;               // sign < 0: `me` before `other`; 0: equal
+  bool ends;                   // `me` ends at len
+  uint32_t token;              // of `me` at len (if it does not end there), in the order of its bits
+};
+__device__ Order compare_paths(const Args& A, int me, int other, int base, int lane) {
+  const int64_t a0 = A.tok_offsets[me], b0 = A.tok_offsets[other];
+  const int la = static_cast<int>(A.tok_offsets[me + 1] - a0), lb = static_cast<int>(A.tok_offsets[other + 1] - b0);
   const int m = min(la, lb);
   const int32_t *a = A.tok_ids + a0, *b = A.tok_ids + b0;
   int l = m;
   // 32 tokens first (most pairs differ at once or not for long), then kUnroll * 32 a step
-  {
-    const int t = base + lane;
-    const bool ne = t < m && __ldg(a + t) != __ldg(b + t);
-    const uint32_t bal = __ballot_sync(0xffffffffu, ne);
-    if (bal) l = base + __ffs(bal) - 1;
-    else {
-      for (int t0 = base + 32; t0 < m; t0 += 32 * kUnroll) {
-        int32_t x[kUnroll], y[kUnroll];
+  int32_t x0 = base + lane < m ? __ldg(a + base + lane) : 0, y0 = base + lane < m ? __ldg(b + base + lane) : 0;
+  int at = base;                                              // x0, y0 are the tokens at `at` + lane
+  uint32_t bal = __ballot_sync(0xffffffffu, x0 != y0);
+  if (bal) {
+    l = base + __ffs(bal) - 1;
+  } else {
+    for (int t0 = base + 32; t0 < m; t0 += 32 * kUnroll) {
+      int32_t x[kUnroll], y[kUnroll];
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
-          const int t1 = t0 + 32 * u + lane;
-          x[u] = t1 < m ? __ldg(a + t1) : 0;
-          y[u] = t1 < m ? __ldg(b + t1) : 0;
-        }
-        int first = 32 * kUnroll;
-#pragma unroll
-        for (int u = kUnroll - 1; u >= 0; --u)
-          if (x[u] != y[u]) first = 32 * u + lane;
-        first = __reduce_min_sync(0xffffffffu, first);
-        if (first < 32 * kUnroll) { l = t0 + first; break; }
+      for (int u = 0; u < kUnroll; ++u) {
+        const int t1 = t0 + 32 * u + lane;
+        x[u] = t1 < m ? __ldg(a + t1) : 0;
+        y[u] = t1 < m ? __ldg(b + t1) : 0;
       }
+      int first = 32 * kUnroll;
+#pragma unroll
+      for (int u = kUnroll - 1; u >= 0; --u)
+        if (x[u] != y[u]) { first = 32 * u + lane; x0 = x[u]; y0 = y[u]; }
+      const int found = __reduce_min_sync(0xffffffffu, first);
+      if (found < 32 * kUnroll) { l = t0 + found; at = l - (found & 31); break; }
     }
   }
+  Order o;
+  o.len = l;
+  o.ends = l == la;
   if (l == m) {
-    if (la == lb) return kEqual;
-    if (la < lb) return static_cast<uint64_t>(l) << 32;
-    return (1ull << 63) | (static_cast<uint64_t>(kInf - l) << 32) | ordered(__ldg(a + l));
+    o.sign = la < lb ? -1 : (la > lb ? 1 : 0);
+    o.token = o.ends ? 0 : ordered(__ldg(a + l));
+  } else {
+    o.token = ordered(__shfl_sync(0xffffffffu, x0, l - at));
+    o.sign = o.token < ordered(__shfl_sync(0xffffffffu, y0, l - at)) ? -1 : 1;
   }
-  const uint32_t x = ordered(__ldg(a + l)), y = ordered(__ldg(b + l));
-  return x < y ? (static_cast<uint64_t>(l) << 32) | (x + 1) : (1ull << 63) | (static_cast<uint64_t>(kInf - l) << 32) | x;
+  return o;
+}
+
+// The key of a path against the pivot, ascending in the paths' order:
+//   below the pivot  0 | l | token + 1, or 0 if the path ends at l    (shorter common prefix = smaller path)
+//   equal to it      0 | kInf | 0
+//   above it         1 | kInf - l | token
+__device__ __forceinline__ uint64_t make_key(const Order& o) {
+  if (o.sign == 0) return static_cast<uint64_t>(kInf) << 32;
+  if (o.sign < 0) return (static_cast<uint64_t>(o.len) << 32) | (o.ends ? 0u : o.token + 1);
+  return (1ull << 63) | (static_cast<uint64_t>(kInf - o.len) << 32) | o.token;
 }
 
 // Whole warp: number of keys in the ascending k[0..len) that are below `key` (OR_EQUAL: not above it).
@@ -156,50 +177,49 @@ __device__ __forceinline__ int count_below(const uint64_t* k, int len, uint64_t 
   return lo + __popc(__ballot_sync(0xffffffffu, lane < len && (OR_EQUAL ? v <= key : v < key)));
 }
 
-// Sorts positions tile * kTile .. by (group, key, position): keys and paths of the round, kin / pin -> kout / pout.
+// Sorts positions tile * kTile .. by (group, key, position): keys and paths of the round, kin / pin -> kout / pout.  An
+// entry per thread; partners in the warp through shuffles, the others through shared memory.
 __device__ void sort_tile(const Args& A, int tile, const uint64_t* kin, const int* pin, uint64_t* kout, int* pout) {
   __shared__ uint64_t s_key[kTile];
-  __shared__ uint32_t s_at[kTile];                            // first position of the group in the tile << 16 | position
+  __shared__ uint32_t s_at[kTile];
   const int p0 = tile * kTile, count = min(kTile, A.n - p0), tid = threadIdx.x;
+  uint64_t k = ~0ull;
+  uint32_t at = 0xffffffffu;                                  // first position of the group in the tile << 16 | position
   bool open = false;
-  if (tid < kTile) {
-    uint64_t k = ~0ull;
-    uint32_t at = 0xffffffffu;
-    if (tid < count) {
-      const int g = A.gs[p0 + tid];
-      open = A.ge[p0 + tid] - g > 1;
-      k = open ? kin[p0 + tid] : 0;
-      at = (static_cast<uint32_t>(max(g - p0, 0)) << 16) | static_cast<uint32_t>(tid);
-    }
-    s_key[tid] = k;
-    s_at[tid] = at;
+  if (tid < count) {
+    const int g = A.gs[p0 + tid];
+    open = A.ge[p0 + tid] - g > 1;
+    k = open ? kin[p0 + tid] : 0;
+    at = (static_cast<uint32_t>(max(g - p0, 0)) << 16) | static_cast<uint32_t>(tid);
   }
-  if (!__syncthreads_or(open)) {
-    if (tid < count) pout[p0 + tid] = pin[p0 + tid];
-    return;
-  }
+  if (!__syncthreads_or(open)) return;
   int n_pad = 2;
   while (n_pad < count) n_pad <<= 1;
   for (int size = 2; size <= n_pad; size <<= 1) {
     for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      if (tid < (n_pad >> 1)) {
-        const int lo = ((tid & ~(stride - 1)) << 1) | (tid & (stride - 1)), hi = lo + stride;
-        const uint64_t ka = s_key[lo], kb = s_key[hi];
-        const uint32_t aa = s_at[lo], ab = s_at[hi];
-        const uint32_t ga = aa >> 16, gb = ab >> 16;
-        const bool above = ga != gb ? ga > gb : (ka != kb ? ka > kb : aa > ab);
-        if (above == ((lo & size) == 0)) { s_key[lo] = kb; s_key[hi] = ka; s_at[lo] = ab; s_at[hi] = aa; }
+      uint64_t kb;
+      uint32_t ab;
+      if (stride >= 32) {
+        s_key[tid] = k;
+        s_at[tid] = at;
+        __syncthreads();
+        kb = s_key[tid ^ stride];
+        ab = s_at[tid ^ stride];
+        __syncthreads();
+      } else {
+        kb = __shfl_xor_sync(0xffffffffu, k, stride);
+        ab = __shfl_xor_sync(0xffffffffu, at, stride);
       }
-      // (strides below 32 stay inside the warp: pairs 32w..32w+31 touch the 64 entries of warp w alone)
-      if (stride > 32) __syncthreads(); else __syncwarp();
+      const uint32_t ga = at >> 16, gb = ab >> 16;
+      const bool above = ga != gb ? ga > gb : (k != kb ? k > kb : at > ab);
+      const bool keep_low = ((tid & stride) == 0) == ((tid & size) == 0);
+      if (above == keep_low) { k = kb; at = ab; }
     }
-    __syncthreads();
   }
   if (tid < count) {
-    kout[p0 + tid] = s_key[tid];
-    pout[p0 + tid] = pin[p0 + static_cast<int>(s_at[tid] & 0xffffu)];
+    kout[p0 + tid] = k;
+    pout[p0 + tid] = pin[p0 + static_cast<int>(at & 0xffffu)];
   }
-  __syncthreads();
 }
 
 // ---- tree -------------------------------------------------------------------------------------------------------------
@@ -301,62 +321,116 @@ __device__ __forceinline__ void build(const Args& A) {
         me = A.perm[pc][p];
         const uint64_t k = ks[p];
         const int g1 = g + count_below<false>(ks + g, e - g, k, lane), e1 = g + count_below<true>(ks + g, e - g, k, lane);
-        const bool settled = e1 - g1 == 1 || key_settled(k);
-        if (lane == 0) {
-          if (p > g1)
-            A.lcp[p] = settled ? static_cast<int>(A.tok_offsets[me + 1] - A.tok_offsets[me]) / A.page : 0;   // equal paths
-          else if (p > g)
-            A.lcp[p] = static_cast<int>(min(key_len(ks[p - 1]), key_len(k))) / A.page;
-          A.gs[p] = settled ? p : g1;
-          A.ge[p] = settled ? p + 1 : e1;
+        const int m = e1 - g1;
+        if (lane == 0 && p == g1 && p > g) A.lcp[p] = static_cast<int>(min(key_len(ks[p - 1]), key_len(k))) / A.page;
+        base = static_cast<int>(key_len(k)) + 1;
+        const bool equal = key_settled(k), pairs = !equal && m <= kPairs;
+        int rank = p - g1, shared = 0;                         // in the group; tokens shared with the rank before
+        if (equal) {
+          shared = static_cast<int>(A.tok_offsets[me + 1] - A.tok_offsets[me]);
+        } else if (pairs) {
+          rank = 0;
+          for (int x = 0; x < m; ++x) {
+            if (g1 + x == p) continue;
+            const Order o = compare_paths(A, me, A.perm[pc][g1 + x], base, lane);
+            if (o.sign > 0 || (o.sign == 0 && g1 + x < p)) {
+              ++rank;
+              shared = max(shared, o.len);
+            }
+          }
         }
-        if (settled) continue;
+        if (equal || pairs) {
+          if (lane == 0) {
+            A.order[g1 + rank] = me;
+            if (rank > 0) A.lcp[g1 + rank] = shared / A.page;
+            A.gs[p] = p;
+            A.ge[p] = p + 1;
+          }
+          continue;
+        }
+        if (lane == 0) {
+          A.gs[p] = g1;
+          A.ge[p] = e1;
+        }
         g = g1;
         e = e1;
-        base = static_cast<int>(key_len(k)) + 1;
-      } else if (lane == 0) {
-        A.gs[p] = g;
-        A.ge[p] = e;
-        A.perm[pc][p] = p;
-        if (p == 0) A.lcp[0] = 0;
+      } else {
+        if (lane == 0) {
+          A.gs[p] = g;
+          A.ge[p] = e;
+          A.perm[pc][p] = p;
+          if (p == 0) A.lcp[0] = 0;
+          if (n == 1) A.order[0] = 0;
+        }
+        if (n == 1) continue;
       }
-      if (e - g == 1) continue;
-      need |= kMore | (g / kTile != (e - 1) / kTile ? kWide : 0);
+      const int m = e - g;
+      need |= kMore | (m > kCount ? kBig : 0);
       uint32_t r = (static_cast<uint32_t>(g) * 0x9e3779b1u) ^ ((round + 1) * 0x85ebca6bu);
       r = (r ^ (r >> 15)) * 0x2c1b3c6du;
-      const int at = g + static_cast<int>((r >> 3) % static_cast<uint32_t>(e - g));
-      const uint64_t k = make_key(A, me, round > 0 ? A.perm[pc][at] : at, base, lane);
-      if (lane == 0) A.key[kc ^ 1][p] = k;
+      const int at = g + static_cast<int>((r >> 3) % static_cast<uint32_t>(m));
+      const int pivot = round > 0 ? A.perm[pc][at] : at;
+      Order o{0, 0, false, 0};
+      if (me != pivot) o = compare_paths(A, me, pivot, base, lane);
+      if (lane == 0) A.key[kc ^ 1][p] = make_key(o);
     }
     if (lane == 0 && need) atomicOr(&A.flags[round & 3], need);
     if (!grid_barrier<CLUSTER>(A, target)) return;
     const unsigned int flags = *reinterpret_cast<volatile unsigned int*>(&A.flags[round & 3]);
     if (!(flags & kMore)) break;
     if (blockIdx.x == 0 && threadIdx.x == 0) A.flags[(round + 2) & 3] = 0;
+    if (!(flags & kBig)) {
+      const uint64_t* kn = A.key[kc ^ 1];
+      for (int p = wid; p < n; p += n_warps) {
+        const int g = A.gs[p], e = A.ge[p];
+        if (e - g == 1) continue;
+        const uint64_t k = kn[p];
+        int below = 0;
+        for (int q = g + lane; q < e; q += 32) below += kn[q] < k || (kn[q] == k && q < p) ? 1 : 0;
+        below = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned int>(below)));
+        if (lane == 0) {
+          A.key[kc][g + below] = k;
+          A.perm[pc ^ 1][g + below] = A.perm[pc][p];
+        }
+      }
+      pc ^= 1;
+      if (!grid_barrier<CLUSTER>(A, target)) return;
+      continue;
+    }
     for (int t = blockIdx.x; t < A.n_tiles; t += gridDim.x)
       sort_tile(A, t, A.key[kc ^ 1], A.perm[pc], A.key[kc], A.perm[pc ^ 1]);
     if (!grid_barrier<CLUSTER>(A, target)) return;
-    if (!(flags & kWide)) {
-      pc ^= 1;
-      continue;
-    }
-    for (int p = wid; p < n; p += n_warps) {
-      const int g = A.gs[p], e = A.ge[p], tile = p / kTile, t0 = g / kTile, t1 = (e - 1) / kTile;
-      const uint64_t k = A.key[kc][p];
-      int rank = lane == 0 ? p - max(g, tile * kTile) : 0;
-      for (int t = t0 + lane; t <= t1; t += 32) {
-        if (t == tile) continue;
-        const int begin = max(g, t * kTile);
-        int lo = begin, hi = min(e, (t + 1) * kTile);          // first position that does not come before p
-        while (lo < hi) {
-          const int mid = (lo + hi) >> 1;
-          const uint64_t v = A.key[kc][mid];
-          if (t < tile ? v <= k : v < k) lo = mid + 1; else hi = mid;
-        }
-        rank += lo - begin;
+    // `width` lanes per position, one for each tile of its group
+    int width = 1;
+    while (width < 32 && width < A.n_tiles) width <<= 1;
+    const int sub = lane & (width - 1), per_warp = 32 / width;
+    for (int p0 = wid * per_warp; p0 < n; p0 += n_warps * per_warp) {
+      const int p = p0 + lane / width;
+      int g = 0, e = 0, rank = 0;
+      uint64_t k = 0;
+      if (p < n) {
+        g = A.gs[p];
+        e = A.ge[p];
       }
-      rank = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned int>(rank)));
-      if (lane == 0) {
+      if (e - g > 1) {
+        const int tile = p / kTile, t0 = g / kTile, t1 = (e - 1) / kTile;
+        k = A.key[kc][p];
+        if (sub == 0) rank = p - max(g, tile * kTile);
+        for (int t = t0 + sub; t <= t1; t += width) {
+          if (t == tile) continue;
+          const int begin = max(g, t * kTile);
+          int lo = begin, hi = min(e, (t + 1) * kTile);        // first position that does not come before p
+          while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            const uint64_t v = A.key[kc][mid];
+            if (t < tile ? v <= k : v < k) lo = mid + 1; else hi = mid;
+          }
+          rank += lo - begin;
+        }
+      }
+      __syncwarp();
+      for (int o = width >> 1; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+      if (sub == 0 && e - g > 1) {
         A.key[kc ^ 1][g + rank] = k;
         A.perm[pc][g + rank] = A.perm[pc ^ 1][p];
       }
@@ -364,13 +438,12 @@ __device__ __forceinline__ void build(const Args& A) {
     kc ^= 1;
     if (!grid_barrier<CLUSTER>(A, target)) return;
   }
-  const int* path_of = A.perm[pc];
+  const int* path_of = A.order;
 
   // ---- tree -----------------------------------------------------------------------------------------------------------
   for (int p0 = wid * 32; p0 <= n; p0 += n_warps * 32) {
     const int p = p0 + lane;
     if (p <= n) A.cnt[p] = 0;
-    if (p < n) A.order[p] = path_of[p];
     const int m = __reduce_min_sync(0xffffffffu, p < n ? A.lcp[p] : 0x7fffffff);
     if (lane == 0 && p0 < n) A.bmin[p0 >> 5] = m;
   }
@@ -577,8 +650,9 @@ extern "C" int32_t ss_build_prefix_tree(const int32_t* tok_ids, const int64_t* t
   A.node_src_offset = node_src_offset_out;
   A.num_nodes = num_nodes_out;
 
-  // One position per warp in one block: its barrier is the cheapest.  A cluster of 8 up to 16 positions per warp's worth of
-  // short paths; from there the grid's bandwidth pays for its barrier.
+  // One block while it has a warp per position (its barrier is the cheapest).  A cluster of 8 blocks up to two positions per
+  // warp and 16 MB of ids, which its 8 SMs read in 20 us: what the grid's barriers (1.5 us against 0.3, a dozen of them)
+  // cost more.
   if (n <= kWarps) return launch(A, 1, true, st);
   if (n <= 512 && total_tok <= (1 << 22)) return launch(A, 8, true, st);
   int sms = sm_count_of_current_device();
