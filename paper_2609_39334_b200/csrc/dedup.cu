@@ -3,25 +3,30 @@
 // Pipeline (all on the caller's stream, no host synchronisation):
 //   1. hash      one warp per path: 64-bit hash of (ctx_key, length, token ids); lanes stride over the tokens,
 //                each token is mixed with its position, lane sums are combined with shuffles
-//   2. sort      LSD radix sort (8-bit digits, 4 passes) of (top 32 hash bits, path index); stable, so equal
-//                keys stay in ascending index order
-//   3. match     one warp per sorted position: binary-search the start of its equal-key run, then look for the
-//                first earlier run member whose full 64-bit hash, ctx_key, length AND token ids are equal
-//                (token ids compared cooperatively by the warp) -> canon
-//   4. compact   exclusive scan of (canon[i] == i) in index order -> ranks; unique list, multiplicities
-//                (integer atomics: order-independent), path_to_unique, slot remap
+//   2. table     open addressing, one entry per distinct hash: the smallest path index with it
+//   3. match     one warp per path: compares itself with the path of its entry - 64-bit hash, ctx_key, length AND token ids
+//                (by the whole warp) -> canon.  If they differ the hash collided, and the warp looks through all earlier
+//                paths with an equal hash.
+//   4. compact   exclusive scan of (canon[i] == i) in index order -> ranks; unique list, multiplicities (counts:
+//                order-independent), path_to_unique, slot remap
 // Hash collisions only cost time: equality is always decided on the token ids themselves.
-// Batches of up to 4096 paths run the same four steps in two launches (the last block to finish a grid-parallel
-// step runs the single-block step that follows it; the sort is a bitonic network in shared memory).
+//
+// Up to kSmallMax paths this takes two launches and no cleared memory: every block of the second builds the whole table in
+// its own shared memory (a microsecond; cheaper than a launch that builds it once), matches its 32 paths, and the block
+// that arrives last compacts.  Above, the first launch inserts into a table in the workspace, the second matches, and the
+// third compacts with a block per 1024 paths.  Latency-bound: a few MB of ids, a handful of dependent trips to L2.
+// Measured, the call: 1024 paths 35 -> 14 us (a bitonic sort of the hashes and binary searches by one block before),
+// 8192 paths 78 -> 28 us (a sort by counting, a compaction by one block).
 #include "common.cuh"
 
 namespace ss {
 namespace dedup {
 
-constexpr int kSortThreads = 256;
-constexpr int kSortItems = 8;                       // rounds per tile
-constexpr int kSortTile = kSortThreads * kSortItems;
-constexpr int kWarpsPerSortBlock = kSortThreads / 32;
+constexpr int kThreads = 1024;                      // match kernels: a warp per path
+constexpr int kWarps = kThreads / 32;
+constexpr int kSmallMax = 4096;
+constexpr int kHashWarps = 8;                       // per block of the hash kernels
+constexpr int kChunk = 1024;                        // paths per block of the compaction
 
 __device__ __forceinline__ uint64_t mix64(uint64_t x) {   // splitmix64 finaliser
   x ^= x >> 30; x *= 0xbf58476d1ce4e5b9ull;
@@ -47,245 +52,79 @@ __device__ __forceinline__ uint64_t hash_path(const int32_t* __restrict__ tok_id
   return h;
 }
 
-__device__ __forceinline__ uint32_t sort_key_of(uint64_t h, uint32_t weak) {
-  return weak ? static_cast<uint32_t>(h) : static_cast<uint32_t>(h >> 32);
-}
+// Entry of the table in the workspace: tag << 32 | smallest path index; all ones when empty.
+constexpr unsigned long long kEmpty = ~0ull;
+__device__ __forceinline__ uint32_t tag_of(uint64_t h) { return static_cast<uint32_t>(h >> 32) ^ static_cast<uint32_t>(h); }
 
+// Hash of every path.  `table` (mask + 1 entries, all ones): inserts; `chunk_count`, `multiplicity`: cleared for the kernels
+// that follow; `arrived`: the counter of small_match_kernel.
 __global__ void hash_kernel(const int32_t* __restrict__ tok_ids, const int64_t* __restrict__ tok_offsets,
                             const int64_t* __restrict__ ctx_key, int n, uint32_t weak, uint64_t* __restrict__ hash64,
-                            uint32_t* __restrict__ keys, uint32_t* __restrict__ idx) {
+                            unsigned long long* table, uint32_t mask, int* __restrict__ chunk_count,
+                            int32_t* __restrict__ multiplicity, unsigned int* __restrict__ arrived) {
   ss::grid_dependency_enter();
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (warp >= n) return;
-  const uint64_t h = hash_path(tok_ids, tok_offsets, ctx_key, warp, weak, lane);
-  if (lane == 0) {
-    hash64[warp] = h;
-    keys[warp] = sort_key_of(h, weak);
-    idx[warp] = warp;
+  const int64_t gtid = static_cast<int64_t>(blockIdx.x) * (kHashWarps * 32) + threadIdx.x;
+  if (gtid == 0 && arrived) *arrived = 0;
+  if (table && gtid < n) {
+    multiplicity[gtid] = 0;
+    if (gtid % kChunk == 0) chunk_count[gtid / kChunk] = 0;
+  }
+  if ((gtid >> 5) >= n) return;
+  const int path = static_cast<int>(gtid >> 5);
+  const uint64_t h = hash_path(tok_ids, tok_offsets, ctx_key, path, weak, lane);
+  if (lane != 0) return;
+  hash64[path] = h;
+  if (!table) return;
+  const unsigned long long mine = (static_cast<unsigned long long>(tag_of(h)) << 32) | static_cast<uint32_t>(path);
+  for (uint32_t s = static_cast<uint32_t>(h) & mask;; s = (s + 1) & mask) {
+    const unsigned long long cur = atomicCAS(&table[s], kEmpty, mine);
+    if (cur == kEmpty) return;
+    if ((cur >> 32) == (mine >> 32)) {                       // (an entry keeps its tag: the minimum is over the index)
+      atomicMin(&table[s], mine);
+      return;
+    }
   }
 }
 
-// ---- radix sort pass -------------------------------------------------------------------------------------
-__global__ void rs_hist(const uint32_t* __restrict__ keys, int n, int shift, int num_tiles, uint32_t* __restrict__ hist) {
-  ss::grid_dependency_enter();
-  __shared__ uint32_t cnt[256];
-  cnt[threadIdx.x] = 0;
-  __syncthreads();
-  const int base = blockIdx.x * kSortTile;
-  for (int r = 0; r < kSortItems; ++r) {
-    const int i = base + r * kSortThreads + threadIdx.x;
-    if (i < n) atomicAdd(&cnt[(keys[i] >> shift) & 255u], 1u);
+// Whole warp: paths i and j have the same context, length and ids.
+__device__ __forceinline__ bool same_path(const int32_t* __restrict__ tok_ids, const int64_t* __restrict__ tok_offsets,
+                                          const int64_t* __restrict__ ctx_key, int i, int j, int lane) {
+  const int64_t a0 = tok_offsets[i], b0 = tok_offsets[j], len = tok_offsets[i + 1] - a0;
+  if (tok_offsets[j + 1] - b0 != len || (ctx_key && ctx_key[i] != ctx_key[j])) return false;
+  constexpr int kUnroll = 4;
+  for (int64_t p = lane; p - lane < len; p += 32 * kUnroll) {
+    int32_t x[kUnroll], y[kUnroll];
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) {
+      const int64_t q = p + 32 * u;
+      x[u] = q < len ? tok_ids[a0 + q] : 0;
+      y[u] = q < len ? tok_ids[b0 + q] : 0;
+    }
+    bool eq = true;
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) eq = eq && x[u] == y[u];
+    if (!__all_sync(0xffffffffu, eq)) return false;
   }
-  __syncthreads();
-  hist[threadIdx.x * num_tiles + blockIdx.x] = cnt[threadIdx.x];
+  return true;
 }
 
-// In-place exclusive sum scan of `count` uint32 by one block (looping with a carry).
-__global__ void scan_u32_single_block(uint32_t* __restrict__ data, int count) {
-  ss::grid_dependency_enter();
-  __shared__ uint32_t warp_tot[32];
-  __shared__ uint32_t carry_s;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (threadIdx.x == 0) carry_s = 0;
-  __syncthreads();
-  for (int base = 0; base < count; base += blockDim.x) {
-    const int i = base + threadIdx.x;
-    const uint32_t v = i < count ? data[i] : 0u;
-    uint32_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) warp_tot[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-      uint32_t t = lane < nw ? warp_tot[lane] : 0u;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, t, o);
-        if (lane >= o) t += y;
-      }
-      warp_tot[lane] = t;                         // inclusive totals of warps
-    }
-    __syncthreads();
-    const uint32_t carry = carry_s;
-    const uint32_t before = carry + (warp ? warp_tot[warp - 1] : 0u) + x - v;
-    if (i < count) data[i] = before;
-    __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) carry_s = before + v;
-    __syncthreads();
-  }
-}
-
-__global__ void rs_scatter(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ idx_in,
-                           uint32_t* __restrict__ keys_out, uint32_t* __restrict__ idx_out, int n, int shift,
-                           int num_tiles, const uint32_t* __restrict__ hist) {
-  ss::grid_dependency_enter();
-  __shared__ uint32_t base[256];
-  __shared__ uint32_t wc[kWarpsPerSortBlock][256];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  base[threadIdx.x] = hist[threadIdx.x * num_tiles + blockIdx.x];
-#pragma unroll
-  for (int w = 0; w < kWarpsPerSortBlock; ++w) wc[w][threadIdx.x] = 0;
-  __syncthreads();
-  const int tile_base = blockIdx.x * kSortTile;
-  for (int r = 0; r < kSortItems; ++r) {
-    const int i = tile_base + r * kSortThreads + threadIdx.x;
-    const bool valid = i < n;
-    uint32_t key = 0, id = 0;
-    if (valid) { key = keys_in[i]; id = idx_in[i]; }
-    const uint32_t digit = valid ? ((key >> shift) & 255u) : 256u;
-    const uint32_t peers = __match_any_sync(0xffffffffu, digit);
-    const uint32_t rank = __popc(peers & ((1u << lane) - 1u));
-    if (valid && rank == 0) wc[warp][digit] = __popc(peers);
-    __syncthreads();
-    if (valid) {
-      uint32_t off = base[digit] + rank;
-      for (int w = 0; w < warp; ++w) off += wc[w][digit];
-      keys_out[off] = key;
-      idx_out[off] = id;
-    }
-    __syncthreads();
-    {
-      uint32_t tot = 0;
-#pragma unroll
-      for (int w = 0; w < kWarpsPerSortBlock; ++w) { tot += wc[w][threadIdx.x]; wc[w][threadIdx.x] = 0; }
-      base[threadIdx.x] += tot;
-    }
-    __syncthreads();
-  }
-}
-
-// ---- exact matching inside equal-key runs ---------------------------------------------------------------
-// Whole warp: canonical representative of the path at sorted position s.
-// (keys, idx, hash64 carry no __restrict__ here: the single-block kernel writes them before it reads them.)
-__device__ __forceinline__ void match_sorted_position(const uint32_t* keys, const uint32_t* idx, int s,
-                                                      const uint64_t* hash64,
-                                                      const int32_t* __restrict__ tok_ids,
-                                                      const int64_t* __restrict__ tok_offsets,
-                                                      const int64_t* __restrict__ ctx_key,
-                                                      int32_t* canon_out, int lane) {
-  const uint32_t key = keys[s];
-  const int i = static_cast<int>(idx[s]);
-  // start of the run of equal keys (lower bound)
-  int lo = 0, hi = s;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (keys[mid] < key) lo = mid + 1; else hi = mid;
-  }
-  const uint64_t hi_ = hash64[i];
-  const int64_t a0 = tok_offsets[i], alen = tok_offsets[i + 1] - a0;
-  const int64_t actx = ctx_key ? ctx_key[i] : 0;
-  int canon = i;
-  for (int b = lo; b < s && canon == i; b += 32) {
+// Whole warp: canonical representative of path i, given the smallest path j <= i in its table entry.
+__device__ __forceinline__ int canon_of(const int32_t* __restrict__ tok_ids, const int64_t* __restrict__ tok_offsets,
+                                        const int64_t* __restrict__ ctx_key, const uint64_t* hash64, uint64_t h, int i, int j,
+                                        int lane) {
+  if (j == i || (hash64[j] == h && same_path(tok_ids, tok_offsets, ctx_key, i, j, lane))) return j;
+  for (int b = 0; b < i; b += 32) {                           // a collision
     const int t = b + lane;
-    bool cand = false;
-    int j = 0;
-    if (t < s) {
-      j = static_cast<int>(idx[t]);
-      cand = hash64[j] == hi_ && (tok_offsets[j + 1] - tok_offsets[j]) == alen && (ctx_key ? ctx_key[j] : 0) == actx;
-    }
-    uint32_t m = __ballot_sync(0xffffffffu, cand);
+    uint32_t m = __ballot_sync(0xffffffffu, t < i && t != j && hash64[t < i ? t : 0] == h);
     while (m) {
-      const int src = __ffs(m) - 1;
+      const int c = b + __ffs(m) - 1;
       m &= m - 1;
-      const int jj = __shfl_sync(0xffffffffu, j, src);
-      const int64_t b0 = tok_offsets[jj];
-      bool same = true;
-      for (int64_t p = 0; p < alen && same; p += 32) {
-        const int64_t q = p + lane;
-        const bool eq = q < alen ? (tok_ids[a0 + q] == tok_ids[b0 + q]) : true;
-        same = __all_sync(0xffffffffu, eq);
-      }
-      if (same) { canon = jj; break; }
+      if (same_path(tok_ids, tok_offsets, ctx_key, i, c, lane)) return c;
     }
   }
-  if (lane == 0) canon_out[i] = canon;
+  return i;
 }
-
-__global__ void match_kernel(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ idx, int n,
-                             const uint64_t* __restrict__ hash64, const int32_t* __restrict__ tok_ids,
-                             const int64_t* __restrict__ tok_offsets, const int64_t* __restrict__ ctx_key,
-                             int32_t* __restrict__ canon_out) {
-  ss::grid_dependency_enter();
-  const int s = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (s >= n) return;
-  match_sorted_position(keys, idx, s, hash64, tok_ids, tok_offsets, ctx_key, canon_out, threadIdx.x & 31);
-}
-
-// ---- compaction ----------------------------------------------------------------------------------------------
-// One block: rank[i] = number of unique paths with a smaller index; also clears the multiplicities.
-__device__ __forceinline__ void rank_block(const int32_t* canon, int n, int32_t* rank, int32_t* multiplicity,
-                                           int32_t* num_unique) {
-  __shared__ int warp_tot[32];
-  __shared__ int carry_s;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (threadIdx.x == 0) carry_s = 0;
-  __syncthreads();
-  for (int base = 0; base < n; base += blockDim.x) {
-    const int i = base + threadIdx.x;
-    const int v = (i < n && canon[i] == i) ? 1 : 0;
-    if (i < n) multiplicity[i] = 0;
-    const uint32_t bal = __ballot_sync(0xffffffffu, v);
-    const int incl_w = __popc(bal & (0xffffffffu >> (31 - lane)));
-    if (lane == 31) warp_tot[warp] = incl_w;
-    __syncthreads();
-    if (warp == 0) {
-      int t = lane < nw ? warp_tot[lane] : 0;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, t, o);
-        if (lane >= o) t += y;
-      }
-      warp_tot[lane] = t;
-    }
-    __syncthreads();
-    const int before = carry_s + (warp ? warp_tot[warp - 1] : 0) + incl_w - v;
-    if (i < n) rank[i] = before;
-    __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) carry_s = before + v;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *num_unique = carry_s;
-}
-
-__global__ void rank_kernel(const int32_t* __restrict__ canon, int n, int32_t* __restrict__ rank,
-                            int32_t* __restrict__ multiplicity, int32_t* __restrict__ num_unique) {
-  ss::grid_dependency_enter();
-  rank_block(canon, n, rank, multiplicity, num_unique);
-}
-
-__device__ __forceinline__ void finalize_path(const int32_t* canon, const int32_t* rank, int i,
-                                              const int32_t* __restrict__ slot_in, int32_t* path_to_unique,
-                                              int32_t* unique_paths, int32_t* multiplicity, int32_t* slot_out) {
-  const int c = canon[i];
-  const int r = rank[c];
-  path_to_unique[i] = r;
-  if (c == i) unique_paths[r] = i;
-  atomicAdd(&multiplicity[r], 1);
-  if (slot_out) slot_out[i] = slot_in[c];
-}
-
-__global__ void finalize_kernel(const int32_t* __restrict__ canon, const int32_t* __restrict__ rank, int n,
-                                const int32_t* __restrict__ slot_in, int32_t* __restrict__ path_to_unique,
-                                int32_t* __restrict__ unique_paths, int32_t* __restrict__ multiplicity,
-                                int32_t* __restrict__ slot_out) {
-  ss::grid_dependency_enter();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  finalize_path(canon, rank, i, slot_in, path_to_unique, unique_paths, multiplicity, slot_out);
-}
-
-// ---- small batches ---------------------------------------------------------------------------------------------
-// A batch of a few thousand paths is launch-latency bound: the multi-launch path above is ~17 dependent launches.
-// Here the same four steps take two: the grid-parallel steps (hash, match) stay grid-parallel, and the block that
-// finishes LAST (a counter in the workspace, zeroed by a memset ahead of the first kernel) runs the single-block step
-// that follows (bitonic sort in shared memory; rank scan + finalize).
-constexpr int kSmallMax = 4096;
-constexpr int kSmallThreads = 1024;
-constexpr int kSmallWarps = kSmallThreads / 32;
 
 // True in every thread of the block that arrives last; its reads come after all other blocks' writes.
 __device__ __forceinline__ bool last_block_arrives(unsigned int* counter) {
@@ -298,114 +137,201 @@ __device__ __forceinline__ bool last_block_arrives(unsigned int* counter) {
   return s_last;
 }
 
-// Sort by counting, for batches too large for one block's shared-memory sort and too small to be worth a radix sort's
-// twelve launches: the rank of a path is the number of paths with a smaller (sort key, index) pair, counted by brute
-// force - n^2 comparisons, 0.27 G at 16384 paths, spread over the whole device (a few microseconds), against a
-// bitonic sort by a single block (~0.25 ms there: one SM, a hundred barrier-separated stages).  One thread per path;
-// the keys go through shared memory in tiles.
-constexpr int kRankThreads = 256;
-constexpr int kRankTile = 2048;
-constexpr int kRankSortMax = 32768;
-
-// Block (bi, bj) counts, for the 256 paths of group bi, the smaller pairs among the 2048 paths of tile bj and adds
-// the counts to rank_acc[] (zeroed before the launch); the block that completes a group - the last of its tiles to
-// arrive at group_done[bi] - scatters the group's keys and indices to their ranks.
-__global__ void __launch_bounds__(kRankThreads)
-rank_sort_kernel(const uint32_t* __restrict__ keys_in, int n, int n_tiles, int* rank_acc, unsigned int* group_done,
-                 uint32_t* __restrict__ keys_out, uint32_t* __restrict__ idx_out) {
-  ss::grid_dependency_enter();
-  __shared__ __align__(16) uint32_t tile[kRankTile];
-  __shared__ bool s_last;
-  const int bi = blockIdx.x / n_tiles, bj = blockIdx.x - bi * n_tiles;
-  const int i = bi * kRankThreads + threadIdx.x;
-  const uint32_t k = i < n ? keys_in[i] : 0xffffffffu;
-  const int base = bj * kRankTile;
-  for (int t = threadIdx.x; t < kRankTile; t += kRankThreads) tile[t] = base + t < n ? keys_in[base + t] : 0xffffffffu;
-  __syncthreads();
-  int cnt = 0;
-  // paths before this one count when their key is <= k, paths after it when it is < k (ties go by index); a tile
-  // that lies wholly on one side of the group's own paths takes the cheap uniform loop
-  if (base + kRankTile <= bi * kRankThreads) {
-#pragma unroll 4
-    for (int t = 0; t < kRankTile; t += 4) {
-      const uint4 v = *reinterpret_cast<const uint4*>(&tile[t]);
-      cnt += (v.x <= k) + (v.y <= k) + (v.z <= k) + (v.w <= k);
-    }
-  } else if (base >= (bi + 1) * kRankThreads) {
-#pragma unroll 4
-    for (int t = 0; t < kRankTile; t += 4) {         // (padding entries are 0xffffffff: never < k)
-      const uint4 v = *reinterpret_cast<const uint4*>(&tile[t]);
-      cnt += (v.x < k) + (v.y < k) + (v.z < k) + (v.w < k);
-    }
-  } else {
-    const int n_here = min(kRankTile, n - base);
-    for (int t = 0; t < n_here; ++t) cnt += (tile[t] < k) || (tile[t] == k && base + t < i);
-  }
-  if (i < n && cnt) atomicAdd(&rank_acc[i], cnt);
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&group_done[bi], 1u) == static_cast<unsigned>(n_tiles - 1);
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  if (i < n) {
-    const int rank = __ldcg(&rank_acc[i]);
-    keys_out[rank] = k;
-    idx_out[rank] = static_cast<uint32_t>(i);
-  }
+// ---- up to kSmallMax paths ---------------------------------------------------------------------------------------
+inline int small_table_size(int n) {
+  int t = 64;
+  while (t < 2 * n) t <<= 1;
+  return t;
 }
+inline size_t small_match_smem(int n) { return static_cast<size_t>(n) * 8 + static_cast<size_t>(small_table_size(n)) * 4; }
 
-__global__ void __launch_bounds__(kSmallThreads)
-small_hash_sort_kernel(const int32_t* __restrict__ tok_ids, const int64_t* __restrict__ tok_offsets,
-                       const int64_t* __restrict__ ctx_key, int n, uint32_t weak, uint64_t* hash64, uint32_t* keys,
-                       uint32_t* idx, unsigned int* counter) {
-  ss::grid_dependency_enter();
-  __shared__ uint64_t skey[kSmallMax];            // (sort key << 32 | path index): distinct, so the order is total
+// Table of all paths in the block's shared memory (s_hash[n], s_tab[mask + 1]), then the canonical representative of path
+// blockIdx.x * kWarps + warp.
+__device__ __forceinline__ void small_match(const int32_t* __restrict__ tok_ids, const int64_t* __restrict__ tok_offsets,
+                                            const int64_t* __restrict__ ctx_key, int n, const uint64_t* hash64,
+                                            int32_t* canon_out, uint64_t* s_hash, int* s_tab, uint32_t mask) {
   const int tid = threadIdx.x, lane = tid & 31;
-  const int p = blockIdx.x * kSmallWarps + (tid >> 5);
-  if (p < n) {
-    const uint64_t h = hash_path(tok_ids, tok_offsets, ctx_key, p, weak, lane);
-    if (lane == 0) hash64[p] = h;
-  }
-  if (!last_block_arrives(counter)) return;
-  int n_pad = 1;
-  while (n_pad < n) n_pad <<= 1;
-  for (int i = tid; i < n_pad; i += blockDim.x)
-    skey[i] = i < n ? (static_cast<uint64_t>(sort_key_of(__ldcg(hash64 + i), weak)) << 32) | static_cast<uint32_t>(i)
-                    : ~0ull;
+  for (int i = tid; i < n; i += kThreads) s_hash[i] = __ldcg(hash64 + i);
+  for (int t = tid; t <= static_cast<int>(mask); t += kThreads) s_tab[t] = -1;
   __syncthreads();
-  for (int size = 2; size <= n_pad; size <<= 1)
-    for (int stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int t = tid; t < (n_pad >> 1); t += blockDim.x) {
-        const int lo = ((t / stride) * (stride << 1)) + (t % stride);
-        const int hi = lo + stride;
-        const bool up = ((lo & size) == 0);
-        const uint64_t a = skey[lo], b = skey[hi];
-        if ((a > b) == up) { skey[lo] = b; skey[hi] = a; }
+  for (int i = tid; i < n; i += kThreads) {
+    const uint64_t h = s_hash[i];
+    for (uint32_t s = static_cast<uint32_t>(h) & mask;; s = (s + 1) & mask) {
+      const int cur = atomicCAS(&s_tab[s], -1, i);
+      if (cur < 0) break;
+      if (s_hash[cur] == h) {
+        atomicMin(&s_tab[s], i);
+        break;
       }
-      __syncthreads();
     }
-  for (int i = tid; i < n; i += blockDim.x) {
-    keys[i] = static_cast<uint32_t>(skey[i] >> 32);
-    idx[i] = static_cast<uint32_t>(skey[i]);
+  }
+  __syncthreads();
+  const int i = blockIdx.x * kWarps + (tid >> 5);
+  if (i >= n) return;
+  const uint64_t h = s_hash[i];
+  uint32_t s = static_cast<uint32_t>(h) & mask;
+  while (s_hash[s_tab[s]] != h) s = (s + 1) & mask;
+  const int c = canon_of(tok_ids, tok_offsets, ctx_key, s_hash, h, i, s_tab[s], lane);
+  if (lane == 0) canon_out[i] = c;
+}
+
+__global__ void __launch_bounds__(kThreads)
+small_match_kernel(const int32_t* __restrict__ tok_ids, const int64_t* __restrict__ tok_offsets,
+                   const int64_t* __restrict__ ctx_key, int n, const uint64_t* __restrict__ hash64, uint32_t mask,
+                   const int32_t* __restrict__ slot_in, int32_t* canon_out, int32_t* path_to_unique, int32_t* unique_paths,
+                   int32_t* multiplicity, int32_t* slot_out, int32_t* num_unique, unsigned int* arrived) {
+  ss::grid_dependency_enter();
+  extern __shared__ __align__(16) uint8_t s_mem[];
+  __shared__ int s_before[kSmallMax / 32];                    // unique paths in front of each group of 32
+  __shared__ int s_total;
+  uint64_t* s_hash = reinterpret_cast<uint64_t*>(s_mem);
+  small_match(tok_ids, tok_offsets, ctx_key, n, hash64, canon_out, s_hash, reinterpret_cast<int*>(s_hash + n), mask);
+  if (!last_block_arrives(arrived)) return;
+  // compaction by the last block; the hashes' shared memory holds ranks and multiplicities
+  const int tid = threadIdx.x, lane = tid & 31, groups = (n + 31) >> 5;
+  int* s_rank = reinterpret_cast<int*>(s_mem);
+  int* s_mult = s_rank + n;
+  for (int i0 = tid & ~31; i0 < n; i0 += kThreads) {
+    const int i = i0 + lane;
+    const uint32_t u = __ballot_sync(0xffffffffu, i < n && __ldcg(canon_out + (i < n ? i : 0)) == i);
+    if (i < n) {
+      s_rank[i] = __popc(u & ((1u << lane) - 1u));
+      s_mult[i] = 0;
+    }
+    if (lane == 0) s_before[i0 >> 5] = __popc(u);
+  }
+  __syncthreads();
+  if (tid < 32) {                                             // 4 groups a lane
+    int v[4], sum = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      v[k] = 4 * lane + k < groups ? s_before[4 * lane + k] : 0;
+      sum += v[k];
+    }
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    int run = incl - sum;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (4 * lane + k < groups) s_before[4 * lane + k] = run;
+      run += v[k];
+    }
+    if (lane == 31) s_total = incl;
+  }
+  __syncthreads();
+  for (int i = tid; i < n; i += kThreads) {
+    const int c = __ldcg(canon_out + i);
+    const int r = s_before[c >> 5] + s_rank[c];
+    path_to_unique[i] = r;
+    if (c == i) unique_paths[r] = i;
+    atomicAdd(&s_mult[r], 1);
+    if (slot_out) slot_out[i] = slot_in[c];
+  }
+  __syncthreads();
+  for (int i = tid; i < s_total; i += kThreads) multiplicity[i] = s_mult[i];
+  for (int i = s_total + tid; i < n; i += kThreads) multiplicity[i] = 0;
+  if (tid == 0) *num_unique = s_total;
+}
+
+// ---- more paths -----------------------------------------------------------------------------------------------------
+// unique[w]: bit b set if path 32 w + b is its own representative; chunk_count[c]: how many of chunk c are.
+__global__ void __launch_bounds__(kThreads)
+match_kernel(const int32_t* __restrict__ tok_ids, const int64_t* __restrict__ tok_offsets, const int64_t* __restrict__ ctx_key,
+             int n, const uint64_t* __restrict__ hash64, const unsigned long long* __restrict__ table, uint32_t mask,
+             int32_t* __restrict__ canon_out, uint32_t* __restrict__ unique, int* chunk_count) {
+  ss::grid_dependency_enter();
+  __shared__ int s_own[kWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * kWarps + warp;
+  int own = 0;
+  if (i < n) {
+    const uint64_t h = hash64[i];
+    const uint32_t tag = tag_of(h);
+    uint32_t s = static_cast<uint32_t>(h) & mask;
+    unsigned long long e = table[s];
+    while (static_cast<uint32_t>(e >> 32) != tag) {
+      s = (s + 1) & mask;
+      e = table[s];
+    }
+    const int c = canon_of(tok_ids, tok_offsets, ctx_key, hash64, h, i, static_cast<int>(static_cast<uint32_t>(e)), lane);
+    if (lane == 0) canon_out[i] = c;
+    own = c == i ? 1 : 0;
+  }
+  if (lane == 0) s_own[warp] = own;
+  __syncthreads();
+  if (warp == 0) {
+    const uint32_t word = __ballot_sync(0xffffffffu, s_own[lane] != 0);
+    if (lane == 0) {
+      unique[blockIdx.x] = word;
+      atomicAdd(&chunk_count[blockIdx.x / (kChunk / kWarps)], __popc(word));
+    }
   }
 }
 
-__global__ void __launch_bounds__(kSmallThreads)
-small_match_finalize_kernel(const uint32_t* __restrict__ keys, const uint32_t* __restrict__ idx, int n,
-                            const uint64_t* __restrict__ hash64, const int32_t* __restrict__ tok_ids,
-                            const int64_t* __restrict__ tok_offsets, const int64_t* __restrict__ ctx_key,
-                            const int32_t* __restrict__ slot_in, int32_t* canon_out, int32_t* rank,
-                            int32_t* path_to_unique, int32_t* unique_paths, int32_t* multiplicity, int32_t* slot_out,
-                            int32_t* num_unique, unsigned int* counter) {
+// Block: exclusive scan of in[0..count) to out (which may be `in`); returns the total.
+__device__ int scan_counts(const int* in, int* out, int count) {
+  __shared__ int warp_tot[32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int carry = 0;
+  for (int base = 0; base < count; base += kChunk) {
+    const int v = base + tid < count ? in[base + tid] : 0;
+    int incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (lane == 31) warp_tot[warp] = incl;
+    __syncthreads();
+    int t = warp_tot[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, t, o);
+      if (lane >= o) t += y;
+    }
+    const int before = __shfl_sync(0xffffffffu, t, (warp + 31) & 31), total = __shfl_sync(0xffffffffu, t, 31);
+    if (base + tid < count) out[base + tid] = carry + (warp ? before : 0) + incl - v;
+    carry += total;
+    __syncthreads();
+  }
+  return carry;
+}
+
+// One block per chunk.  The rank of any path c: the unique paths in the chunks before its own (scanned by every block in
+// its shared memory, or in place by a launch of its own where that would take several steps), plus those in front of it in
+// its chunk (32 words).
+constexpr int kMaxChunksShared = 512;
+__global__ void __launch_bounds__(kChunk) scan_chunks_kernel(int* chunk_count, int n_chunks, int32_t* num_unique) {
   ss::grid_dependency_enter();
-  const int s = blockIdx.x * kSmallWarps + (threadIdx.x >> 5);
-  if (s < n) match_sorted_position(keys, idx, s, hash64, tok_ids, tok_offsets, ctx_key, canon_out, threadIdx.x & 31);
-  if (!last_block_arrives(counter)) return;
-  rank_block(canon_out, n, rank, multiplicity, num_unique);     // canon_out was not read before: no stale L1 lines
-  __syncthreads();
-  for (int i = threadIdx.x; i < n; i += blockDim.x)
-    finalize_path(canon_out, rank, i, slot_in, path_to_unique, unique_paths, multiplicity, slot_out);
+  const int total = scan_counts(chunk_count, chunk_count, n_chunks);
+  if (threadIdx.x == 0) *num_unique = total;
+}
+__global__ void __launch_bounds__(kChunk)
+compact_kernel(const int32_t* __restrict__ canon, int n, const uint32_t* __restrict__ unique, const int* chunk_count,
+               int n_chunks, const int32_t* __restrict__ slot_in, int32_t* __restrict__ path_to_unique,
+               int32_t* __restrict__ unique_paths, int32_t* multiplicity, int32_t* __restrict__ slot_out,
+               int32_t* __restrict__ num_unique) {
+  ss::grid_dependency_enter();
+  __shared__ int s_start[kMaxChunksShared];
+  const int tid = threadIdx.x;
+  const int* start = chunk_count;
+  if (n_chunks <= kMaxChunksShared) {
+    const int total = scan_counts(chunk_count, s_start, n_chunks);
+    if (blockIdx.x == 0 && tid == 0) *num_unique = total;
+    start = s_start;
+  }
+  const int i = blockIdx.x * kChunk + tid;
+  if (i >= n) return;
+  const int c = canon[i], w0 = c / kChunk * (kChunk / 32), w1 = c >> 5;
+  int r = start[c / kChunk] + __popc(unique[w1] & ((1u << (c & 31)) - 1u));
+  for (int w = w0; w < w1; ++w) r += __popc(unique[w]);
+  path_to_unique[i] = r;
+  if (c == i) unique_paths[r] = i;
+  atomicAdd(&multiplicity[r], 1);
+  if (slot_out) slot_out[i] = slot_in[c];
 }
 
 // ---- ss_gather_unique_paths ------------------------------------------------------------------------------------
@@ -482,23 +408,37 @@ gather_unique_kernel(const int32_t* __restrict__ unique_paths, const int32_t* __
 __global__ void zero_scalar_kernel(int32_t* p) {
   ss::grid_dependency_enter(); *p = 0; }
 
+// Shared memory of small_match_kernel beyond 48 KB, once per device.
+static int32_t small_smem_ready() {
+  static bool configured[kDeviceSlots] = {false};
+  const int slot = current_device_slot();
+  if (slot >= 0 && configured[slot]) return SS_OK;
+  if (cudaFuncSetAttribute(small_match_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(small_match_smem(kSmallMax))) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return SS_ERR_CUDA;
+  }
+  if (slot >= 0) configured[slot] = true;
+  return SS_OK;
+}
+
 struct Layout {
-  size_t hash64, keys_a, keys_b, idx_a, idx_b, hist, rank, total;
-  int num_tiles;
+  size_t counters, hash64, table, unique, chunk_count, total;
+  uint32_t mask;                                    // table entries - 1
 };
 
 static Layout layout(int n) {
   Layout L;
   const size_t m = n > 0 ? n : 1;
-  L.num_tiles = static_cast<int>((m + kSortTile - 1) / kSortTile);
+  size_t entries = 1;
+  while (entries < 2 * m) entries <<= 1;
+  L.mask = static_cast<uint32_t>(entries - 1);
   size_t off = 0;
+  L.counters = off; off = align_up(off + 64);
   L.hash64 = off; off = align_up(off + m * 8);
-  L.keys_a = off; off = align_up(off + m * 4);
-  L.keys_b = off; off = align_up(off + m * 4);
-  L.idx_a = off; off = align_up(off + m * 4);
-  L.idx_b = off; off = align_up(off + m * 4);
-  L.hist = off; off = align_up(off + static_cast<size_t>(256) * L.num_tiles * 4);
-  L.rank = off; off = align_up(off + m * 4);
+  L.table = off; off = align_up(off + (n > kSmallMax ? entries * 8 : 0));
+  L.unique = off; off = align_up(off + (m + 31) / 32 * 4);
+  L.chunk_count = off; off = align_up(off + (m + kChunk - 1) / kChunk * 4);
   L.total = off;
   return L;
 }
@@ -535,69 +475,35 @@ extern "C" int32_t ss_dedup_paths(const int32_t* tok_ids, const int64_t* tok_off
   if (workspace_bytes < L.total) return SS_ERR_WORKSPACE_TOO_SMALL;
   char* ws = static_cast<char*>(workspace);
   uint64_t* hash64 = reinterpret_cast<uint64_t*>(ws + L.hash64);
-  uint32_t* keys_a = reinterpret_cast<uint32_t*>(ws + L.keys_a);
-  uint32_t* keys_b = reinterpret_cast<uint32_t*>(ws + L.keys_b);
-  uint32_t* idx_a = reinterpret_cast<uint32_t*>(ws + L.idx_a);
-  uint32_t* idx_b = reinterpret_cast<uint32_t*>(ws + L.idx_b);
-  uint32_t* hist = reinterpret_cast<uint32_t*>(ws + L.hist);
-  int32_t* rank = reinterpret_cast<int32_t*>(ws + L.rank);
-
   const int n = n_paths;
   const uint32_t weak = (flags & SS_FLAG_WEAK_HASH) ? 1u : 0u;
+  const int hash_blocks = (n + kHashWarps - 1) / kHashWarps, match_blocks = (n + kWarps - 1) / kWarps;
   if (n <= kSmallMax) {
-    unsigned int* counters = reinterpret_cast<unsigned int*>(hist);      // the sort histogram is unused on this path
-    if (cudaMemsetAsync(counters, 0, 2 * sizeof(unsigned int), st) != cudaSuccess) {
-      (void)cudaGetLastError();
-      return SS_ERR_CUDA;
-    }
-    const int blocks = (n + kSmallWarps - 1) / kSmallWarps;
-    SS_LAUNCH(small_hash_sort_kernel, blocks, kSmallThreads, 0, st, tok_ids, tok_offsets, ctx_key, n, weak, hash64, keys_a,
-              idx_a, counters);
-    SS_LAUNCH(small_match_finalize_kernel, blocks, kSmallThreads, 0, st, keys_a, idx_a, n, hash64, tok_ids, tok_offsets,
-              ctx_key, slot_in, canon_out, rank, path_to_unique_out, unique_paths_out, multiplicity_out, slot_out,
-              num_unique_out, counters + 1);
+    unsigned int* arrived = reinterpret_cast<unsigned int*>(ws + L.counters);
+    const int32_t rc = small_smem_ready();
+    if (rc != SS_OK) return rc;
+    SS_LAUNCH(hash_kernel, hash_blocks, kHashWarps * 32, 0, st, tok_ids, tok_offsets, ctx_key, n, weak, hash64,
+              static_cast<unsigned long long*>(nullptr), 0u, static_cast<int*>(nullptr), static_cast<int32_t*>(nullptr), arrived);
+    SS_LAUNCH(small_match_kernel, match_blocks, kThreads, small_match_smem(n), st, tok_ids, tok_offsets, ctx_key, n, hash64,
+              static_cast<uint32_t>(small_table_size(n) - 1), slot_in, canon_out, path_to_unique_out, unique_paths_out,
+              multiplicity_out, slot_out, num_unique_out, arrived);
     return SS_OK;
   }
-  const int warps_per_block = 8;
-  const int warp_blocks = (n + warps_per_block - 1) / warps_per_block;
-  SS_LAUNCH(hash_kernel, warp_blocks, warps_per_block * 32, 0, st, tok_ids, tok_offsets, ctx_key, n, weak, hash64,
-            keys_a, idx_a);
-  if (n <= kRankSortMax) {                          // three launches: hash, sort by counting, match + rank + finalize
-    unsigned int* counters = reinterpret_cast<unsigned int*>(hist);      // the sort histogram is unused on this path
-    if (cudaMemsetAsync(counters, 0, 2 * sizeof(unsigned int), st) != cudaSuccess) {
-      (void)cudaGetLastError();
-      return SS_ERR_CUDA;
-    }
-    // (idx_a holds the identity permutation the radix sort starts from: free here, it accumulates the ranks; the
-    //  group counters follow the two arrival counters in the histogram region)
-    const int n_groups = (n + kRankThreads - 1) / kRankThreads, n_tiles = (n + kRankTile - 1) / kRankTile;
-    if (cudaMemsetAsync(idx_a, 0, static_cast<size_t>(n) * sizeof(uint32_t), st) != cudaSuccess ||
-        cudaMemsetAsync(counters + 2, 0, static_cast<size_t>(n_groups) * sizeof(unsigned int), st) != cudaSuccess) {
-      (void)cudaGetLastError();
-      return SS_ERR_CUDA;
-    }
-    SS_LAUNCH(rank_sort_kernel, n_groups * n_tiles, kRankThreads, 0, st, keys_a, n, n_tiles, reinterpret_cast<int*>(idx_a),
-              counters + 2, keys_b, idx_b);
-    SS_LAUNCH(small_match_finalize_kernel, (n + kSmallWarps - 1) / kSmallWarps, kSmallThreads, 0, st, keys_b, idx_b, n,
-              hash64, tok_ids, tok_offsets, ctx_key, slot_in, canon_out, rank, path_to_unique_out, unique_paths_out,
-              multiplicity_out, slot_out, num_unique_out, counters + 1);
-    return SS_OK;
+  unsigned long long* table = reinterpret_cast<unsigned long long*>(ws + L.table);
+  uint32_t* unique = reinterpret_cast<uint32_t*>(ws + L.unique);
+  int* chunk_count = reinterpret_cast<int*>(ws + L.chunk_count);
+  const int n_chunks = (n + kChunk - 1) / kChunk;
+  if (cudaMemsetAsync(table, 0xff, (static_cast<size_t>(L.mask) + 1) * 8, st) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return SS_ERR_CUDA;
   }
-  const int passes = weak ? 1 : 4;
-  uint32_t *kin = keys_a, *kout = keys_b, *iin = idx_a, *iout = idx_b;
-  for (int p = 0; p < passes; ++p) {
-    const int shift = 8 * p;
-    SS_LAUNCH(rs_hist, L.num_tiles, kSortThreads, 0, st, kin, n, shift, L.num_tiles, hist);
-    SS_LAUNCH(scan_u32_single_block, 1, 1024, 0, st, hist, 256 * L.num_tiles);
-    SS_LAUNCH(rs_scatter, L.num_tiles, kSortThreads, 0, st, kin, iin, kout, iout, n, shift, L.num_tiles, hist);
-    uint32_t* t = kin; kin = kout; kout = t;
-    t = iin; iin = iout; iout = t;
-  }
-  SS_LAUNCH(match_kernel, warp_blocks, warps_per_block * 32, 0, st, kin, iin, n, hash64, tok_ids, tok_offsets,
-            ctx_key, canon_out);
-  SS_LAUNCH(rank_kernel, 1, 1024, 0, st, canon_out, n, rank, multiplicity_out, num_unique_out);
-  SS_LAUNCH(finalize_kernel, (n + 255) / 256, 256, 0, st, canon_out, rank, n, slot_in, path_to_unique_out,
-            unique_paths_out, multiplicity_out, slot_out);
+  SS_LAUNCH(hash_kernel, hash_blocks, kHashWarps * 32, 0, st, tok_ids, tok_offsets, ctx_key, n, weak, hash64, table, L.mask,
+            chunk_count, multiplicity_out, static_cast<unsigned int*>(nullptr));
+  SS_LAUNCH(match_kernel, match_blocks, kThreads, 0, st, tok_ids, tok_offsets, ctx_key, n, hash64, table, L.mask, canon_out,
+            unique, chunk_count);
+  if (n_chunks > kMaxChunksShared) SS_LAUNCH(scan_chunks_kernel, 1, kChunk, 0, st, chunk_count, n_chunks, num_unique_out);
+  SS_LAUNCH(compact_kernel, n_chunks, kChunk, 0, st, canon_out, n, unique, chunk_count, n_chunks, slot_in, path_to_unique_out,
+            unique_paths_out, multiplicity_out, slot_out, num_unique_out);
   return SS_OK;
 }
 
@@ -618,7 +524,7 @@ namespace ss {
 namespace dedup {
 
 constexpr int kStaticMaxPaths = SS_DEDUP_STATIC_MAX_PATHS;
-constexpr size_t kStaticScratchBytes = 2u << 20;           // 2 MiB; layout(kStaticMaxPaths).total is about 1.8 MiB
+constexpr size_t kStaticScratchBytes = 2u << 20;           // 2 MiB; layout(kStaticMaxPaths).total is about 1.6 MiB
 static __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
 
 constexpr int kMaxDevices = 64;
@@ -656,8 +562,8 @@ extern "C" int32_t ss_dedup_paths_static(const int32_t* tok_ids, const int64_t* 
   void* scratch = nullptr;
   const int32_t rc = static_scratch_address(&scratch);
   if (rc != SS_OK) return rc;
-  // Nothing in the scratch has to start at zero: every region is fully written before it is read (histograms,
-  // keys, ranks), and the multiplicities that do start at zero are an output cleared by the rank kernel.
+  // Nothing in the scratch has to start at zero: what must be clear (the table, counters and counts) is cleared by the
+  // call itself.
   return ss_dedup_paths(tok_ids, tok_offsets, ctx_key, slot_in, n_paths, flags, canon_out, path_to_unique_out,
                         unique_paths_out, multiplicity_out, slot_out, num_unique_out, scratch, kStaticScratchBytes,
                         stream);
