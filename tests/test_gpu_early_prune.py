@@ -102,3 +102,29 @@ def test_topk_and_early_prune_report_segments_outside_the_candidates():
     B.ss_topk_prune(scores, torch.tensor([0, 10, 25, 40], dtype=torch.int32, device=dev), 3, n, k, surv, keep, ws)
     torch.cuda.synchronize()
     assert B.ss_last_device_status(ws) == B.SS_OK
+
+
+@pytest.mark.parametrize("sizes,k", [([63, 1, 64, 65, 2], 5), ([1, 1, 1000, 1, 1, 30], 7), ([1023, 1024, 1025], 300),
+                                     ([2047, 2049], 1), ([100] * 300, 25)])
+def test_segments_at_the_edges_of_the_register_sort(sizes, k):
+    """Segments below, at and above one candidate per thread (the block size follows the average), candidates before the
+    first and after the last segment, against the oracle; selection and pruning share the sort."""
+    rng = np.random.default_rng(sum(sizes) + k)
+    seg = (np.concatenate([[0], np.cumsum(sizes)]) + 3).astype(np.int32)
+    n = int(seg[-1]) + 5
+    sc = (rng.integers(0, 30, size=n) / 32.0).astype(np.float32)
+    sc[rng.random(n) < 0.02] = 1.0
+    dev = torch.device(DEV)
+    surv = torch.full((len(sizes), k), -9, dtype=torch.int32, device=dev)
+    keep = torch.full((n,), 7, dtype=torch.uint8, device=dev)
+    ws = B.alloc_workspace(B.ss_topk_workspace_bytes(n), dev)
+    B.ss_topk_prune(torch.from_numpy(sc).to(dev), torch.from_numpy(seg).to(dev), len(sizes), n, k, surv, keep, ws)
+    s_ref, k_ref = oracle.topk(sc[3:-5], seg - 3, k)
+    assert np.array_equal(surv.cpu().numpy(), np.where(s_ref >= 0, s_ref + 3, -1))
+    assert np.array_equal(keep.cpu().numpy(), np.concatenate([np.zeros(3), k_ref, np.zeros(5)]))
+    for frac in (0.3, 1.0):
+        ver = (rng.random(n) < frac).astype(np.uint8)
+        got = run(sc, ver, seg, k)
+        want = oracle.early_prune(sc[3:-5], ver[3:-5], seg - 3, k)
+        assert np.array_equal(got[0], np.concatenate([np.zeros(3), want[0], np.zeros(5)]))
+        assert np.array_equal(got[1], np.where(want[1] >= 0, want[1] + 3, -1)) and np.array_equal(got[2], want[2])
