@@ -37,7 +37,8 @@ struct alignas(8) TileItem {
   int32_t kv_end;
   int32_t limit0;     // keys visible to the tile's first token; token i sees limit0 + i * (kind == chain)
   int32_t slot_off;   // stacked: partial slot relative to the token's slot base; chain: -1 (final output)
-  int32_t src0;       // chain: row of q holding the tile's first token (stacked: rows come from dec_src[])
+  int32_t src0;       // chain: row of q holding the tile's first token; stacked (rows come from dec_src[]): index into
+                      // node_pages of the node's first page
   int32_t pad;
 };
 

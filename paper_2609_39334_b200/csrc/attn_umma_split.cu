@@ -571,7 +571,7 @@ tile_items_umma_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const _
             seg_first[n_seg] = first;
           } else {
             seg_first[0] = 0;
-            seg_off[0] = P.node_page_offsets[v.node];
+            seg_off[0] = v.src0;
             seg_first[1] = 0x7fffffff;
             n_seg = 1;
           }

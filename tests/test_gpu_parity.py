@@ -697,3 +697,30 @@ def test_attention_pool_blocks_off_the_8_row_grid():
     r = pipe.results()
     ref = oracle.dedup(w.tok_ids, w.tok_offsets, w.ctx_key, w.slot_in)
     check_attention(r, w, ref, max_paths=64)
+
+
+# =========================================================================================================
+# the planner's small and general form
+# =========================================================================================================
+@pytest.mark.parametrize("paths", [1, 31, 33, 1023, 1025, 2046, 2047, 2048])
+def test_planner_at_the_edges_of_its_small_form(paths):
+    """One root with `paths` leaves (paths + 1 nodes; the one-launch planner takes up to 2048 of each, two per thread):
+    decode, verification and leaves of 0, one chunk, a chunk and a page, and several chunks."""
+    lens = [0, 1, 16, 255, 256, 257, 272, 600]
+    w = synth.build_tree_workload("planner", 7000 + paths, 4, 2, [48], [paths], 1, (0, 0),
+                                  lambda i, n, rng: 1 if i % 5 else 3, device="cpu", poison=False)
+    leaf = w.path_leaf_node
+    w.node_kv_len[leaf] = np.asarray([lens[i % len(lens)] if w.path_q_len[i] == 1 else 3 + (i * 7) % 90 for i in range(paths)], np.int32)
+    pages = (w.node_kv_len.astype(np.int64) + 15) // 16
+    w.node_page_offsets[1:] = np.cumsum(pages)
+    rng = np.random.default_rng(paths)
+    w.num_pages = int(pages.sum())
+    w.node_pages = rng.permutation(w.num_pages).astype(np.int32)
+    w.kv_pool = torch.randn((w.num_pages, 2, 2, 16, 128), generator=torch.Generator().manual_seed(paths)).to(torch.bfloat16)
+    own = w.node_kv_len[leaf].astype(np.int64)
+    w.tok_offsets[1:] = np.cumsum(own)
+    w.tok_ids = rng.integers(0, 1 << 30, size=int(own.sum()), dtype=np.int64).astype(np.int32)
+    w.ctx_key[:] = np.arange(paths)                              # (the empty leaves are not duplicates of one another)
+    r, ref = attention_only(w)
+    assert r["num_unique"] == paths
+    check_attention(r, w, ref, max_paths=40)
