@@ -444,6 +444,10 @@ tile_items_umma_split_kernel(const __grid_constant__ CUtensorMap tmap_k, const _
             if (ragged) {                                         // zero the V rows past the end of the source
               const int n_keys = it.kv_end - (it.kv_begin + j * kTile);
               const int s = gj % kStagesV;
+              // The softmax may be two tiles ahead of P V and so of the V ring, where the parity of this tile's copy is also
+              // that of the one before the last: the stage must be this tile's before its barrier is asked (otherwise the
+              // rows are cleared first and the copy then puts the undefined ones back).
+              if (gj >= kStagesV) ok = mbar_wait(&C.pv_done[(gj - kStagesV) % kRing], ((gj - kStagesV) / kRing) & 1, abort_flag) && ok;
               ok = mbar_wait(&C.v_full[s], (gj / kStagesV) & 1, abort_flag) && ok;
               uint8_t* vs = smem + kOffV + s * kStageBytes;
               const int n_chunks = (kTile - n_keys) * 16;         // 16-byte chunks to clear (both halves)

@@ -724,3 +724,21 @@ def test_planner_at_the_edges_of_its_small_form(paths):
     r, ref = attention_only(w)
     assert r["num_unique"] == paths
     check_attention(r, w, ref, max_paths=40)
+
+
+def test_ragged_ends_do_not_race_with_late_value_copies():
+    """Verification items whose last tile ends early, on a tree that keeps every SM's copy pipeline loaded: the undefined
+    rows behind the last key (NaN here) must be cleared after their copy has landed, however late it is.  Repeated runs
+    must be finite and equal bit for bit."""
+    w = synth.build_tree_workload("ragged", 990, 32, 8, [4096], [256], 8, (128, 1024), lambda i, n, rng: 1 if i < n // 2 else 64,
+                                  dup_frac=0.2, device=DEV)
+    pipe = DevicePipeline(w, DEV)
+    first = None
+    for _ in range(8):
+        pipe.out.zero_()
+        pipe.step()
+        live = pipe.out[:int(pipe.u_q_offsets[int(pipe.num_unique.item())].item())]
+        assert bool(torch.isfinite(live.float()).all())
+        bits = live.view(torch.int16).clone()
+        assert first is None or torch.equal(bits, first)
+        first = bits
