@@ -134,53 +134,94 @@ __device__ __forceinline__ void merge_row(const Params& P, int d, int h, int lan
   row_store_final(r, P, P.dec_tok[d], h, lane);
 }
 
-// The same merge for the (up to 8) q heads [h0, h0 + n_rows) of decode token `d` at once (one whole warp).  The rows
-// are independent, so their loads are issued together: merging them one after another costs two memory round trips
-// per row, which is what a leaf item's last warp would otherwise wait for.
-__device__ __forceinline__ void merge_rows8(const Params& P, int d, int h0, int n_rows, int lane) {
-  int s0 = P.dec_slot_base[d], s1 = P.dec_slot_base[d + 1];
-  SS_CHECK_OR(s0 >= 0 && s0 <= s1 && s1 <= P.caps.slots && P.dec_tok[d] >= 0 && P.dec_tok[d] < P.total_q, &P.hdr->status,
-              return);
-  float m[8];
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    m[r] = -INFINITY;
-    if (r < n_rows)
-      for (int s = s0 + lane; s < s1; s += 32) m[r] = fmaxf(m[r], __ldcg(P.part_lse + static_cast<int64_t>(s) * P.Hq + h0 + r));
+// The same merge for up to 8 rows at once (one whole warp): lane r < n_rows brings decode token `d` and q head `h` of row r.
+// Three trips to memory for up to 2 partials a row (slots; log-sum-exps and values together), one more for every further
+// two: a merge is nothing but latency.  Out of line (inlined it takes registers and instruction-cache space from the leaf
+// kernel's page loop), with its arguments by value: through a reference to the kernel's parameters every one of them would
+// be a load (5 us a call, measured).
+struct MergeArgs {       // what a merge needs of Params, in registers (it is called out of line)
+  const int32_t *dec_slot_base, *dec_tok;
+  const float *part_o, *part_lse;
+  __nv_bfloat16* out;
+  float* lse;
+  int32_t Hq;
+#ifdef SS_CHECKED
+  int64_t slots, total_q;
+  int32_t* status;
+#endif
+};
+__device__ __forceinline__ MergeArgs merge_args(const Params& P) {
+  MergeArgs M{P.dec_slot_base, P.dec_tok, P.part_o, P.part_lse, P.out, P.lse, P.Hq};
+#ifdef SS_CHECKED
+  M.slots = P.caps.slots;
+  M.total_q = P.total_q;
+  M.status = &P.hdr->status;
+#endif
+  return M;
+}
+static __device__ __noinline__ void merge_rows8(const MergeArgs P, int d, int h, int n_rows, int lane) {
+  int s0 = 0, ns = 0, q_row = -1;
+  if (lane < n_rows) {
+    s0 = __ldcg(P.dec_slot_base + d);
+    ns = __ldcg(P.dec_slot_base + d + 1) - s0;
+    q_row = __ldcg(P.dec_tok + d);
+    SS_CHECK_OR(s0 >= 0 && ns >= 0 && s0 + ns <= P.slots && q_row >= 0 && q_row < P.total_q, P.status, { ns = 0; q_row = -1; });
   }
+  const int ns_max = __reduce_max_sync(0xffffffffu, ns);
+  // lane r + 8 k looks after slot 4 p + k of row r
+  const int r = lane & 7, k = lane >> 3;
+  const int my_s0 = __shfl_sync(0xffffffffu, s0, r), my_ns = __shfl_sync(0xffffffffu, ns, r), my_h = __shfl_sync(0xffffffffu, h, r);
+  auto lse_of = [&](int p) {
+    return 4 * p + k < my_ns ? __ldcg(P.part_lse + static_cast<int64_t>(my_s0 + 4 * p + k) * P.Hq + my_h) : -INFINITY;
+  };
+  auto value = [&](int row, int slot) {                        // (row: a constant after unrolling)
+    const int rs0 = __shfl_sync(0xffffffffu, s0, row), rns = __shfl_sync(0xffffffffu, ns, row), rh = __shfl_sync(0xffffffffu, h, row);
+    return slot < rns ? __ldcg(reinterpret_cast<const float4*>(P.part_o + (static_cast<int64_t>(rs0 + slot) * P.Hq + rh) * kHeadDim + 4 * lane))
+                      : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  float lse = lse_of(0), m = lse;
+  for (int p = 1; 4 * p < ns_max; ++p) m = fmaxf(m, lse_of(p));
+  float4 v[2][8];
 #pragma unroll
-  for (int r = 0; r < 8; ++r) m[r] = warp_max(m[r]);
-  float acc[8][4], l[8];
+  for (int x = 0; x < 8; ++x) { v[0][x] = value(x, 0); v[1][x] = value(x, 1); }
+  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
+  m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+  float4 acc[8];
 #pragma unroll
-  for (int r = 0; r < 8; ++r) { acc[r][0] = acc[r][1] = acc[r][2] = acc[r][3] = 0.f; l[r] = 0.f; }
-  for (int s = s0; s < s1; ++s) {
-    float ls[8];
-    float4 o[8];
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      ls[r] = -INFINITY;
-      o[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (r < n_rows) {
-        ls[r] = __ldcg(P.part_lse + static_cast<int64_t>(s) * P.Hq + h0 + r);
-        o[r] = __ldcg(reinterpret_cast<const float4*>(P.part_o + (static_cast<int64_t>(s) * P.Hq + h0 + r) * kHeadDim + 4 * lane));
-      }
+  for (int x = 0; x < 8; ++x) acc[x] = make_float4(0.f, 0.f, 0.f, 0.f);
+  float l = 0.f, w = 0.f;
+#pragma unroll 1
+  for (int s = 0; s < ns_max; s += 2) {
+    if ((s & 3) == 0) {
+      if (s) lse = lse_of(s >> 2);
+      w = lse == -INFINITY ? 0.f : __expf(lse - m);            // (m = -inf only if every one is)
+      l += w;
     }
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      const float wgt = ls[r] == -INFINITY ? 0.f : __expf(ls[r] - m[r]);   // (m = -inf only if every ls is)
-      l[r] += wgt;
-      acc[r][0] += wgt * o[r].x; acc[r][1] += wgt * o[r].y; acc[r][2] += wgt * o[r].z; acc[r][3] += wgt * o[r].w;
+    for (int x = 0; x < 8; ++x) {
+      const float w0 = __shfl_sync(0xffffffffu, w, x + 8 * (s & 3)), w1 = __shfl_sync(0xffffffffu, w, x + 8 * (s & 3) + 8);
+      if (w0 != 0.f) { acc[x].x += w0 * v[0][x].x; acc[x].y += w0 * v[0][x].y; acc[x].z += w0 * v[0][x].z; acc[x].w += w0 * v[0][x].w; }
+      if (w1 != 0.f) { acc[x].x += w1 * v[1][x].x; acc[x].y += w1 * v[1][x].y; acc[x].z += w1 * v[1][x].z; acc[x].w += w1 * v[1][x].w; }
+    }
+    if (s + 2 < ns_max) {
+#pragma unroll
+      for (int x = 0; x < 8; ++x) { v[0][x] = value(x, s + 2); v[1][x] = value(x, s + 3); }
     }
   }
-  const int64_t q_row = P.dec_tok[d];
+  l += __shfl_xor_sync(0xffffffffu, l, 8);
+  l += __shfl_xor_sync(0xffffffffu, l, 16);
 #pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    if (r >= n_rows) continue;
-    RowState rs;
-    rs.acc[0] = acc[r][0]; rs.acc[1] = acc[r][1]; rs.acc[2] = acc[r][2]; rs.acc[3] = acc[r][3];
-    rs.l = l[r];
-    rs.m = m[r];
-    row_store_final(rs, P, q_row, h0 + r, lane);
+  for (int x = 0; x < 8; ++x) {
+    const int row = __shfl_sync(0xffffffffu, q_row, x), rh = __shfl_sync(0xffffffffu, h, x);
+    const float sum = __shfl_sync(0xffffffffu, l, x), top = __shfl_sync(0xffffffffu, m, x);
+    if (row < 0) continue;
+    const float inv = sum > 0.f ? 1.f / sum : 0.f;
+    const __nv_bfloat162 a = __floats2bfloat162_rn(acc[x].x * inv, acc[x].y * inv), b = __floats2bfloat162_rn(acc[x].z * inv, acc[x].w * inv);
+    uint2 u;
+    u.x = *reinterpret_cast<const uint32_t*>(&a);
+    u.y = *reinterpret_cast<const uint32_t*>(&b);
+    *reinterpret_cast<uint2*>(P.out + (static_cast<int64_t>(row) * P.Hq + rh) * kHeadDim + 4 * lane) = u;
+    if (P.lse && lane == 0) P.lse[static_cast<int64_t>(row) * P.Hq + rh] = sum > 0.f ? top + __logf(sum) : -INFINITY;
   }
 }
 
