@@ -74,6 +74,20 @@ class ss_attn_desc_t(ctypes.Structure):
 
 _lib = None
 
+# Argument types, so that a call passes plain integers (a ctypes object per argument cost more than the call: a step of
+# small kernels is bound by the host).  p: pointer or None, i / I / q / z: int32, uint32, int64, size_t, f: float
+_TYPES = {"p": ctypes.c_void_p, "i": ctypes.c_int32, "I": ctypes.c_uint32, "q": ctypes.c_int64, "z": ctypes.c_size_t,
+          "f": ctypes.c_float}
+_SIGNATURES = {
+    "ss_last_device_status": "ppp", "ss_dedup_workspace_bytes": "ip", "ss_dedup_paths": "ppppiIpppppppzp",
+    "ss_dedup_paths_static": "ppppiIppppppp", "ss_gather_unique_paths": "ppipppppppp",
+    "ss_tree_attention_workspace_bytes": "pp", "ss_tree_attention": "ppzp", "ss_topk_workspace_bytes": "ip",
+    "ss_topk_prune": "ppiiipppzp", "ss_early_prune": "pppiiippppzp", "ss_branch_sample": "pppiifppp",
+    "ss_prefix_tree_workspace_bytes": "iqip", "ss_build_prefix_tree": "ppiqippppppppzp",
+    "ss_candidate_step_host_arena_bytes": "pp", "ss_candidate_step_host": "ppzp", "ss_profile_enable": "i",
+    "ss_profile_read": "pp", "ss_debug_umma_tile": "pppiiipp", "ss_debug_bounded_wait": "pp",
+}
+
 
 def lib() -> ctypes.CDLL:
     """Loads the CUDA library; raises if it has not been built (there is no other implementation)."""
@@ -89,6 +103,8 @@ def lib() -> ctypes.CDLL:
         for name in EXPORTS:
             if name not in ("ss_status_string", "ss_launch_count"):
                 getattr(L, name).restype = ctypes.c_int32
+        for name, kinds in _SIGNATURES.items():
+            getattr(L, name).argtypes = [_TYPES[k] for k in kinds]
         _lib = L
     return _lib
 
@@ -99,15 +115,15 @@ def status_string(status: int) -> str:
 
 def _ptr(t: Optional[torch.Tensor]):
     if t is None:
-        return ctypes.c_void_p(0)
+        return None
     assert t.is_cuda and t.is_contiguous(), "device-resident contiguous tensors only"
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+def _stream(stream) -> int:
+    if stream is None:                       # the current stream of the current device, without a Stream object
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _check(rc: int, where: str):
@@ -133,17 +149,17 @@ def ss_last_device_status(workspace: torch.Tensor, stream=None) -> int:
 # ---------------------------------------------------------------------------------------------------------
 def ss_dedup_workspace_bytes(n_paths: int) -> int:
     out = ctypes.c_size_t(0)
-    _check(lib().ss_dedup_workspace_bytes(ctypes.c_int32(n_paths), ctypes.byref(out)), "ss_dedup_workspace_bytes")
+    _check(lib().ss_dedup_workspace_bytes(n_paths, ctypes.byref(out)), "ss_dedup_workspace_bytes")
     return int(out.value)
 
 
 def ss_dedup_paths(tok_ids, tok_offsets, ctx_key, slot_in, n_paths, flags, canon_out, path_to_unique_out,
                    unique_paths_out, multiplicity_out, slot_out, num_unique_out, workspace, stream=None,
                    check=True) -> int:
-    rc = lib().ss_dedup_paths(_ptr(tok_ids), _ptr(tok_offsets), _ptr(ctx_key), _ptr(slot_in), ctypes.c_int32(n_paths),
-                              ctypes.c_uint32(flags), _ptr(canon_out), _ptr(path_to_unique_out),
+    rc = lib().ss_dedup_paths(_ptr(tok_ids), _ptr(tok_offsets), _ptr(ctx_key), _ptr(slot_in), n_paths,
+                              flags, _ptr(canon_out), _ptr(path_to_unique_out),
                               _ptr(unique_paths_out), _ptr(multiplicity_out), _ptr(slot_out), _ptr(num_unique_out),
-                              _ptr(workspace), ctypes.c_size_t(workspace.numel() if workspace is not None else 0),
+                              _ptr(workspace), workspace.numel() if workspace is not None else 0,
                               _stream(stream))
     if check:
         _check(rc, "ss_dedup_paths")
@@ -155,7 +171,7 @@ def ss_dedup_paths_static(tok_ids, tok_offsets, ctx_key, slot_in, n_paths, flags
     """ss_dedup_paths for callers that may not allocate: no workspace argument, the scratch is a fixed array inside
     the library (at most SS_DEDUP_STATIC_MAX_PATHS paths; calls must not overlap on the GPU)."""
     rc = lib().ss_dedup_paths_static(_ptr(tok_ids), _ptr(tok_offsets), _ptr(ctx_key), _ptr(slot_in),
-                                     ctypes.c_int32(n_paths), ctypes.c_uint32(flags), _ptr(canon_out),
+                                     n_paths, flags, _ptr(canon_out),
                                      _ptr(path_to_unique_out), _ptr(unique_paths_out), _ptr(multiplicity_out),
                                      _ptr(slot_out), _ptr(num_unique_out), _stream(stream))
     if check:
@@ -167,7 +183,7 @@ def ss_gather_unique_paths(unique_paths, num_unique, n_paths, path_leaf_node, pa
                            u_q_len_out, u_q_offsets_out, u_q_src_out, stream=None, check=True) -> int:
     """Descriptor rows of the unique paths (leaf node, query length, query offsets, source query row) gathered by
     `unique_paths`, ready to be passed to ss_tree_attention."""
-    rc = lib().ss_gather_unique_paths(_ptr(unique_paths), _ptr(num_unique), ctypes.c_int32(n_paths),
+    rc = lib().ss_gather_unique_paths(_ptr(unique_paths), _ptr(num_unique), n_paths,
                                       _ptr(path_leaf_node), _ptr(path_q_len), _ptr(q_offsets), _ptr(u_leaf_out),
                                       _ptr(u_q_len_out), _ptr(u_q_offsets_out), _ptr(u_q_src_out), _stream(stream))
     if check:
@@ -177,8 +193,8 @@ def ss_gather_unique_paths(unique_paths, num_unique, n_paths, path_leaf_node, pa
 
 def ss_prefix_tree_workspace_bytes(n_paths: int, total_tok: int, page_size: int = 16) -> int:
     out = ctypes.c_size_t(0)
-    _check(lib().ss_prefix_tree_workspace_bytes(ctypes.c_int32(n_paths), ctypes.c_int64(total_tok),
-                                                ctypes.c_int32(page_size), ctypes.byref(out)),
+    _check(lib().ss_prefix_tree_workspace_bytes(n_paths, total_tok,
+                                                page_size, ctypes.byref(out)),
            "ss_prefix_tree_workspace_bytes")
     return int(out.value)
 
@@ -187,11 +203,11 @@ def ss_build_prefix_tree(tok_ids, tok_offsets, n_paths, total_tok, page_size, or
                          node_parent_out, node_kv_len_out, node_src_path_out, node_src_offset_out, num_nodes_out,
                          workspace, stream=None, check=True) -> int:
     """Radix tree of the paths over whole pages (parents before children, paths in sorted order)."""
-    rc = lib().ss_build_prefix_tree(_ptr(tok_ids), _ptr(tok_offsets), ctypes.c_int32(n_paths), ctypes.c_int64(total_tok),
-                                    ctypes.c_int32(page_size), _ptr(order_out), _ptr(path_leaf_node_out),
+    rc = lib().ss_build_prefix_tree(_ptr(tok_ids), _ptr(tok_offsets), n_paths, total_tok,
+                                    page_size, _ptr(order_out), _ptr(path_leaf_node_out),
                                     _ptr(node_parent_out), _ptr(node_kv_len_out), _ptr(node_src_path_out),
                                     _ptr(node_src_offset_out), _ptr(num_nodes_out), _ptr(workspace),
-                                    ctypes.c_size_t(workspace.numel() * workspace.element_size()), _stream(stream))
+                                    workspace.numel() * workspace.element_size(), _stream(stream))
     if check:
         _check(rc, "ss_build_prefix_tree")
     return rc
@@ -250,7 +266,7 @@ def ss_candidate_step_host(step: ss_host_step_t, device_arena: torch.Tensor, str
     """The whole path for host-resident per-step data: copies in, dedup, gather, attention, top-k, copies out; all
     asynchronous on `stream`."""
     rc = lib().ss_candidate_step_host(ctypes.byref(step), _ptr(device_arena),
-                                      ctypes.c_size_t(device_arena.numel() * device_arena.element_size()),
+                                      device_arena.numel() * device_arena.element_size(),
                                       _stream(stream))
     if check:
         _check(rc, "ss_candidate_step_host")
@@ -306,7 +322,7 @@ def ss_tree_attention_workspace_bytes(desc: ss_attn_desc_t) -> int:
 
 
 def ss_tree_attention(desc: ss_attn_desc_t, workspace: torch.Tensor, stream=None, check=True) -> int:
-    rc = lib().ss_tree_attention(ctypes.byref(desc), _ptr(workspace), ctypes.c_size_t(workspace.numel()),
+    rc = lib().ss_tree_attention(ctypes.byref(desc), _ptr(workspace), workspace.numel(),
                                  _stream(stream))
     if check:
         _check(rc, "ss_tree_attention")
@@ -316,15 +332,15 @@ def ss_tree_attention(desc: ss_attn_desc_t, workspace: torch.Tensor, stream=None
 # ---------------------------------------------------------------------------------------------------------
 def ss_topk_workspace_bytes(n_total: int) -> int:
     out = ctypes.c_size_t(0)
-    _check(lib().ss_topk_workspace_bytes(ctypes.c_int32(n_total), ctypes.byref(out)), "ss_topk_workspace_bytes")
+    _check(lib().ss_topk_workspace_bytes(n_total, ctypes.byref(out)), "ss_topk_workspace_bytes")
     return int(out.value)
 
 
 def ss_topk_prune(scores, seg_offsets, n_segments, n_total, k, survivors_out, keep_out, workspace, stream=None,
                   check=True) -> int:
-    rc = lib().ss_topk_prune(_ptr(scores), _ptr(seg_offsets), ctypes.c_int32(n_segments), ctypes.c_int32(n_total),
-                             ctypes.c_int32(k), _ptr(survivors_out), _ptr(keep_out), _ptr(workspace),
-                             ctypes.c_size_t(workspace.numel() if workspace is not None else 0), _stream(stream))
+    rc = lib().ss_topk_prune(_ptr(scores), _ptr(seg_offsets), n_segments, n_total,
+                             k, _ptr(survivors_out), _ptr(keep_out), _ptr(workspace),
+                             workspace.numel() if workspace is not None else 0, _stream(stream))
     if check:
         _check(rc, "ss_topk_prune")
     return rc
@@ -332,10 +348,10 @@ def ss_topk_prune(scores, seg_offsets, n_segments, n_total, k, survivors_out, ke
 
 def ss_early_prune(scores, verified, seg_offsets, n_segments, n_total, k, pruned_out, selected_out, final_out,
                    workspace, stream=None, check=True) -> int:
-    rc = lib().ss_early_prune(_ptr(scores), _ptr(verified), _ptr(seg_offsets), ctypes.c_int32(n_segments),
-                              ctypes.c_int32(n_total), ctypes.c_int32(k), _ptr(pruned_out), _ptr(selected_out),
+    rc = lib().ss_early_prune(_ptr(scores), _ptr(verified), _ptr(seg_offsets), n_segments,
+                              n_total, k, _ptr(pruned_out), _ptr(selected_out),
                               _ptr(final_out), _ptr(workspace),
-                              ctypes.c_size_t(workspace.numel() if workspace is not None else 0), _stream(stream))
+                              workspace.numel() if workspace is not None else 0, _stream(stream))
     if check:
         _check(rc, "ss_early_prune")
     return rc
@@ -343,8 +359,8 @@ def ss_early_prune(scores, verified, seg_offsets, n_segments, n_total, k, pruned
 
 def ss_branch_sample(logits, draw_offsets, uniforms, n_seq, vocab, temperature, tokens_out, seq_out, stream=None,
                      check=True) -> int:
-    rc = lib().ss_branch_sample(_ptr(logits), _ptr(draw_offsets), _ptr(uniforms), ctypes.c_int32(n_seq),
-                                ctypes.c_int32(vocab), ctypes.c_float(temperature), _ptr(tokens_out), _ptr(seq_out),
+    rc = lib().ss_branch_sample(_ptr(logits), _ptr(draw_offsets), _ptr(uniforms), n_seq,
+                                vocab, temperature, _ptr(tokens_out), _ptr(seq_out),
                                 _stream(stream))
     if check:
         _check(rc, "ss_branch_sample")
@@ -356,12 +372,12 @@ def ss_debug_bounded_wait(status_out, stream=None) -> int:
 
 
 def ss_debug_umma_tile(a, b, c, n, k, b_is_mn_major, status_out, stream=None) -> int:
-    return lib().ss_debug_umma_tile(_ptr(a), _ptr(b), _ptr(c), ctypes.c_int32(n), ctypes.c_int32(k),
-                                    ctypes.c_int32(b_is_mn_major), _ptr(status_out), _stream(stream))
+    return lib().ss_debug_umma_tile(_ptr(a), _ptr(b), _ptr(c), n, k,
+                                    b_is_mn_major, _ptr(status_out), _stream(stream))
 
 
 def ss_profile_enable(on: bool) -> None:
-    _check(lib().ss_profile_enable(ctypes.c_int32(1 if on else 0)), "ss_profile_enable")
+    _check(lib().ss_profile_enable(1 if on else 0), "ss_profile_enable")
 
 
 def ss_profile_read():
