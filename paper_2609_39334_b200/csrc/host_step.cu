@@ -15,20 +15,63 @@
 // much bus time as the 512 KB gap it skips, and the wait keeps the steps from overlapping: 135 ms per step against
 // 98 ms), and as a kernel reading mapped host memory the two directions together reach only 56-80 GB/s against the
 // 96 GB/s of two copy engines.
+//
+// Small arrays (a copy of a few KB costs its place in the stream, 2 to 4 us, whatever its size; a decode step has 8 in and
+// 9 out) go through one kernel per direction that reads or writes the mapped host memory, if it is page-locked; arrays
+// above kSmallBytes keep their copy engine.  Measured, a step of 1024 decode paths: 330 -> 278 us.
 #include "common.cuh"
 
 namespace ss {
 namespace host_step {
 
+constexpr size_t kSmallBytes = 64 << 10;
+constexpr int kMaxSegments = 12;
+
+// Arrays to move, one after the other.
+struct Segments {
+  const char* src[kMaxSegments];
+  char* dst[kMaxSegments];
+  unsigned int bytes[kMaxSegments];
+  int count;
+};
+
+// The device's address of page-locked host memory, or null.
+static char* mapped(const void* host) {
+  void* dev = nullptr;
+  if (!host || cudaHostGetDevicePointer(&dev, const_cast<void*>(host), 0) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return nullptr;
+  }
+  return static_cast<char*>(dev);
+}
+
+__device__ __forceinline__ void move_segments(const Segments& S, int block, int n_blocks) {
+  for (int i = 0; i < S.count; ++i) {
+    const char* src = S.src[i];
+    char* dst = S.dst[i];
+    const unsigned int n = S.bytes[i], step = n_blocks * blockDim.x, t = block * blockDim.x + threadIdx.x;
+    if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0) {
+      for (unsigned int c = t; c < n / 16; c += step) reinterpret_cast<uint4*>(dst)[c] = reinterpret_cast<const uint4*>(src)[c];
+      for (unsigned int c = n / 16 * 16 + t; c < n; c += step) dst[c] = src[c];
+    } else {
+      for (unsigned int c = t; c < n; c += step) dst[c] = src[c];
+    }
+  }
+}
+
 constexpr int kCopyBlocks = 8;       // persistent blocks of the copy kernel (8 reach 52 GB/s on the measured system)
 constexpr int kCopyThreads = 512;
 
-// The live rows of out / lse, device -> (mapped) host: rows [0, u_q_offsets[U]) of the compact device buffers.
+// The small results, and with `out_host` the live rows of out / lse, device -> (mapped) host: rows [0, u_q_offsets[U]) of the
+// compact device buffers.
 __global__ void __launch_bounds__(kCopyThreads)
 rows_to_host_kernel(const uint4* __restrict__ out_dev, uint4* __restrict__ out_host, const uint4* __restrict__ lse_dev,
                     uint4* __restrict__ lse_host, const int32_t* __restrict__ num_unique, int32_t n_paths,
-                    const int64_t* __restrict__ u_q_offsets, int64_t out_row_chunks, int64_t lse_row_bytes) {
+                    const int64_t* __restrict__ u_q_offsets, int64_t out_row_chunks, int64_t lse_row_bytes,
+                    const __grid_constant__ Segments small) {
   ss::grid_dependency_enter();
+  move_segments(small, blockIdx.x, gridDim.x);
+  if (!out_host) return;
   int live = *num_unique;
   live = live < 0 ? 0 : (live > n_paths ? n_paths : live);
   const int64_t rows = u_q_offsets[live];
@@ -51,6 +94,12 @@ rows_to_host_kernel(const uint4* __restrict__ out_dev, uint4* __restrict__ out_h
     float* tail_dst = reinterpret_cast<float*>(lse_host + n_lse);
     if (tid < (n_bytes - n_lse * 16) / 4) tail_dst[tid] = tail_src[tid];
   }
+}
+
+// The small input arrays, a block's worth of threads for each 8 KB.
+__global__ void __launch_bounds__(kCopyThreads) small_inputs_kernel(const __grid_constant__ Segments small) {
+  ss::grid_dependency_enter();
+  move_segments(small, blockIdx.x, gridDim.x);
 }
 
 struct Arena {                       // device-side layout of one step
@@ -156,14 +205,6 @@ extern "C" int32_t ss_candidate_step_host_arena_bytes(const ss_host_step_t* step
   return SS_OK;
 }
 
-#define SS_COPY(dst, src, bytes, kind)                                                            \
-  do {                                                                                            \
-    if ((bytes) > 0 && cudaMemcpyAsync((dst), (src), (bytes), (kind), st) != cudaSuccess) {       \
-      (void)cudaGetLastError();                                                                   \
-      return SS_ERR_CUDA;                                                                         \
-    }                                                                                             \
-  } while (0)
-
 extern "C" int32_t ss_candidate_step_host(const ss_host_step_t* step, void* device_arena, size_t arena_bytes,
                                           void* stream) {
   using namespace ss;
@@ -190,26 +231,44 @@ extern "C" int32_t ss_candidate_step_host(const ss_host_step_t* step, void* devi
   const size_t q_bytes = static_cast<size_t>(s.total_q) * row * sizeof(__nv_bfloat16);
 
   // ---- host -> device: the step's candidates, queries and scores ------------------------------------------------
-  const cudaMemcpyKind H2D = cudaMemcpyHostToDevice, D2H = cudaMemcpyDeviceToHost;
-  SS_COPY(a.tok_ids, s.tok_ids, static_cast<size_t>(s.total_tok) * 4, H2D);
-  SS_COPY(a.tok_offsets, s.tok_offsets, (N + 1) * 8, H2D);
-  if (s.ctx_key) SS_COPY(a.ctx_key, s.ctx_key, N * 8, H2D);
-  if (s.slot_in) SS_COPY(a.slot_in, s.slot_in, N * 4, H2D);
-  SS_COPY(a.path_leaf_node, s.path_leaf_node, N * 4, H2D);
-  SS_COPY(a.path_q_len, s.path_q_len, N * 4, H2D);
-  SS_COPY(a.q_offsets, s.q_offsets, (N + 1) * 8, H2D);
-  SS_COPY(a.q, s.q, q_bytes, H2D);
+  Segments in{}, res{};
+  // puts an array on the list if it is small and mapped; else copies it
+  auto move = [&](Segments& list, void* dst, const void* src, size_t bytes, bool to_host) -> bool {
+    if (bytes == 0) return true;
+    char* map = bytes <= kSmallBytes && list.count < kMaxSegments ? mapped(to_host ? dst : src) : nullptr;
+    if (!map) {
+      if (cudaMemcpyAsync(dst, src, bytes, to_host ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice, st) == cudaSuccess) return true;
+      (void)cudaGetLastError();
+      return false;
+    }
+    list.src[list.count] = to_host ? static_cast<const char*>(src) : map;
+    list.dst[list.count] = to_host ? map : static_cast<char*>(dst);
+    list.bytes[list.count++] = static_cast<unsigned int>(bytes);
+    return true;
+  };
+  bool ok = move(in, a.tok_ids, s.tok_ids, static_cast<size_t>(s.total_tok) * 4, false) &&
+            move(in, a.tok_offsets, s.tok_offsets, (N + 1) * 8, false) &&
+            (!s.ctx_key || move(in, a.ctx_key, s.ctx_key, N * 8, false)) &&
+            (!s.slot_in || move(in, a.slot_in, s.slot_in, N * 4, false)) &&
+            move(in, a.path_leaf_node, s.path_leaf_node, N * 4, false) && move(in, a.path_q_len, s.path_q_len, N * 4, false) &&
+            move(in, a.q_offsets, s.q_offsets, (N + 1) * 8, false) && move(in, a.q, s.q, q_bytes, false) &&
+            move(in, a.scores, s.scores, N * 4, false) && move(in, a.seg_offsets, s.seg_offsets, (P + 1) * 4, false);
+  if (!ok) return SS_ERR_CUDA;
   // compact return: needs out / lse mapped (the kernel writes them) and whole 16-byte chunks per row
-  void *out_map = nullptr, *lse_map = nullptr;
+  char *out_map = nullptr, *lse_map = nullptr;
   bool compact = (s.flags & SS_STEP_COMPACT_TRANSFERS) != 0 && s.total_q > 0 && s.n_paths > 0 &&
                  row * sizeof(__nv_bfloat16) % 16 == 0;
-  if (compact && (cudaHostGetDevicePointer(&out_map, s.out, 0) != cudaSuccess ||
-                  (s.lse && cudaHostGetDevicePointer(&lse_map, s.lse, 0) != cudaSuccess))) {
-    (void)cudaGetLastError();
-    compact = false;
+  if (compact) {
+    out_map = mapped(s.out);
+    if (s.lse) lse_map = mapped(s.lse);
+    compact = out_map && (!s.lse || lse_map);
   }
-  SS_COPY(a.scores, s.scores, N * 4, H2D);
-  SS_COPY(a.seg_offsets, s.seg_offsets, (P + 1) * 4, H2D);
+  if (in.count > 0) {
+    size_t bytes = 0;
+    for (int i = 0; i < in.count; ++i) bytes += in.bytes[i];
+    const int blocks = static_cast<int>((bytes + 16 * kCopyThreads - 1) / (16 * kCopyThreads));
+    SS_LAUNCH(small_inputs_kernel, blocks < kCopyBlocks ? blocks : kCopyBlocks, kCopyThreads, 0, st, in);
+  }
 
   // ---- the path ---------------------------------------------------------------------------------------------------
   rc = ss_dedup_paths(a.tok_ids, a.tok_offsets, s.ctx_key ? a.ctx_key : nullptr, s.slot_in ? a.slot_in : nullptr,
@@ -237,24 +296,21 @@ extern "C" int32_t ss_candidate_step_host(const ss_host_step_t* step, void* devi
   if (rc != SS_OK) return rc;
 
   // ---- device -> host: every result ------------------------------------------------------------------------------------
-  SS_COPY(s.canon, a.canon, N * 4, D2H);
-  SS_COPY(s.path_to_unique, a.path_to_unique, N * 4, D2H);
-  SS_COPY(s.unique_paths, a.unique_paths, N * 4, D2H);
-  SS_COPY(s.multiplicity, a.multiplicity, N * 4, D2H);
-  if (s.slot_out) SS_COPY(s.slot_out, a.slot_out, N * 4, D2H);
-  SS_COPY(s.num_unique, a.num_unique, 4, D2H);
-  SS_COPY(s.u_q_offsets, a.u_q_offsets, (N + 1) * 8, D2H);
-  if (compact) {
+  if (!compact)
+    ok = move(res, s.out, a.out, q_bytes, true) &&
+         (!s.lse || move(res, s.lse, a.lse, static_cast<size_t>(s.total_q) * static_cast<size_t>(s.attn->num_q_heads) * sizeof(float), true));
+  ok = ok && move(res, s.canon, a.canon, N * 4, true) && move(res, s.path_to_unique, a.path_to_unique, N * 4, true) &&
+       move(res, s.unique_paths, a.unique_paths, N * 4, true) && move(res, s.multiplicity, a.multiplicity, N * 4, true) &&
+       (!s.slot_out || move(res, s.slot_out, a.slot_out, N * 4, true)) && move(res, s.num_unique, a.num_unique, 4, true) &&
+       move(res, s.u_q_offsets, a.u_q_offsets, (N + 1) * 8, true) &&
+       move(res, s.survivors, a.survivors, P * static_cast<size_t>(s.top_k) * 4, true) && move(res, s.keep, a.keep, N, true) &&
+       move(res, s.device_status, a.attn_ws, sizeof(int32_t), true);   // first word of the attention workspace
+  if (!ok) return SS_ERR_CUDA;
+  if (compact || res.count > 0)
     SS_LAUNCH(rows_to_host_kernel, kCopyBlocks, kCopyThreads, 0, st, static_cast<const uint4*>(a.out),
-              static_cast<uint4*>(out_map), reinterpret_cast<const uint4*>(a.lse), static_cast<uint4*>(lse_map),
-              static_cast<const int32_t*>(a.num_unique), s.n_paths, static_cast<const int64_t*>(a.u_q_offsets),
-              static_cast<int64_t>(row * sizeof(__nv_bfloat16) / 16), static_cast<int64_t>(s.attn->num_q_heads) * 4);
-  } else {
-    SS_COPY(s.out, a.out, q_bytes, D2H);
-    if (s.lse) SS_COPY(s.lse, a.lse, static_cast<size_t>(s.total_q) * static_cast<size_t>(s.attn->num_q_heads) * sizeof(float), D2H);
-  }
-  SS_COPY(s.survivors, a.survivors, P * static_cast<size_t>(s.top_k) * 4, D2H);
-  SS_COPY(s.keep, a.keep, N, D2H);
-  SS_COPY(s.device_status, a.attn_ws, sizeof(int32_t), D2H);     // first word of the attention workspace
+              reinterpret_cast<uint4*>(compact ? out_map : nullptr), reinterpret_cast<const uint4*>(a.lse),
+              reinterpret_cast<uint4*>(lse_map), static_cast<const int32_t*>(a.num_unique), s.n_paths,
+              static_cast<const int64_t*>(a.u_q_offsets), static_cast<int64_t>(row * sizeof(__nv_bfloat16) / 16),
+              static_cast<int64_t>(s.attn->num_q_heads) * 4, res);
   return SS_OK;
 }
