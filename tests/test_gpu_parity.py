@@ -742,3 +742,15 @@ def test_ragged_ends_do_not_race_with_late_value_copies():
         bits = live.view(torch.int16).clone()
         assert first is None or torch.equal(bits, first)
         first = bits
+
+
+@pytest.mark.parametrize("flags", [0, B.SS_FLAG_WEAK_HASH])
+@pytest.mark.parametrize("n,max_len", [(95, 3), (96, 2), (97, 3), (64, 400)])
+def test_dedup_at_the_edge_of_the_one_launch_form(n, max_len, flags):
+    rng = np.random.default_rng(n * 7 + max_len)
+    ids, off, ctx, slot = dedup_case(rng, n, 2, max_len, 2)
+    got = run_dedup(ids, off, ctx, slot, flags)
+    want = oracle.dedup(ids, off, ctx, slot)
+    assert got["num_unique"] == want["num_unique"]
+    for key in ("canon", "path_to_unique", "unique_paths", "multiplicity", "slot_out"):
+        assert np.array_equal(got[key], want[key]), key
