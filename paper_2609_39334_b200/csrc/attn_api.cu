@@ -72,17 +72,13 @@ static Layout carve(const ss_attn_desc_t* d, char* base, Params* P) {
   const int64_t cap_dec = d->max_decode_paths > 0 ? (d->max_decode_paths < d->num_paths ? d->max_decode_paths : d->num_paths)
                                                   : d->num_paths;
   const int target = 2 * sm_count_of_current_device();   // (the size query and the call must see the same device)
-  // Keys per leaf item.  (Finer items - 128 or 64 keys - were measured on the small configurations, where a warp of
-  // the leaf kernel gets fewer than two items: the extra partials, counters and merges cost more than the better
-  // balance gains, 0.50 -> 0.41 of the HBM rate at 64 keys; whole-leaf items of up to 512 keys: no gain either.)
-  const int leaf_chunk = kLeafChunk;
   Caps caps;
   caps.dec = static_cast<int32_t>(cap_dec);
   const int64_t stacked = static_cast<int64_t>(Hkv) * (cap_dec * max_depth / tpt + d->num_nodes) + target + Hkv * kMaxRootSplits;
   const int64_t chain = static_cast<int64_t>(Hkv) * (d->total_q / tpt + d->num_paths);
   caps.tile_items = static_cast<int32_t>(stacked + chain);
-  caps.leaf_items = static_cast<int32_t>(static_cast<int64_t>(Hkv) * (d->total_node_pages * kPage / leaf_chunk + cap_dec));
-  caps.slots = cap_dec * (kMaxRootSplits + max_depth) + d->total_node_pages * kPage / leaf_chunk;
+  caps.leaf_items = static_cast<int32_t>(static_cast<int64_t>(Hkv) * (d->total_node_pages * kPage / kLeafChunk + cap_dec));
+  caps.slots = cap_dec * (kMaxRootSplits + max_depth) + d->total_node_pages * kPage / kLeafChunk;
 
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes); return base ? base + o : nullptr; };
@@ -120,7 +116,6 @@ static Layout carve(const ss_attn_desc_t* d, char* base, Params* P) {
     P->part_lse = reinterpret_cast<float*>(part_lse);
     P->caps = caps;
     P->target_tiles = target;
-    P->leaf_chunk = leaf_chunk;
   }
   Layout L;
   L.total = off;

@@ -11,7 +11,7 @@
 // fetches whatever the number of blocks) and then writes its share of the item lists.  Larger inputs take four launches
 // (nodes, paths and emit grid-parallel, scan in one block).  Bound: the latency of seven phases behind barriers, and of
 // code that runs once (instruction fetches).  Measured, against one block that shared the phases of the general path and
-// searched a path for every item: 922 unique paths 20.9 -> 14.2 us, 256 verification paths 29.1 -> 10.8, 8 paths 12.0 -> 8.8.
+// searched a path for every item: 922 unique paths 20.9 -> 11.5 us, 256 verification paths 29.1 -> 8.2, 8 paths 12.0 -> 8.1.
 // The header (status word first) is cleared by the host-side launcher before the first of the four kernels; the
 // small planner builds it in shared memory and its block 0 writes it out whole.
 #include "attn_plan.cuh"
@@ -327,7 +327,7 @@ __device__ __forceinline__ void plan_scan_phase(const Params& P, int32_t* stage)
     int splits = 1, own = 0, split_len = len;
     if (nd > 0 && len > 0) {
       if (tiles == 0) {
-        own = ceil_div(len, P.leaf_chunk);             // private leaf of one decode path
+        own = ceil_div(len, kLeafChunk);             // private leaf of one decode path
       } else {
         if (P.node_depth[n] == 0) node_split(P, len, total_tiles, splits, split_len);
         own = splits;
@@ -358,7 +358,7 @@ __device__ __forceinline__ void plan_scan_phase(const Params& P, int32_t* stage)
       const int leaf = P.path_leaf_node[p];
       slots = P.node_level_off[leaf] + P.node_own_slots[leaf];
       if (P.node_npaths[leaf] == 1 && P.node_kv_len[leaf] > 0)
-        leaf_items = ceil_div(P.node_kv_len[leaf], P.leaf_chunk) * P.Hkv;
+        leaf_items = ceil_div(P.node_kv_len[leaf], kLeafChunk) * P.Hkv;
     } else if (cls == kClassChain) {
       chain_items = ceil_div(P.path_q_len[p], tpt) * P.Hkv;
     }
@@ -420,7 +420,7 @@ __device__ __forceinline__ void plan_emit_phase(const Params& P) {
     P.dec_src[rank] = static_cast<int32_t>(P.q_src_offsets ? P.q_src_offsets[p] : P.q_offsets[p]);
     P.dec_slot_base[rank] = P.path_slot_base[p];
     const bool own_leaf = P.node_npaths[leaf] == 1 && len > 0;
-    P.dec_leaf_chunks[rank] = own_leaf ? ceil_div(len, P.leaf_chunk) : 0;
+    P.dec_leaf_chunks[rank] = own_leaf ? ceil_div(len, kLeafChunk) : 0;
     for (int g = 0; g < P.Hkv; ++g) P.leaf_arrive[static_cast<int64_t>(rank) * P.Hkv + g] = 0;
   }
   // Leaf and chain items, one thread per ITEM (consecutive threads write consecutive descriptors: a thread per path
@@ -443,11 +443,11 @@ __device__ __forceinline__ void plan_emit_phase(const Params& P) {
     const int leaf = P.path_leaf_node[p];
     const int len = P.node_kv_len[leaf];
     LeafItem it;
-    it.page0 = static_cast<int32_t>(P.node_page_offsets[leaf]) + c * (P.leaf_chunk / kPage);
+    it.page0 = static_cast<int32_t>(P.node_page_offsets[leaf]) + c * (kLeafChunk / kPage);
     it.node = leaf;
     it.g = g;
-    it.kv_begin = c * P.leaf_chunk;
-    it.kv_end = min(len, (c + 1) * P.leaf_chunk);
+    it.kv_begin = c * kLeafChunk;
+    it.kv_end = min(len, (c + 1) * kLeafChunk);
     it.slot = P.path_slot_base[p] + P.node_level_off[leaf] + c;
     it.q_src = static_cast<int32_t>(P.q_src_offsets ? P.q_src_offsets[p] : P.q_offsets[p]);
     it.dec = P.path_dec_rank[p];
@@ -539,8 +539,8 @@ inline size_t small_plan_smem(int N, int NP) {
 }
 // Blocks: what is left to share is the emission, a warp per path and per node.
 inline int small_plan_blocks(int N, int NP) {
-  const int b = (N + NP + 127) / 128;
-  return b < 1 ? 1 : (b > 24 ? 24 : b);
+  const int b = (N + NP + 31) / 32;
+  return b < 1 ? 1 : (b > 64 ? 64 : b);
 }
 constexpr int kLeafClasses = 17;               // pages of the last chunk of a leaf: 0 .. 16
 
@@ -645,27 +645,40 @@ __global__ void __launch_bounds__(kScanThreads) plan_small_kernel(const __grid_c
   const int live = live_paths(P);
   bool bad = false;
 #pragma unroll 1
-  for (int n = tid; n < N; n += kScanThreads) {
-    const int parent = P.node_parent[n], len = P.node_kv_len[n];
-    const int64_t o0 = P.node_page_offsets[n], o1 = P.node_page_offsets[n + 1];
-    bad = bad || parent >= n || parent < -1 || len < 0 || o1 < o0 || (o1 - o0) * kPage < len || o1 > P.total_node_pages || o0 < 0;
-    n_parent[n] = parent;
-    n_len[n] = len;
-    n_page0[n] = static_cast<int32_t>(o0);
-    n_first[n] = 0x7fffffff;
-    n_last[n] = -1;
-    n_paths[n] = n_dec[n] = 0;
-  }
-#pragma unroll 1
-  for (int p = tid; p < NP; p += kScanThreads) {
-    const int leaf = P.path_leaf_node[p], T = P.path_q_len[p];
-    const int64_t r0 = P.q_offsets[p], r1 = P.q_offsets[p + 1], src = P.q_src_offsets ? P.q_src_offsets[p] : r0;
-    bool ok = leaf >= 0 && leaf < N && T >= 1 && r1 - r0 == T && r0 >= 0 && r1 <= P.total_q;
-    if (P.q_src_offsets) ok = ok && src >= 0 && src + T <= P.q_src_rows && src + T <= 0x7fffffffLL;
-    p_leaf[p] = ok ? leaf : -1;
-    p_T[p] = T;
-    p_row[p] = static_cast<int32_t>(r0);
-    p_src[p] = static_cast<int32_t>(src);
+  for (int i = tid; i < max(N, NP); i += kScanThreads) {       // (node i and path i: their loads go out together)
+    const int n = min(i, N - 1), p = min(i, NP - 1);
+    int parent = 0, len = 0, leaf = 0, T = 0;
+    int64_t o0 = 0, o1 = 0, r0 = 0, r1 = 0, src = 0;
+    if (N > 0) {
+      parent = P.node_parent[n];
+      len = P.node_kv_len[n];
+      o0 = P.node_page_offsets[n];
+      o1 = P.node_page_offsets[n + 1];
+    }
+    if (NP > 0) {
+      leaf = P.path_leaf_node[p];
+      T = P.path_q_len[p];
+      r0 = P.q_offsets[p];
+      r1 = P.q_offsets[p + 1];
+      src = P.q_src_offsets ? P.q_src_offsets[p] : r0;
+    }
+    if (i < N) {
+      bad = bad || parent >= n || parent < -1 || len < 0 || o1 < o0 || (o1 - o0) * kPage < len || o1 > P.total_node_pages || o0 < 0;
+      n_parent[n] = parent;
+      n_len[n] = len;
+      n_page0[n] = static_cast<int32_t>(o0);
+      n_first[n] = 0x7fffffff;
+      n_last[n] = -1;
+      n_paths[n] = n_dec[n] = 0;
+    }
+    if (i < NP) {
+      bool ok = leaf >= 0 && leaf < N && T >= 1 && r1 - r0 == T && r0 >= 0 && r1 <= P.total_q;
+      if (P.q_src_offsets) ok = ok && src >= 0 && src + T <= P.q_src_rows && src + T <= 0x7fffffffLL;
+      p_leaf[p] = ok ? leaf : -1;
+      p_T[p] = T;
+      p_row[p] = static_cast<int32_t>(r0);
+      p_src[p] = static_cast<int32_t>(src);
+    }
   }
   if (P.flags & SS_FLAG_VALIDATE) {
     for (int64_t i = tid; i < P.total_node_pages; i += kScanThreads) {
@@ -758,7 +771,7 @@ __global__ void __launch_bounds__(kScanThreads) plan_small_kernel(const __grid_c
         if (n_parent[n] < 0) node_split(P, len, total_tiles, splits, split_len);
         own = splits;
       } else if (n_dec[n] > 0 && len > 0) {
-        own = ceil_div(len, P.leaf_chunk);                     // private leaf of one decode path
+        own = ceil_div(len, kLeafChunk);                     // private leaf of one decode path
       }
       n_splits[n] = splits;
       n_split_len[n] = split_len;
@@ -787,8 +800,8 @@ __global__ void __launch_bounds__(kScanThreads) plan_small_kernel(const __grid_c
 #pragma unroll 1
           for (int a = leaf; a >= 0; a = n_parent[a]) slots += n_own[a];
           if (n_paths[leaf] == 1 && len > 0) {
-            full = len / P.leaf_chunk;
-            c = ceil_div(len - full * P.leaf_chunk, kPage);
+            full = len / kLeafChunk;
+            c = ceil_div(len - full * kLeafChunk, kPage);
           }
         } else if (p_class[i] == kClassChain) {
           chain = ceil_div(p_T[i], tpt) * Hkv;
@@ -852,22 +865,22 @@ __global__ void __launch_bounds__(kScanThreads) plan_small_kernel(const __grid_c
             P.dec_tok[rank] = p_row[p];
             P.dec_src[rank] = p_src[p];
             P.dec_slot_base[rank] = slot;
-            P.dec_leaf_chunks[rank] = own_leaf ? ceil_div(len, P.leaf_chunk) : 0;
+            P.dec_leaf_chunks[rank] = own_leaf ? ceil_div(len, kLeafChunk) : 0;
           }
           for (int g = lane; g < Hkv; g += 32) P.leaf_arrive[static_cast<int64_t>(rank) * Hkv + g] = 0;
           if (!own_leaf) continue;
           // whole chunks first, then the last chunks of all leaves, longest first: the leaf kernel hands its items out in
           // this order, and the short ones level out its warps' ends (922 leaves of 32 to 512 keys: 71.6 -> 68.9 us)
-          const int full = len / P.leaf_chunk, last = p_last[p], n_items = (full + (last >= 0 ? 1 : 0)) * Hkv;
+          const int full = len / kLeafChunk, last = p_last[p], n_items = (full + (last >= 0 ? 1 : 0)) * Hkv;
 #pragma unroll 1
           for (int x = lane; x < n_items; x += 32) {
             const int c = x / Hkv, g = x - c * Hkv;
             LeafItem it;
-            it.page0 = n_page0[leaf] + c * (P.leaf_chunk / kPage);
+            it.page0 = n_page0[leaf] + c * (kLeafChunk / kPage);
             it.node = leaf;
             it.g = g;
-            it.kv_begin = c * P.leaf_chunk;
-            it.kv_end = min(len, (c + 1) * P.leaf_chunk);
+            it.kv_begin = c * kLeafChunk;
+            it.kv_end = min(len, (c + 1) * kLeafChunk);
             it.slot = slot + n_level[leaf] + c;
             it.q_src = p_src[p];
             it.dec = rank;
