@@ -6,16 +6,16 @@
 // (a cooperative launch).  No token is hashed and none that is known to be shared is read twice.
 //
 //   sort    The paths are sorted by refinement (a multikey quicksort with longest common prefixes as keys).  All
-//           positions start in one group.  In a round every group of two or more picks one of its paths as the pivot, and
-//           every other member compares itself with it, from the length that the group is known to share: a warp per path,
-//           streaming both.  Its key - below or above the pivot, common length, first differing token - sorts the group;
+//           positions start in one group; round 0 sorts by the first token.  In a round every group of two or more picks one
+//           of its paths as the pivot, and every other member compares itself with it, from the length that the group is known
+//           to share: a warp per path, streaming both.  Its key - below or above the pivot, common length, first differing token - sorts the group;
 //           members with equal keys share that many tokens plus one, and make a group of the next round.  Members that equal
 //           the pivot, or that end where they differ from it, are settled.  Neighbours that were told apart in a round share
 //           exactly the smaller of their two lengths, so the common prefixes of the sorted neighbours, which the tree is made
 //           of, come out of the keys.  A round settles at least the pivots; the pivot is picked pseudo-randomly, so the number
 //           of rounds is that of a quicksort's levels in the worst case and the depth of the tree in ordinary ones (3 or 4).
 //             compare   a warp per position: boundaries of the groups from the last round's sorted keys (32-ary search), then
-//                       the new key; a group of up to 8 that has been through a round is finished at once, every member
+//                       the new key; a group of up to 8 that has met a pivot is finished at once, every member
 //                       against every other (its rank is the number below it, what it shares with the rank before the
 //                       most that it shares with any of them)
 //             ranks     a warp per position counts the smaller keys of its group; with groups of more than 256 a block per
@@ -26,8 +26,8 @@
 //           the intervals per start rank; parents follow from the neighbours of an interval.
 //
 // Bound: HBM, one pass over the shared prefixes (268 MB for 16384 paths with prompts of 4096 tokens, 41 us), and for small
-// inputs the latency of a dozen dependent phases.  Measured: 16384 paths / 76 M ids 169 us (of which 61 the pass over the
-// prompts; page hashes, a bitonic sort with a string comparator and a pass over the neighbours: 1729), 64 paths 26 us (135).
+// inputs the latency of a dozen dependent phases.  Measured: 16384 paths / 76 M ids 151 us (of which 61 the pass over the
+// prompts; page hashes, a bitonic sort with a string comparator and a pass over the neighbours: 1729), 64 paths 25 us (135).
 #include "common.cuh"
 
 namespace ss {
@@ -35,8 +35,10 @@ namespace ptree {
 
 constexpr int kThreads = 1024;
 constexpr int kWarps = kThreads / 32;
-constexpr int kTile = 1024;                       // positions that a block sorts in shared memory
-constexpr int kUnroll = 8;                        // 128-byte loads in flight per warp and path
+constexpr int kTile = 1024;                       // positions that are sorted in shared memory together (16384 paths: 1024 151
+                                                  // us, 512 159, 256 173; below a few thousand 2 to 4 us less with 256)
+constexpr int kUnroll = 8;                        // 128-byte loads in flight per warp and path (16384 paths: 8 151 us, 16 148;
+                                                  // 512 paths 46.8 and 48.1)
 constexpr int kPairs = 8;                         // a group of up to this many is finished with all pairs: 7 comparisons in a
                                                   // row (9 us) against two or three more rounds (8 us each)
 constexpr int kCount = 256;                       // ranks by counting up to this group size: 8 keys a lane (1.2 us) against a
@@ -58,7 +60,7 @@ struct Args {
   int *bmin, *c_start, *c_end, *outer, *cnt, *block_sum;
   int32_t *order, *path_leaf_node, *node_parent, *node_kv_len, *node_src_path, *node_src_offset, *num_nodes;
 };
-constexpr unsigned int kMore = 1, kBig = 2;
+constexpr unsigned int kMore = 1, kBig = 2, kMixed = 4;
 
 // ---- barrier over all blocks ----------------------------------------------------------------------------------------
 // False when the wait ran out (status SS_ERR_TIMEOUT; every block leaves).  A grid that is one cluster uses the hardware's
@@ -177,12 +179,13 @@ __device__ __forceinline__ int count_below(const uint64_t* k, int len, uint64_t 
   return lo + __popc(__ballot_sync(0xffffffffu, lane < len && (OR_EQUAL ? v <= key : v < key)));
 }
 
-// Sorts positions tile * kTile .. by (group, key, position): keys and paths of the round, kin / pin -> kout / pout.  An
-// entry per thread; partners in the warp through shuffles, the others through shared memory.
-__device__ void sort_tile(const Args& A, int tile, const uint64_t* kin, const int* pin, uint64_t* kout, int* pout) {
-  __shared__ uint64_t s_key[kTile];
-  __shared__ uint32_t s_at[kTile];
-  const int p0 = tile * kTile, count = min(kTile, A.n - p0), tid = threadIdx.x;
+// Sorts the positions of kThreads / kTile tiles, each by (group, key, position): keys and paths of the round, kin / pin ->
+// kout / pout.  An entry per thread; partners in the warp through shuffles, the others through shared memory.
+__device__ void sort_tiles(const Args& A, int first_tile, const uint64_t* kin, const int* pin, uint64_t* kout, int* pout) {
+  __shared__ uint64_t s_key[kThreads];
+  __shared__ uint32_t s_at[kThreads];
+  const int tid = threadIdx.x % kTile, at0 = threadIdx.x - tid;   // position in the tile, the tile's place in shared memory
+  const int p0 = (first_tile + threadIdx.x / kTile) * kTile, count = min(kTile, A.n - p0);
   uint64_t k = ~0ull;
   uint32_t at = 0xffffffffu;                                  // first position of the group in the tile << 16 | position
   bool open = false;
@@ -193,18 +196,18 @@ __device__ void sort_tile(const Args& A, int tile, const uint64_t* kin, const in
     at = (static_cast<uint32_t>(max(g - p0, 0)) << 16) | static_cast<uint32_t>(tid);
   }
   if (!__syncthreads_or(open)) return;
-  int n_pad = 2;
-  while (n_pad < count) n_pad <<= 1;
+  int n_pad = 2;                                              // (of the block's first tile, the fullest)
+  while (n_pad < min(kTile, A.n - first_tile * kTile)) n_pad <<= 1;
   for (int size = 2; size <= n_pad; size <<= 1) {
     for (int stride = size >> 1; stride > 0; stride >>= 1) {
       uint64_t kb;
       uint32_t ab;
       if (stride >= 32) {
-        s_key[tid] = k;
-        s_at[tid] = at;
+        s_key[at0 + tid] = k;
+        s_at[at0 + tid] = at;
         __syncthreads();
-        kb = s_key[tid ^ stride];
-        ab = s_at[tid ^ stride];
+        kb = s_key[at0 + (tid ^ stride)];
+        ab = s_at[at0 + (tid ^ stride)];
         __syncthreads();
       } else {
         kb = __shfl_xor_sync(0xffffffffu, k, stride);
@@ -312,19 +315,37 @@ __device__ __forceinline__ void build(const Args& A) {
   for (unsigned int round = 0;; ++round) {
     const uint64_t* ks = A.key[kc];
     unsigned int need = 0;
-    for (int p = wid; p < n; p += n_warps) {
-      int g = 0, e = n, base = 0, me = p;
-      if (round > 0) {
-        g = A.gs[p];
-        e = A.ge[p];
-        if (e - g == 1) continue;                              // settled
+    if (round == 0) {
+      // Against the empty path: the key is the first token (a warp that compares two long paths of one problem would hold
+      // up all others).  If all of them begin alike there is nothing to sort.
+      auto first_key = [&](int i) {
+        const int64_t o = A.tok_offsets[i];
+        return make_key(A.tok_offsets[i + 1] > o ? Order{0, 1, false, ordered(__ldg(A.tok_ids + o))} : Order{0, 0, true, 0});
+      };
+      const uint64_t key0 = first_key(0);
+      for (int p = blockIdx.x * kThreads + threadIdx.x; p < n; p += gridDim.x * kThreads) {
+        const uint64_t k = first_key(p);
+        A.key[0][p] = A.key[1][p] = k;
+        A.perm[pc][p] = p;
+        A.gs[p] = 0;
+        A.ge[p] = n;
+        if (p == 0) A.lcp[0] = 0;
+        if (n == 1) A.order[0] = 0;
+        else need |= kMore | (n > kCount ? kBig : 0) | (k != key0 ? kMixed : 0);
+      }
+      need = __reduce_or_sync(0xffffffffu, need);
+    }
+    for (int p = wid; round > 0 && p < n; p += n_warps) {
+      int g = A.gs[p], e = A.ge[p], base, me;
+      if (e - g == 1) continue;                                // settled
+      {
         me = A.perm[pc][p];
         const uint64_t k = ks[p];
         const int g1 = g + count_below<false>(ks + g, e - g, k, lane), e1 = g + count_below<true>(ks + g, e - g, k, lane);
         const int m = e1 - g1;
         if (lane == 0 && p == g1 && p > g) A.lcp[p] = static_cast<int>(min(key_len(ks[p - 1]), key_len(k))) / A.page;
         base = static_cast<int>(key_len(k)) + 1;
-        const bool equal = key_settled(k), pairs = !equal && m <= kPairs;
+        const bool equal = key_settled(k), pairs = !equal && (m == 1 || (m <= kPairs && round > 1));
         int rank = p - g1, shared = 0;                         // in the group; tokens shared with the rank before
         if (equal) {
           shared = static_cast<int>(A.tok_offsets[me + 1] - A.tok_offsets[me]);
@@ -354,22 +375,13 @@ __device__ __forceinline__ void build(const Args& A) {
         }
         g = g1;
         e = e1;
-      } else {
-        if (lane == 0) {
-          A.gs[p] = g;
-          A.ge[p] = e;
-          A.perm[pc][p] = p;
-          if (p == 0) A.lcp[0] = 0;
-          if (n == 1) A.order[0] = 0;
-        }
-        if (n == 1) continue;
       }
       const int m = e - g;
       need |= kMore | (m > kCount ? kBig : 0);
       uint32_t r = (static_cast<uint32_t>(g) * 0x9e3779b1u) ^ ((round + 1) * 0x85ebca6bu);
       r = (r ^ (r >> 15)) * 0x2c1b3c6du;
       const int at = g + static_cast<int>((r >> 3) % static_cast<uint32_t>(m));
-      const int pivot = round > 0 ? A.perm[pc][at] : at;
+      const int pivot = A.perm[pc][at];
       Order o{0, 0, false, 0};
       if (me != pivot) o = compare_paths(A, me, pivot, base, lane);
       if (lane == 0) A.key[kc ^ 1][p] = make_key(o);
@@ -379,6 +391,7 @@ __device__ __forceinline__ void build(const Args& A) {
     const unsigned int flags = *reinterpret_cast<volatile unsigned int*>(&A.flags[round & 3]);
     if (!(flags & kMore)) break;
     if (blockIdx.x == 0 && threadIdx.x == 0) A.flags[(round + 2) & 3] = 0;
+    if (round == 0 && !(flags & kMixed)) continue;
     if (!(flags & kBig)) {
       const uint64_t* kn = A.key[kc ^ 1];
       for (int p = wid; p < n; p += n_warps) {
@@ -397,8 +410,8 @@ __device__ __forceinline__ void build(const Args& A) {
       if (!grid_barrier<CLUSTER>(A, target)) return;
       continue;
     }
-    for (int t = blockIdx.x; t < A.n_tiles; t += gridDim.x)
-      sort_tile(A, t, A.key[kc ^ 1], A.perm[pc], A.key[kc], A.perm[pc ^ 1]);
+    for (int t = blockIdx.x * (kThreads / kTile); t < A.n_tiles; t += gridDim.x * (kThreads / kTile))
+      sort_tiles(A, t, A.key[kc ^ 1], A.perm[pc], A.key[kc], A.perm[pc ^ 1]);
     if (!grid_barrier<CLUSTER>(A, target)) return;
     // `width` lanes per position, one for each tile of its group
     int width = 1;
