@@ -25,7 +25,7 @@
 // 8 fp64 instructions with the summation; the table is copied 16 times so that every lane reads its own bank pair.
 // Bound: issue slots.  An fp64 instruction holds two, so 32 logits take ~30 clocks of a sub-partition, 120 us for
 // 922 x 151936 logits (the loop alone, measured; 4 bytes a logit from HBM would take 85).  Measured, the call: 922 rows
-// 582 -> 186 us, 16 rows 91 -> 18 us, against one block of 1024 threads per row with a pass for the maximum, CUDA's exp
+// 582 -> 183 us, 16 rows 91 -> 13 us, against one block of 1024 threads per row with a pass for the maximum, CUDA's exp
 // and a block-wide scan for every 4096 tokens.
 #include <cooperative_groups.h>
 
@@ -404,6 +404,35 @@ static int32_t launch(Args A, bool vec, int row0, int n_seq, int clusters, cudaS
   return SS_OK;
 }
 
+// Clusters of CL blocks that the current device holds at a time (asked once per device; 74 of 2, 33 of 4, 15 of 8 on 148 SMs).
+template <int CL>
+static int resident_clusters(bool vec) {
+  static std::atomic<int> cached[2][kDeviceSlots];
+  const int slot = current_device_slot();
+  if (slot >= 0) {
+    const int n = cached[vec][slot].load(std::memory_order_relaxed);
+    if (n > 0) return n;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(CL);
+  cfg.blockDim = dim3(kThreads);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CL;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  const cudaError_t rc = vec ? cudaOccupancyMaxActiveClusters(&n, branch_sample_kernel<CL, true>, &cfg)
+                             : cudaOccupancyMaxActiveClusters(&n, branch_sample_kernel<CL, false>, &cfg);
+  if (rc != cudaSuccess || n < 1) {
+    (void)cudaGetLastError();
+    n = 1;
+  }
+  if (slot >= 0) cached[vec][slot].store(n, std::memory_order_relaxed);
+  return n;
+}
+
 }  // namespace sample
 }  // namespace ss
 
@@ -432,13 +461,13 @@ extern "C" int32_t ss_branch_sample(const float* logits, const int64_t* draw_off
   const bool vec = reinterpret_cast<uintptr_t>(logits) % 16 == 0 && vocab % 4 == 0;
   cudaStream_t st = as_stream(stream);
   const int sms = sm_count_of_current_device();
-  // Whole rounds of one row per SM, then the rows that are left over on clusters as large as they fit: a GPC of 18 SMs
-  // holds 2 clusters of 8 blocks, 4 of 4, 9 of 2 (one block per SM), and there are 8.  (Clusters for all rows: the
-  // launch and the barriers of a block that has an eighth of a row cost more than the uneven last round, 250-400 us
-  // instead of 186 for 922 rows; persistent clusters depend on all of them being placed at once.)
+  // Whole rounds of one row per SM, then the rows that are left over on clusters as large as fit at once (a cluster that has
+  // to wait for another doubles the time: 16 rows 18 us on clusters of 8, of which 15 fit, 13 on clusters of 4).
+  // Clusters for all rows cost more than the uneven last round: 250-400 us instead of 186 for 922 rows.
   constexpr int kMaxSlice = kMaxSegs * kSeg * kWarps;           // vocabulary that one block can take (262144)
   const int blocks_min = (vocab + kMaxSlice - 1) / kMaxSlice;   // 1 .. 8
-  auto cluster_size = [&](int rows) { return rows <= 16 ? 8 : rows <= 32 ? 4 : rows <= 72 ? 2 : 1; };
+  const int n8 = resident_clusters<8>(vec), n4 = resident_clusters<4>(vec), n2 = resident_clusters<2>(vec);
+  auto cluster_size = [&](int rows) { return rows <= n8 ? 8 : rows <= n4 ? 4 : rows <= n2 ? 2 : 1; };
   int whole = blocks_min > 1 ? 0 : n_seq / sms * sms;
   if (blocks_min == 1 && cluster_size(n_seq - whole) == 1) whole = n_seq;
   if (whole > 0) {
@@ -448,7 +477,7 @@ extern "C" int32_t ss_branch_sample(const float* logits, const int64_t* draw_off
   const int rest = n_seq - whole;
   if (rest == 0) return SS_OK;
   const int size = cluster_size(rest) > blocks_min ? cluster_size(rest) : blocks_min;
-  if (size > 4) return launch<8>(A, vec, whole, n_seq, rest < 16 ? rest : 16, st);
-  if (size > 2) return launch<4>(A, vec, whole, n_seq, rest < 32 ? rest : 32, st);
-  return launch<2>(A, vec, whole, n_seq, rest < 72 ? rest : 72, st);
+  if (size > 4) return launch<8>(A, vec, whole, n_seq, rest < n8 ? rest : n8, st);
+  if (size > 2) return launch<4>(A, vec, whole, n_seq, rest < n4 ? rest : n4, st);
+  return launch<2>(A, vec, whole, n_seq, rest < n2 ? rest : n2, st);
 }
