@@ -84,10 +84,11 @@ static Layout carve(const ss_attn_desc_t* d, char* base, Params* P) {
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes); return base ? base + o : nullptr; };
   const size_t N = static_cast<size_t>(d->num_nodes) + 1, NP = static_cast<size_t>(d->num_paths) + 1;
   char* hdr = take(sizeof(PlanHeader));
-  char* node_arrays[11];
-  for (int i = 0; i < 11; ++i) node_arrays[i] = take(N * 4);
-  char* path_arrays[6];
-  for (int i = 0; i < 6; ++i) path_arrays[i] = take(NP * 4);
+  char* node_arrays[kPlanNodeArrays];
+  for (int i = 0; i < kPlanNodeArrays; ++i) node_arrays[i] = take(N * 4);
+  char* path_arrays[kPlanPathArrays];
+  for (int i = 0; i < kPlanPathArrays; ++i) path_arrays[i] = take(NP * 4);
+  char* path_kv_len = take(NP * 4);
   char* dec_tok = take((static_cast<size_t>(cap_dec) + 1) * 4);
   char* dec_src = take((static_cast<size_t>(cap_dec) + 1) * 4);
   char* dec_slot = take((static_cast<size_t>(cap_dec) + 1) * 4);
@@ -99,12 +100,16 @@ static Layout carve(const ss_attn_desc_t* d, char* base, Params* P) {
   char* part_lse = take(static_cast<size_t>(caps.slots) * d->num_q_heads * 4);
   if (P) {
     P->hdr = reinterpret_cast<PlanHeader*>(hdr);
-    int32_t** np[11] = {&P->node_start, &P->node_depth, &P->node_first, &P->node_last, &P->node_npaths, &P->node_ndec,
-                        &P->node_own_slots, &P->node_level_off, &P->node_item_base, &P->node_splits, &P->node_split_len};
-    for (int i = 0; i < 11; ++i) *np[i] = reinterpret_cast<int32_t*>(node_arrays[i]);
-    int32_t** pp[6] = {&P->path_class, &P->path_kv_len, &P->path_dec_rank, &P->path_slot_base, &P->path_leaf_base,
-                       &P->path_chain_base};
-    for (int i = 0; i < 6; ++i) *pp[i] = reinterpret_cast<int32_t*>(path_arrays[i]);
+    for (int i = 0; i < kPlanNodeArrays; ++i) P->plan.node_array(i) = reinterpret_cast<int32_t*>(node_arrays[i]);
+    for (int i = 0; i < kPlanPathArrays; ++i) P->plan.path_array(i) = reinterpret_cast<int32_t*>(path_arrays[i]);
+    P->plan.sums = N > NP ? P->plan.n_last : reinterpret_cast<int32_t*>(path_kv_len);   // (8 of every 2048: fits where any fit)
+    P->plan.n_parent = const_cast<int32_t*>(d->node_parent);
+    P->plan.n_len = const_cast<int32_t*>(d->node_kv_len);
+    P->plan.p_leaf = const_cast<int32_t*>(d->path_leaf_node);
+    P->plan.p_T = const_cast<int32_t*>(d->path_q_len);
+    P->node_start = P->plan.n_start;
+    P->path_class = P->plan.p_class;
+    P->path_kv_len = reinterpret_cast<int32_t*>(path_kv_len);
     P->dec_tok = reinterpret_cast<int32_t*>(dec_tok);
     P->dec_src = reinterpret_cast<int32_t*>(dec_src);
     P->dec_slot_base = reinterpret_cast<int32_t*>(dec_slot);
@@ -190,6 +195,7 @@ extern "C" int32_t ss_tree_attention(const ss_attn_desc_t* d, void* workspace, s
   cudaStream_t st = as_stream(stream);
   int sms = sm_count_of_current_device();
   if (d->max_sms > 0 && d->max_sms < sms) sms = d->max_sms;
+  P.sms = sms;
   const bool timed = prof_begin_call();
   const int call = g_prof.used;
   // phase boundaries: event e is recorded before phase e, event SS_NUM_PHASES after the last one

@@ -1,173 +1,41 @@
 // Device-side planner of ss_tree_attention: turns the tree + per-path arrays into work lists (tile items, leaf
 // items), partial-slot assignments and per-path classes.  Running it on the device means the live path count can
-// come straight from ss_dedup_paths without a host round trip.  Four phases:
-//   nodes   depth and prefix length of every node, range checks, counters reset
-//   paths   class and key length of every path, membership counts of its chain nodes
-//   scan    (one block) every prefix sum: decode ranks, per-node tile items and KV splits, partial slots, leaf
-//           items, chain items; capacity checks; totals into the header
-//   emit    writes the item lists and the per-decode-token arrays
-// Trees of up to kSmallPlan nodes and paths are planned in ONE launch of a few blocks, each of which makes the WHOLE plan in
-// its own shared memory (redundantly: that needs no communication, and the phases cost their latency and instruction
-// fetches whatever the number of blocks) and then writes its share of the item lists.  Larger inputs take four launches
-// (nodes, paths and emit grid-parallel, scan in one block).  Bound: the latency of seven phases behind barriers, and of
-// code that runs once (instruction fetches).  Measured, against one block that shared the phases of the general path and
-// searched a path for every item: 922 unique paths 20.9 -> 11.5 us, 256 verification paths 29.1 -> 8.2, 8 paths 12.0 -> 8.1.
-// The header (status word first) is cleared by the host-side launcher before the first of the four kernels; the
-// small planner builds it in shared memory and its block 0 writes it out whole.
+// come straight from ss_dedup_paths without a host round trip.  Phases:
+//   inputs  read and checked
+//   nodes   keys before every node, depth check
+//   paths   class of every path, membership counts of its chain nodes
+//   tiles   per-node tile counts, KV splits, partial slots
+//   scan    every prefix sum: decode ranks, tile items, partial slots, leaf items; capacity checks; totals
+//   emit    the item lists and the per-decode-token arrays, a warp per path and per node
+// Two forms of the same code:
+//   small   (up to kSmallPlan nodes and paths)  one launch of a few blocks, each of which makes the WHOLE plan in its own shared
+//           memory (redundantly: that needs no communication, and the phases cost their latency and instruction fetches whatever
+//           the number of blocks) and then writes its share of the item lists
+//   large   (any size)  one cluster makes the plan, its arrays in the workspace (2048 nodes and paths are what shared
+//           memory holds), the cluster's hardware barrier between the phases; a second kernel writes the items, which
+//           needs more warps than a cluster has
+// Bound: the latency of the phases behind barriers, and of code that runs once (instruction fetches).  Measured, small: 922
+// unique paths 20.9 -> 11.5 us, 256 verification paths 29.1 -> 8.2, 8 paths 12.0 -> 8.1 (against one block that shared the
+// phases of a chain of five kernels and searched a path for every item).  Large, against that chain with its scan in one
+// block, between events: 2912 paths 42.6 -> 29.8 us, 6400 57.8 -> 29.8, 25600 183 -> 57, 64000 452 -> 101; as ONE cooperative
+// kernel with a barrier over the grid 40.7 and 43.9 for the first two (seven barriers, a memset, no overlap with its
+// neighbours' launches).
+// The header (status word first) is cleared and written by the planner itself.
+#include <cooperative_groups.h>
 #include "attn_plan.cuh"
 
 namespace ss {
 namespace attn {
 
-constexpr int kScanThreads = 1024;
-constexpr int kGridThreads = 256;
+namespace cg = cooperative_groups;
 
-// In-place exclusive scan of a[0..n) by one whole block: every thread sums a contiguous chunk, the chunk sums are
-// scanned across the block, then every thread rewrites its chunk.  Returns the total to every thread.
-__device__ int block_excl_scan_chunks(int32_t* a, int n) {
-  __shared__ int warp_tot[32];
-  __shared__ int total_s;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int chunk = (n + blockDim.x - 1) / blockDim.x;
-  const int lo = min(n, static_cast<int>(threadIdx.x) * chunk), hi = min(n, lo + chunk);
-  __syncthreads();
-  int sum = 0;
-  for (int i = lo; i < hi; ++i) sum += a[i];
-  int x = sum;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) warp_tot[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    int t = lane < nw ? warp_tot[lane] : 0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, t, o);
-      if (lane >= o) t += y;
-    }
-    warp_tot[lane] = t;
-    if (lane == 31) total_s = t;
-  }
-  __syncthreads();
-  int run = (warp ? warp_tot[warp - 1] : 0) + x - sum;
-  for (int i = lo; i < hi; ++i) {
-    const int v = a[i];
-    a[i] = run;
-    run += v;
-  }
-  __syncthreads();
-  return total_s;
-}
-
-// Two scans of arrays in GLOBAL memory of up to 16 entries per thread at once: a thread keeps its 16 consecutive entries of
-// each array in registers (128-bit loads, all issued before the first is used; 128-bit stores), so a pair of scans
-// costs two trips to memory instead of the six of two staged scans.  The arrays must be 16-byte aligned.
-constexpr int kScanRegs = 16;
-__device__ void block_excl_scan2_regs(int32_t* a0, int32_t* a1, int n, int (&total)[2]) {   // (two arrays per call: 32 of a thread's 64 registers)
-  __shared__ int warp_tot4[32][2];
-  __shared__ int total4_s[2];
-  int32_t* a[2] = {a0, a1};
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int lo = static_cast<int>(threadIdx.x) * kScanRegs;
-  int v[2][kScanRegs];
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-#pragma unroll
-    for (int i = 0; i < kScanRegs; i += 4) {
-      if (lo + i + 4 <= n) {
-        const int4 q = *reinterpret_cast<const int4*>(a[k] + lo + i);
-        v[k][i] = q.x; v[k][i + 1] = q.y; v[k][i + 2] = q.z; v[k][i + 3] = q.w;
-      } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) v[k][i + j] = (lo + i + j < n) ? a[k][lo + i + j] : 0;
-      }
-    }
-  }
-  int sum[2], x[2];
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    sum[k] = 0;
-#pragma unroll
-    for (int i = 0; i < kScanRegs; ++i) sum[k] += v[k][i];
-    x[k] = sum[k];
-  }
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int y = __shfl_up_sync(0xffffffffu, x[k], o);
-      if (lane >= o) x[k] += y;
-    }
-  }
-  if (lane == 31) {
-#pragma unroll
-    for (int k = 0; k < 2; ++k) warp_tot4[warp][k] = x[k];
-  }
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      int t = lane < nw ? warp_tot4[lane][k] : 0;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, t, o);
-        if (lane >= o) t += y;
-      }
-      warp_tot4[lane][k] = t;
-      if (lane == 31) total4_s[k] = t;
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    int run = (warp ? warp_tot4[warp - 1][k] : 0) + x[k] - sum[k];
-#pragma unroll
-    for (int i = 0; i < kScanRegs; i += 4) {
-      int4 q;
-      q.x = run; run += v[k][i];
-      q.y = run; run += v[k][i + 1];
-      q.z = run; run += v[k][i + 2];
-      q.w = run; run += v[k][i + 3];
-      if (lo + i + 4 <= n) {
-        *reinterpret_cast<int4*>(a[k] + lo + i) = q;
-      } else {
-        if (lo + i < n) a[k][lo + i] = q.x;
-        if (lo + i + 1 < n) a[k][lo + i + 1] = q.y;
-        if (lo + i + 2 < n) a[k][lo + i + 2] = q.z;
-      }
-    }
-    total[k] = total4_s[k];
-  }
-  __syncthreads();
-}
-
-// The same scan for an array in GLOBAL memory: it goes through the block's staging buffer in shared memory when it
-// fits (coalesced in, scanned on chip, coalesced out) - every thread walking its own contiguous chunk of a global
-// array makes each load touch 32 different sectors, which cost the one-block scan kernel most of its time.
-constexpr int kScanStage = 16384;                  // entries of the staging buffer (64 KB, dynamic shared memory)
-__device__ int block_excl_scan(int32_t* a, int n, int32_t* stage) {
-  if (n > kScanStage) return block_excl_scan_chunks(a, n);
-  __syncthreads();
-  for (int i = threadIdx.x; i < n; i += blockDim.x) stage[i] = a[i];
-  const int total = block_excl_scan_chunks(stage, n);      // (starts and ends with a barrier)
-  for (int i = threadIdx.x; i < n; i += blockDim.x) a[i] = stage[i];
-  __syncthreads();
-  return total;
-}
-
-// Block-uniform read of the status word (every thread gets the same answer, so an early return cannot leave
-// part of the block waiting at a later barrier).
-__device__ bool block_failed(const PlanHeader* hdr) {
-  __shared__ int s_status;
-  __syncthreads();
-  if (threadIdx.x == 0) s_status = *reinterpret_cast<const volatile int32_t*>(&hdr->status);
-  __syncthreads();
-  return s_status != SS_OK;
-}
+constexpr int kThreads = 1024;
+constexpr int kSmallPlan = 2048;               // nodes and paths: two of each per thread
+constexpr int kScanChunk = 2 * kThreads;       // entries of one block scan
+constexpr int kLeafClasses = 17;               // pages of the last chunk of a leaf: 0 .. 16
+constexpr int kSums = 7;
+constexpr int kLargeBlocks = 8;                // one cluster
+constexpr int kEmitThreads = 256;
 
 __device__ __forceinline__ int live_paths(const Params& P) {
   int live = P.num_paths;
@@ -191,394 +59,44 @@ __device__ __forceinline__ void node_split(const Params& P, int len, int total_t
   }
 }
 
-// ---- nodes: depth and number of keys before the node -------------------------------------------------------------
-__device__ __forceinline__ void plan_nodes_phase(const Params& P) {
-  PlanHeader* hdr = P.hdr;
-  const int64_t gtid = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t gsize = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  if (gtid == 0) hdr->live_paths = live_paths(P);
-  for (int64_t n64 = gtid; n64 < P.num_nodes; n64 += gsize) {
-    const int n = static_cast<int>(n64);
-    int d = 0, start = 0;
-    int a = P.node_parent[n];
-    bool bad = (a >= n || a < -1 || P.node_kv_len[n] < 0);
-    while (!bad && a >= 0 && d < SS_MAX_DEPTH) {
-      start += P.node_kv_len[a];
-      ++d;
-      const int na = P.node_parent[a];
-      if (na >= a || na < -1) { bad = true; break; }
-      a = na;
-    }
-    if (bad) set_status(&hdr->status, SS_ERR_BAD_INPUT);
-    else if (a >= 0 || d + 1 > SS_MAX_DEPTH) set_status(&hdr->status, SS_ERR_UNSUPPORTED);
-    const int64_t np = P.node_page_offsets[n + 1] - P.node_page_offsets[n];
-    if (!bad && (np < 0 || np * kPage < P.node_kv_len[n] || P.node_page_offsets[n + 1] > P.total_node_pages ||
-                 P.node_page_offsets[n] < 0))
-      set_status(&hdr->status, SS_ERR_BAD_INPUT);
-    P.node_depth[n] = d;
-    P.node_start[n] = start;
-    P.node_first[n] = 0x7fffffff;
-    P.node_last[n] = -1;
-    P.node_npaths[n] = 0;
-    P.node_ndec[n] = 0;
-  }
-  if (P.flags & SS_FLAG_VALIDATE) {
-    for (int64_t i = gtid; i < P.total_node_pages; i += gsize) {
-      const int pg = P.node_pages[i];
-      if (pg < 0 || pg >= P.num_pages) set_status(&hdr->status, SS_ERR_BAD_INPUT);
-    }
-  }
-}
-
-// ---- paths: class, kv length, membership counts of every chain node ------------------------------------------------
-__device__ __forceinline__ void plan_paths_phase(const Params& P) {
-  PlanHeader* hdr = P.hdr;
-  const int live = live_paths(P);
-  const int N = P.num_nodes;
-  const bool force_generic = (P.flags & SS_FLAG_FORCE_GENERIC) != 0;
-  const int64_t gsize = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  for (int64_t p64 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; p64 < live; p64 += gsize) {
-    const int p = static_cast<int>(p64);
-    const int leaf = P.path_leaf_node[p];
-    const int T = P.path_q_len[p];
-    bool bad_src = false;
-    if (P.q_src_offsets) {
-      const int64_t s0 = P.q_src_offsets[p];
-      bad_src = s0 < 0 || s0 + T > P.q_src_rows || s0 + T > 0x7fffffffLL;
-    }
-    if (leaf < 0 || leaf >= N || T < 1 || P.q_offsets[p + 1] - P.q_offsets[p] != T || P.q_offsets[p] < 0 ||
-        P.q_offsets[p + 1] > P.total_q || bad_src) {
-      set_status(&hdr->status, SS_ERR_BAD_INPUT);
-      P.path_class[p] = kClassGeneric;
-      continue;
-    }
-    bool inner_whole_pages = true;
-    for (int a = P.node_parent[leaf]; a >= 0; a = P.node_parent[a])
-      if (P.node_kv_len[a] % kPage) inner_whole_pages = false;
-    int cls;
-    if (force_generic) cls = kClassGeneric;
-    else if (T == 1) cls = (P.G <= 16) ? kClassDecode : kClassGeneric;
-    else cls = inner_whole_pages ? kClassChain : kClassGeneric;
-    P.path_class[p] = cls;
-    P.path_kv_len[p] = P.node_start[leaf] + P.node_kv_len[leaf];
-    if (cls == kClassGeneric) atomicAdd(&hdr->n_generic_rows, T);
-    for (int a = leaf; a >= 0; a = P.node_parent[a]) {
-      atomicMin(&P.node_first[a], p);
-      atomicMax(&P.node_last[a], p);
-      atomicAdd(&P.node_npaths[a], 1);
-      if (cls == kClassDecode) atomicAdd(&P.node_ndec[a], 1);
-    }
-  }
-}
-
-// ---- every prefix sum -------------------------------------------------------------------------------------------------
-__device__ __forceinline__ void plan_scan_phase(const Params& P, int32_t* stage) {   // one whole block; block-uniform
-                                                                                     // returns only; stage: see block_excl_scan
-  __shared__ int s_total_tiles;
-  PlanHeader* hdr = P.hdr;
-  if (block_failed(hdr)) return;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int live = live_paths(P);
-  const int N = P.num_nodes;
-  const int tpt = P.tok_per_tile;
-  if (tid == 0) s_total_tiles = 0;
-
-#ifdef SS_STAMPS
-  long long pt = clock64();
-  int pi = 24;
-#define PLAN_MARK() do { __syncthreads(); if (tid == 0) { const long long t = clock64(); hdr->stamp[pi] = t - pt; pt = t; } ++pi; } while (0)
-#else
-#define PLAN_MARK() do { } while (0)
-#endif
-  // decode ranks (scanned together with the per-path counts below where one pass can take all four arrays)
-  const bool fused = live <= nt * kScanRegs &&
-                     ((reinterpret_cast<uintptr_t>(P.path_slot_base) | reinterpret_cast<uintptr_t>(P.path_leaf_base) |
-                       reinterpret_cast<uintptr_t>(P.path_chain_base) | reinterpret_cast<uintptr_t>(P.path_dec_rank)) & 15) == 0;
-  for (int p = tid; p < live; p += nt) P.path_dec_rank[p] = (P.path_class[p] == kClassDecode) ? 1 : 0;
-  if (!fused) {
-    const int n_dec = block_excl_scan(P.path_dec_rank, live, stage);
-    if (tid == 0) {
-      P.path_dec_rank[live] = n_dec;
-      hdr->n_dec = n_dec;
-      if (n_dec > P.caps.dec) set_status(&hdr->status, SS_ERR_WORKSPACE_TOO_SMALL);
-    }
-  }
-
-  PLAN_MARK();   // 8: decode ranks
-  // nodes: role, tiles
-  for (int n = tid; n < N; n += nt) {
-    const int np = P.node_npaths[n];
-    if (np > 0 && P.node_last[n] - P.node_first[n] + 1 != np) set_status(&hdr->status, SS_ERR_BAD_INPUT);
-    const int nd = P.node_ndec[n], len = P.node_kv_len[n];
-    int tiles = 0;
-    if (nd > 0 && len > 0) {
-      const bool leaf_only = (np == 1 && P.path_leaf_node[P.node_first[n]] == n);
-      if (!leaf_only) tiles = ceil_div(nd, tpt);
-    }
-    P.node_item_base[n] = tiles;                     // tiles for now; becomes the item base after the scan
-    if (tiles) atomicAdd(&s_total_tiles, tiles);
-  }
-  if (block_failed(hdr)) return;
-  PLAN_MARK();   // 9: node tiles
-  const int total_tiles = s_total_tiles * P.Hkv;
-  for (int n = tid; n < N; n += nt) {
-    const int nd = P.node_ndec[n], len = P.node_kv_len[n];
-    const int tiles = P.node_item_base[n];
-    int splits = 1, own = 0, split_len = len;
-    if (nd > 0 && len > 0) {
-      if (tiles == 0) {
-        own = ceil_div(len, kLeafChunk);             // private leaf of one decode path
-      } else {
-        if (P.node_depth[n] == 0) node_split(P, len, total_tiles, splits, split_len);
-        own = splits;
-      }
-    }
-    P.node_splits[n] = splits;
-    P.node_split_len[n] = split_len;
-    P.node_own_slots[n] = own;
-    P.node_item_base[n] = tiles * splits * P.Hkv;
-  }
-  __syncthreads();
-  PLAN_MARK();   // 10: splits
-  for (int n = tid; n < N; n += nt) {
-    int off = 0;
-    for (int a = P.node_parent[n]; a >= 0; a = P.node_parent[a]) off += P.node_own_slots[a];
-    P.node_level_off[n] = off;
-  }
-  PLAN_MARK();   // 11: level offsets
-  const int n_stacked = block_excl_scan(P.node_item_base, N, stage);
-  PLAN_MARK();   // 12: item base scan
-  if (tid == 0) P.node_item_base[N] = n_stacked;
-
-  // decode paths: partial slots, leaf items; chain paths: tile items
-  for (int p = tid; p < live; p += nt) {
-    int slots = 0, leaf_items = 0, chain_items = 0;
-    const int cls = P.path_class[p];
-    if (cls == kClassDecode) {
-      const int leaf = P.path_leaf_node[p];
-      slots = P.node_level_off[leaf] + P.node_own_slots[leaf];
-      if (P.node_npaths[leaf] == 1 && P.node_kv_len[leaf] > 0)
-        leaf_items = ceil_div(P.node_kv_len[leaf], kLeafChunk) * P.Hkv;
-    } else if (cls == kClassChain) {
-      chain_items = ceil_div(P.path_q_len[p], tpt) * P.Hkv;
-    }
-    P.path_slot_base[p] = slots;
-    P.path_leaf_base[p] = leaf_items;
-    P.path_chain_base[p] = chain_items;
-  }
-  PLAN_MARK();   // 13: per-path counts
-  int n_slots, n_leaf_items, n_chain;
-  if (fused) {
-    int t2[2];
-    block_excl_scan2_regs(P.path_slot_base, P.path_leaf_base, live, t2);
-    n_slots = t2[0];
-    n_leaf_items = t2[1];
-    block_excl_scan2_regs(P.path_chain_base, P.path_dec_rank, live, t2);
-    n_chain = t2[0];
-    if (tid == 0) {
-      P.path_dec_rank[live] = t2[1];
-      hdr->n_dec = t2[1];
-      if (t2[1] > P.caps.dec) set_status(&hdr->status, SS_ERR_WORKSPACE_TOO_SMALL);
-    }
-  } else {
-    n_slots = block_excl_scan(P.path_slot_base, live, stage);
-    n_leaf_items = block_excl_scan(P.path_leaf_base, live, stage);
-    n_chain = block_excl_scan(P.path_chain_base, live, stage);
-  }
-  PLAN_MARK();   // 14: three scans
-  if (tid == 0) {
-    hdr->n_slots = n_slots;
-    hdr->n_stacked_items = n_stacked;
-    if (n_slots > P.caps.slots || n_leaf_items > P.caps.leaf_items || n_stacked + n_chain > P.caps.tile_items) {
-      set_status(&hdr->status, SS_ERR_WORKSPACE_TOO_SMALL);     // the executors see the status and do nothing
-    } else {
-      hdr->n_leaf_items = n_leaf_items;
-      hdr->n_tile_items = n_stacked + n_chain;
-    }
-  }
-}
-
-// ---- item lists ---------------------------------------------------------------------------------------------------------
-__device__ __forceinline__ void plan_emit_phase(const Params& P) {
-  PlanHeader* hdr = P.hdr;
-  const int live = live_paths(P);
-  const int N = P.num_nodes;
-  const int tpt = P.tok_per_tile;
-  const int n_stacked = hdr->n_stacked_items;
-  const int64_t gtid = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t gsize = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  if (gtid == 0) P.dec_slot_base[hdr->n_dec] = hdr->n_slots;
-
-  // per decode token: output row, query row, partial slots, leaf chunks, arrival counters
-  for (int64_t p64 = gtid; p64 < live; p64 += gsize) {
-    const int p = static_cast<int>(p64);
-    if (P.path_class[p] != kClassDecode) continue;
-    const int rank = P.path_dec_rank[p];
-    const int leaf = P.path_leaf_node[p];
-    const int len = P.node_kv_len[leaf];
-    P.dec_tok[rank] = static_cast<int32_t>(P.q_offsets[p]);
-    P.dec_src[rank] = static_cast<int32_t>(P.q_src_offsets ? P.q_src_offsets[p] : P.q_offsets[p]);
-    P.dec_slot_base[rank] = P.path_slot_base[p];
-    const bool own_leaf = P.node_npaths[leaf] == 1 && len > 0;
-    P.dec_leaf_chunks[rank] = own_leaf ? ceil_div(len, kLeafChunk) : 0;
-    for (int g = 0; g < P.Hkv; ++g) P.leaf_arrive[static_cast<int64_t>(rank) * P.Hkv + g] = 0;
-  }
-  // Leaf and chain items, one thread per ITEM (consecutive threads write consecutive descriptors: a thread per path
-  // writing its own run of descriptors makes every store instruction touch 32 different sectors, and that alone cost
-  // tens of microseconds on one SM).  Item e -> path by binary search over the exclusive scans.
-  auto path_of = [&](const int32_t* base, int e) {
-    int lo = 0, hi = live;                    // last p with base[p] <= e (paths without items share their successor's base)
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (base[mid] <= e) lo = mid; else hi = mid;
-    }
-    return lo;
-  };
-  const int n_leaf_items = hdr->n_leaf_items;
-  for (int64_t e64 = gtid; e64 < n_leaf_items; e64 += gsize) {
-    const int e = static_cast<int>(e64);
-    const int p = path_of(P.path_leaf_base, e);
-    const int local = e - P.path_leaf_base[p];
-    const int c = local / P.Hkv, g = local - c * P.Hkv;
-    const int leaf = P.path_leaf_node[p];
-    const int len = P.node_kv_len[leaf];
-    LeafItem it;
-    it.page0 = static_cast<int32_t>(P.node_page_offsets[leaf]) + c * (kLeafChunk / kPage);
-    it.node = leaf;
-    it.g = g;
-    it.kv_begin = c * kLeafChunk;
-    it.kv_end = min(len, (c + 1) * kLeafChunk);
-    it.slot = P.path_slot_base[p] + P.node_level_off[leaf] + c;
-    it.q_src = static_cast<int32_t>(P.q_src_offsets ? P.q_src_offsets[p] : P.q_offsets[p]);
-    it.dec = P.path_dec_rank[p];
-    P.leaf_items[e] = it;
-  }
-  const int n_chain_items = hdr->n_tile_items - n_stacked;
-  for (int64_t e64 = gtid; e64 < n_chain_items; e64 += gsize) {
-    const int e = static_cast<int>(e64);
-    const int p = path_of(P.path_chain_base, e);
-    const int local = e - P.path_chain_base[p];
-    const int T = P.path_q_len[p];
-    const int L = P.path_kv_len[p];
-    const int tiles = ceil_div(T, tpt);
-    const int g = local / tiles, t = local - g * tiles;
-    const int32_t src_row = static_cast<int32_t>(P.q_src_offsets ? P.q_src_offsets[p] : P.q_offsets[p]);
-    TileItem it;
-    it.node = P.path_leaf_node[p];
-    it.tok0 = static_cast<int32_t>(P.q_offsets[p]) + t * tpt;
-    it.n_tok = min(tpt, T - t * tpt);
-    it.kind_g = (kItemChain << 16) | g;
-    it.kv_begin = 0;
-    it.limit0 = L - T + t * tpt + 1;
-    it.kv_end = max(0, min(L, it.limit0 + it.n_tok - 1));
-    it.slot_off = -1;
-    it.src0 = src_row + t * tpt;
-    it.pad = 0;
-    P.tile_items[n_stacked + e] = it;
-  }
-
-  // stacked items: item e -> node by binary search over the exclusive scan of per-node item counts
-  for (int64_t e64 = gtid; e64 < n_stacked; e64 += gsize) {
-    const int e = static_cast<int>(e64);
-    int lo = 0, hi = N;                       // last n with base[n] <= e and base[n+1] > e
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (P.node_item_base[mid] <= e) lo = mid; else hi = mid;
-    }
-    const int n = lo;
-    const int local = e - P.node_item_base[n];
-    const int splits = P.node_splits[n];
-    const int split = local % splits;
-    const int rest = local / splits;
-    const int g = rest % P.Hkv;
-    const int tile = rest / P.Hkv;
-    const int len = P.node_kv_len[n];
-    const int split_len = P.node_split_len[n];
-    const int nd = P.node_ndec[n];
-    TileItem it;
-    it.node = n;
-    it.tok0 = P.path_dec_rank[P.node_first[n]] + tile * tpt;
-    it.n_tok = min(tpt, nd - tile * tpt);
-    it.kind_g = (kItemStacked << 16) | g;
-    it.kv_begin = split * split_len;
-    it.kv_end = min(len, (split + 1) * split_len);
-    it.limit0 = it.kv_end;
-    it.slot_off = P.node_level_off[n] + split;
-    it.src0 = static_cast<int32_t>(P.node_page_offsets[n]);
-    it.pad = 0;
-    P.tile_items[e] = it;
-  }
-}
-
-// ---- general path: four launches ------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kGridThreads) plan_nodes_kernel(const Params P) {
-  ss::grid_dependency_enter();
-  plan_nodes_phase(P);
-}
-__global__ void __launch_bounds__(kGridThreads) plan_paths_kernel(const Params P) {
-  ss::grid_dependency_enter();
-  if (P.hdr->status != SS_OK) return;          // no barrier in this kernel: a per-thread return is safe
-  plan_paths_phase(P);
-}
-__global__ void __launch_bounds__(kScanThreads) plan_scan_kernel(const Params P) {
-  ss::grid_dependency_enter();
-  extern __shared__ __align__(16) int32_t scan_stage[];
-  plan_scan_phase(P, scan_stage);
-}
-__global__ void __launch_bounds__(kGridThreads) plan_emit_kernel(const Params P) {
-  ss::grid_dependency_enter();
-  if (P.hdr->status != SS_OK) return;          // no barrier in this kernel
-  plan_emit_phase(P);
-}
-
-// ---- small trees: one launch, everything in shared memory ---------------------------------------------------------
-constexpr int kSmallPlan = 2048;               // nodes and paths: two of each per thread
-constexpr int kSmallNodeArrays = 14, kSmallPathArrays = 10;
-inline size_t small_plan_smem(int N, int NP) {
-  return static_cast<size_t>(4) * (static_cast<size_t>(N) * kSmallNodeArrays + static_cast<size_t>(NP) * kSmallPathArrays) + 64;
-}
-// Blocks: what is left to share is the emission, a warp per path and per node.
-inline int small_plan_blocks(int N, int NP) {
-  const int b = (N + NP + 31) / 32;
-  return b < 1 ? 1 : (b > 64 ? 64 : b);
-}
-constexpr int kLeafClasses = 17;               // pages of the last chunk of a leaf: 0 .. 16
-
-// Six exclusive scans at once over the block's entries 2 tid, 2 tid + 1 (v -> positions), and the totals; in the same two
-// barriers the rank of each entry among all of them, larger classes cls[] first (order[]: deterministic, but not index
-// order within a class).
-struct SmallScan {
-  int tot[6][32];              // per warp, then exclusive over the warps
-  int total[6];
+// Seven exclusive scans at once over the block's entries 2 tid, 2 tid + 1 (v -> positions), and the totals; with RANK, in the
+// same two barriers, the rank of each entry among all of them, larger classes cls[] first (order[]: deterministic, but not
+// index order within a class).
+struct BlockScan {
+  int tot[kSums][32];          // per warp, then exclusive over the warps
+  int total[kSums];
   int hist[kLeafClasses][64];  // per class and group of 32 entries, then exclusive over the groups
   int cls_total[kLeafClasses];
 };
-__device__ __forceinline__ void small_scan(SmallScan& S, int (&v)[6][2], const int (&cls)[2], int (&order)[2]) {
+template <bool RANK>
+__device__ __forceinline__ void block_scan(BlockScan& S, int (&v)[kSums][2], const int (&cls)[2], int (&order)[2]) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int sum[6], x[6];
+  int sum[kSums], x[kSums];
 #pragma unroll
-  for (int k = 0; k < 6; ++k) x[k] = sum[k] = v[k][0] + v[k][1];
+  for (int k = 0; k < kSums; ++k) x[k] = sum[k] = v[k][0] + v[k][1];
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
+    for (int k = 0; k < kSums; ++k) {
       const int y = __shfl_up_sync(0xffffffffu, x[k], o);
       if (lane >= o) x[k] += y;
     }
   }
   if (lane == 31) {
 #pragma unroll
-    for (int k = 0; k < 6; ++k) S.tot[k][warp] = x[k];
+    for (int k = 0; k < kSums; ++k) S.tot[k][warp] = x[k];
   }
-  int in_group[2];
+  int in_group[2] = {0, 0};
+  if (RANK) {
 #pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    const uint32_t peers = __match_any_sync(0xffffffffu, cls[e]);
-    in_group[e] = __popc(peers & ((1u << lane) - 1u));
-    if (in_group[e] == 0) S.hist[cls[e]][2 * warp + e] = __popc(peers);   // (the rest was cleared by the caller)
+    for (int e = 0; e < 2; ++e) {
+      const uint32_t peers = __match_any_sync(0xffffffffu, cls[e]);
+      in_group[e] = __popc(peers & ((1u << lane) - 1u));
+      if (in_group[e] == 0) S.hist[cls[e]][2 * warp + e] = __popc(peers);   // (the rest was cleared by the caller)
+    }
   }
   __syncthreads();
-  if (warp < 6) {
+  if (warp < kSums) {
     const int t = S.tot[warp][lane];
     int y = t;
 #pragma unroll
@@ -588,7 +106,7 @@ __device__ __forceinline__ void small_scan(SmallScan& S, int (&v)[6][2], const i
     }
     S.tot[warp][lane] = y - t;
     if (lane == 31) S.total[warp] = y;
-  } else if (warp >= 8 && warp < 8 + kLeafClasses) {
+  } else if (RANK && warp >= 8 && warp < 8 + kLeafClasses) {
     int* h = S.hist[warp - 8];
     const int a = h[2 * lane], b = h[2 * lane + 1];
     int y = a + b;
@@ -603,49 +121,57 @@ __device__ __forceinline__ void small_scan(SmallScan& S, int (&v)[6][2], const i
   }
   __syncthreads();
 #pragma unroll
-  for (int k = 0; k < 6; ++k) {
+  for (int k = 0; k < kSums; ++k) {
     const int first = S.tot[k][warp] + x[k] - sum[k];
     v[k][1] = first + v[k][0];
     v[k][0] = first;
   }
-  int above = lane < kLeafClasses ? S.cls_total[lane] : 0;      // lane r: entries of the classes > r
-  const int own = above;
+  if (RANK) {
+    int above = lane < kLeafClasses ? S.cls_total[lane] : 0;    // lane r: entries of the classes > r
+    const int own = above;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int z = __shfl_down_sync(0xffffffffu, above, o);
-    if (lane + o < 32) above += z;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int z = __shfl_down_sync(0xffffffffu, above, o);
+      if (lane + o < 32) above += z;
+    }
+    above -= own;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) order[e] = __shfl_sync(0xffffffffu, above, cls[e]) + S.hist[cls[e]][2 * warp + e] + in_group[e];
   }
-  above -= own;
-#pragma unroll
-  for (int e = 0; e < 2; ++e) order[e] = __shfl_sync(0xffffffffu, above, cls[e]) + S.hist[cls[e]][2 * warp + e] + in_group[e];
 }
 
-__global__ void __launch_bounds__(kScanThreads) plan_small_kernel(const __grid_constant__ Params P) {
-  ss::grid_dependency_enter();
-  extern __shared__ __align__(16) int32_t plan_smem[];
-  __shared__ PlanHeader s_hdr;
-  __shared__ SmallScan s_scan;
-  __shared__ int s_total_tiles, s_generic;
+// The plan up to the item lists.  `A`: its arrays, in shared memory (small) or in the workspace; `bad_phase`: a word per phase
+// in the block's shared memory; `totals` (tiles of the shared nodes, rows of GENERIC paths): in shared memory, of block 0 of
+// the cluster in the large form.  All start at zero.  False: it failed, the status says why.
+template <bool LARGE>
+__device__ __forceinline__ bool make_plan(const Params& P, const PlanArrays& A, PlanHeader* hdr, BlockScan& S, int* bad_phase,
+                                          int* totals) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int N = P.num_nodes, NP = P.num_paths, Hkv = P.Hkv, tpt = P.tok_per_tile;
-  int32_t* w = plan_smem;
-  auto take = [&](int n) { int32_t* r = w; w += n; return r; };
-  int32_t *n_parent = take(N), *n_len = take(N), *n_page0 = take(N), *n_start = take(N), *n_first = take(N), *n_last = take(N),
-          *n_paths = take(N), *n_dec = take(N), *n_own = take(N), *n_level = take(N), *n_tiles = take(N), *n_splits = take(N),
-          *n_split_len = take(N), *n_base = take(N);
-  int32_t *p_leaf = take(NP), *p_T = take(NP), *p_row = take(NP), *p_src = take(NP), *p_class = take(NP), *p_rank = take(NP),
-          *p_slot = take(NP), *p_full = take(NP), *p_chain = take(NP), *p_last = take(NP);
+  const int first = LARGE ? static_cast<int>(blockIdx.x) * kThreads + tid : tid;
+  const int stride = LARGE ? kLargeBlocks * kThreads : kThreads;
+  int phase = 0;
+  // Ends a phase: true in every thread of every block that plans if `bad` was set in any of them.  (The large form tells
+  // every block, in a word of the phase's own: a block that is already in the next phase must not change what others read.)
+  auto phase_failed = [&](bool bad, int code) -> bool {
+    if (LARGE) {
+      if (bad) {
+        for (int r = 0; r < kLargeBlocks; ++r) *cg::this_cluster().map_shared_rank(&bad_phase[phase], r) = 1;
+        set_status(&hdr->status, code);
+      }
+      cg::this_cluster().sync();
+      return bad_phase[phase++] != 0;
+    }
+    const bool any = __syncthreads_or(bad) != 0;
+    if (any && tid == 0) hdr->status = code;
+    return any;
+  };
 
-  for (int x = tid; x < static_cast<int>(sizeof(PlanHeader) / 4); x += kScanThreads) reinterpret_cast<int32_t*>(&s_hdr)[x] = 0;
-  for (int x = tid; x < kLeafClasses * 64; x += kScanThreads) (&s_scan.hist[0][0])[x] = 0;
-  if (tid == 0) s_total_tiles = s_generic = 0;
-  SS_STAMP_BEGIN(P.hdr, 0);
-
-  // ---- inputs (one trip: the per-path arrays are read up to their capacity, beside the live count) -----------------------
+  // ---- inputs (the per-path arrays up to their capacity, beside the live count: one trip) ---------------------------------
   const int live = live_paths(P);
   bool bad = false;
 #pragma unroll 1
-  for (int i = tid; i < max(N, NP); i += kScanThreads) {       // (node i and path i: their loads go out together)
+  for (int i = first; i < max(N, NP); i += stride) {           // (node i and path i: their loads go out together)
     const int n = min(i, N - 1), p = min(i, NP - 1);
     int parent = 0, len = 0, leaf = 0, T = 0;
     int64_t o0 = 0, o1 = 0, r0 = 0, r1 = 0, src = 0;
@@ -664,325 +190,387 @@ __global__ void __launch_bounds__(kScanThreads) plan_small_kernel(const __grid_c
     }
     if (i < N) {
       bad = bad || parent >= n || parent < -1 || len < 0 || o1 < o0 || (o1 - o0) * kPage < len || o1 > P.total_node_pages || o0 < 0;
-      n_parent[n] = parent;
-      n_len[n] = len;
-      n_page0[n] = static_cast<int32_t>(o0);
-      n_first[n] = 0x7fffffff;
-      n_last[n] = -1;
-      n_paths[n] = n_dec[n] = 0;
+      if (!LARGE) {
+        A.n_parent[n] = parent;
+        A.n_len[n] = len;
+        A.n_page0[n] = static_cast<int32_t>(o0);
+      }
+      A.n_first[n] = 0x7fffffff;
+      A.n_last[n] = -1;
+      A.n_paths[n] = A.n_dec[n] = 0;
     }
     if (i < NP) {
       bool ok = leaf >= 0 && leaf < N && T >= 1 && r1 - r0 == T && r0 >= 0 && r1 <= P.total_q;
       if (P.q_src_offsets) ok = ok && src >= 0 && src + T <= P.q_src_rows && src + T <= 0x7fffffffLL;
-      p_leaf[p] = ok ? leaf : -1;
-      p_T[p] = T;
-      p_row[p] = static_cast<int32_t>(r0);
-      p_src[p] = static_cast<int32_t>(src);
+      bad = bad || (i < live && !ok);
+      if (!LARGE) {
+        A.p_leaf[p] = leaf;
+        A.p_T[p] = T;
+        A.p_row[p] = static_cast<int32_t>(r0);
+        A.p_src[p] = static_cast<int32_t>(src);
+      }
     }
   }
   if (P.flags & SS_FLAG_VALIDATE) {
-    for (int64_t i = tid; i < P.total_node_pages; i += kScanThreads) {
+    for (int64_t i = first; i < P.total_node_pages; i += stride) {
       const int pg = P.node_pages[i];
       bad = bad || pg < 0 || pg >= P.num_pages;
     }
   }
-  bool failed = __syncthreads_or(bad) != 0;
-  if (failed && tid == 0) s_hdr.status = SS_ERR_BAD_INPUT;
+  if (phase_failed(bad, SS_ERR_BAD_INPUT)) return false;
 
-  // ---- nodes: keys before the node (parents come first, so every walk ends) -------------------------------------------------
-  if (!failed) {
-    bool deep = false;
+  // ---- nodes: keys before the node (parents come first, so every walk ends) ---------------------------------------------------
+  bad = false;
 #pragma unroll 1
-    for (int n = tid; n < N; n += kScanThreads) {
-      int d = 1, start = 0;
+  for (int n = first; n < N; n += stride) {
+    int d = 1, start = 0;
 #pragma unroll 1
-      for (int a = n_parent[n]; a >= 0 && d <= SS_MAX_DEPTH; a = n_parent[a]) { start += n_len[a]; ++d; }
-      deep = deep || d > SS_MAX_DEPTH;
-      n_start[n] = start;
-    }
-    failed = __syncthreads_or(deep) != 0;
-    if (failed && tid == 0) s_hdr.status = SS_ERR_UNSUPPORTED;
+    for (int a = A.n_parent[n]; a >= 0 && d <= SS_MAX_DEPTH; a = A.n_parent[a]) { start += A.n_len[a]; ++d; }
+    bad = bad || d > SS_MAX_DEPTH;
+    A.n_start[n] = start;
   }
+  if (phase_failed(bad, SS_ERR_UNSUPPORTED)) return false;
 
-  // ---- paths: class, membership of every chain node (lanes with the same node are counted together) ---------------------
-  if (!failed) {
-    bad = false;
+  // ---- paths: class, membership of every chain node (lanes with the same node are counted together) -----------------------
 #pragma unroll 1
-    for (int p0 = 0; p0 < live; p0 += kScanThreads) {
-      const int p = p0 + tid;
-      const int leaf = p < live ? p_leaf[p] : -1, T = p < live ? p_T[p] : 0;
-      bad = bad || (p < live && leaf < 0);
-      const bool force = (P.flags & SS_FLAG_FORCE_GENERIC) != 0;
-      const bool dec = leaf >= 0 && T == 1 && P.G <= 16 && !force;
-      const uint32_t decs = __ballot_sync(0xffffffffu, dec);
-      bool whole = true;                                       // inner nodes are whole pages
-      int a = leaf;
+  for (int p0 = first - tid; p0 < live; p0 += stride) {
+    const int p = p0 + tid;
+    const int leaf = p < live ? A.p_leaf[p] : -1, T = p < live ? A.p_T[p] : 0;
+    const bool force = (P.flags & SS_FLAG_FORCE_GENERIC) != 0;
+    const bool dec = leaf >= 0 && T == 1 && P.G <= 16 && !force;
+    const uint32_t decs = __ballot_sync(0xffffffffu, dec);
+    bool whole = true;                                         // inner nodes are whole pages
+    int a = leaf;
 #pragma unroll 1
-      while (__any_sync(0xffffffffu, a >= 0)) {
-        const uint32_t peers = __match_any_sync(0xffffffffu, a);
-        if (a >= 0) {
-          if ((peers & ((1u << lane) - 1u)) == 0) {
-            atomicMin(&n_first[a], p);
-            atomicMax(&n_last[a], p + 31 - __clz(peers) - lane);
-            atomicAdd(&n_paths[a], __popc(peers));
-            if (peers & decs) atomicAdd(&n_dec[a], __popc(peers & decs));
-          }
-          if (a != leaf && n_len[a] % kPage) whole = false;
-          a = n_parent[a];
+    while (__any_sync(0xffffffffu, a >= 0)) {
+      const uint32_t peers = __match_any_sync(0xffffffffu, a);
+      if (a >= 0) {
+        if ((peers & ((1u << lane) - 1u)) == 0) {
+          atomicMin(&A.n_first[a], p);
+          atomicMax(&A.n_last[a], p + 31 - __clz(peers) - lane);
+          atomicAdd(&A.n_paths[a], __popc(peers));
+          if (peers & decs) atomicAdd(&A.n_dec[a], __popc(peers & decs));
         }
-      }
-      if (leaf >= 0) {
-        const int cls = dec ? kClassDecode : (force || T == 1 || !whole ? kClassGeneric : kClassChain);
-        p_class[p] = cls;
-        if (cls == kClassGeneric) atomicAdd(&s_generic, T);
+        if (a != leaf && A.n_len[a] % kPage) whole = false;
+        a = A.n_parent[a];
       }
     }
-    failed = __syncthreads_or(bad) != 0;
-    if (failed && tid == 0) s_hdr.status = SS_ERR_BAD_INPUT;
+    if (leaf >= 0) {
+      const int cls = dec ? kClassDecode : (force || T == 1 || !whole ? kClassGeneric : kClassChain);
+      A.p_class[p] = cls;
+      if (cls == kClassGeneric) atomicAdd(&totals[1], T);
+    }
   }
+  phase_failed(false, SS_OK);
 
-  // ---- nodes: tiles ----------------------------------------------------------------------------------------------------
-  if (!failed) {
-    bad = false;
-    int mine = 0;
+  // ---- nodes: tiles (what other blocks' atomics counted is read from L2) ----------------------------------------------------
+  auto count = [](const int32_t* c) { return LARGE ? __ldcg(c) : *c; };
+  bad = false;
+  int mine = 0;
 #pragma unroll 1
-    for (int n = tid; n < N; n += kScanThreads) {
-      const int np = n_paths[n], nd = n_dec[n];
-      bad = bad || (np > 0 && n_last[n] - n_first[n] + 1 != np);
-      int tiles = 0;
-      if (nd > 0 && n_len[n] > 0 && !(np == 1 && p_leaf[n_first[n]] == n)) tiles = ceil_div(nd, tpt);
-      n_tiles[n] = tiles;
-      mine += tiles;
-    }
-    mine = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned>(mine)));
-    if (lane == 0 && mine) atomicAdd(&s_total_tiles, mine);
-    failed = __syncthreads_or(bad) != 0;
-    if (failed && tid == 0) s_hdr.status = SS_ERR_BAD_INPUT;
+  for (int n = first; n < N; n += stride) {
+    const int np = count(A.n_paths + n), nd = count(A.n_dec + n), p0 = count(A.n_first + n);
+    bad = bad || (np > 0 && count(A.n_last + n) - p0 + 1 != np);
+    int tiles = 0;
+    if (nd > 0 && A.n_len[n] > 0 && !(np == 1 && A.p_leaf[p0] == n)) tiles = ceil_div(nd, tpt);
+    A.n_tiles[n] = tiles;
+    mine += tiles;
   }
+  mine = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned>(mine)));
+  if (lane == 0 && mine) atomicAdd(&totals[0], mine);
+  if (phase_failed(bad, SS_ERR_BAD_INPUT)) return false;
 
-  // ---- nodes: KV splits, partial slots -----------------------------------------------------------------------------------
-  if (!failed) {
-    const int total_tiles = s_total_tiles * Hkv;
+  // ---- nodes: KV splits, partial slots ------------------------------------------------------------------------------------------
+  const int total_tiles = totals[0] * Hkv;
 #pragma unroll 1
-    for (int n = tid; n < N; n += kScanThreads) {
-      const int len = n_len[n], tiles = n_tiles[n];
-      int splits = 1, own = 0, split_len = len;
-      if (tiles > 0) {
-        if (n_parent[n] < 0) node_split(P, len, total_tiles, splits, split_len);
-        own = splits;
-      } else if (n_dec[n] > 0 && len > 0) {
-        own = ceil_div(len, kLeafChunk);                     // private leaf of one decode path
-      }
-      n_splits[n] = splits;
-      n_split_len[n] = split_len;
-      n_own[n] = own;
+  for (int n = first; n < N; n += stride) {
+    const int len = A.n_len[n], tiles = A.n_tiles[n];
+    int splits = 1, own = 0, split_len = len;
+    if (tiles > 0) {
+      if (A.n_parent[n] < 0) node_split(P, len, total_tiles, splits, split_len);
+      own = splits;
+    } else if (count(A.n_dec + n) > 0 && len > 0) {
+      own = ceil_div(len, kLeafChunk);                         // private leaf of one decode path
     }
-    __syncthreads();
+    A.n_splits[n] = splits;
+    A.n_split_len[n] = split_len;
+    A.n_own[n] = own;
+  }
+  phase_failed(false, SS_OK);
 
-    // ---- every prefix sum: entries 2 tid, 2 tid + 1 of the nodes and of the paths ------------------------------------------
-    int v[6][2], cls[2] = {0, 0}, order[2];
+  // ---- every prefix sum: entries 2 tid, 2 tid + 1 of the nodes and of the paths, a chunk per block at a time ----------------
+  // sums: items of the roots, of the other nodes, decode paths, partial slots, whole leaf chunks, chain items, last chunks
+  const int n_chunks = LARGE ? max(1, ceil_div(max(N, live), kScanChunk)) : 1;
+#pragma unroll 1
+  for (int chunk = LARGE ? blockIdx.x : 0; chunk < n_chunks; chunk += LARGE ? gridDim.x : 1) {
+    int v[kSums][2], cls[2] = {0, 0}, order[2];
 #pragma unroll 1
     for (int e = 0; e < 2; ++e) {
-      const int i = 2 * tid + e;
+      const int i = chunk * kScanChunk + 2 * tid + e;
       int root_items = 0, node_items = 0, slots = 0, full = 0, chain = 0, dec = 0, c = 0;
       if (i < N) {
         int off = 0;
 #pragma unroll 1
-        for (int a = n_parent[i]; a >= 0; a = n_parent[a]) off += n_own[a];
-        n_level[i] = off;
-        const int items = n_tiles[i] * n_splits[i] * Hkv;
-        if (n_parent[i] < 0) root_items = items; else node_items = items;
+        for (int a = A.n_parent[i]; a >= 0; a = A.n_parent[a]) off += A.n_own[a];
+        A.n_level[i] = off;
+        const int items = A.n_tiles[i] * A.n_splits[i] * Hkv;
+        if (A.n_parent[i] < 0) root_items = items; else node_items = items;
       }
       if (i < live) {
-        const int leaf = p_leaf[i], len = n_len[leaf];
-        if (p_class[i] == kClassDecode) {
+        const int leaf = A.p_leaf[i], len = A.n_len[leaf];
+        if (A.p_class[i] == kClassDecode) {
           dec = 1;
 #pragma unroll 1
-          for (int a = leaf; a >= 0; a = n_parent[a]) slots += n_own[a];
-          if (n_paths[leaf] == 1 && len > 0) {
+          for (int a = leaf; a >= 0; a = A.n_parent[a]) slots += A.n_own[a];
+          if (count(A.n_paths + leaf) == 1 && len > 0) {
             full = len / kLeafChunk;
             c = ceil_div(len - full * kLeafChunk, kPage);
           }
-        } else if (p_class[i] == kClassChain) {
-          chain = ceil_div(p_T[i], tpt) * Hkv;
+        } else if (A.p_class[i] == kClassChain) {
+          chain = ceil_div(A.p_T[i], tpt) * Hkv;
         }
       }
+      const int last = c > 0 ? 1 : 0;
       if (e == 0) {
-        v[0][0] = root_items; v[1][0] = node_items; v[2][0] = dec; v[3][0] = slots; v[4][0] = full; v[5][0] = chain; cls[0] = c;
+        v[0][0] = root_items; v[1][0] = node_items; v[2][0] = dec; v[3][0] = slots; v[4][0] = full; v[5][0] = chain; v[6][0] = last; cls[0] = c;
       } else {
-        v[0][1] = root_items; v[1][1] = node_items; v[2][1] = dec; v[3][1] = slots; v[4][1] = full; v[5][1] = chain; cls[1] = c;
+        v[0][1] = root_items; v[1][1] = node_items; v[2][1] = dec; v[3][1] = slots; v[4][1] = full; v[5][1] = chain; v[6][1] = last; cls[1] = c;
       }
     }
-    small_scan(s_scan, v, cls, order);
+    block_scan<!LARGE>(S, v, cls, order);
+    const int roots = LARGE ? 0 : S.total[0];
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
-      const int i = 2 * tid + e;
-      if (i < N) n_base[i] = n_parent[i] < 0 ? v[0][e] : s_scan.total[0] + v[1][e];   // the roots' items come first
+      const int i = chunk * kScanChunk + 2 * tid + e;
+      if (i < N) A.n_base[i] = A.n_parent[i] < 0 ? v[0][e] : roots + v[1][e];   // the roots' items come first
       if (i < live) {
-        p_rank[i] = v[2][e];
-        p_slot[i] = v[3][e];
-        p_full[i] = v[4][e];
-        p_chain[i] = v[5][e];
-        p_last[i] = cls[e] > 0 ? order[e] : -1;
+        A.p_rank[i] = v[2][e];
+        A.p_slot[i] = v[3][e];
+        A.p_items[i] = A.p_class[i] == kClassChain ? v[5][e] : v[4][e];
+        A.p_last[i] = cls[e] > 0 ? (LARGE ? v[6][e] : order[e]) : -1;
       }
     }
+    if (LARGE && tid < kSums) A.sums[chunk * 8 + tid] = S.total[tid];
     __syncthreads();
   }
-
-  if (!failed) {
-    const int n_stacked = s_scan.total[0] + s_scan.total[1], n_dec_tok = s_scan.total[2], n_slots = s_scan.total[3];
-    const int n_full = s_scan.total[4] * Hkv, n_chain = s_scan.total[5];
-    int n_last_chunks = 0;
-    for (int r = 1; r < kLeafClasses; ++r) n_last_chunks += s_scan.cls_total[r];
-    const int n_leaf_items = n_full + n_last_chunks * Hkv;
-    failed = n_dec_tok > P.caps.dec || n_slots > P.caps.slots || n_leaf_items > P.caps.leaf_items || n_stacked + n_chain > P.caps.tile_items;
-    if (tid == 0) {
-      s_hdr.status = failed ? SS_ERR_WORKSPACE_TOO_SMALL : SS_OK;
-      s_hdr.n_dec = n_dec_tok;
-      s_hdr.n_slots = n_slots;
-      s_hdr.n_stacked_items = n_stacked;
-      s_hdr.n_generic_rows = s_generic;
-      if (!failed) {
-        s_hdr.n_leaf_items = n_leaf_items;
-        s_hdr.n_tile_items = n_stacked + n_chain;
+  if (LARGE) {
+    phase_failed(false, SS_OK);
+    // totals, and for each chunk of this block what lies in front of it
+#pragma unroll 1
+    for (int chunk = blockIdx.x; chunk == static_cast<int>(blockIdx.x) || chunk < n_chunks; chunk += gridDim.x) {
+      if (warp < kSums) {
+        int before = 0, all = 0;
+        for (int c = lane; c < n_chunks; c += 32) {
+          const int x = __ldcg(A.sums + c * 8 + warp);
+          all += x;
+          if (c < chunk) before += x;
+        }
+        before = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned>(before)));
+        all = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned>(all)));
+        if (lane == 0) {
+          S.tot[warp][0] = before;
+          S.total[warp] = all;
+        }
       }
+      __syncthreads();
+      if (chunk < n_chunks) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int i = chunk * kScanChunk + 2 * tid + e;
+          if (i < N) A.n_base[i] += A.n_parent[i] < 0 ? S.tot[0][0] : S.total[0] + S.tot[1][0];
+          if (i < live) {
+            A.p_rank[i] += S.tot[2][0];
+            A.p_slot[i] += S.tot[3][0];
+            A.p_items[i] += S.tot[A.p_class[i] == kClassChain ? 5 : 4][0];
+            if (A.p_last[i] >= 0) A.p_last[i] += S.tot[6][0];
+          }
+        }
+      }
+      __syncthreads();
     }
-    if (!failed) {
-      // ---- emission: a warp per path and per node --------------------------------------------------------------------------
-      const int wid = blockIdx.x * (kScanThreads / 32) + warp, nw = gridDim.x * (kScanThreads / 32);
-      if (wid == 0 && lane == 0) P.dec_slot_base[n_dec_tok] = n_slots;
+  }
+  if (tid == 0 && (!LARGE || blockIdx.x == 0)) {
+    const int* total = S.total;
+    const int n_stacked = total[0] + total[1], n_full = total[4] * Hkv, n_leaf_items = n_full + total[6] * Hkv;
+    const bool small_ws = total[2] > P.caps.dec || total[3] > P.caps.slots || n_leaf_items > P.caps.leaf_items ||
+                          n_stacked + total[5] > P.caps.tile_items;
+    if (small_ws) hdr->status = SS_ERR_WORKSPACE_TOO_SMALL;    // nothing is emitted, the executors see the status and do nothing
+    hdr->live_paths = live;
+    hdr->n_dec = total[2];
+    hdr->n_slots = total[3];
+    hdr->n_stacked_items = n_stacked;
+    hdr->n_generic_rows = totals[1];
+    hdr->n_full_leaf_items = n_full;
+    hdr->n_leaf_items = small_ws ? 0 : n_leaf_items;
+    hdr->n_tile_items = small_ws ? 0 : n_stacked + total[5];
+  }
+  return true;
+}
+
+// The item lists and the per-decode-token arrays: a warp per path and per node, of all blocks of the grid.
+template <bool LARGE>
+__device__ __forceinline__ void emit_items(const Params& P, const PlanArrays& A, const PlanHeader* hdr) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int N = P.num_nodes, Hkv = P.Hkv, tpt = P.tok_per_tile;
+  const int live = hdr->live_paths, n_stacked = hdr->n_stacked_items, n_full = hdr->n_full_leaf_items;
+  const int wid = blockIdx.x * (blockDim.x / 32) + warp, nw = gridDim.x * (blockDim.x / 32);
+  auto page0_of = [&](int n) { return LARGE ? static_cast<int32_t>(P.node_page_offsets[n]) : A.n_page0[n]; };
+  if (wid == 0 && lane == 0) P.dec_slot_base[hdr->n_dec] = hdr->n_slots;
 #pragma unroll 1
-      for (int p = wid; p < live; p += nw) {
-        const int leaf = p_leaf[p], len = n_len[leaf], cls = p_class[p], L = n_start[leaf] + len;
-        if (lane == 0) {                                       // (read by the generic rows and the exact second pass)
-          P.path_class[p] = cls;
-          P.path_kv_len[p] = L;
-        }
-        if (cls == kClassDecode) {
-          const int rank = p_rank[p], slot = p_slot[p];
-          const bool own_leaf = n_paths[leaf] == 1 && len > 0;
-          if (lane == 0) {
-            P.dec_tok[rank] = p_row[p];
-            P.dec_src[rank] = p_src[p];
-            P.dec_slot_base[rank] = slot;
-            P.dec_leaf_chunks[rank] = own_leaf ? ceil_div(len, kLeafChunk) : 0;
-          }
-          for (int g = lane; g < Hkv; g += 32) P.leaf_arrive[static_cast<int64_t>(rank) * Hkv + g] = 0;
-          if (!own_leaf) continue;
-          // whole chunks first, then the last chunks of all leaves, longest first: the leaf kernel hands its items out in
-          // this order, and the short ones level out its warps' ends (922 leaves of 32 to 512 keys: 71.6 -> 68.9 us)
-          const int full = len / kLeafChunk, last = p_last[p], n_items = (full + (last >= 0 ? 1 : 0)) * Hkv;
-#pragma unroll 1
-          for (int x = lane; x < n_items; x += 32) {
-            const int c = x / Hkv, g = x - c * Hkv;
-            LeafItem it;
-            it.page0 = n_page0[leaf] + c * (kLeafChunk / kPage);
-            it.node = leaf;
-            it.g = g;
-            it.kv_begin = c * kLeafChunk;
-            it.kv_end = min(len, (c + 1) * kLeafChunk);
-            it.slot = slot + n_level[leaf] + c;
-            it.q_src = p_src[p];
-            it.dec = rank;
-            P.leaf_items[c < full ? p_full[p] * Hkv + x : n_full + last * Hkv + g] = it;
-          }
-        } else if (cls == kClassChain) {
-          const int T = p_T[p], tiles = ceil_div(T, tpt);
-#pragma unroll 1
-          for (int x = lane; x < tiles * Hkv; x += 32) {
-            const int g = x / tiles, t = x - g * tiles;
-            TileItem it;
-            it.node = leaf;
-            it.tok0 = p_row[p] + t * tpt;
-            it.n_tok = min(tpt, T - t * tpt);
-            it.kind_g = (kItemChain << 16) | g;
-            it.kv_begin = 0;
-            it.limit0 = L - T + t * tpt + 1;
-            it.kv_end = max(0, min(L, it.limit0 + it.n_tok - 1));
-            it.slot_off = -1;
-            it.src0 = p_src[p] + t * tpt;
-            it.pad = 0;
-            P.tile_items[n_stacked + p_chain[p] + x] = it;
-          }
-        }
+  for (int p = wid; p < live; p += nw) {
+    const int leaf = A.p_leaf[p], len = A.n_len[leaf], cls = A.p_class[p], L = A.n_start[leaf] + len;
+    if (lane == 0) {                                           // (read by the generic rows and the exact second pass)
+      if (!LARGE) P.path_class[p] = cls;
+      P.path_kv_len[p] = L;
+    }
+    const int row = LARGE ? static_cast<int32_t>(P.q_offsets[p]) : A.p_row[p];
+    const int src = !LARGE ? A.p_src[p] : P.q_src_offsets ? static_cast<int32_t>(P.q_src_offsets[p]) : row;
+    if (cls == kClassDecode) {
+      const int rank = A.p_rank[p], slot = A.p_slot[p];
+      const bool own_leaf = A.n_paths[leaf] == 1 && len > 0;
+      if (lane == 0) {
+        P.dec_tok[rank] = row;
+        P.dec_src[rank] = src;
+        P.dec_slot_base[rank] = slot;
+        P.dec_leaf_chunks[rank] = own_leaf ? ceil_div(len, kLeafChunk) : 0;
       }
+      for (int g = lane; g < Hkv; g += 32) P.leaf_arrive[static_cast<int64_t>(rank) * Hkv + g] = 0;
+      if (!own_leaf) continue;
+      // whole chunks first, then the last chunks of all leaves - in the small form longest first: the leaf kernel hands its
+      // items out in this order, and the short ones level out its warps' ends (922 leaves of 32 to 512 keys: 71.6 -> 68.9 us)
+      const int page0 = page0_of(leaf), full = len / kLeafChunk, last = A.p_last[p], n_items = (full + (last >= 0 ? 1 : 0)) * Hkv;
 #pragma unroll 1
-      for (int n = wid; n < N; n += nw) {
-        if (lane == 0) P.node_start[n] = n_start[n];
-        const int tiles = n_tiles[n];
-        if (tiles == 0) continue;
-        const int splits = n_splits[n], split_len = n_split_len[n], len = n_len[n], nd = n_dec[n], rank0 = p_rank[n_first[n]];
+      for (int x = lane; x < n_items; x += 32) {
+        const int c = x / Hkv, g = x - c * Hkv;
+        LeafItem it;
+        it.page0 = page0 + c * (kLeafChunk / kPage);
+        it.node = leaf;
+        it.g = g;
+        it.kv_begin = c * kLeafChunk;
+        it.kv_end = min(len, (c + 1) * kLeafChunk);
+        it.slot = slot + A.n_level[leaf] + c;
+        it.q_src = src;
+        it.dec = rank;
+        P.leaf_items[c < full ? A.p_items[p] * Hkv + x : n_full + last * Hkv + g] = it;
+      }
+    } else if (cls == kClassChain) {
+      const int T = A.p_T[p], tiles = ceil_div(T, tpt);
 #pragma unroll 1
-        for (int x = lane; x < tiles * splits * Hkv; x += 32) {
-          const int rest = x / splits, split = x - rest * splits, tile = rest / Hkv, g = rest - tile * Hkv;
-          TileItem it;
-          it.node = n;
-          it.tok0 = rank0 + tile * tpt;
-          it.n_tok = min(tpt, nd - tile * tpt);
-          it.kind_g = (kItemStacked << 16) | g;
-          it.kv_begin = split * split_len;
-          it.kv_end = min(len, (split + 1) * split_len);
-          it.limit0 = it.kv_end;
-          it.slot_off = n_level[n] + split;
-          it.src0 = n_page0[n];
-          it.pad = 0;
-          P.tile_items[n_base[n] + x] = it;
-        }
+      for (int x = lane; x < tiles * Hkv; x += 32) {
+        const int g = x / tiles, t = x - g * tiles;
+        TileItem it;
+        it.node = leaf;
+        it.tok0 = row + t * tpt;
+        it.n_tok = min(tpt, T - t * tpt);
+        it.kind_g = (kItemChain << 16) | g;
+        it.kv_begin = 0;
+        it.limit0 = L - T + t * tpt + 1;
+        it.kv_end = max(0, min(L, it.limit0 + it.n_tok - 1));
+        it.slot_off = -1;
+        it.src0 = src + t * tpt;
+        it.pad = 0;
+        P.tile_items[n_stacked + A.p_items[p] + x] = it;
       }
     }
   }
+#pragma unroll 1
+  for (int n = wid; n < N; n += nw) {
+    if (!LARGE && lane == 0) P.node_start[n] = A.n_start[n];
+    const int tiles = A.n_tiles[n];
+    if (tiles == 0) continue;
+    const int page0 = page0_of(n), splits = A.n_splits[n], split_len = A.n_split_len[n], len = A.n_len[n], nd = A.n_dec[n],
+              rank0 = A.p_rank[A.n_first[n]];
+#pragma unroll 1
+    for (int x = lane; x < tiles * splits * Hkv; x += 32) {
+      const int rest = x / splits, split = x - rest * splits, tile = rest / Hkv, g = rest - tile * Hkv;
+      TileItem it;
+      it.node = n;
+      it.tok0 = rank0 + tile * tpt;
+      it.n_tok = min(tpt, nd - tile * tpt);
+      it.kind_g = (kItemStacked << 16) | g;
+      it.kv_begin = split * split_len;
+      it.kv_end = min(len, (split + 1) * split_len);
+      it.limit0 = it.kv_end;
+      it.slot_off = A.n_level[n] + split;
+      it.src0 = page0;
+      it.pad = 0;
+      P.tile_items[A.n_base[n] + x] = it;
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kThreads) plan_small_kernel(const __grid_constant__ Params P) {
+  ss::grid_dependency_enter();
+  extern __shared__ __align__(16) int32_t plan_smem[];
+  __shared__ PlanHeader s_hdr;
+  __shared__ BlockScan s_scan;
+  __shared__ int s_totals[2];
+  const int tid = threadIdx.x;
+  PlanArrays A;
+  int32_t* w = plan_smem;
+  for (int x = 0; x < kPlanNodeArrays + kPlanNodeInputs; ++x, w += P.num_nodes) A.node_array(x) = w;
+  for (int x = 0; x < kPlanPathArrays + kPlanPathInputs; ++x, w += P.num_paths) A.path_array(x) = w;
+  A.sums = nullptr;
+  for (int x = tid; x < kPlanHeaderWords; x += kThreads) reinterpret_cast<int32_t*>(&s_hdr)[x] = 0;
+  for (int x = tid; x < kLeafClasses * 64; x += kThreads) (&s_scan.hist[0][0])[x] = 0;
+  if (tid < 2) s_totals[tid] = 0;
+  SS_STAMP_BEGIN(P.hdr, 0);
+  make_plan<false>(P, A, &s_hdr, s_scan, nullptr, s_totals);
+  __syncthreads();
+  if (s_hdr.status == SS_OK) emit_items<false>(P, A, &s_hdr);
   if (blockIdx.x != 0) return;
-  if (tid == 0) s_hdr.live_paths = live;
 #ifdef SS_STAMPS
   __syncthreads();
   if (tid == 0) { s_hdr.stamp[0] = P.hdr->stamp[0]; s_hdr.stamp[1] = ss_globaltimer(); }
 #endif
   __syncthreads();
-  for (int x = tid; x < static_cast<int>(sizeof(PlanHeader) / 4); x += kScanThreads)
+  for (int x = tid; x < kPlanHeaderWords; x += kThreads)
     reinterpret_cast<int32_t*>(P.hdr)[x] = reinterpret_cast<const int32_t*>(&s_hdr)[x];
 }
 
+__global__ void __cluster_dims__(kLargeBlocks, 1, 1) __launch_bounds__(kThreads) plan_large_kernel(const __grid_constant__ Params P) {
+  ss::grid_dependency_enter();
+  __shared__ BlockScan s_scan;
+  __shared__ int s_bad[8], s_totals[2];
+  const int tid = threadIdx.x;
+  if (tid < 8) s_bad[tid] = 0;
+  if (tid < 2) s_totals[tid] = 0;
+  if (blockIdx.x == 0 && tid < kPlanHeaderWords) reinterpret_cast<int32_t*>(P.hdr)[tid] = 0;
+  cg::this_cluster().sync();
+  SS_STAMP_BEGIN(P.hdr, 0);
+  make_plan<true>(P, P.plan, P.hdr, s_scan, s_bad, cg::this_cluster().map_shared_rank(s_totals, 0));
+}
+
+__global__ void __launch_bounds__(kEmitThreads) plan_emit_kernel(const __grid_constant__ Params P) {
+  ss::grid_dependency_enter();
+  if (P.hdr->status == SS_OK) emit_items<true>(P, P.plan, P.hdr);
+  SS_STAMP_END(P.hdr, 1);
+}
+
 int32_t launch_plan(const Params& P, cudaStream_t st) {
-  if (P.num_nodes <= kSmallPlan && P.num_paths <= kSmallPlan) {     // (this kernel writes the whole header itself)
+  const int N = P.num_nodes, NP = P.num_paths;
+  if (N <= kSmallPlan && NP <= kSmallPlan) {                   // (this kernel writes the whole header itself)
+    auto smem = [](int n, int np) { return static_cast<size_t>(4) * (static_cast<size_t>(n) * (kPlanNodeArrays + kPlanNodeInputs) +
+                                         static_cast<size_t>(np) * (kPlanPathArrays + kPlanPathInputs)) + 64; };
     static bool configured[kDeviceSlots] = {false};
     const int dev_slot = current_device_slot();
     if (dev_slot < 0 || !configured[dev_slot]) {
       if (cudaFuncSetAttribute(plan_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               static_cast<int>(small_plan_smem(kSmallPlan, kSmallPlan))) != cudaSuccess) {
+                               static_cast<int>(smem(kSmallPlan, kSmallPlan))) != cudaSuccess) {
         (void)cudaGetLastError();
         return SS_ERR_CUDA;
       }
       if (dev_slot >= 0) configured[dev_slot] = true;
     }
-    SS_LAUNCH(plan_small_kernel, small_plan_blocks(P.num_nodes, P.num_paths), kScanThreads,
-              small_plan_smem(P.num_nodes, P.num_paths), st, P);
+    int blocks = (N + NP + 31) / 32;                           // what is left to share is the emission, a warp per path and node
+    blocks = blocks < 1 ? 1 : (blocks > 64 ? 64 : blocks);
+    SS_LAUNCH(plan_small_kernel, blocks, kThreads, smem(N, NP), st, P);
     return SS_OK;
   }
-  if (cudaMemsetAsync(P.hdr, 0, sizeof(PlanHeader), st) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return SS_ERR_CUDA;
-  }
-  const int64_t work = P.num_nodes > P.num_paths ? P.num_nodes : P.num_paths;
-  int blocks = static_cast<int>((work + kGridThreads - 1) / kGridThreads);
-  if (blocks < 1) blocks = 1;
-  if (blocks > 1184) blocks = 1184;
-  SS_LAUNCH(plan_nodes_kernel, blocks, kGridThreads, 0, st, P);
-  SS_LAUNCH(plan_paths_kernel, blocks, kGridThreads, 0, st, P);
-  {
-    static bool configured[kDeviceSlots] = {false};
-    const int dev_slot = current_device_slot();
-    if (dev_slot < 0 || !configured[dev_slot]) {
-      if (cudaFuncSetAttribute(plan_scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kScanStage * 4) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return SS_ERR_CUDA;
-      }
-      if (dev_slot >= 0) configured[dev_slot] = true;
-    }
-  }
-  SS_LAUNCH(plan_scan_kernel, 1, kScanThreads, kScanStage * 4, st, P);
-  // one thread per ITEM (there are an order of magnitude more items than paths; their number is known on the device
-  // only): a grid that covers the typical item count in one or two strides
-  SS_LAUNCH(plan_emit_kernel, blocks < 64 ? 8 * blocks : 1184, kGridThreads, 0, st, P);
+  SS_LAUNCH(plan_large_kernel, kLargeBlocks, kThreads, 0, st, P);
+  int64_t blocks = (static_cast<int64_t>(N) + NP + kEmitThreads / 32 - 1) / (kEmitThreads / 32);
+  if (blocks > P.sms * 8) blocks = P.sms * 8;
+  SS_LAUNCH(plan_emit_kernel, static_cast<int>(blocks), kEmitThreads, 0, st, P);
   return SS_OK;
 }
 

@@ -66,12 +66,15 @@ struct PlanHeader {       // first bytes of the workspace; status MUST be the fi
   int32_t tile_counter;   // work-stealing counters (reset by the planner)
   int32_t leaf_counter;
   int32_t n_stacked_items; // tile items [0, n_stacked_items) are stacked items, the rest chain items
-  int32_t pad[6];
+  int32_t n_full_leaf_items;  // leaf items of whole chunks: they come first
+  int32_t pad[5];
 #ifdef SS_STAMPS
-  unsigned long long stamp[40];  // instrumented build: %globaltimer at kernel starts / ends (see SS_STAMP); 8..23 (24..31: phases of the planner's scan; 32..36: of the one-block planner):
+  unsigned long long stamp[40];  // instrumented build: %globaltimer at kernel starts / ends (see SS_STAMP); 8..23:
                                  // clock sums of one softmax thread per tile-kernel block (where an item's time goes)
 #endif
 };
+
+constexpr int kPlanHeaderWords = sizeof(PlanHeader) / 4;
 
 // Instrumented build (-DSS_STAMPS): the first thread of a kernel records when it started (after its predecessor
 // completed), every block when it ended; slots 0/1 planner, 2/3 tile kernel, 4/5 leaf kernel, 6/7 merge.
@@ -91,6 +94,31 @@ __device__ __forceinline__ unsigned long long ss_globaltimer() {
 struct Caps {             // host-computed capacities of the plan arrays
   int32_t dec, tile_items, leaf_items;
   int64_t slots;
+};
+
+// The planner's arrays, per node and per path.  The large planner has those that it computes in the workspace and reads the
+// others where the caller has them; the small one copies everything to shared memory.
+constexpr int kPlanNodeArrays = 11, kPlanPathArrays = 5;               // computed
+constexpr int kPlanNodeInputs = 3, kPlanPathInputs = 4;
+struct PlanArrays {
+  // keys before the node, first / last path, paths and decode paths below, own partial slots, slots of the chain above, tiles,
+  // KV splits, their length, first tile item; parent, length, first page
+  int32_t *n_start, *n_first, *n_last, *n_paths, *n_dec, *n_own, *n_level, *n_tiles, *n_splits, *n_split_len, *n_base;
+  int32_t *n_parent, *n_len, *n_page0;
+  // class, decode rank, first slot, whole leaf chunks or chain items before it, rank of its last leaf chunk (-1: none); leaf,
+  // query tokens, output row, query row
+  int32_t *p_class, *p_rank, *p_slot, *p_items, *p_last;
+  int32_t *p_leaf, *p_T, *p_row, *p_src;
+  int32_t* sums;             // large planner: totals of every scan chunk, 8 apart (in an array that has no other use by then)
+  __host__ __device__ int32_t*& node_array(int i) {
+    int32_t** const a[kPlanNodeArrays + kPlanNodeInputs] = {&n_start, &n_first, &n_last, &n_paths, &n_dec, &n_own, &n_level,
+                                                            &n_tiles, &n_splits, &n_split_len, &n_base, &n_parent, &n_len, &n_page0};
+    return *a[i];
+  }
+  __host__ __device__ int32_t*& path_array(int i) {
+    int32_t** const a[kPlanPathArrays + kPlanPathInputs] = {&p_class, &p_rank, &p_slot, &p_items, &p_last, &p_leaf, &p_T, &p_row, &p_src};
+    return *a[i];
+  }
 };
 
 // Everything a kernel needs, passed by value.
@@ -115,12 +143,12 @@ struct Params {
   __nv_bfloat16* out;
   float* lse;
   int32_t target_tiles;      // the planner splits root nodes until about this many tile items exist
+  int32_t sms;               // SMs the call may use
   Caps caps;
   // ---- workspace regions ----
   PlanHeader* hdr;
-  int32_t *node_start, *node_depth, *node_first, *node_last, *node_npaths, *node_ndec, *node_own_slots,
-      *node_level_off, *node_item_base, *node_splits, *node_split_len;
-  int32_t *path_class, *path_kv_len, *path_dec_rank, *path_slot_base, *path_leaf_base, *path_chain_base;
+  int32_t *node_start, *path_class, *path_kv_len;   // keys before each node; read by the generic rows and the exact second pass
+  PlanArrays plan;           // the large planner's arrays
   int32_t *dec_tok, *dec_src, *dec_slot_base;   // per decode token: output row, query row, first partial slot
   int32_t *dec_leaf_chunks;  // per decode token: leaf items per kv head (0: empty or shared leaf)
   int32_t *leaf_arrive;      // [decode token][kv head]: leaf items that have written their partial (zeroed by the planner)

@@ -700,12 +700,12 @@ def test_attention_pool_blocks_off_the_8_row_grid():
 
 
 # =========================================================================================================
-# the planner's small and general form
+# the planner's small and large form
 # =========================================================================================================
-@pytest.mark.parametrize("paths", [1, 31, 33, 1023, 1025, 2046, 2047, 2048])
-def test_planner_at_the_edges_of_its_small_form(paths):
-    """One root with `paths` leaves (paths + 1 nodes; the one-launch planner takes up to 2048 of each, two per thread):
-    decode, verification and leaves of 0, one chunk, a chunk and a page, and several chunks."""
+@pytest.mark.parametrize("paths", [1, 31, 33, 1023, 1025, 2046, 2047, 2048, 4095, 4097, 6200])
+def test_planner_at_the_edges_of_its_forms(paths):
+    """One root with `paths` leaves (paths + 1 nodes; the small planner takes up to 2048 of each, the large one scans
+    chunks of 2048): decode, verification and leaves of 0, one chunk, a chunk and a page, and several chunks."""
     lens = [0, 1, 16, 255, 256, 257, 272, 600]
     w = synth.build_tree_workload("planner", 7000 + paths, 4, 2, [48], [paths], 1, (0, 0),
                                   lambda i, n, rng: 1 if i % 5 else 3, device="cpu", poison=False)
