@@ -17,7 +17,7 @@
 // Bound: the latency of the phases behind barriers, and of code that runs once (instruction fetches).  Measured, small: 922
 // unique paths 20.9 -> 11.5 us, 256 verification paths 29.1 -> 8.2, 8 paths 12.0 -> 8.1 (against one block that shared the
 // phases of a chain of five kernels and searched a path for every item).  Large, against that chain with its scan in one
-// block, between events: 2912 paths 42.6 -> 29.8 us, 6400 57.8 -> 29.8, 25600 183 -> 57, 64000 452 -> 101; as ONE cooperative
+// block, between events: 2912 paths 42.6 -> 29.2 us, 6400 57.8 -> 29.3, 25600 183 -> 54, 64000 452 -> 99; as ONE cooperative
 // kernel with a barrier over the grid 40.7 and 43.9 for the first two (seven barriers, a memset, no overlap with its
 // neighbours' launches).
 // The header (status word first) is cleared and written by the planner itself.
@@ -346,8 +346,8 @@ __device__ __forceinline__ bool make_plan(const Params& P, const PlanArrays& A, 
       if (i < live) {
         A.p_rank[i] = v[2][e];
         A.p_slot[i] = v[3][e];
-        A.p_items[i] = A.p_class[i] == kClassChain ? v[5][e] : v[4][e];
-        A.p_last[i] = cls[e] > 0 ? (LARGE ? v[6][e] : order[e]) : -1;
+        A.p_items[i] = A.p_class[i] == kClassChain ? v[5][e] : v[4][e] + (LARGE ? v[6][e] : 0);
+        if (!LARGE) A.p_last[i] = cls[e] > 0 ? order[e] : -1;
       }
     }
     if (LARGE && tid < kSums) A.sums[chunk * 8 + tid] = S.total[tid];
@@ -381,8 +381,7 @@ __device__ __forceinline__ bool make_plan(const Params& P, const PlanArrays& A, 
           if (i < live) {
             A.p_rank[i] += S.tot[2][0];
             A.p_slot[i] += S.tot[3][0];
-            A.p_items[i] += S.tot[A.p_class[i] == kClassChain ? 5 : 4][0];
-            if (A.p_last[i] >= 0) A.p_last[i] += S.tot[6][0];
+            A.p_items[i] += A.p_class[i] == kClassChain ? S.tot[5][0] : S.tot[4][0] + S.tot[6][0];
           }
         }
       }
@@ -436,9 +435,12 @@ __device__ __forceinline__ void emit_items(const Params& P, const PlanArrays& A,
       }
       for (int g = lane; g < Hkv; g += 32) P.leaf_arrive[static_cast<int64_t>(rank) * Hkv + g] = 0;
       if (!own_leaf) continue;
-      // whole chunks first, then the last chunks of all leaves - in the small form longest first: the leaf kernel hands its
-      // items out in this order, and the short ones level out its warps' ends (922 leaves of 32 to 512 keys: 71.6 -> 68.9 us)
-      const int page0 = page0_of(leaf), full = len / kLeafChunk, last = A.p_last[p], n_items = (full + (last >= 0 ? 1 : 0)) * Hkv;
+      // The leaf kernel hands its items out in this order.  Small form: whole chunks first, then the last chunks of all leaves,
+      // longest first, so that the short ones level out the warps' ends (922 leaves of 32 to 512 keys: 71.6 -> 68.9 us).  Large
+      // form: leaf after leaf; with many items per warp the order by length only costs (6550 leaves of 128 to 1024 keys: 2.46 ms,
+      // whole chunks first 2.43, leaf after leaf 2.37)
+      const int page0 = page0_of(leaf), full = len / kLeafChunk, n_items = ceil_div(len, kLeafChunk) * Hkv;
+      const int last = LARGE ? 0 : A.p_last[p];
 #pragma unroll 1
       for (int x = lane; x < n_items; x += 32) {
         const int c = x / Hkv, g = x - c * Hkv;
@@ -451,7 +453,7 @@ __device__ __forceinline__ void emit_items(const Params& P, const PlanArrays& A,
         it.slot = slot + A.n_level[leaf] + c;
         it.q_src = src;
         it.dec = rank;
-        P.leaf_items[c < full ? A.p_items[p] * Hkv + x : n_full + last * Hkv + g] = it;
+        P.leaf_items[LARGE || c < full ? A.p_items[p] * Hkv + x : n_full + last * Hkv + g] = it;
       }
     } else if (cls == kClassChain) {
       const int T = A.p_T[p], tiles = ceil_div(T, tpt);

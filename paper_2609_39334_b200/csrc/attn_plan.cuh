@@ -105,7 +105,8 @@ struct PlanArrays {
   // KV splits, their length, first tile item; parent, length, first page
   int32_t *n_start, *n_first, *n_last, *n_paths, *n_dec, *n_own, *n_level, *n_tiles, *n_splits, *n_split_len, *n_base;
   int32_t *n_parent, *n_len, *n_page0;
-  // class, decode rank, first slot, whole leaf chunks or chain items before it, rank of its last leaf chunk (-1: none); leaf,
+  // class, decode rank, first slot, leaf items (small: whole chunks only) or chain items before it, rank of its last
+  // leaf chunk (small; -1: none); leaf,
   // query tokens, output row, query row
   int32_t *p_class, *p_rank, *p_slot, *p_items, *p_last;
   int32_t *p_leaf, *p_T, *p_row, *p_src;
