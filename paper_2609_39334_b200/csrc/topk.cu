@@ -17,6 +17,7 @@ namespace topk {
 
 constexpr int kMaxThreads = 1024;
 constexpr int kSmemKeys = 4096;     // 32 KB of shared memory
+constexpr uint64_t kUnverified = 0xffffffff80000000ull;   // | index: a NaN's key has the same high word, bit 31 clear
 
 __device__ __forceinline__ uint64_t make_key(float f, uint32_t local_idx) {
   uint32_t ordered;                           // ascending in the score
@@ -197,12 +198,11 @@ early_prune_kernel(const float* __restrict__ scores, const uint8_t* __restrict__
   const bool all_verified = nver == g.n;
   for (int j = (all_verified ? nver : 0) + tid; j < k; j += nt) out[j] = -1;
   sorted(g.n, smem_keys, scratch + 2 * static_cast<int64_t>(g.lo),
-         [&](int i) {                             // (an unverified one: behind every score's key, still distinct)
-           return verified[g.lo + i] ? make_key(scores[g.lo + i], static_cast<uint32_t>(i))
-                                     : (0xffffffffull << 32) | static_cast<uint32_t>(i);
+         [&](int i) {                             // (an unverified one: behind every score's key, a NaN's too, still distinct)
+           return verified[g.lo + i] ? make_key(scores[g.lo + i], static_cast<uint32_t>(i)) : kUnverified | static_cast<uint32_t>(i);
          },
          [&](int j, uint64_t key) {
-           const int cand = g.lo + static_cast<int>(key & 0xffffffffu);
+           const int cand = g.lo + static_cast<int>(key & 0x7fffffffu);
            pruned[cand] = j < nver && nver > k && j >= k ? 1 : 0;
            if (all_verified && j < k) out[j] = cand;
          });

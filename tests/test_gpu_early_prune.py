@@ -128,3 +128,20 @@ def test_segments_at_the_edges_of_the_register_sort(sizes, k):
         want = oracle.early_prune(sc[3:-5], ver[3:-5], seg - 3, k)
         assert np.array_equal(got[0], np.concatenate([np.zeros(3), want[0], np.zeros(5)]))
         assert np.array_equal(got[1], np.where(want[1] >= 0, want[1] + 3, -1)) and np.array_equal(got[2], want[2])
+
+
+@pytest.mark.parametrize("sizes,k", [([3], 1), ([8] * 40, 2), ([64, 300, 1000], 20), ([3000, 10], 5), ([5000, 9000], 40)])
+def test_nan_scores_among_unverified_candidates(sizes, k):
+    """A verified NaN ranks below every score but above what has not been verified, wherever their indices lie: in the register
+    sort, in shared memory (3000) and in the workspace (5000, 9000)."""
+    rng = np.random.default_rng(sum(sizes) + k)
+    seg = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int32)
+    n = int(seg[-1])
+    for nan_frac, frac in ((0.5, 0.5), (0.1, 0.9), (0.9, 0.3), (0.3, 1.0)):
+        sc = (rng.integers(0, 9, size=n) / 8.0).astype(np.float32) * np.float32(0.99)
+        sc[rng.random(n) < nan_frac] = np.nan
+        ver = (rng.random(n) < frac).astype(np.uint8)
+        if n == 3:
+            sc, ver = np.asarray([0.9, np.nan, 0.5], np.float32), np.asarray([0, 1, 1], np.uint8)
+        for g, w in zip(run(sc, ver, seg, k), oracle.early_prune(sc, ver, seg, k)):
+            assert np.array_equal(g, w)
