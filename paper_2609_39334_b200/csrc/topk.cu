@@ -6,8 +6,8 @@
 // candidate per thread is sorted in registers (a bitonic network, partners in the warp through shuffles, the others through
 // shared memory), a larger one in shared memory (up to kSmemKeys) or in the caller's workspace; then the first k indices
 // and the mask are written.
-// Latency-bound.  One launch and nothing else: the blocks themselves clear what lies outside every segment, and block 0
-// checks all segments and writes the status word.  Measured: 64 segments of 256 half
+// Latency-bound.  One launch and nothing else: block 0 checks all segments, writes the status word and clears the mask
+// outside every segment.  Measured: 64 segments of 256 half
 // verified 16.4 -> 10.3 us a call (two memsets in front of the kernel before), 4 segments of 256 9.1 -> 5.8 us in the kernel
 // (a shared-memory network with a barrier per stage before).
 #include "common.cuh"
@@ -69,32 +69,52 @@ __device__ uint64_t sort_registers(uint64_t k, int n_pad, uint64_t* s_key) {
 }
 
 // A block's segment.  One that does not lie inside [0, n_total] is reported and treated as empty: its offsets index the mask
-// and the scratch region, so following them would write out of bounds.  Clears `mask` outside every segment (before the
-// first, after the last, where a bad one lies); block 0 looks at all segments and writes the status word.
+// and the scratch region, so following them would write out of bounds.  Block 0 looks at all segments, writes the status word
+// and clears `mask` where NO valid segment lies, so that it never writes what another block does: in front of the first and
+// behind the last one, or, with a bad one among them, wherever `covered` (kSmemKeys words) says.
 struct Segment {
   int lo, n;
 };
-__device__ __forceinline__ Segment open_segment(const int32_t* __restrict__ seg_offsets, int n_total, uint8_t* mask,
-                                                int32_t* status) {
-  const int s = blockIdx.x, last = gridDim.x - 1, nt = blockDim.x;
-  const int lo = seg_offsets[s], hi = seg_offsets[s + 1];
-  const bool bad = lo < 0 || hi < lo || hi > n_total;
-  auto clear = [&](int from, int to) {
-    for (int i = max(from, 0) + static_cast<int>(threadIdx.x); i < min(to, n_total); i += nt) mask[i] = 0;
-  };
-  if (bad) clear(lo, hi);
-  if (s == 0) {
-    clear(0, lo);
-    bool any = false;
-    for (int x = threadIdx.x; x <= last; x += nt) {
-      const int l = seg_offsets[x], h = seg_offsets[x + 1];
-      any = any || l < 0 || h < l || h > n_total;
+__device__ __forceinline__ bool valid_segment(int lo, int hi, int n_total) { return lo >= 0 && hi >= lo && hi <= n_total; }
+__device__ __noinline__ void clear_uncovered(const int32_t* __restrict__ seg_offsets, int n_segments, int n_total, uint8_t* mask,
+                                             uint32_t* covered) {
+  constexpr int kWindow = kSmemKeys * 64;                     // candidates a pass, a bit each
+  const int tid = threadIdx.x, nt = blockDim.x;
+  for (int base = 0; base < n_total; base = base > n_total - kWindow ? n_total : base + kWindow) {
+    const int end = n_total - base < kWindow ? n_total : base + kWindow;
+    for (int i = tid; i < kWindow / 32; i += nt) covered[i] = 0;
+    __syncthreads();
+    for (int x = tid; x < n_segments; x += nt) {
+      if (!valid_segment(seg_offsets[x], seg_offsets[x + 1], n_total)) continue;
+      const int l = max(seg_offsets[x], base) - base, h = min(seg_offsets[x + 1], end) - base;
+      for (int w = l >> 5; l < h && w <= (h - 1) >> 5; ++w) {
+        const uint32_t from = 0xffffffffu << (w == l >> 5 ? l & 31 : 0), to = 0xffffffffu >> (w == (h - 1) >> 5 ? 31 - ((h - 1) & 31) : 0);
+        atomicOr(&covered[w], from & to);
+      }
     }
+    __syncthreads();
+    for (int i = tid; i < end - base; i += nt)
+      if (!((covered[i >> 5] >> (i & 31)) & 1u)) mask[base + i] = 0;
+    __syncthreads();
+  }
+}
+__device__ __forceinline__ Segment open_segment(const int32_t* __restrict__ seg_offsets, int n_total, uint8_t* mask,
+                                                int32_t* status, uint64_t* smem_keys) {
+  const int s = blockIdx.x, n_segments = gridDim.x, nt = blockDim.x;
+  const int lo = seg_offsets[s], hi = seg_offsets[s + 1];
+  if (s == 0) {
+    bool any = false;
+    for (int x = threadIdx.x; x < n_segments; x += nt) any = any || !valid_segment(seg_offsets[x], seg_offsets[x + 1], n_total);
     any = __syncthreads_or(any) != 0;
     if (threadIdx.x == 0) *status = any ? SS_ERR_BAD_INPUT : SS_OK;
+    if (any) {
+      clear_uncovered(seg_offsets, n_segments, n_total, mask, reinterpret_cast<uint32_t*>(smem_keys));
+    } else {
+      for (int i = threadIdx.x; i < lo; i += nt) mask[i] = 0;
+      for (int i = seg_offsets[n_segments] + static_cast<int>(threadIdx.x); i < n_total; i += nt) mask[i] = 0;
+    }
   }
-  if (s == last) clear(hi, n_total);
-  return Segment{lo, bad ? 0 : hi - lo};
+  return Segment{lo, valid_segment(lo, hi, n_total) ? hi - lo : 0};
 }
 
 // Calls rank(j, key) for the key of every rank j < n, n keys from make(i).  `scratch`: where neither the registers nor
@@ -122,7 +142,7 @@ topk_kernel(const float* __restrict__ scores, const int32_t* __restrict__ seg_of
             int32_t* __restrict__ status) {
   ss::grid_dependency_enter();
   __shared__ uint64_t smem_keys[kSmemKeys];
-  const Segment g = open_segment(seg_offsets, n_total, keep, status);
+  const Segment g = open_segment(seg_offsets, n_total, keep, status, smem_keys);
   int32_t* out = survivors + static_cast<int64_t>(blockIdx.x) * k;
   for (int j = g.n + threadIdx.x; j < k; j += blockDim.x) out[j] = -1;
   if (g.n == 0) return;
@@ -152,7 +172,7 @@ early_prune_kernel(const float* __restrict__ scores, const uint8_t* __restrict__
   __shared__ int s_nver, s_nperfect, s_warp[32];
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) { s_nver = 0; s_nperfect = 0; }
-  const Segment g = open_segment(seg_offsets, n_total, pruned, status);
+  const Segment g = open_segment(seg_offsets, n_total, pruned, status, smem_keys);
   int32_t* out = selected + static_cast<int64_t>(blockIdx.x) * k;
   if (g.n == 0) {
     for (int j = tid; j < k; j += nt) out[j] = -1;

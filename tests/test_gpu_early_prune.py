@@ -145,3 +145,36 @@ def test_nan_scores_among_unverified_candidates(sizes, k):
             sc, ver = np.asarray([0.9, np.nan, 0.5], np.float32), np.asarray([0, 1, 1], np.uint8)
         for g, w in zip(run(sc, ver, seg, k), oracle.early_prune(sc, ver, seg, k)):
             assert np.array_equal(g, w)
+
+
+@pytest.mark.parametrize("off,n", [([0, 20, 10], 30), ([25, 5, 20], 30), ([0, 300, 100, 200], 200), ([0, 10, -5], 40), ([-3, 10, 30], 40),
+                                   ([0, 0] + [100] * 60000 + [0], 150), ([0, 0] + [100] * 60000 + [50], 150),
+                                   ([300100, 400000, 700000, 100, 262200], 600000)])
+def test_bad_segments_leave_the_masks_of_valid_ones_alone(off, n):
+    """A segment that runs backwards or out of [0, n) counts as empty: the masks of the valid ones hold what they would hold
+    without it, and everything outside them is 0 - also where a block behind thousands of others has the bad segment, and
+    where more candidates are to be looked at than a pass of the clearing takes."""
+    rng = np.random.default_rng(n)
+    k, P = 5, len(off) - 1
+    sc = (rng.integers(0, 30, size=n) / 32.0).astype(np.float32)
+    ver = (rng.random(n) < 0.7).astype(np.uint8)
+    keep_ref, pruned_ref = np.zeros(n, np.uint8), np.zeros(n, np.uint8)
+    surv_ref, sel_ref, fin_ref = np.full((P, k), -1, np.int32), np.full((P, k), -1, np.int32), np.ones(P, np.uint8)
+    for s in range(P):
+        lo, hi = off[s], off[s + 1]
+        if not 0 <= lo < hi <= n:
+            continue
+        x, y = oracle.topk(sc[lo:hi], np.asarray([0, hi - lo], np.int32), k)
+        keep_ref[lo:hi], surv_ref[s] = y, np.where(x[0] >= 0, x[0] + lo, -1)
+        x, y, z = oracle.early_prune(sc[lo:hi], ver[lo:hi], np.asarray([0, hi - lo], np.int32), k)
+        pruned_ref[lo:hi], sel_ref[s], fin_ref[s] = x, np.where(y[0] >= 0, y[0] + lo, -1), z[0]
+    dev = torch.device(DEV)
+    surv = torch.full((P, k), -9, dtype=torch.int32, device=dev)
+    ws = B.alloc_workspace(B.ss_topk_workspace_bytes(n), dev)
+    for _ in range(10):
+        keep = torch.full((n,), 7, dtype=torch.uint8, device=dev)
+        B.ss_topk_prune(torch.from_numpy(sc).to(dev), torch.tensor(off, dtype=torch.int32, device=dev), P, n, k, surv, keep, ws)
+        assert B.ss_last_device_status(ws) == B.SS_ERR_BAD_INPUT
+        assert np.array_equal(keep.cpu().numpy(), keep_ref) and np.array_equal(surv.cpu().numpy(), surv_ref)
+        for g, w in zip(run(sc, ver, off, k), (pruned_ref, sel_ref, fin_ref)):
+            assert np.array_equal(g, w)
