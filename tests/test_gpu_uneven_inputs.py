@@ -1,0 +1,40 @@
+"""Calls far from the usual proportions must not fall off a cliff: each is timed against an ordinary call with the same work,
+with a bound that leaves a factor of two for the machine's noise.  (What they return is compared with the oracle elsewhere.)"""
+import numpy as np
+import pytest
+import torch
+
+from paper_2609_39334_b200 import binding as B
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def device_us(fn, reps=5):
+    """Least time of a call on the device, warmed up."""
+    best = float("inf")
+    for _ in range(reps + 1):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        fn()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) * 1e3)
+    return best
+
+
+@pytest.mark.parametrize("call", ["topk", "early_prune"])
+def test_one_large_segment_among_many_small_ones(call):
+    """The block size follows the average segment; the largest one is sorted by such a block (measured 1.5 times the large
+    segment alone, which has four times the threads; 4.5 with blocks of 64)."""
+    def us(sizes):
+        seg = torch.tensor(np.concatenate([[0], np.cumsum(sizes)]), dtype=torch.int32, device=DEV)
+        n, P, k = int(seg[-1]), len(sizes), 8
+        sc, ver = torch.rand(n, device=DEV) * 0.9, torch.ones(n, dtype=torch.uint8, device=DEV)
+        mask, fin = torch.empty(n, dtype=torch.uint8, device=DEV), torch.empty(P, dtype=torch.uint8, device=DEV)
+        sel = torch.empty((P, k), dtype=torch.int32, device=DEV)
+        ws = B.alloc_workspace(B.ss_topk_workspace_bytes(n), torch.device(DEV))
+        if call == "topk":
+            return device_us(lambda: B.ss_topk_prune(sc, seg, P, n, k, sel, mask, ws))
+        return device_us(lambda: B.ss_early_prune(sc, ver, seg, P, n, k, mask, sel, fin, ws))
+    assert us([4096] + [16] * 1000) < 3 * us([4096])
