@@ -103,6 +103,7 @@ __device__ __forceinline__ Segment open_segment(const int32_t* __restrict__ seg_
   const int s = blockIdx.x, n_segments = gridDim.x, nt = blockDim.x;
   const int lo = seg_offsets[s], hi = seg_offsets[s + 1];
   if (s == 0) {
+    const int tail = seg_offsets[n_segments];                 // (loaded with the others, not behind the barrier)
     bool any = false;
     for (int x = threadIdx.x; x < n_segments; x += nt) any = any || !valid_segment(seg_offsets[x], seg_offsets[x + 1], n_total);
     any = __syncthreads_or(any) != 0;
@@ -111,7 +112,7 @@ __device__ __forceinline__ Segment open_segment(const int32_t* __restrict__ seg_
       clear_uncovered(seg_offsets, n_segments, n_total, mask, reinterpret_cast<uint32_t*>(smem_keys));
     } else {
       for (int i = threadIdx.x; i < lo; i += nt) mask[i] = 0;
-      for (int i = seg_offsets[n_segments] + static_cast<int>(threadIdx.x); i < n_total; i += nt) mask[i] = 0;
+      for (int i = tail + static_cast<int>(threadIdx.x); i < n_total; i += nt) mask[i] = 0;
     }
   }
   return Segment{lo, valid_segment(lo, hi, n_total) ? hi - lo : 0};
@@ -229,12 +230,14 @@ early_prune_kernel(const float* __restrict__ scores, const uint8_t* __restrict__
   if (tid == 0) final_out[blockIdx.x] = all_verified ? 1 : 0;
 }
 
-// Threads per block: one per candidate of a segment of average size, but at least kMinThreads, since any one segment may be
-// far above the average: one of 4096 candidates among 1000 of 16 takes 236 us with 64 threads and 76 with 256, while segments
-// of 8 or 16 gain nothing from smaller blocks (shared memory allows 7 blocks an SM either way).
+// Threads per block: one per candidate of a segment of average size, but at least kMinThreads where there are so many candidates,
+// since any one segment may be far above the average: one of 4096 among 1000 of 16 takes 236 us with 64 threads and 76 with 256,
+// while small segments gain nothing from smaller blocks (shared memory allows 7 blocks an SM either way) but at the bare
+// latency of a handful of candidates.
 constexpr int kMinThreads = 256;
 static int block_threads(int n_total, int n_segments) {
-  int t = kMinThreads;
+  int t = 64;
+  while (t < kMinThreads && t < n_total) t <<= 1;
   while (t < kMaxThreads && static_cast<int64_t>(t) * n_segments < n_total) t <<= 1;
   return t;
 }
