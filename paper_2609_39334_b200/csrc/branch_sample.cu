@@ -130,9 +130,9 @@ __device__ __forceinline__ double slice_sums(const float* __restrict__ row, cons
     float mn = l[0];
 #pragma unroll
     for (int x = 0; x < 8; ++x) { mx = fmaxf(mx, l[x]); mn = fminf(mn, l[x]); }
-    if (__any_sync(0xffffffffu, !(mn >= A.lowest))) {          // masked tokens, or past the end
+    if (__any_sync(0xffffffffu, !(mn >= A.lowest))) {          // masked tokens, or past the end (a NaN stays one)
 #pragma unroll
-      for (int x = 0; x < 8; ++x) l[x] = fmaxf(l[x], A.lowest);
+      for (int x = 0; x < 8; ++x) l[x] = l[x] < A.lowest ? A.lowest : l[x];
     }
 #pragma unroll
     for (int x = 0; x < 8; x += 2) {

@@ -105,3 +105,30 @@ def test_branch_sample_slices_segments_and_ranges(V, kind):
     sure = margin > 1e-12
     assert np.array_equal(got[sure], want_tok[sure])
     assert np.array_equal(got[u == 0.0], want_tok[u == 0.0])
+
+
+@pytest.mark.parametrize("V", [5, 700, 9000, 151936])
+@pytest.mark.parametrize("masked", [False, True])
+def test_a_row_with_a_nan_draws_its_last_token(V, masked):
+    """No cumulative sum exceeds a target that is NaN, wherever the NaN lies: beside ordinary tokens, beside masked ones, in a
+    segment that ends with the row, or alone.  The rows around it are not touched."""
+    rng = np.random.default_rng(V)
+    S = 9
+    logits = (rng.normal(size=(S, V)) * 3).astype(np.float32)
+    if masked:
+        logits[rng.random((S, V)) < 0.3] = -np.inf
+        logits[:, 1] = 0.5
+    for s, at in ((1, 0), (3, V - 1), (5, V // 2), (6, slice(None))):
+        logits[s, at] = np.nan
+    off = np.arange(S + 1, dtype=np.int64) * 6
+    u = rng.random(6 * S).astype(np.float32)
+    u[::6] = 0.0
+    tok, _ = run(logits, off, u, 0.8)
+    got = tok.cpu().numpy().reshape(S, 6)
+    want, _, margin = oracle.branch_sample(logits, off, u, 0.8)
+    want, sure = want.reshape(S, 6), margin.reshape(S, 6) > 1e-12
+    for s in range(S):
+        if np.isnan(logits[s]).any():
+            assert (got[s] == V - 1).all() and (want[s] == V - 1).all()
+        else:
+            assert np.array_equal(got[s][sure[s]], want[s][sure[s]])
