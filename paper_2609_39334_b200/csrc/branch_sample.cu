@@ -309,8 +309,12 @@ __device__ __forceinline__ void draws(const Args& A, Sums<CL>* sums, const doubl
       const double before = start + in_front;
       const int n_seg = (L.n_half + 1) >> 1;                   // at most kMaxSegs
       const double end_s = lane < n_seg ? seg_end[lane] : 0.0;
-      const uint32_t hit = __ballot_sync(0xffffffffu, lane < n_seg && before + end_s > t);
-      const int s = hit ? __ffs(hit) - 1 : n_seg - 1;
+      // (the slice was chosen by start + (in_front + sum), a segment is by (start + in_front) + sum so far: rounded differently,
+      //  the slice's end may not be above t here.  Then it is the last segment that added anything - behind it all is masked)
+      uint32_t hit = __ballot_sync(0xffffffffu, lane < n_seg && before + end_s > t);
+      const double last_end = __shfl_sync(0xffffffffu, end_s, max(n_seg - 1, 0));
+      if (!hit) hit = __ballot_sync(0xffffffffu, lane < n_seg && end_s == last_end);
+      const int s = __ffs(hit) - 1;
       if (s >= 0) {
         const double in_slice = s ? __shfl_sync(0xffffffffu, end_s, max(s - 1, 0)) : 0.0;
         const int base = L.v0 + s * kSeg, end = min(A.vocab, L.v0 + A.slice);

@@ -132,3 +132,38 @@ def test_a_row_with_a_nan_draws_its_last_token(V, masked):
             assert (got[s] == V - 1).all() and (want[s] == V - 1).all()
         else:
             assert np.array_equal(got[s][sure[s]], want[s][sure[s]])
+
+
+def test_targets_between_two_roundings_of_a_slice_end():
+    """The end of a warp's slice is rounded one way when the slice is chosen and another when its segment is.  Rows are made whose
+    target (u = 1/2) lies between the two: three terms S, f, x in three slices with fl(S + fl(f + x)) above fl(fl(S + f) + x) = a,
+    the rest of x's slice masked, and a tail that makes the total 2 a (64 rows scan the rounding of the table's exponentials).
+    The draw is x or the tail's first token, never a masked one.  Slices of 1024 tokens, 32 of them over a cluster of two blocks."""
+    V, S_rows = 32768, 64
+    dev = torch.device(DEV)
+    rng = np.random.default_rng(7)
+    at_s, at_f, at_x, at_y = 10, 16 * 1024 + 3, 17 * 1024 + 5, [20 * 1024 + i for i in range(3)]
+    off = torch.arange(S_rows + 1, dtype=torch.int64, device=dev)
+    u = torch.full((S_rows,), 0.5, device=dev)
+    tok = torch.empty(S_rows, dtype=torch.int32, device=dev)
+    seq = torch.empty(S_rows, dtype=torch.int64, device=dev)
+    tried = 0
+    while tried < 60:
+        l = rng.normal(size=3).astype(np.float32)
+        s, f, x = (float(v) for v in np.exp(l.astype(np.float64)))
+        a = (s + f) + x
+        if not s + (f + x) > a:
+            continue
+        tried += 1
+        logits = torch.full((S_rows, V), -float("inf"), device=dev)
+        cols = np.empty((S_rows, 6), np.float32)
+        for r in range(S_rows):
+            left = a + (r - S_rows // 2) * a * 2.0 ** -53          # the tail's sum, about a
+            cols[r, :3] = l
+            for i, share in enumerate((1.0 - 2.0 ** -20, 1.0 - 2.0 ** -14, 1.0)):
+                y = np.float32(np.log(left * share))
+                left -= float(np.exp(np.float64(y)))
+                cols[r, 3 + i] = y
+        logits[:, [at_s, at_f, at_x] + at_y] = torch.from_numpy(cols).to(dev)
+        B.ss_branch_sample(logits, off, u, S_rows, V, 1.0, tok, seq)
+        assert set(tok.tolist()) <= {at_x, at_y[0]}
