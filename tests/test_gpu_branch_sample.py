@@ -167,3 +167,20 @@ def test_targets_between_two_roundings_of_a_slice_end():
         logits[:, [at_s, at_f, at_x] + at_y] = torch.from_numpy(cols).to(dev)
         B.ss_branch_sample(logits, off, u, S_rows, V, 1.0, tok, seq)
         assert set(tok.tolist()) <= {at_x, at_y[0]}
+
+
+@pytest.mark.parametrize("S", [2, 40, 160])
+@pytest.mark.parametrize("V,live", [(151936, 10), (32001, 1), (9000, 8500)])
+def test_uniform_zero_draws_the_first_token_with_any_probability(S, V, live):
+    """u = 0: the first token whose term is not 0 in fp64, behind masked ones and ones that underflow to 0 (1000 below the
+    maximum at T = 0.8); one that is merely tiny (590 below: 1e-320) counts.  Rows on clusters of 8, 2 and 1 blocks."""
+    rng = np.random.default_rng(V)
+    logits = np.full((S, V), -np.inf, np.float32)
+    logits[:, V - live:] = (rng.normal(size=(S, live)) * 3).astype(np.float32)
+    logits[1::2, : V // 2] = -900.0
+    logits[::4, (V - live) // 2] = logits[::4].max(axis=1) - 590.0
+    off = np.arange(S + 1, dtype=np.int64) * 2
+    u = np.tile(np.asarray([0.0, 0.5], np.float32), S)
+    tok, _ = run(logits, off, u, 0.8)
+    want, _, _ = oracle.branch_sample(logits, off, u, 0.8)
+    assert np.array_equal(tok.cpu().numpy()[::2], want[::2])
