@@ -16,7 +16,7 @@
 // of a split barrier, so that neither the barrier nor a draw is waited for; the warps that draw change from row to row.
 // There is no pass for the maximum: fp64 holds 2^(logit * c) itself for rows whose largest exponent lies in
 // [kLowTop, kHighTop], which every ordinary row does; a row outside (or a temperature outside [1e-3, 1e6]) is summed again
-// relative to its maximum with the library's exp.
+// relative to its maximum, and its draws are taken by the warps in whose slices they fall.
 //
 // The exponential (after Tang, "Table-driven implementation of the exponential function in IEEE floating-point
 // arithmetic", ACM TOMS 15, 1989): K = the integer nearest to 128 * x from ONE fp32 FMA (it only has to be near), r =
@@ -42,6 +42,7 @@ constexpr int kSeg = 512;                                     // tokens per segm
 constexpr int kMaxSegs = 32;                                  // per slice
 constexpr int kMaxVocab = 2097152;
 constexpr int kTable = 128;
+constexpr int kLater = -1;                                    // not a token
 constexpr float kLowTop = -200.f, kHighTop = 900.f;           // exponent range of a row's largest term
 constexpr float kLowest = -1020.f;                            // smaller exponents count as this one (2^-820 of the sum)
 constexpr double kTiny = 1e-300;                              // above 2^-1020: what a masked token counts for
@@ -57,7 +58,8 @@ struct Args {
   double inv_temperature;
   double ck;                   // kTable * log2(e) / temperature
   float ckf, lowest;           // lowest: the logit whose exponent is kLowest
-  bool fast;                   // the temperature allows the table path
+  double lowest_below;         // the same for l - dm
+  bool fast;                   // the temperature allows sums that are not relative to the row's maximum
 };
 
 template <int CL>
@@ -69,28 +71,39 @@ struct Sums {                          // of one row
 template <int CL>
 struct Shared {
   double table[kTable * 16];
-  Sums<CL> sums[4];                    // rows in turn (a warp may be two rows ahead of one that reads its running sums);
-};                                     // [3]: a row outside the table path's range
+  Sums<CL> sums[3];                    // rows in turn (a warp may be two rows ahead of one that reads its running sums)
+};
 
-// 2^(l * c) for -1021 < l * c < 1021 (see the head of the file); `bank` = table + (lane & 15)
-__device__ __forceinline__ double exp2_table(float l, const Args& A, const double* bank) {
-  constexpr float kRound = 12582912.f;                        // 1.5 * 2^23: the sum's low bits are the nearest integer
+// 2^(K / 128) * 2^(r / 128) (see the head of the file); `bits`: K in the low bits, nothing in the ones above that the shift keeps;
+// `bank` = table + (lane & 15)
+__device__ __forceinline__ double exp2_parts(int bits, double r, const double* bank) {
   constexpr double a1 = 0.005415212348124257, a2 = 1.466226238764014e-05, a3 = 2.6466431340771855e-08,
                    a4 = 3.5830331985890313e-11;
-  const int bits = __float_as_int(fmaf(l, A.ckf, kRound));    // 0x4b400000 + K
-  const double K = __hiloint2double(0x43300000, bits) - (4503599627370496.0 + 1262485504.0);   // 2^52 + bits - (2^52 + 0x4b400000)
-  const double r = fma(static_cast<double>(l), A.ck, -K);
   const double t0 = bank[(bits & (kTable - 1)) * 16];
-  // K / 128 into the exponent field: the table has K % 128 taken off again, and the bits of 0x4b400000 that the shift
-  // keeps are zero
+  // K / 128 into the exponent field: the table has K % 128 taken off again
   const double t = __hiloint2double(__double2hiint(t0) + (bits << 13), __double2loint(t0));
   double q = fma(a4, r, a3);
   q = fma(q, r, a2);
   q = fma(q, r, a1);
   return fma(t * r, q, t);
 }
-// The term relative to the row's maximum (rows outside the table path's range).  Tokens past the end (and masked ones)
-// count as 2^-1020 on the table path, exactly 0 here.
+// 2^(l * c) for -1021 < l * c < 1021
+__device__ __forceinline__ double exp2_table(float l, const Args& A, const double* bank) {
+  constexpr float kRound = 12582912.f;                        // 1.5 * 2^23: the sum's low bits are the nearest integer
+  const int bits = __float_as_int(fmaf(l, A.ckf, kRound));    // 0x4b400000 + K
+  const double K = __hiloint2double(0x43300000, bits) - (4503599627370496.0 + 1262485504.0);   // 2^52 + bits - (2^52 + 0x4b400000)
+  return exp2_parts(bits, fma(static_cast<double>(l), A.ck, -K), bank);
+}
+// 2^((l - dm) * c) for l <= dm at any temperature: K from an fp64 sum.
+__device__ __forceinline__ double exp2_below(float l, double dm, const Args& A, const double* bank) {
+  constexpr double kRound = 6755399441055744.0;               // 1.5 * 2^52
+  double d = static_cast<double>(l) - dm;
+  d = d < A.lowest_below ? A.lowest_below : d;                // (a NaN stays one)
+  const double k = fma(d, A.ck, kRound);
+  return exp2_parts(__double2loint(k), fma(d, A.ck, -(k - kRound)), bank);
+}
+// The term relative to the row's maximum, exactly 0 where fp64 has nothing smaller (the table gives 2^-1020 at least, also for
+// masked tokens and past the end).
 __device__ __noinline__ double term_exact(float l, double dmax, double inv_temperature) {
   return exp((static_cast<double>(l) - dmax) * inv_temperature);
 }
@@ -132,7 +145,7 @@ __device__ __forceinline__ double slice_sums(const float* __restrict__ row, cons
     for (int x = 0; x < 8; ++x) { mx = fmaxf(mx, l[x]); mn = fminf(mn, l[x]); }
     if (__any_sync(0xffffffffu, !(mn >= A.lowest))) {          // masked tokens, or past the end (a NaN stays one)
 #pragma unroll
-      for (int x = 0; x < 8; ++x) l[x] = l[x] < A.lowest ? A.lowest : l[x];
+      for (int x = 0; x < 8; ++x) asm("max.NaN.f32 %0, %1, %2;" : "=f"(l[x]) : "f"(l[x]), "f"(A.lowest));
     }
 #pragma unroll
     for (int x = 0; x < 8; x += 2) {
@@ -155,19 +168,31 @@ __device__ __forceinline__ double slice_sums(const float* __restrict__ row, cons
   }
   return end;
 }
-// The same relative to the row's maximum.
+// The same relative to the row's maximum dm.
 template <bool VEC>
-__device__ __noinline__ double slice_sums_exact(const float* __restrict__ row, const Args& A, double* seg_end, int v0,
-                                                int n_half, int lane, double dmax) {
-  double end = 0.0;
+__device__ __forceinline__ double slice_sums_below(const float* __restrict__ row, const Args& A, const double* bank,
+                                                   double* seg_end, int v0, int n_half, int lane, double dm, float& mx) {
+  double end = 0.0, s0 = 0.0, s1 = 0.0;
+  mx = -INFINITY;
+  float next[8];
+  load_half<VEC>(row, v0, A.vocab, lane, next);
+#pragma unroll 1
   for (int h = 0; h < n_half; ++h) {
     float l[8];
-    load_half<VEC>(row, v0 + h * (kSeg / 2), A.vocab, lane, l);
-    double sum = 0.0;
-#pragma unroll 1
-    for (int x = 0; x < 8; ++x) sum += term_exact(l[x], dmax, A.inv_temperature);
-    end += warp_sum_d(sum);
-    if (lane == 0) seg_end[h >> 1] = end;
+#pragma unroll
+    for (int x = 0; x < 8; ++x) l[x] = next[x];
+    if (h + 1 < n_half) load_half<VEC>(row, v0 + (h + 1) * (kSeg / 2), A.vocab, lane, next);
+#pragma unroll
+    for (int x = 0; x < 8; x += 2) {
+      mx = fmaxf(mx, fmaxf(l[x], l[x + 1]));
+      s0 += exp2_below(l[x], dm, A, bank);
+      s1 += exp2_below(l[x + 1], dm, A, bank);
+    }
+    if ((h & 1) || h + 1 == n_half) {
+      end += warp_sum_d(s0 + s1);
+      s0 = s1 = 0.0;
+      if (lane == 0) seg_end[h >> 1] = end;
+    }
   }
   return end;
 }
@@ -198,42 +223,48 @@ __device__ __forceinline__ Slice slice_of(const Args& A, int slice) {
   return Slice{v0, (min(A.slice, A.vocab - v0) + kSeg / 2 - 1) / (kSeg / 2)};
 }
 
-// The token of target t, which lies in the segment [base, min(base + kSeg, end)); `before`: the sum in front of it.
-template <bool FAST, bool VEC>
-__device__ __forceinline__ int token_in_segment(const float* __restrict__ row, const Args& A, const double* bank,
-                                                double dmax, int base, int end, double before, double t, int lane) {
-  double e[4][4], run[4], incl[4];                            // terms; sums of the lane's share of a group of 128; scanned
+// A lane's terms of the segment [base, min(base + kSeg, end)) (BELOW: relative to dm), the sums of its share of each group of 128 tokens, and their
+// scans over the warp.
+struct Terms {
+  double e[4][4], run[4], incl[4];
+};
+template <bool BELOW, bool VEC>
+__device__ __forceinline__ void segment_terms(Terms& T, const float* __restrict__ row, const Args& A, const double* bank,
+                                              double dm, int base, int end, int lane) {
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     float l[8];
     load_half<VEC>(row, base + h * (kSeg / 2), end, lane, l);
 #pragma unroll
     for (int x = 0; x < 8; ++x)
-      e[2 * h + (x >> 2)][x & 3] = FAST ? exp2_table(fmaxf(l[x], A.lowest), A, bank) : term_exact(l[x], dmax, A.inv_temperature);
+      T.e[2 * h + (x >> 2)][x & 3] = BELOW ? exp2_below(l[x], dm, A, bank) : exp2_table(fmaxf(l[x], A.lowest), A, bank);
   }
 #pragma unroll
-  for (int j = 0; j < 4; ++j) incl[j] = run[j] = (e[j][0] + e[j][1]) + (e[j][2] + e[j][3]);
+  for (int j = 0; j < 4; ++j) T.incl[j] = T.run[j] = (T.e[j][0] + T.e[j][1]) + (T.e[j][2] + T.e[j][3]);
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const double y = __shfl_up_sync(0xffffffffu, incl[j], o);
-      if (lane >= o) incl[j] += y;
+      const double y = __shfl_up_sync(0xffffffffu, T.incl[j], o);
+      if (lane >= o) T.incl[j] += y;
     }
   }
+}
+// The token of target t, which lies in the segment at `base`; `before`: the sum in front of it.
+__device__ __forceinline__ int pick(const Terms& T, const Args& A, int base, double before, double t) {
   int token = -1;                                              // if rounding leaves t above everything: the last that counts
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    const uint32_t some = __ballot_sync(0xffffffffu, run[j] > kTiny);
-    const uint32_t over = __ballot_sync(0xffffffffu, run[j] > kTiny && before + incl[j] > t);
+    const uint32_t some = __ballot_sync(0xffffffffu, T.run[j] > kTiny);
+    const uint32_t over = __ballot_sync(0xffffffffu, T.run[j] > kTiny && before + T.incl[j] > t);
     if (some) {
       const int f = over ? __ffs(over) - 1 : 31 - __clz(some);
-      double c = before + (incl[j] - run[j]);
+      double c = before + (T.incl[j] - T.run[j]);
       int hit = -1, tail = 0;
 #pragma unroll
       for (int x = 0; x < 4; ++x) {
-        c += e[j][x];
-        if (e[j][x] > kTiny) {
+        c += T.e[j][x];
+        if (T.e[j][x] > kTiny) {
           tail = x;
           if (hit < 0 && c > t) hit = x;
         }
@@ -241,15 +272,9 @@ __device__ __forceinline__ int token_in_segment(const float* __restrict__ row, c
       token = base + 128 * j + 4 * f + __shfl_sync(0xffffffffu, hit < 0 ? tail : hit, f);
       if (over) return token;
     }
-    before += __shfl_sync(0xffffffffu, incl[j], 31);
+    before += __shfl_sync(0xffffffffu, T.incl[j], 31);
   }
   return token < 0 ? A.vocab - 1 : token;
-}
-
-template <bool VEC>
-__device__ __noinline__ int token_in_segment_exact(const float* __restrict__ row, const Args& A, double dmax, int base, int end,
-                                                   double before, double t, int lane) {
-  return token_in_segment<false, VEC>(row, A, nullptr, dmax, base, end, before, t, lane);
 }
 
 // The row's first token whose term is not 0 at all (the sums do not tell: a masked term counts as 2^-1020 in them).  It is in
@@ -277,32 +302,13 @@ __device__ __noinline__ int first_positive(const float* __restrict__ row, const 
   return A.vocab - 1;
 }
 
-// This warp's share of the draws of row `seq`; `at`: which of `sums` holds the row.
-template <int CL, bool VEC>
-__device__ __forceinline__ void draws(const Args& A, Sums<CL>* sums, const double* bank, int at, int64_t seq, int slice, int lane) {
-  constexpr int kSlices = CL * kWarps;
-  cg::cluster_group cl = cg::this_cluster();
-  const float* row = A.logits + seq * A.vocab;
-  const int64_t d0 = A.draw_offsets[seq], d1 = A.draw_offsets[seq + 1];
-  const int turn = static_cast<int>((slice + seq) % kSlices);
-  float mx = -INFINITY;
-  for (int i = lane; i < kSlices; i += 32) mx = fmaxf(mx, sums[at].slice_max[i]);
-  mx = warp_max(mx);
-  const double dmax = static_cast<double>(mx);
-  const float top = mx * A.ckf * (1.f / kTable);
-  const bool fast = A.fast && top >= kLowTop && top <= kHighTop;
-  if (!fast) {                                                 // again, relative to the row's maximum (the cluster agrees)
-    const Slice L = slice_of(A, slice);
-    const double sum = slice_sums_exact<VEC>(row, A, sums[3].seg_end[slice % kWarps], L.v0, L.n_half, lane, dmax);
-    publish<CL>(cl, sums[3], slice, lane, sum, sums[at].slice_max[slice]);
-    at = 3;
-    cl.sync();
-  }
-  if (d0 + turn >= d1) return;
-  Sums<CL>& S = sums[at];
-  // Cumulative sums at the ends of the slices: the first lanes add up a block's, then the blocks in turn.  A slice ends at
-  // (start of its block) + (sum of the block's slices so far), so the ends ascend whatever the rounding.
-  double in_block = 0.0, end_b = 0.0, Z = 0.0;
+// Cumulative sums at the ends of the cluster's blocks (lane b < CL: block b's) and the row's total: the first lanes add up a
+// block's slices, then the blocks in turn.  A slice ends at (start of its block) + (sum of the block's slices so far), so the
+// ends ascend whatever the rounding.
+template <int CL>
+__device__ __forceinline__ void block_ends(const Sums<CL>& S, int lane, double& end_b, double& Z) {
+  double in_block = 0.0;
+  end_b = Z = 0.0;
   if (lane < CL)
     for (int w = 0; w < kWarps; ++w) in_block += S.slice_sum[lane * kWarps + w];
 #pragma unroll
@@ -310,11 +316,111 @@ __device__ __forceinline__ void draws(const Args& A, Sums<CL>* sums, const doubl
     Z += __shfl_sync(0xffffffffu, in_block, b);
     if (lane == b) end_b = Z;
   }
+}
+
+// A row outside the table's range, with its maximum mx: the sums once more, relative to it, and then the draws that fall into
+// this warp's slice, a segment of it at a time (it is evaluated once for all draws in it).
+template <int CL, bool VEC>
+__device__ __forceinline__ void row_below(const Args& A, Sums<CL>& S, const double* bank, int64_t seq, int slice, int lane,
+                                          float mx) {
+  constexpr int kSlices = CL * kWarps;
+  const float* row = A.logits + seq * A.vocab;
+  const int64_t d0 = A.draw_offsets[seq], d1 = A.draw_offsets[seq + 1];
+  const Slice L = slice_of(A, slice);
+  const double dm = static_cast<double>(mx);                   // (if it is not finite the sum is a NaN)
+  cg::cluster_group cl = cg::this_cluster();
+  {
+    float own;
+    const double sum = slice_sums_below<VEC>(row, A, bank, S.seg_end[slice % kWarps], L.v0, L.n_half, lane, dm, own);
+    own = warp_max(own);
+    cl.sync();                                                 // (nobody reads the sums of the row before any more)
+    publish<CL>(cl, S, slice, lane, sum, own);
+    cl.sync();
+  }
+  double end_b, Z;
+  block_ends<CL>(S, lane, end_b, Z);
+  if (slice == 0) {                                            // draws that no segment holds
+    for (int64_t c = d0; c < d1; c += 32) {
+      const double t = c + lane < d1 ? static_cast<double>(A.uniforms[c + lane]) * Z : 0.0;
+      const uint32_t zero = __ballot_sync(0xffffffffu, c + lane < d1 && t == 0.0);
+      int token = A.vocab - 1;
+      if (zero) {
+        const int first = first_positive(row, A, S.slice_max, kSlices, dm, lane);
+        if (t == 0.0) token = first;
+      }
+      if (c + lane < d1 && (t == 0.0 || !(t < Z))) {
+        A.tokens_out[c + lane] = token;
+        A.seq_out[c + lane] = seq;
+      }
+    }
+  }
+  const int block = slice / kWarps, warp = slice % kWarps, n_seg = (L.n_half + 1) >> 1;
+  const double block_start = __shfl_sync(0xffffffffu, end_b, max(block - 1, 0)), start = block ? block_start : 0.0;
+  double in_front = 0.0;
+  for (int w = 0; w < warp; ++w) in_front += S.slice_sum[block * kWarps + w];
+  const double before = start + in_front, slice_end = start + (in_front + S.slice_sum[slice]);
+  const double end_s = lane < n_seg ? S.seg_end[warp][lane] : 0.0;
+  const double last_end = __shfl_sync(0xffffffffu, end_s, max(n_seg - 1, 0));
+  const int s_last = __ffs(__ballot_sync(0xffffffffu, lane < n_seg && end_s == last_end)) - 1;   // (see draws; -1: no segment, or NaN)
+  Terms T;
+#pragma unroll 1
+  for (int s = 0; s <= s_last; ++s) {
+    const double in_slice = s ? __shfl_sync(0xffffffffu, end_s, max(s - 1, 0)) : 0.0, seg_end = before + __shfl_sync(0xffffffffu, end_s, s);
+    const double from = before + in_slice, to = s == s_last ? slice_end : fmin(seg_end, slice_end);
+    bool evaluated = false;
+#pragma unroll 1
+    for (int64_t c = d0; c < d1; c += 32) {
+      const double t = c + lane < d1 ? static_cast<double>(A.uniforms[c + lane]) * Z : 0.0;
+      const bool mine = c + lane < d1 && t != 0.0 && (t >= from || (slice == 0 && s == 0)) && t < to;
+      uint32_t members = __ballot_sync(0xffffffffu, mine);
+      if (!members) continue;
+      const int base = L.v0 + s * kSeg, end = min(A.vocab, L.v0 + A.slice);
+      if (!evaluated) {
+        segment_terms<true, VEC>(T, row, A, bank, dm, base, end, lane);
+        evaluated = true;
+      }
+      int token = 0;
+      for (; members; members &= members - 1) {
+        const int i = __ffs(members) - 1;
+        const int k = pick(T, A, base, from, __shfl_sync(0xffffffffu, t, i));
+        if (lane == i) token = k;
+      }
+      if (mine) {
+        A.tokens_out[c + lane] = token;
+        A.seq_out[c + lane] = seq;
+      }
+    }
+  }
+}
+
+// This warp's share of the draws of row `seq`; `at`: which of `sums` holds the row.  True, with nothing drawn, if the row is
+// outside the table's range (the cluster agrees).
+template <int CL, bool VEC>
+__device__ __forceinline__ bool draws(const Args& A, Sums<CL>* sums, const double* bank, int at, int64_t seq, int slice, int lane) {
+  constexpr int kSlices = CL * kWarps;
+  const int64_t d0 = A.draw_offsets[seq], d1 = A.draw_offsets[seq + 1];
+  const int turn = static_cast<int>((slice + seq) % kSlices);
+  float mx = -INFINITY;
+  for (int i = lane; i < kSlices; i += 32) mx = fmaxf(mx, sums[at].slice_max[i]);
+  mx = warp_max(mx);
+  const float top = mx * A.ckf * (1.f / kTable);
+  if (!(A.fast && top >= kLowTop && top <= kHighTop)) {        // its first draw's outputs say so meanwhile, and keep the maximum
+    if (slice == 0 && lane == 0) {
+      A.tokens_out[d0] = kLater;
+      A.seq_out[d0] = __float_as_int(mx);
+    }
+    return true;
+  }
+  if (d0 + turn >= d1) return false;
+  const float* row = A.logits + seq * A.vocab;
+  Sums<CL>& S = sums[at];
+  double end_b, Z;
+  block_ends<CL>(S, lane, end_b, Z);
   for (int64_t d = d0 + turn; d < d1; d += kSlices) {
     const double t = static_cast<double>(A.uniforms[d]) * Z;
     int token = A.vocab - 1;                                   // the answer if t is not below the total
     if (t == 0.0) {                                            // the first term that is not 0 at all
-      token = first_positive(row, A, S.slice_max, kSlices, dmax, lane);
+      token = first_positive(row, A, S.slice_max, kSlices, static_cast<double>(mx), lane);
     } else if (t < Z) {
       const int b = __ffs(__ballot_sync(0xffffffffu, lane < CL && end_b > t)) - 1;
       const double start = b ? __shfl_sync(0xffffffffu, end_b, max(b - 1, 0)) : 0.0;
@@ -326,7 +432,7 @@ __device__ __forceinline__ void draws(const Args& A, Sums<CL>* sums, const doubl
         in_front = e;
       }
       const Slice L = slice_of(A, b * kWarps + w);
-      const double* seg_end = cl.map_shared_rank(&S, b)->seg_end[w];
+      const double* seg_end = cg::this_cluster().map_shared_rank(&S, b)->seg_end[w];
       const double before = start + in_front;
       const int n_seg = (L.n_half + 1) >> 1;                   // at most kMaxSegs
       const double end_s = lane < n_seg ? seg_end[lane] : 0.0;
@@ -338,9 +444,10 @@ __device__ __forceinline__ void draws(const Args& A, Sums<CL>* sums, const doubl
       const int s = __ffs(hit) - 1;
       if (s >= 0) {
         const double in_slice = s ? __shfl_sync(0xffffffffu, end_s, max(s - 1, 0)) : 0.0;
-        const int base = L.v0 + s * kSeg, end = min(A.vocab, L.v0 + A.slice);
-        token = fast ? token_in_segment<true, VEC>(row, A, bank, dmax, base, end, before + in_slice, t, lane)
-                     : token_in_segment_exact<VEC>(row, A, dmax, base, end, before + in_slice, t, lane);
+        const int base = L.v0 + s * kSeg;
+        Terms T;
+        segment_terms<false, VEC>(T, row, A, bank, 0.0, base, min(A.vocab, L.v0 + A.slice), lane);
+        token = pick(T, A, base, before + in_slice, t);
       }
     }
     if (lane == 0) {
@@ -348,6 +455,7 @@ __device__ __forceinline__ void draws(const Args& A, Sums<CL>* sums, const doubl
       A.seq_out[d] = seq;
     }
   }
+  return false;
 }
 
 template <int CL, bool VEC>
@@ -380,6 +488,7 @@ branch_sample_kernel(const __grid_constant__ Args A) {
   cl.sync();                                                   // (the table; and every block runs before it is written to)
 
   int at = 0, prev_at = 0;
+  bool later = false;                                          // a row outside the table's range: for when the others are done
   for (;;) {
     double sum = 0.0;
     float mx = -INFINITY;
@@ -402,7 +511,7 @@ branch_sample_kernel(const __grid_constant__ Args A) {
     }
     if (prev >= 0) {
       cluster_wait();
-      draws<CL, VEC>(A, S.sums, bank, prev_at, prev, slice, lane);
+      later |= draws<CL, VEC>(A, S.sums, bank, prev_at, prev, slice, lane);
     }
     if (!more) break;
     publish<CL>(cl, S.sums[at], slice, lane, sum, mx);
@@ -411,6 +520,14 @@ branch_sample_kernel(const __grid_constant__ Args A) {
     prev_at = at;
     at = at == 2 ? 0 : at + 1;
     row = after;
+  }
+  if (later) {                                                 // (the cluster agrees)
+    cl.sync();                                                 // (the marks; and nobody reads the running sums any more)
+    for (int64_t r = next_row(row0); r < A.n_seq; r = next_row(r + gridDim.x / CL)) {
+      const int64_t d = A.draw_offsets[r];
+      if (__ldcg(A.tokens_out + d) != kLater) continue;        // (read in front of row_below's barriers, written behind them)
+      row_below<CL, VEC>(A, S.sums[0], bank, r, slice, lane, __int_as_float(static_cast<int>(__ldcg(A.seq_out + d))));
+    }
   }
   if (CL > 1) cl.sync();                                       // (a block's running sums may still be read by another)
 }
@@ -483,6 +600,7 @@ extern "C" int32_t ss_branch_sample(const float* logits, const int64_t* draw_off
   A.ckf = static_cast<float>(A.ck);
   A.lowest = static_cast<float>(kLowest / c);
   A.fast = T >= 1e-3 && T <= 1e6;
+  A.lowest_below = kLowest / c;
   const bool vec = reinterpret_cast<uintptr_t>(logits) % 16 == 0 && vocab % 4 == 0;
   cudaStream_t st = as_stream(stream);
   const int sms = sm_count_of_current_device();

@@ -184,3 +184,34 @@ def test_uniform_zero_draws_the_first_token_with_any_probability(S, V, live):
     tok, _ = run(logits, off, u, 0.8)
     want, _, _ = oracle.branch_sample(logits, off, u, 0.8)
     assert np.array_equal(tok.cpu().numpy()[::2], want[::2])
+
+
+@pytest.mark.parametrize("S", [3, 30, 70, 160])
+@pytest.mark.parametrize("V", [700, 9001, 70000])
+@pytest.mark.parametrize("kind,T", [("up", 0.8), ("up", 1.1e-3), ("down", 0.8), ("cold", 9e-4), ("cold", 1e-12), ("cold", 2e-30), ("hot", 5e6),
+                                    ("hot", 9e29), ("tiny", 1e-32), ("huge", 1e32)])
+def test_rows_outside_the_table_path(S, V, kind, T):
+    """Rows whose largest exponent is out of range are summed again relative to their maximum: by the table (up, down, cold,
+    hot) or by CUDA's exp (temperatures beyond 1e-30 and 1e30), on blocks and on clusters of 2, 4 and 8.  Scores are scaled so
+    that there is something to choose from; every third row is an ordinary one, every fourth is partly masked."""
+    rng = np.random.default_rng(S + V)
+    logits = (rng.normal(size=(S, V)) * 3).astype(np.float32)
+    if kind in ("cold", "tiny"):
+        logits = (logits * T).astype(np.float32)
+    elif kind in ("hot", "huge"):
+        logits = (logits.astype(np.float64) * T / 4).astype(np.float32)
+    else:
+        rows = np.arange(S) % 3 != 1
+        logits[rows] += np.float32({"up": 3000.0, "down": -900.0}[kind])
+    logits[::4][rng.random(logits[::4].shape) < 0.3] = -np.inf
+    logits[::4, V // 2] = logits[::4].max(axis=1)
+    pot = rng.integers(0, 6, size=S)
+    pot[0] = 70
+    off = np.concatenate([[0], np.cumsum(pot)]).astype(np.int64)
+    u = rng.random(int(off[-1])).astype(np.float32)
+    u[:60:9] = 0.0
+    tok, seq = run(logits, off, u, T)
+    want_tok, want_seq, margin = oracle.branch_sample(logits, off, u, float(np.float32(T)))
+    got, sure = tok.cpu().numpy(), margin > 1e-12
+    assert np.array_equal(seq.cpu().numpy(), want_seq)
+    assert np.array_equal(got[sure], want_tok[sure]) and np.array_equal(got[u == 0.0], want_tok[u == 0.0])
