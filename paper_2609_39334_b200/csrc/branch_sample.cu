@@ -55,6 +55,7 @@ struct Args {
   int64_t* seq_out;
   int n_seq, row0, vocab;
   int slice;                   // tokens per warp, a multiple of kSeg / 2
+  int many;                    // draws of a row from which its segments are gone through instead
   double inv_temperature;
   double ck;                   // kTable * log2(e) / temperature
   float ckf, lowest;           // lowest: the logit whose exponent is kLowest
@@ -72,6 +73,7 @@ template <int CL>
 struct Shared {
   double table[kTable * 16];
   Sums<CL> sums[3];                    // rows in turn (a warp may be two rows ahead of one that reads its running sums)
+  int queue[kWarps][64];               // see row_below
 };
 
 // 2^(K / 128) * 2^(r / 128) (see the head of the file); `bits`: K in the low bits, nothing in the ones above that the shift keeps;
@@ -318,33 +320,74 @@ __device__ __forceinline__ void block_ends(const Sums<CL>& S, int lane, double& 
   }
 }
 
-// A row outside the table's range, with its maximum mx: the sums once more, relative to it, and then the draws that fall into
-// this warp's slice, a segment of it at a time (it is evaluated once for all draws in it).
+// The token of every lane's own target, or -1 where rounding leaves it to `pick`.
+__device__ __forceinline__ int pick_each(const Terms& T, int base, double before, double t) {
+  double in_front = before;                                    // the group of 128, then the lane of it, that holds t
+  int j = 0;
+#pragma unroll
+  for (int x = 0; x < 3; ++x) {
+    const double e = in_front + __shfl_sync(0xffffffffu, T.incl[x], 31);
+    if (j == x && !(e > t)) {
+      ++j;
+      in_front = e;
+    }
+  }
+  int f = 0;
+#pragma unroll
+  for (int step = 16; step > 0; step >>= 1) {
+    double v = 0.0;
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      const double y = __shfl_sync(0xffffffffu, T.incl[x], f + step - 1);
+      if (j == x) v = y;
+    }
+    if (!(in_front + v > t)) f += step;
+  }
+  double c = 0.0, e[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+  for (int x = 0; x < 4; ++x) {
+    const double y = in_front + (__shfl_sync(0xffffffffu, T.incl[x], f) - __shfl_sync(0xffffffffu, T.run[x], f));
+    if (j == x) c = y;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const double z = __shfl_sync(0xffffffffu, T.e[x][k], f);
+      if (j == x) e[k] = z;
+    }
+  }
+  int token = -1;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    c += e[k];
+    if (token < 0 && e[k] > kTiny && c > t) token = base + 128 * j + 4 * f + k;
+  }
+  return token;
+}
+
+// A row outside the table's range or with many draws, mx its maximum: the sums once more, relative to it, and then the draws
+// that fall into this warp's slice, a segment at a time: it is evaluated once for all of them.  `queue`: 64 words of the warp's.
 template <int CL, bool VEC>
-__device__ __forceinline__ void row_below(const Args& A, Sums<CL>& S, const double* bank, int64_t seq, int slice, int lane,
-                                          float mx) {
+__device__ __forceinline__ void row_below(const Args& A, Sums<CL>& S, int* queue, const double* bank, int64_t seq, int slice,
+                                          int lane, float mx) {
   constexpr int kSlices = CL * kWarps;
   const float* row = A.logits + seq * A.vocab;
   const int64_t d0 = A.draw_offsets[seq], d1 = A.draw_offsets[seq + 1];
-  const Slice L = slice_of(A, slice);
   const double dm = static_cast<double>(mx);                   // (if it is not finite the sum is a NaN)
   cg::cluster_group cl = cg::this_cluster();
   {
-    float own;
-    const double sum = slice_sums_below<VEC>(row, A, bank, S.seg_end[slice % kWarps], L.v0, L.n_half, lane, dm, own);
-    own = warp_max(own);
+    const Slice L = slice_of(A, slice);
+    float top;
     cl.sync();                                                 // (nobody reads the sums of the row before any more)
-    publish<CL>(cl, S, slice, lane, sum, own);
+    const double sum = slice_sums_below<VEC>(row, A, bank, S.seg_end[slice % kWarps], L.v0, L.n_half, lane, dm, top);
+    publish<CL>(cl, S, slice, lane, sum, warp_max(top));
     cl.sync();
   }
   double end_b, Z;
   block_ends<CL>(S, lane, end_b, Z);
   if (slice == 0) {                                            // draws that no segment holds
     for (int64_t c = d0; c < d1; c += 32) {
-      const double t = c + lane < d1 ? static_cast<double>(A.uniforms[c + lane]) * Z : 0.0;
-      const uint32_t zero = __ballot_sync(0xffffffffu, c + lane < d1 && t == 0.0);
+      const double t = c + lane < d1 ? static_cast<double>(A.uniforms[c + lane]) * Z : 1.0;
       int token = A.vocab - 1;
-      if (zero) {
+      if (__any_sync(0xffffffffu, t == 0.0)) {
         const int first = first_positive(row, A, S.slice_max, kSlices, dm, lane);
         if (t == 0.0) token = first;
       }
@@ -354,47 +397,79 @@ __device__ __forceinline__ void row_below(const Args& A, Sums<CL>& S, const doub
       }
     }
   }
-  const int block = slice / kWarps, warp = slice % kWarps, n_seg = (L.n_half + 1) >> 1;
+  // The slice and its segments, by the same sums as in `draws`.  A vocabulary of few slices: several warps share the draws of one.
+  const int used = static_cast<int>((static_cast<int64_t>(A.vocab) + A.slice - 1) / A.slice), parts = kSlices / used;
+  const int own = slice % used, part = slice / used, block = own / kWarps, warp = own % kWarps;
+  if (part >= parts) return;
+  const Slice L = slice_of(A, own);
+  const int n_seg = (L.n_half + 1) >> 1;
   const double block_start = __shfl_sync(0xffffffffu, end_b, max(block - 1, 0)), start = block ? block_start : 0.0;
   double in_front = 0.0;
   for (int w = 0; w < warp; ++w) in_front += S.slice_sum[block * kWarps + w];
-  const double before = start + in_front, slice_end = start + (in_front + S.slice_sum[slice]);
-  const double end_s = lane < n_seg ? S.seg_end[warp][lane] : 0.0;
+  const double before = start + in_front, slice_end = start + (in_front + S.slice_sum[own]);
+  const double end_s = lane < n_seg ? cl.map_shared_rank(&S, block)->seg_end[warp][lane] : 0.0;
   const double last_end = __shfl_sync(0xffffffffu, end_s, max(n_seg - 1, 0));
-  const int s_last = __ffs(__ballot_sync(0xffffffffu, lane < n_seg && end_s == last_end)) - 1;   // (see draws; -1: no segment, or NaN)
-  Terms T;
+  const int s_last = __ffs(__ballot_sync(0xffffffffu, lane < n_seg && end_s == last_end)) - 1;   // (-1: no segment, or a NaN)
 #pragma unroll 1
   for (int s = 0; s <= s_last; ++s) {
-    const double in_slice = s ? __shfl_sync(0xffffffffu, end_s, max(s - 1, 0)) : 0.0, seg_end = before + __shfl_sync(0xffffffffu, end_s, s);
-    const double from = before + in_slice, to = s == s_last ? slice_end : fmin(seg_end, slice_end);
+    const double in_slice = __shfl_sync(0xffffffffu, end_s, max(s - 1, 0)), seg_end = before + __shfl_sync(0xffffffffu, end_s, s);
+    const double from = s ? before + in_slice : before, to = s == s_last ? slice_end : fmin(seg_end, slice_end);
+    const double low = own == 0 && s == 0 ? -INFINITY : from;
+    const int base = L.v0 + s * kSeg;
+    Terms T;
     bool evaluated = false;
+    int waiting = 0;                                           // draws in the queue, which are looked up 32 at a time
+    auto look_up = [&](int count) {
+      if (!evaluated) segment_terms<true, VEC>(T, row, A, bank, dm, base, min(A.vocab, L.v0 + A.slice), lane);
+      evaluated = true;
+      __syncwarp();
+      const int64_t d = d0 + (lane < count ? queue[lane] : queue[0]);
+      const double t = static_cast<double>(__ldg(A.uniforms + d)) * Z;
+      int token = pick_each(T, base, from, t);
+      for (uint32_t open = __ballot_sync(0xffffffffu, token < 0); open; open &= open - 1) {
+        const int i = __ffs(open) - 1;
+        const int one = pick(T, A, base, from, __shfl_sync(0xffffffffu, t, i));
+        if (lane == i) token = one;
+      }
+      if (lane < count) {
+        A.tokens_out[d] = token;
+        A.seq_out[d] = seq;
+      }
+      __syncwarp();
+    };
+    constexpr int kAhead = 4;
 #pragma unroll 1
-    for (int64_t c = d0; c < d1; c += 32) {
-      const double t = c + lane < d1 ? static_cast<double>(A.uniforms[c + lane]) * Z : 0.0;
-      const bool mine = c + lane < d1 && t != 0.0 && (t >= from || (slice == 0 && s == 0)) && t < to;
-      uint32_t members = __ballot_sync(0xffffffffu, mine);
-      if (!members) continue;
-      const int base = L.v0 + s * kSeg, end = min(A.vocab, L.v0 + A.slice);
-      if (!evaluated) {
-        segment_terms<true, VEC>(T, row, A, bank, dm, base, end, lane);
-        evaluated = true;
+    for (int64_t c0 = d0 + 32 * part; c0 < d1; c0 += 32 * kAhead * parts) {
+      float u[kAhead];
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k) {
+        const int64_t d = c0 + 32 * parts * k + lane;
+        u[k] = d < d1 ? __ldg(A.uniforms + d) : 2.f;           // (2: above every segment)
       }
-      int token = 0;
-      for (; members; members &= members - 1) {
-        const int i = __ffs(members) - 1;
-        const int k = pick(T, A, base, from, __shfl_sync(0xffffffffu, t, i));
-        if (lane == i) token = k;
-      }
-      if (mine) {
-        A.tokens_out[c + lane] = token;
-        A.seq_out[c + lane] = seq;
+#pragma unroll
+      for (int k = 0; k < kAhead; ++k) {
+        const double t = static_cast<double>(u[k]) * Z;
+        const bool mine = t != 0.0 && t >= low && t < to;
+        const uint32_t members = __ballot_sync(0xffffffffu, mine);
+        if (!members) continue;
+        if (mine) queue[waiting + __popc(members & ((1u << lane) - 1u))] = static_cast<int>(c0 - d0) + 32 * parts * k + lane;
+        waiting += __popc(members);
+        if (waiting >= 32) {
+          look_up(32);
+          waiting -= 32;
+          const int moved = queue[32 + lane];
+          __syncwarp();
+          queue[lane] = moved;
+          __syncwarp();
+        }
       }
     }
+    if (waiting > 0) look_up(waiting);
   }
 }
 
 // This warp's share of the draws of row `seq`; `at`: which of `sums` holds the row.  True, with nothing drawn, if the row is
-// outside the table's range (the cluster agrees).
+// outside the table's range or has many draws (the cluster agrees).
 template <int CL, bool VEC>
 __device__ __forceinline__ bool draws(const Args& A, Sums<CL>* sums, const double* bank, int at, int64_t seq, int slice, int lane) {
   constexpr int kSlices = CL * kWarps;
@@ -404,7 +479,7 @@ __device__ __forceinline__ bool draws(const Args& A, Sums<CL>* sums, const doubl
   for (int i = lane; i < kSlices; i += 32) mx = fmaxf(mx, sums[at].slice_max[i]);
   mx = warp_max(mx);
   const float top = mx * A.ckf * (1.f / kTable);
-  if (!(A.fast && top >= kLowTop && top <= kHighTop)) {        // its first draw's outputs say so meanwhile, and keep the maximum
+  if (!(A.fast && top >= kLowTop && top <= kHighTop) || d1 - d0 > A.many) {   // its first draw's outputs say so meanwhile, and keep the maximum
     if (slice == 0 && lane == 0) {
       A.tokens_out[d0] = kLater;
       A.seq_out[d0] = __float_as_int(mx);
@@ -526,7 +601,7 @@ branch_sample_kernel(const __grid_constant__ Args A) {
     for (int64_t r = next_row(row0); r < A.n_seq; r = next_row(r + gridDim.x / CL)) {
       const int64_t d = A.draw_offsets[r];
       if (__ldcg(A.tokens_out + d) != kLater) continue;        // (read in front of row_below's barriers, written behind them)
-      row_below<CL, VEC>(A, S.sums[0], bank, r, slice, lane, __int_as_float(static_cast<int>(__ldcg(A.seq_out + d))));
+      row_below<CL, VEC>(A, S.sums[0], S.queue[warp], bank, r, slice, lane, __int_as_float(static_cast<int>(__ldcg(A.seq_out + d))));
     }
   }
   if (CL > 1) cl.sync();                                       // (a block's running sums may still be read by another)
@@ -537,6 +612,13 @@ template <int CL>
 static int32_t launch(Args A, bool vec, int row0, int n_seq, int clusters, cudaStream_t st) {
   constexpr int kUnit = kSeg / 2;
   A.slice = (A.vocab + CL * kWarps * kUnit - 1) / (CL * kWarps * kUnit) * kUnit;
+  // A draw by itself costs a warp 2.9 us, going through the segments of its slice a second pass over it and 2.5 us a segment.
+  // 200 rows of 32000, 128 / 256 / 1024 draws each: 49 / 81 / 269 us one by one, 53 / 58 / 102 by segment (blocks of 1024 threads
+  // with the row's sums in shared memory: 68 / 68 / 74); 200 rows of 151936, 256 / 512 / 1024: 109 / 171 / 291 and 175 / 207 / 263
+  // (315 / 320 / 331).  Clusters of 4 and 8 blocks have enough warps, one by one is as fast up to 20000 draws, but where most
+  // of them would have no slice (4 rows of 300, 4096 draws: 74 and 42).
+  const bool idle = static_cast<int64_t>(CL) * kWarps / 2 * A.slice >= A.vocab;
+  A.many = CL <= 2 || idle ? CL * kWarps * (4 + A.slice / 384) : INT32_MAX;
   A.row0 = row0;
   A.n_seq = n_seq;
   if (vec)

@@ -215,3 +215,24 @@ def test_rows_outside_the_table_path(S, V, kind, T):
     got, sure = tok.cpu().numpy(), margin > 1e-12
     assert np.array_equal(seq.cpu().numpy(), want_seq)
     assert np.array_equal(got[sure], want_tok[sure]) and np.array_equal(got[u == 0.0], want_tok[u == 0.0])
+
+
+@pytest.mark.parametrize("S,V,most", [(150, 300, 900), (150, 5000, 700), (151, 32001, 900), (70, 32000, 1200), (40, 700, 3000), (3, 600, 5000)])
+@pytest.mark.parametrize("peak", [0.0, 12.0])
+def test_many_draws_of_a_row(S, V, most, peak):
+    """Rows with more draws than are looked up one by one, beside rows with few, none and just as many as a queue holds; flat
+    rows and rows with nearly all of their probability on one token."""
+    rng = np.random.default_rng(S + V)
+    logits = (rng.normal(size=(S, V)) * 2).astype(np.float32)
+    logits[:, V // 3] += np.float32(peak)
+    logits[::5, : V // 4] = -np.inf
+    pot = rng.integers(0, most + 1, size=S)
+    pot[1::7] = rng.integers(0, 70, size=len(pot[1::7]))
+    off = np.concatenate([[0], np.cumsum(pot)]).astype(np.int64)
+    u = rng.random(int(off[-1])).astype(np.float32)
+    u[::97] = 0.0
+    tok, seq = run(logits, off, u, 0.9)
+    want_tok, want_seq, margin = oracle.branch_sample(logits, off, u, float(np.float32(0.9)))
+    got, sure = tok.cpu().numpy(), margin > 1e-12
+    assert np.array_equal(seq.cpu().numpy(), want_seq)
+    assert np.array_equal(got[sure], want_tok[sure]) and np.array_equal(got[u == 0.0], want_tok[u == 0.0])

@@ -61,3 +61,9 @@ def test_rows_outside_the_table_path(shift, T):
     """They take a second pass; measured 1.9 times an ordinary row (3.9 with CUDA's exp in the second pass)."""
     logits = torch.randn((600, 151936), device=DEV) * 3
     assert sample_us(logits + shift, 2, T=T) < 3 * sample_us(logits, 2)
+
+
+def test_thousands_of_draws_of_a_row():
+    """Measured 118 us against 373 one draw after the other; 182 for the ordinary case to compare with."""
+    many, rows = torch.randn((64, 32000), device=DEV) * 3, torch.randn((922, 151936), device=DEV) * 3
+    assert sample_us(many, 4096) < 1.3 * sample_us(rows, 2)
