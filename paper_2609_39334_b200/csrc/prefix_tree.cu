@@ -19,7 +19,8 @@
 //                       against every other (its rank is the number below it, what it shares with the rank before the
 //                       most that it shares with any of them)
 //             ranks     a warp per position counts the smaller keys of its group; with groups of more than 256 a block per
-//                       1024 positions sorts (group, key, position) first and the lanes search the tiles of the group
+//                       1024 positions sorts (group, key, position), then the sorted runs are merged by ranks, 4 at a time: a lane
+//                       per position and run counts the keys in front by binary search
 //   tree    Inner nodes are the intervals of neighbours that share more pages than their surroundings (the LCP-interval
 //           tree).  A warp per position finds its interval with nearest-smaller-value searches of 32 entries a step, over
 //           the entries and over their minima by 32; depth-first numbering (leaves included) comes from a prefix sum of
@@ -43,6 +44,9 @@ constexpr int kPairs = 8;                         // a group of up to this many 
                                                   // row (9 us) against two or three more rounds (8 us each)
 constexpr int kCount = 256;                       // ranks by counting up to this group size: 8 keys a lane (1.2 us) against a
                                                   // tile sort (13 us); beyond, counting grows with the square
+constexpr int kFan = 4;                           // sorted runs merged in a pass.  1M paths of 6 tokens: all 1024 tiles at once 34.4 ms
+                                                  // (a search in every tile for every position), 4 2.3, 8 2.6, 2 2.4; 64000 paths 344 us,
+                                                  // 225, 229, 236; 16384 (16 tiles) 145 at once, 145, 143, 152
 constexpr uint32_t kInf = 0x7fffffffu;            // "common length" of a path with itself
 constexpr unsigned long long kBarrierLimitNs = 4000000000ull;
 
@@ -413,43 +417,47 @@ __device__ __forceinline__ void build(const Args& A) {
     for (int t = blockIdx.x * (kThreads / kTile); t < A.n_tiles; t += gridDim.x * (kThreads / kTile))
       sort_tiles(A, t, A.key[kc ^ 1], A.perm[pc], A.key[kc], A.perm[pc ^ 1]);
     if (!grid_barrier<CLUSTER>(A, target)) return;
-    // `width` lanes per position, one for each tile of its group
-    int width = 1;
-    while (width < 32 && width < A.n_tiles) width <<= 1;
-    const int sub = lane & (width - 1), per_warp = 32 / width;
-    for (int p0 = wid * per_warp; p0 < n; p0 += n_warps * per_warp) {
-      const int p = p0 + lane / width;
-      int g = 0, e = 0, rank = 0;
-      uint64_t k = 0;
-      if (p < n) {
-        g = A.gs[p];
-        e = A.ge[p];
-      }
-      if (e - g > 1) {
-        const int tile = p / kTile, t0 = g / kTile, t1 = (e - 1) / kTile;
-        k = A.key[kc][p];
-        if (sub == 0) rank = p - max(g, tile * kTile);
-        for (int t = t0 + sub; t <= t1; t += width) {
-          if (t == tile) continue;
-          const int begin = max(g, t * kTile);
-          int lo = begin, hi = min(e, (t + 1) * kTile);        // first position that does not come before p
-          while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            const uint64_t v = A.key[kc][mid];
-            if (t < tile ? v <= k : v < k) lo = mid + 1; else hi = mid;
+    // Sorted runs of `span` positions are merged, kFan at a time: a lane for each run that may hold keys of the position's group.
+    pc ^= 1;
+    for (int span = kTile; span < n; span *= kFan) {
+      const int sub = lane & (kFan - 1);
+      for (int p0 = wid * (32 / kFan); p0 < n; p0 += n_warps * (32 / kFan)) {
+        const int p = p0 + lane / kFan;
+        int g = 0, e = 0, rank = 0, first = 0;
+        uint64_t k = 0;
+        if (p < n) {
+          g = A.gs[p];
+          e = A.ge[p];
+        }
+        if (e - g > 1) {
+          const int run = p / span, other = run / kFan * kFan + sub;
+          first = max(g, run / kFan * kFan * span);
+          k = A.key[kc][p];
+          if (other == run) {
+            rank = p - max(g, run * span);
+          } else if (other * span < e && (other + 1) * span > g) {
+            const int begin = max(g, other * span);
+            int lo = begin, hi = min(e, (other + 1) * span);   // first position that does not come before p
+            while (lo < hi) {
+              const int mid = (lo + hi) >> 1;
+              const uint64_t v = A.key[kc][mid];
+              if (other < run ? v <= k : v < k) lo = mid + 1; else hi = mid;
+            }
+            rank = lo - begin;
           }
-          rank += lo - begin;
+        }
+        __syncwarp();
+#pragma unroll
+        for (int o = kFan >> 1; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+        if (sub == 0 && e - g > 1) {
+          A.key[kc ^ 1][first + rank] = k;
+          A.perm[pc ^ 1][first + rank] = A.perm[pc][p];
         }
       }
-      __syncwarp();
-      for (int o = width >> 1; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
-      if (sub == 0 && e - g > 1) {
-        A.key[kc ^ 1][g + rank] = k;
-        A.perm[pc][g + rank] = A.perm[pc ^ 1][p];
-      }
+      kc ^= 1;
+      pc ^= 1;
+      if (!grid_barrier<CLUSTER>(A, target)) return;
     }
-    kc ^= 1;
-    if (!grid_barrier<CLUSTER>(A, target)) return;
   }
   const int* path_of = A.order;
 

@@ -223,3 +223,12 @@ def test_prefix_tree_grids_tiles_and_pivots(n):
             s = [int(x) for x in rng.integers(0, 3, size=int(rng.integers(0, 12)))]
         seqs.append(s)
     check(*csr(seqs), 4)
+
+
+@pytest.mark.parametrize("n,alphabet", [(4096, 3), (4097, 150000), (5000, 2), (16385, 3), (70000, 150000), (70000, 5), (300000, 4)])
+def test_prefix_tree_merges_of_sorted_runs(n, alphabet):
+    """Groups over up to 293 tiles of 1024 positions (1, 2 and more passes of merges, partly filled runs), and groups that begin
+    and end inside tiles: few different tokens, many equal paths and empty ones."""
+    rng = np.random.default_rng(n + alphabet)
+    off = np.concatenate([[0], np.cumsum(rng.integers(0, 9, size=n))]).astype(np.int64)
+    check(rng.integers(0, alphabet, size=int(off[-1])).astype(np.int32), off, 1)
