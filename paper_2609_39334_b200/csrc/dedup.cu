@@ -78,10 +78,13 @@ __global__ void hash_kernel(const int32_t* __restrict__ tok_ids, const int64_t* 
   if (!table) return;
   const unsigned long long mine = (static_cast<unsigned long long>(tag_of(h)) << 32) | static_cast<uint32_t>(path);
   for (uint32_t s = static_cast<uint32_t>(h) & mask;; s = (s + 1) & mask) {
-    const unsigned long long cur = atomicCAS(&table[s], kEmpty, mine);
+    // (the entry is looked at first: of many equal paths most then find a smaller one there.  With the counts below: 1M equal paths
+    //  3.0 -> 0.5 ms; different ones 0.54 either way)
+    unsigned long long cur = __ldcg(&table[s]);
+    if (cur == kEmpty) cur = atomicCAS(&table[s], kEmpty, mine);
     if (cur == kEmpty) return;
     if ((cur >> 32) == (mine >> 32)) {                       // (an entry keeps its tag: the minimum is over the index)
-      atomicMin(&table[s], mine);
+      if (cur > mine) atomicMin(&table[s], mine);
       return;
     }
   }
@@ -360,13 +363,24 @@ compact_kernel(const int32_t* __restrict__ canon, int n, const uint32_t* __restr
     start = s_start;
   }
   const int i = blockIdx.x * kChunk + tid;
+  const uint32_t warp_paths = __ballot_sync(0xffffffffu, i < n);
   if (i >= n) return;
   const int c = canon[i], w0 = c / kChunk * (kChunk / 32), w1 = c >> 5;
   int r = start[c / kChunk] + __popc(unique[w1] & ((1u << (c & 31)) - 1u));
   for (int w = w0; w < w1; ++w) r += __popc(unique[w]);
   path_to_unique[i] = r;
   if (c == i) unique_paths[r] = i;
-  atomicAdd(&multiplicity[r], 1);
+  // (one atomic for the warp's paths that equal its first one, and so on twice: groups of many paths would else be bound by
+  //  atomics on one address)
+  uint32_t left = warp_paths;
+#pragma unroll
+  for (int round = 0; round < 2; ++round) {
+    const int leader = left ? __ffs(left) - 1 : 0;
+    const uint32_t same = __ballot_sync(warp_paths, r == __shfl_sync(warp_paths, r, leader)) & left;
+    if (same && (tid & 31) == leader) atomicAdd(&multiplicity[r], __popc(same));
+    left &= ~same;
+  }
+  if ((left >> (tid & 31)) & 1u) atomicAdd(&multiplicity[r], 1);
   if (slot_out) slot_out[i] = slot_in[c];
 }
 

@@ -219,6 +219,20 @@ def test_dedup_edge_cases():
     assert list(got["canon"]) == [0, 0]
 
 
+@pytest.mark.parametrize("n", [4097, 5120, 20001])
+@pytest.mark.parametrize("groups", [1, 2, 3, 40])
+def test_dedup_large_groups(n, groups):
+    """Groups of thousands of equal paths: a warp's equal paths are counted together, at most two groups of it, the rest one by
+    one (40 groups); the last warp is partly filled."""
+    rng = np.random.default_rng(n + groups)
+    ids = rng.integers(0, groups, size=n).astype(np.int32)
+    off = np.arange(n + 1, dtype=np.int64)
+    got, want = run_dedup(ids, off, None, None), oracle.dedup(ids, off)
+    assert got["num_unique"] == want["num_unique"]
+    for key in ("canon", "path_to_unique", "unique_paths", "multiplicity"):
+        assert np.array_equal(got[key], want[key]), key
+
+
 def test_dedup_paper_example_on_gpu():
     got = run_dedup(np.asarray([1055, 1055, 1055, 429], np.int32), np.arange(5, dtype=np.int64), np.zeros(4, np.int64), None)
     assert list(got["multiplicity"]) == [3, 1]
