@@ -71,15 +71,19 @@ __device__ uint64_t sort_registers(uint64_t k, int n_pad, uint64_t* s_key) {
 // A block's segment.  One that does not lie inside [0, n_total] is reported and treated as empty: its offsets index the mask
 // and the scratch region, so following them would write out of bounds.  Block 0 looks at all segments, writes the status word
 // and clears `mask` where NO valid segment lies, so that it never writes what another block does: in front of the first and
-// behind the last one, or, with a bad one among them, wherever `covered` (kSmemKeys words) says.
+// behind the last one here, or, with a bad one among them (`gaps`), by clear_uncovered when its own segment is done - not
+// before: the compiler then makes the sort slower for everybody (512 segments of 1024: 31.9 us instead of 25.0).
 struct Segment {
   int lo, n;
+  bool gaps;
 };
 __device__ __forceinline__ bool valid_segment(int lo, int hi, int n_total) { return lo >= 0 && hi >= lo && hi <= n_total; }
 __device__ __noinline__ void clear_uncovered(const int32_t* __restrict__ seg_offsets, int n_segments, int n_total, uint8_t* mask,
-                                             uint32_t* covered) {
+                                             uint64_t* smem_keys) {
   constexpr int kWindow = kSmemKeys * 64;                     // candidates a pass, a bit each
+  uint32_t* covered = reinterpret_cast<uint32_t*>(smem_keys);
   const int tid = threadIdx.x, nt = blockDim.x;
+  __syncthreads();
   for (int base = 0; base < n_total; base = base > n_total - kWindow ? n_total : base + kWindow) {
     const int end = n_total - base < kWindow ? n_total : base + kWindow;
     for (int i = tid; i < kWindow / 32; i += nt) covered[i] = 0;
@@ -99,23 +103,21 @@ __device__ __noinline__ void clear_uncovered(const int32_t* __restrict__ seg_off
   }
 }
 __device__ __forceinline__ Segment open_segment(const int32_t* __restrict__ seg_offsets, int n_total, uint8_t* mask,
-                                                int32_t* status, uint64_t* smem_keys) {
+                                                int32_t* status) {
   const int s = blockIdx.x, n_segments = gridDim.x, nt = blockDim.x;
   const int lo = seg_offsets[s], hi = seg_offsets[s + 1];
+  bool any = false;
   if (s == 0) {
     const int tail = seg_offsets[n_segments];                 // (loaded with the others, not behind the barrier)
-    bool any = false;
     for (int x = threadIdx.x; x < n_segments; x += nt) any = any || !valid_segment(seg_offsets[x], seg_offsets[x + 1], n_total);
     any = __syncthreads_or(any) != 0;
     if (threadIdx.x == 0) *status = any ? SS_ERR_BAD_INPUT : SS_OK;
-    if (any) {
-      clear_uncovered(seg_offsets, n_segments, n_total, mask, reinterpret_cast<uint32_t*>(smem_keys));
-    } else {
+    if (!any) {
       for (int i = threadIdx.x; i < lo; i += nt) mask[i] = 0;
       for (int i = tail + static_cast<int>(threadIdx.x); i < n_total; i += nt) mask[i] = 0;
     }
   }
-  return Segment{lo, valid_segment(lo, hi, n_total) ? hi - lo : 0};
+  return Segment{lo, valid_segment(lo, hi, n_total) ? hi - lo : 0, any};
 }
 
 // Calls rank(j, key) for the key of every rank j < n, n keys from make(i).  `scratch`: where neither the registers nor
@@ -143,18 +145,19 @@ topk_kernel(const float* __restrict__ scores, const int32_t* __restrict__ seg_of
             int32_t* __restrict__ status) {
   ss::grid_dependency_enter();
   __shared__ uint64_t smem_keys[kSmemKeys];
-  const Segment g = open_segment(seg_offsets, n_total, keep, status, smem_keys);
+  const Segment g = open_segment(seg_offsets, n_total, keep, status);
   int32_t* out = survivors + static_cast<int64_t>(blockIdx.x) * k;
   for (int j = g.n + threadIdx.x; j < k; j += blockDim.x) out[j] = -1;
-  if (g.n == 0) return;
   // (a segment's scratch region starts at 2 lo: pow2ceil(n) < 2n keeps the regions of different segments apart)
-  sorted(g.n, smem_keys, scratch + 2 * static_cast<int64_t>(g.lo),
-         [&](int i) { return make_key(scores[g.lo + i], static_cast<uint32_t>(i)); },
-         [&](int j, uint64_t key) {
-           const int cand = g.lo + static_cast<int>(key & 0xffffffffu);
-           keep[cand] = j < k ? 1 : 0;
-           if (j < k) out[j] = cand;
-         });
+  if (g.n > 0)
+    sorted(g.n, smem_keys, scratch + 2 * static_cast<int64_t>(g.lo),
+           [&](int i) { return make_key(scores[g.lo + i], static_cast<uint32_t>(i)); },
+           [&](int j, uint64_t key) {
+             const int cand = g.lo + static_cast<int>(key & 0xffffffffu);
+             keep[cand] = j < k ? 1 : 0;
+             if (j < k) out[j] = cand;
+           });
+  if (g.gaps) clear_uncovered(seg_offsets, gridDim.x, n_total, keep, smem_keys);
 }
 
 // Early pruning with partially verified candidates (paper, Section "Early Pruning of Search Tree").  Same sort as
@@ -163,17 +166,12 @@ topk_kernel(const float* __restrict__ scores, const int32_t* __restrict__ seg_of
 //           other candidate of the segment is pruned, the segment is final;
 //   rule 1: more than k verified -> the verified candidates ranked below the k best are pruned;
 //   all verified -> final, selected = the k best.
-__global__ void __launch_bounds__(kMaxThreads)
-early_prune_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ verified,
-                   const int32_t* __restrict__ seg_offsets, int n_total, int k, uint8_t* __restrict__ pruned,
-                   int32_t* __restrict__ selected, uint8_t* __restrict__ final_out, uint64_t* __restrict__ scratch,
-                   int32_t* __restrict__ status) {
-  ss::grid_dependency_enter();
-  __shared__ uint64_t smem_keys[kSmemKeys];
-  __shared__ int s_nver, s_nperfect, s_warp[32];
+__device__ __forceinline__ void early_prune_segment(const float* __restrict__ scores, const uint8_t* __restrict__ verified,
+                                                    const Segment g, int k, uint8_t* __restrict__ pruned,
+                                                    int32_t* __restrict__ selected, uint8_t* __restrict__ final_out,
+                                                    uint64_t* __restrict__ scratch, uint64_t* smem_keys, int& s_nver, int& s_nperfect) {
+  __shared__ int s_warp[32];
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) { s_nver = 0; s_nperfect = 0; }
-  const Segment g = open_segment(seg_offsets, n_total, pruned, status, smem_keys);
   int32_t* out = selected + static_cast<int64_t>(blockIdx.x) * k;
   if (g.n == 0) {
     for (int j = tid; j < k; j += nt) out[j] = -1;
@@ -229,15 +227,28 @@ early_prune_kernel(const float* __restrict__ scores, const uint8_t* __restrict__
          });
   if (tid == 0) final_out[blockIdx.x] = all_verified ? 1 : 0;
 }
+__global__ void __launch_bounds__(kMaxThreads)
+early_prune_kernel(const float* __restrict__ scores, const uint8_t* __restrict__ verified,
+                   const int32_t* __restrict__ seg_offsets, int n_total, int k, uint8_t* __restrict__ pruned,
+                   int32_t* __restrict__ selected, uint8_t* __restrict__ final_out, uint64_t* __restrict__ scratch,
+                   int32_t* __restrict__ status) {
+  ss::grid_dependency_enter();
+  __shared__ uint64_t smem_keys[kSmemKeys];
+  __shared__ int s_nver, s_nperfect;
+  if (threadIdx.x == 0) { s_nver = 0; s_nperfect = 0; }
+  const Segment g = open_segment(seg_offsets, n_total, pruned, status);
+  early_prune_segment(scores, verified, g, k, pruned, selected, final_out, scratch, smem_keys, s_nver, s_nperfect);
+  if (g.gaps) clear_uncovered(seg_offsets, gridDim.x, n_total, pruned, smem_keys);
+}
 
-// Threads per block: one per candidate of a segment of average size, but at least kMinThreads where there are so many candidates,
-// since any one segment may be far above the average: one of 4096 among 1000 of 16 takes 236 us with 64 threads and 76 with 256,
-// while small segments gain nothing from smaller blocks (shared memory allows 7 blocks an SM either way) but at the bare
-// latency of a handful of candidates.
-constexpr int kMinThreads = 256;
+// Threads per block: one per candidate of a segment of average size, but more where there are so many candidates, since any one
+// segment may be far above the average: one of 4096 among 1000 of 16 takes 236 us with 64 threads and 76 with 256.  Few
+// candidates get 128: a decode step of 16 segments of 64 takes 1 us more with 256 (107.0 us, 106.1 with 64 or 128), whose blocks
+// are in the way of the kernels around them.  512 segments of 16: 2.6 us with 64, 3.3 with 256.
 static int block_threads(int n_total, int n_segments) {
+  const int least = n_total <= 2048 ? 128 : 256;
   int t = 64;
-  while (t < kMinThreads && t < n_total) t <<= 1;
+  while (t < least && t < n_total) t <<= 1;
   while (t < kMaxThreads && static_cast<int64_t>(t) * n_segments < n_total) t <<= 1;
   return t;
 }
