@@ -367,7 +367,7 @@ int32_t ss_build_prefix_tree(const int32_t* tok_ids, const int64_t* tok_offsets,
  *   ss_tree_attention (queries read in place through the gathered offsets)  ->  ss_topk_prune  ->
  *   asynchronous copies device -> host of every result.
  * With SS_STEP_COMPACT_TRANSFERS in `flags`, and out / lse page-locked AND mapped into the device's address space
- * (memory from cudaHostAlloc / cudaHostRegister), only the live rows of out / lse come back - the first
+ * (memory from cudaHostAlloc / cudaHostRegister, starting on 16 bytes), only the live rows of out / lse come back - the first
  * u_q_offsets[num_unique]: a duplicate candidate gets no forward pass, hence no output of its own - written by a small
  * kernel straight into the host buffers; the rest of out / lse is left untouched.  (Buffers the device cannot address
  * are returned whole, as without the flag.)

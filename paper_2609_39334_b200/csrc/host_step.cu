@@ -254,14 +254,14 @@ extern "C" int32_t ss_candidate_step_host(const ss_host_step_t* step, void* devi
             move(in, a.q_offsets, s.q_offsets, (N + 1) * 8, false) && move(in, a.q, s.q, q_bytes, false) &&
             move(in, a.scores, s.scores, N * 4, false) && move(in, a.seg_offsets, s.seg_offsets, (P + 1) * 4, false);
   if (!ok) return SS_ERR_CUDA;
-  // compact return: needs out / lse mapped (the kernel writes them) and whole 16-byte chunks per row
+  // compact return: needs out / lse mapped (the kernel writes them, 16 bytes at a time) and whole 16-byte chunks per row
   char *out_map = nullptr, *lse_map = nullptr;
   bool compact = (s.flags & SS_STEP_COMPACT_TRANSFERS) != 0 && s.total_q > 0 && s.n_paths > 0 &&
                  row * sizeof(__nv_bfloat16) % 16 == 0;
   if (compact) {
     out_map = mapped(s.out);
     if (s.lse) lse_map = mapped(s.lse);
-    compact = out_map && (!s.lse || lse_map);
+    compact = out_map && (!s.lse || lse_map) && ((reinterpret_cast<uintptr_t>(out_map) | reinterpret_cast<uintptr_t>(lse_map)) & 15) == 0;
   }
   if (in.count > 0) {
     size_t bytes = 0;

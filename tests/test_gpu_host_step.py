@@ -90,3 +90,41 @@ def test_host_step_with_compact_transfers_returns_only_live_rows(cfg):
         assert np.array_equal(r["out"], r_dev["out"]) and np.array_equal(r["lse"], r_dev["lse"])
         for key in ("canon", "path_to_unique", "unique_paths", "multiplicity", "slot_out", "survivors", "keep"):
             assert np.array_equal(r[key], r_dev[key]), key
+
+
+def shifted(t, offset, pinned=True):
+    """A copy of `t` that starts `offset` elements into a page-locked (or pageable) buffer."""
+    buf = torch.empty(t.numel() + offset, dtype=t.dtype, pin_memory=pinned)
+    view = buf[offset:].view(t.shape)
+    view.copy_(t)
+    return view
+
+
+@pytest.mark.parametrize("compact", [False, True])
+@pytest.mark.parametrize("kind", ["off_16_bytes", "some_pageable", "all_pageable"])
+def test_host_step_takes_any_host_buffers(kind, compact):
+    """Buffers that do not start on 16 bytes, or are not page-locked, all of them or some: kernels move what is page-locked, the
+    rest is copied; out / lse come back whole where a kernel cannot write their rows 16 bytes at a time."""
+    w = synth.make_config(2)
+    pipe = DevicePipeline(w, DEV)
+    pipe.step()
+    r_dev = pipe.results()
+    host = HostStepPipeline(pipe, depth=1, compact=compact)
+    s = host.sets[0]
+    for part in ("h_in", "h_out"):
+        for i, (name, t) in enumerate(list(s[part].items())):
+            if kind == "off_16_bytes":
+                s[part][name] = shifted(t, 1)
+            elif kind == "all_pageable" or i % 2:
+                s[part][name] = shifted(t, 0, pinned=False)
+    s["step"] = B.make_host_step(pipe.desc, n_paths=pipe.N, n_segments=pipe.P, top_k=w.top_k, total_tok=int(w.tok_offsets[-1]),
+                                 total_q=w.total_q, host_in=s["h_in"], host_out=s["h_out"], dedup_flags=pipe.dedup_flags,
+                                 flags=B.SS_STEP_COMPACT_TRANSFERS if compact else 0)
+    for _ in range(2):
+        for t in s["h_out"].values():
+            t.zero_()
+        host.submit(0)
+        r = host.results(0)
+        assert np.array_equal(r["out"], r_dev["out"]) and np.array_equal(r["lse"], r_dev["lse"])
+        for key in ("canon", "path_to_unique", "unique_paths", "multiplicity", "slot_out", "survivors", "keep"):
+            assert np.array_equal(r[key], r_dev[key]), key
