@@ -18,13 +18,16 @@
 //
 // Small arrays (a copy of a few KB costs its place in the stream, 2 to 4 us, whatever its size; a decode step has 8 in and
 // 9 out) go through one kernel per direction that reads or writes the mapped host memory, if it is page-locked; arrays
-// above kSmallBytes keep their copy engine.  Measured, a step of 1024 decode paths: 330 -> 278 us.
+// above kSmallBytes keep their copy engine.  Measured, a step of 1024 decode paths: 330 -> 278 us.  Arrays that do not start on 16
+// bytes are moved a byte per thread, which still beats the copies up to a few KB (8 paths 138 -> 67 us a step, 1024 265 -> 216; 4096
+// with three sets in flight 350 -> 457).
 #include "common.cuh"
 
 namespace ss {
 namespace host_step {
 
-constexpr size_t kSmallBytes = 64 << 10;
+constexpr size_t kSmallBytes = 64 << 10;      // three sets in flight, 4096 decode paths: 4 KB 471 us a step, 16 KB 420, 64 KB 350, 256 KB
+                                              // 350; one at a time, 1024 paths: 227, 207, 206, 208; 16384: 2341, 2332, 2297, 2282
 constexpr int kMaxSegments = 12;
 
 // Arrays to move, one after the other.
@@ -35,14 +38,20 @@ struct Segments {
   int count;
 };
 
-// The device's address of page-locked host memory, or null.
-static char* mapped(const void* host) {
-  void* dev = nullptr;
-  if (!host || cudaHostGetDevicePointer(&dev, const_cast<void*>(host), 0) != cudaSuccess) {
+// The device's address of `bytes` of host memory, or null if they are not page-locked, to the last byte (an array may run past the
+// end of a registered range: a copy then reports it, a kernel would fault.  Pages are locked whole, so one that lies in a page
+// is only asked for once; a lookup costs the host 0.1 us).
+static char* mapped(const void* host, size_t bytes) {
+  if (!host || bytes == 0) return nullptr;
+  char* at = static_cast<char*>(const_cast<void*>(host));
+  char* end = at + bytes - 1;
+  void *first = nullptr, *last = nullptr;
+  const bool one_page = ((reinterpret_cast<uintptr_t>(at) ^ reinterpret_cast<uintptr_t>(end)) >> 12) == 0;
+  if (cudaHostGetDevicePointer(&first, at, 0) != cudaSuccess || (!one_page && cudaHostGetDevicePointer(&last, end, 0) != cudaSuccess)) {
     (void)cudaGetLastError();
     return nullptr;
   }
-  return static_cast<char*>(dev);
+  return one_page || static_cast<char*>(last) - static_cast<char*>(first) == end - at ? static_cast<char*>(first) : nullptr;
 }
 
 __device__ __forceinline__ void move_segments(const Segments& S, int block, int n_blocks) {
@@ -229,13 +238,14 @@ extern "C" int32_t ss_candidate_step_host(const ss_host_step_t* step, void* devi
   const size_t N = static_cast<size_t>(s.n_paths), P = static_cast<size_t>(s.n_segments);
   const size_t row = static_cast<size_t>(s.attn->num_q_heads) * static_cast<size_t>(s.attn->head_dim);
   const size_t q_bytes = static_cast<size_t>(s.total_q) * row * sizeof(__nv_bfloat16);
+  const size_t lse_bytes = static_cast<size_t>(s.total_q) * static_cast<size_t>(s.attn->num_q_heads) * sizeof(float);
 
   // ---- host -> device: the step's candidates, queries and scores ------------------------------------------------
   Segments in{}, res{};
   // puts an array on the list if it is small and mapped; else copies it
   auto move = [&](Segments& list, void* dst, const void* src, size_t bytes, bool to_host) -> bool {
     if (bytes == 0) return true;
-    char* map = bytes <= kSmallBytes && list.count < kMaxSegments ? mapped(to_host ? dst : src) : nullptr;
+    char* map = bytes <= kSmallBytes && list.count < kMaxSegments ? mapped(to_host ? dst : src, bytes) : nullptr;
     if (!map) {
       if (cudaMemcpyAsync(dst, src, bytes, to_host ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice, st) == cudaSuccess) return true;
       (void)cudaGetLastError();
@@ -259,8 +269,8 @@ extern "C" int32_t ss_candidate_step_host(const ss_host_step_t* step, void* devi
   bool compact = (s.flags & SS_STEP_COMPACT_TRANSFERS) != 0 && s.total_q > 0 && s.n_paths > 0 &&
                  row * sizeof(__nv_bfloat16) % 16 == 0;
   if (compact) {
-    out_map = mapped(s.out);
-    if (s.lse) lse_map = mapped(s.lse);
+    out_map = mapped(s.out, q_bytes);
+    if (s.lse) lse_map = mapped(s.lse, lse_bytes);
     compact = out_map && (!s.lse || lse_map) && ((reinterpret_cast<uintptr_t>(out_map) | reinterpret_cast<uintptr_t>(lse_map)) & 15) == 0;
   }
   if (in.count > 0) {
@@ -298,7 +308,7 @@ extern "C" int32_t ss_candidate_step_host(const ss_host_step_t* step, void* devi
   // ---- device -> host: every result ------------------------------------------------------------------------------------
   if (!compact)
     ok = move(res, s.out, a.out, q_bytes, true) &&
-         (!s.lse || move(res, s.lse, a.lse, static_cast<size_t>(s.total_q) * static_cast<size_t>(s.attn->num_q_heads) * sizeof(float), true));
+         (!s.lse || move(res, s.lse, a.lse, lse_bytes, true));
   ok = ok && move(res, s.canon, a.canon, N * 4, true) && move(res, s.path_to_unique, a.path_to_unique, N * 4, true) &&
        move(res, s.unique_paths, a.unique_paths, N * 4, true) && move(res, s.multiplicity, a.multiplicity, N * 4, true) &&
        (!s.slot_out || move(res, s.slot_out, a.slot_out, N * 4, true)) && move(res, s.num_unique, a.num_unique, 4, true) &&
