@@ -120,9 +120,15 @@ def _ptr(t: Optional[torch.Tensor]):
     return t.data_ptr()
 
 
+# (of the current device, without a Stream object; torch has no public name for it)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream) -> int:
-    if stream is None:                       # the current stream of the current device, without a Stream object
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
+        stream = torch.cuda.current_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 

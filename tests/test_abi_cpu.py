@@ -116,6 +116,17 @@ def test_binding_fails_loudly_without_library(monkeypatch):
         B.lib()
 
 
+def test_current_stream_with_and_without_torchs_private_name(monkeypatch):
+    class Stream:
+        cuda_stream = 77
+    monkeypatch.setattr(B, "_raw_stream", lambda device: 40 + device)
+    monkeypatch.setattr(B.torch.cuda, "current_device", lambda: 2)
+    monkeypatch.setattr(B.torch.cuda, "current_stream", lambda: Stream())
+    assert B._stream(None) == 42 and B._stream(Stream()) == 77 and B._stream(5) == 5
+    monkeypatch.setattr(B, "_raw_stream", None)
+    assert B._stream(None) == 77
+
+
 def test_every_kernel_waits_for_its_predecessor_first():
     """Kernels are launched with programmatic stream serialization; stream order then rests on every kernel calling
     grid_dependency_enter() before anything else (a kernel that skipped it could finish before its predecessor)."""
