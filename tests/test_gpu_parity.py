@@ -740,6 +740,69 @@ def test_planner_at_the_edges_of_its_forms(paths):
     check_attention(r, w, ref, max_paths=40)
 
 
+@pytest.mark.parametrize("levels,fanout,problems", [([48, 32], [10, 40], 8), ([48, 20], [10, 40], 8), ([16, 16, 32], [3, 30, 9], 6),
+                                                    ([32], [7], 330)])
+def test_large_planner_levels_roots_and_classes(levels, fanout, problems):
+    """More than 2048 nodes and paths below several levels and roots: items of inner nodes behind those of all roots, across
+    scan chunks and blocks; one path in seven is verified (GENERIC rows where an inner node is not whole pages), the
+    others decode; duplicates, so that fewer paths live than there are."""
+    w = synth.build_tree_workload("large", 8100 + problems, 4, 2, levels, fanout, problems, (0, 40),
+                                  lambda i, n, rng: 5 if i % 7 == 0 else 1, dup_frac=0.1)
+    assert w.num_nodes > 2048 and w.num_paths > 2048
+    r, ref = attention_only(w)
+    check_attention(r, w, ref, max_paths=90)
+    # one row per warp, without plan items: the same rows
+    r1, _ = attention_only(w, flags=B.SS_FLAG_FORCE_GENERIC)
+    fin = np.isfinite(r1["lse"])
+    assert np.array_equal(np.isfinite(r["lse"]), fin) and np.abs(r["lse"][fin] - r1["lse"][fin]).max() <= 2e-5
+    assert (np.abs(r["out"] - r1["out"]) <= 2 * (TIGHT_ABS + TIGHT_REL * np.abs(r1["out"]))).all()
+
+
+@pytest.mark.parametrize("problems", [2, 60])
+def test_both_planners_report_what_the_device_sees(problems):
+    """Each check of the planner, in the form for small trees and in the one for large ones: an error is recorded, nothing is
+    written (not even behind a workspace sized by a hint that is too low), and the next good call is as if nothing was."""
+    w = synth.build_tree_workload("report", 8200, 4, 2, [32, 16], [4, 12], problems, (1, 30), lambda i, n, rng: 1 + 3 * (i % 9 == 0))
+    assert (w.num_paths > 2048) == (problems == 60)
+    pipe = DevicePipeline(w, DEV, attn_flags=B.SS_FLAG_VALIDATE)
+    pipe.step()
+    good = pipe.results()
+    depth, pipe.desc.max_depth = pipe.desc.max_depth, 0        # (as deep as it may be)
+    need = B.ss_tree_attention_workspace_bytes(pipe.desc)
+    canary = torch.full((4096,), 0x5A, dtype=torch.uint8, device=DEV)
+
+    def status(need):
+        ws_all = torch.cat([B.alloc_workspace(need, DEV)[:need + (-need) % 256], canary])
+        ws = ws_all[:ws_all.numel() - 4096]
+        pipe.out.fill_(7.0)
+        B.ss_tree_attention(pipe.desc, ws)
+        got = B.ss_last_device_status(ws)
+        assert bool((ws_all[-4096:] == 0x5A).all())
+        assert got == B.SS_OK or bool((pipe.out == 7.0).all())
+        return got
+
+    nodes, last = w.num_nodes, w.num_paths - 1
+    chain = 20                                                # nodes hung below one another: deeper than 16
+    root2 = int(np.flatnonzero(w.node_parent < 0)[-1])
+    for tensor, at, value, want in ((pipe.node_pages, -1, w.num_pages, B.SS_ERR_BAD_INPUT), (pipe.node_pages, 0, -1, B.SS_ERR_BAD_INPUT),
+                                    (pipe.node_parent, nodes - 1, nodes - 1, B.SS_ERR_BAD_INPUT),
+                                    (pipe.node_parent, 1, -2, B.SS_ERR_BAD_INPUT), (pipe.node_kv_len, nodes - 1, 10 ** 6, B.SS_ERR_BAD_INPUT),
+                                    (pipe.u_leaf, last, nodes, B.SS_ERR_BAD_INPUT), (pipe.u_q_len, 0, 0, B.SS_ERR_BAD_INPUT),
+                                    (pipe.u_leaf, 0, nodes - 1, B.SS_ERR_BAD_INPUT),                   # not contiguous
+                                    (pipe.node_parent, slice(root2 + 1, root2 + 1 + chain), None, B.SS_ERR_UNSUPPORTED)):
+        keep = tensor[at].clone()
+        tensor[at] = torch.arange(at.start - 1, at.stop - 1, dtype=torch.int32, device=DEV) if value is None else value
+        assert status(need) == want, (at, value)
+        tensor[at] = keep
+        assert status(need) == B.SS_OK
+    pipe.desc.max_decode_paths = 5
+    assert status(B.ss_tree_attention_workspace_bytes(pipe.desc)) == B.SS_ERR_WORKSPACE_TOO_SMALL
+    pipe.desc.max_decode_paths, pipe.desc.max_depth = int((w.path_q_len == 1).sum()), depth
+    pipe.step()
+    r = pipe.results()
+    assert np.array_equal(r["out"], good["out"]) and np.array_equal(r["lse"], good["lse"])
+
+
 def test_ragged_ends_do_not_race_with_late_value_copies():
     """Verification items whose last tile ends early, on a tree that keeps every SM's copy pipeline loaded: the undefined
     rows behind the last key (NaN here) must be cleared after their copy has landed, however late it is.  Repeated runs
