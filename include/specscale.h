@@ -343,8 +343,10 @@ int32_t ss_branch_sample(const float* logits, const int64_t* draw_offsets, const
  *                                                                        and the position where they start in it
  *   num_nodes_out       int32 [1]           n_paths leaves + the inner nodes (0 after a device-side error)
  *   workspace           >= ss_prefix_tree_workspace_bytes(...) bytes, 256-byte aligned; its first word is the device
- *                       status (ss_last_device_status): SS_ERR_BAD_INPUT if the internal 64-bit page hashes collided
- *                       in a way that mis-ordered two paths (the tree is then withheld, never wrong)
+ *                       status (ss_last_device_status): SS_ERR_TIMEOUT if the blocks waited for one another for more
+ *                       than 4 seconds (the tree is then withheld: *num_nodes_out = 0)
+ * More than 512 paths, or 4 M token ids, take one cooperative launch of up to a block of 1024 threads per SM: it starts when
+ * the device has room for all of them at once, so it waits for another stream's kernel that holds SMs for long.
  * Errors (host): SS_ERR_INVALID_ARG, SS_ERR_WORKSPACE_TOO_SMALL, SS_ERR_CUDA.
  * ======================================================================================================= */
 #define SS_PREFIX_TREE_MAX_PATHS (1 << 20)

@@ -66,7 +66,7 @@ struct PlanHeader {       // first bytes of the workspace; status MUST be the fi
   int32_t tile_counter;   // work-stealing counters (reset by the planner)
   int32_t leaf_counter;
   int32_t n_stacked_items; // tile items [0, n_stacked_items) are stacked items, the rest chain items
-  int32_t n_full_leaf_items;  // leaf items of whole chunks: they come first
+  int32_t n_full_leaf_items;  // leaf items of whole chunks (they come first in the small planner's list; the large one's goes leaf by leaf)
   int32_t pad[5];
 #ifdef SS_STAMPS
   unsigned long long stamp[40];  // instrumented build: %globaltimer at kernel starts / ends (see SS_STAMP); 8..23:

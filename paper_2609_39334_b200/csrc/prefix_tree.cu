@@ -27,7 +27,7 @@
 //           the intervals per start rank; parents follow from the neighbours of an interval.
 //
 // Bound: HBM, one pass over the shared prefixes (268 MB for 16384 paths with prompts of 4096 tokens, 41 us), and for small
-// inputs the latency of a dozen dependent phases.  Measured: 16384 paths / 76 M ids 151 us (of which 61 the pass over the
+// inputs the latency of a dozen dependent phases.  Measured: 16384 paths / 76 M ids 149 us (of which 61 the pass over the
 // prompts; page hashes, a bitonic sort with a string comparator and a pass over the neighbours: 1729), 64 paths 25 us (135).
 #include "common.cuh"
 
