@@ -1,5 +1,8 @@
-"""Calls far from the usual proportions must not fall off a cliff: each is timed against an ordinary call with the same work,
-with a bound that leaves a factor of two for the machine's noise.  (What they return is compared with the oracle elsewhere.)"""
+"""Calls far from the usual proportions must not fall off a cliff: each is timed against an ordinary call, with a bound well above
+the measured ratio and below the one that was a fault, and again if another user of the machine got in between.  (What they
+return is compared with the oracle elsewhere.)"""
+import os
+
 import numpy as np
 import pytest
 import torch
@@ -23,10 +26,23 @@ def device_us(fn, reps=5):
     return best
 
 
+def check_ratio(unusual, ordinary, bound):
+    """unusual() < bound * ordinary(), both in microseconds, in one of four tries."""
+    ratios = []
+    for _ in range(4):
+        ratios.append(unusual() / ordinary())
+        if ratios[-1] < bound:
+            break
+    if os.environ.get("SS_PARITY_LOG"):
+        with open(os.environ["SS_PARITY_LOG"], "a") as f:
+            f.write(f"ratio {ratios} bound {bound}\n")
+    assert min(ratios) < bound, ratios
+
+
 @pytest.mark.parametrize("call", ["topk", "early_prune"])
 def test_one_large_segment_among_many_small_ones(call):
-    """The block size follows the average segment; the largest one is sorted by such a block (measured 1.5 times the large
-    segment alone, which has four times the threads; 4.5 with blocks of 64)."""
+    """The block size follows the average segment; the largest one is sorted by such a block: 1.4 times the large segment alone,
+    which has four times the threads (3.9 with blocks of 64)."""
     def us(sizes):
         seg = torch.tensor(np.concatenate([[0], np.cumsum(sizes)]), dtype=torch.int32, device=DEV)
         n, P, k = int(seg[-1]), len(sizes), 8
@@ -37,7 +53,7 @@ def test_one_large_segment_among_many_small_ones(call):
         if call == "topk":
             return device_us(lambda: B.ss_topk_prune(sc, seg, P, n, k, sel, mask, ws))
         return device_us(lambda: B.ss_early_prune(sc, ver, seg, P, n, k, mask, sel, fin, ws))
-    assert us([4096] + [16] * 1000) < 3 * us([4096])
+    check_ratio(lambda: us([4096] + [16] * 1000), lambda: us([4096]), 3)
 
 
 def sample_us(logits, draws_each, T=0.8, u=None):
@@ -50,38 +66,38 @@ def sample_us(logits, draws_each, T=0.8, u=None):
 
 
 def test_uniform_zero_behind_a_long_mask():
-    """Measured 1.4 times a draw in the middle; 140 with a pass over the row by one warp."""
+    """1.4 times a draw in the middle (88 with a pass over the row by one warp)."""
     logits = torch.randn((16, 151936), device=DEV)
     logits[:, :-10] = -float("inf")
-    assert sample_us(logits, 4, u=0.0) < 8 * sample_us(logits, 4, u=0.5)
+    check_ratio(lambda: sample_us(logits, 4, u=0.0), lambda: sample_us(logits, 4, u=0.5), 8)
 
 
 @pytest.mark.parametrize("shift,T", [(3000.0, 0.8), (0.0, 1e-4)])
 def test_rows_outside_the_table_path(shift, T):
-    """They take a second pass; measured 1.9 times an ordinary row (3.9 with CUDA's exp in the second pass)."""
+    """They take a second pass: 2.3 and 1.9 times an ordinary row (3.6 and 3.4 with CUDA's exp in the second pass)."""
     logits = torch.randn((600, 151936), device=DEV) * 3
-    assert sample_us(logits + shift, 2, T=T) < 3 * sample_us(logits, 2)
+    check_ratio(lambda: sample_us(logits + shift, 2, T=T), lambda: sample_us(logits, 2), 3)
 
 
 def test_thousands_of_draws_of_a_row():
-    """Measured 118 us against 373 one draw after the other; 182 for the ordinary case to compare with."""
+    """64 rows with 4096 draws each, in the time of 922 large rows: 0.66 times (1.8 one draw after the other)."""
     many, rows = torch.randn((64, 32000), device=DEV) * 3, torch.randn((922, 151936), device=DEV) * 3
-    assert sample_us(many, 4096) < 1.3 * sample_us(rows, 2)
+    check_ratio(lambda: sample_us(many, 4096), lambda: sample_us(rows, 2), 1.3)
 
 
 def test_prefix_tree_of_a_million_short_paths():
-    """Measured 2.3 ms, 10 times 100000 of them 2.5; 34 where every position searched every sorted tile."""
+    """10.6 times 100000 of them (69 where every position searched every sorted tile)."""
     def us(n):
         off = torch.arange(n + 1, dtype=torch.int64, device=DEV) * 6
         ids = torch.randint(0, 150000, (6 * n,), dtype=torch.int32, device=DEV)
         out = [torch.empty(2 * n, dtype=torch.int32, device=DEV) for _ in range(7)]
         ws = B.alloc_workspace(B.ss_prefix_tree_workspace_bytes(n, 6 * n, 16), torch.device(DEV))
         return device_us(lambda: B.ss_build_prefix_tree(ids, off, n, 6 * n, 16, *out, ws))
-    assert us(1 << 20) < 25 * us(100000)
+    check_ratio(lambda: us(1 << 20), lambda: us(100000), 25)
 
 
 def test_dedup_of_a_million_equal_paths():
-    """Measured 0.93 times a million different ones (5.6 with an atomic on one address for each, 1.3 before hashes were tabled)."""
+    """1.1 times a million different ones (6.9 with atomics on one address for each)."""
     def us(distinct):
         n = 1 << 20
         ids = torch.arange(n, dtype=torch.int32, device=DEV) % distinct
@@ -89,4 +105,4 @@ def test_dedup_of_a_million_equal_paths():
         out = [torch.empty(n, dtype=torch.int32, device=DEV) for _ in range(4)]
         num, ws = torch.empty(1, dtype=torch.int32, device=DEV), B.alloc_workspace(B.ss_dedup_workspace_bytes(n), torch.device(DEV))
         return device_us(lambda: B.ss_dedup_paths(ids, off, None, None, n, 0, *out, None, num, ws))
-    assert us(1) < 2 * us(1 << 20)
+    check_ratio(lambda: us(1), lambda: us(1 << 20), 2)
