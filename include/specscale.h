@@ -359,6 +359,51 @@ int32_t ss_build_prefix_tree(const int32_t* tok_ids, const int64_t* tok_offsets,
                              size_t workspace_bytes, void* stream);
 
 /* =========================================================================================================
+ * ss_candidate_step - one pass of the whole path for per-step data that lives in DEVICE memory.
+ *
+ * Paper: as for ss_candidate_step_host below.  Results are those of ss_dedup_paths, ss_gather_unique_paths, ss_tree_attention and
+ * ss_topk_prune in this order, on the arguments of the same names; up to 4096 candidates the parts that do not need one another
+ * share launches.  `attn` is passed to ss_tree_attention as it is: its per-path arrays are the u_* arrays and num_unique of this
+ * struct where a step is wanted.  Nothing is allocated, and the call does not synchronise.
+ * Errors: those of the four calls.
+ * ======================================================================================================= */
+typedef struct ss_device_step {
+  uint32_t struct_size;              /* = sizeof(ss_device_step_t) */
+  uint32_t dedup_flags;              /* 0 or SS_FLAG_WEAK_HASH */
+  const ss_attn_desc_t* attn;        /* host */
+  int32_t n_paths, n_segments, top_k, reserved;
+  size_t dedup_workspace_bytes, attn_workspace_bytes, topk_workspace_bytes;
+  /* inputs, device memory */
+  const int32_t* tok_ids;
+  const int64_t* tok_offsets;
+  const int64_t* ctx_key;
+  const int32_t* slot_in;
+  const int32_t* path_leaf_node;
+  const int32_t* path_q_len;
+  const int64_t* q_offsets;
+  const float* scores;
+  const int32_t* seg_offsets;
+  /* results, device memory */
+  int32_t* canon;
+  int32_t* path_to_unique;
+  int32_t* unique_paths;
+  int32_t* multiplicity;
+  int32_t* slot_out;
+  int32_t* num_unique;
+  int32_t* u_leaf;
+  int32_t* u_q_len;
+  int64_t* u_q_offsets;
+  int64_t* u_q_src;
+  int32_t* survivors;
+  uint8_t* keep;
+  void* dedup_workspace;
+  void* attn_workspace;
+  void* topk_workspace;
+} ss_device_step_t;
+
+int32_t ss_candidate_step(const ss_device_step_t* step /* host */, void* stream);
+
+/* =========================================================================================================
  * ss_candidate_step_host - one pass of the whole path for per-step data that lives in HOST memory.
  *
  * Paper: the system overview figure and Sections "Computation Deduplication", "Lazy Verification" and "Early

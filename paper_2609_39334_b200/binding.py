@@ -39,7 +39,7 @@ EXPORTS = [
     "ss_launch_count", "ss_debug_umma_tile", "ss_debug_bounded_wait", "ss_profile_enable", "ss_profile_read",
     "ss_dedup_paths_static", "ss_debug_tile_kernel_occupancy", "ss_early_prune",
     "ss_branch_sample", "ss_gather_unique_paths", "ss_candidate_step_host_arena_bytes", "ss_candidate_step_host",
-    "ss_prefix_tree_workspace_bytes", "ss_build_prefix_tree",
+    "ss_prefix_tree_workspace_bytes", "ss_build_prefix_tree", "ss_candidate_step",
 ]
 PHASES = ["plan", "tiles", "leaves", "generic", "merge"]
 
@@ -84,7 +84,7 @@ _SIGNATURES = {
     "ss_tree_attention_workspace_bytes": "pp", "ss_tree_attention": "ppzp", "ss_topk_workspace_bytes": "ip",
     "ss_topk_prune": "ppiiipppzp", "ss_early_prune": "pppiiippppzp", "ss_branch_sample": "pppiifppp",
     "ss_prefix_tree_workspace_bytes": "iqip", "ss_build_prefix_tree": "ppiqippppppppzp",
-    "ss_candidate_step_host_arena_bytes": "pp", "ss_candidate_step_host": "ppzp", "ss_profile_enable": "i",
+    "ss_candidate_step": "pp", "ss_candidate_step_host_arena_bytes": "pp", "ss_candidate_step_host": "ppzp", "ss_profile_enable": "i",
     "ss_profile_read": "pp", "ss_debug_umma_tile": "pppiiipp", "ss_debug_bounded_wait": "pp",
 }
 
@@ -216,6 +216,29 @@ def ss_build_prefix_tree(tok_ids, tok_offsets, n_paths, total_tok, page_size, or
                                     workspace.numel() * workspace.element_size(), _stream(stream))
     if check:
         _check(rc, "ss_build_prefix_tree")
+    return rc
+
+
+class ss_device_step_t(ctypes.Structure):
+    _fields_ = [
+        ("struct_size", ctypes.c_uint32), ("dedup_flags", ctypes.c_uint32),
+        ("attn", ctypes.c_void_p),
+        ("n_paths", ctypes.c_int32), ("n_segments", ctypes.c_int32), ("top_k", ctypes.c_int32),
+        ("reserved", ctypes.c_int32),
+        ("dedup_workspace_bytes", ctypes.c_size_t), ("attn_workspace_bytes", ctypes.c_size_t),
+        ("topk_workspace_bytes", ctypes.c_size_t),
+    ] + [(n, ctypes.c_void_p) for n in (
+        "tok_ids", "tok_offsets", "ctx_key", "slot_in", "path_leaf_node", "path_q_len", "q_offsets", "scores",
+        "seg_offsets", "canon", "path_to_unique", "unique_paths", "multiplicity", "slot_out", "num_unique", "u_leaf",
+        "u_q_len", "u_q_offsets", "u_q_src", "survivors", "keep", "dedup_workspace", "attn_workspace",
+        "topk_workspace")]
+
+
+def ss_candidate_step(step: ss_device_step_t, stream=None, check=True) -> int:
+    """Deduplication, gather, attention and selection as one call (see the header); `step` holds device pointers."""
+    rc = lib().ss_candidate_step(ctypes.byref(step), _stream(stream))
+    if check:
+        _check(rc, "ss_candidate_step")
     return rc
 
 

@@ -17,7 +17,7 @@
 // third compacts with a block per 1024 paths.  Latency-bound: a few MB of ids, a handful of dependent trips to L2.
 // Measured, the call: 1024 paths 35 -> 14 us (a bitonic sort of the hashes and binary searches by one block before),
 // 8192 paths 78 -> 28 us (a sort by counting, a compaction by one block).
-#include "common.cuh"
+#include "topk.cuh"
 
 namespace ss {
 namespace dedup {
@@ -40,9 +40,16 @@ __device__ __forceinline__ uint64_t hash_path(const int32_t* __restrict__ tok_id
                                               const int64_t* __restrict__ ctx_key, int path, uint32_t weak, int lane) {
   const int64_t lo = tok_offsets[path], hi = tok_offsets[path + 1];
   uint64_t acc = 0;
-  for (int64_t j = lo + lane; j < hi; j += 32) {
-    const uint64_t t = static_cast<uint32_t>(tok_ids[j]);
-    acc += mix64(t * 0x9e3779b97f4a7c15ull + static_cast<uint64_t>(j - lo + 1) * 0xd1b54a32d192ed03ull);
+  constexpr int kUnroll = 8;                    // loads in flight: paths of 300 tokens are one or two trips to memory, not ten
+  for (int64_t j0 = lo + lane; j0 < hi; j0 += 32 * kUnroll) {
+    uint32_t t[kUnroll];
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) t[u] = j0 + 32 * u < hi ? static_cast<uint32_t>(tok_ids[j0 + 32 * u]) : 0u;
+#pragma unroll
+    for (int u = 0; u < kUnroll; ++u) {
+      const int64_t j = j0 + 32 * u;
+      if (j < hi) acc += mix64(t[u] * 0x9e3779b97f4a7c15ull + static_cast<uint64_t>(j - lo + 1) * 0xd1b54a32d192ed03ull);
+    }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -90,12 +97,43 @@ __global__ void hash_kernel(const int32_t* __restrict__ tok_ids, const int64_t* 
   }
 }
 
+// The selection of a step, which needs nothing from the deduplication nor it from the selection: blocks of the first launch.
+struct Selection {
+  const float* scores;
+  const int32_t* seg_offsets;
+  int n_segments, k;
+  int32_t* survivors;
+  uint8_t* keep;
+  uint64_t* scratch;
+  int32_t* status;
+};
+__device__ __forceinline__ void selection_block(const Selection& T, int s, int n) {
+  __shared__ uint64_t smem_keys[topk::kSmemKeys];
+  topk::select_segment(s, T.n_segments, T.scores, T.seg_offsets, n, T.k, T.survivors, T.keep, T.scratch, T.status, smem_keys);
+}
+// Hash of every path, as above without a table, and the selection's blocks behind those of the hash.
+__global__ void __launch_bounds__(kHashWarps * 32)
+hash_select_kernel(const int32_t* __restrict__ tok_ids, const int64_t* __restrict__ tok_offsets,
+                   const int64_t* __restrict__ ctx_key, int n, uint32_t weak, uint64_t* __restrict__ hash64,
+                   unsigned int* __restrict__ arrived, int hash_blocks, const __grid_constant__ Selection T) {
+  ss::grid_dependency_enter();
+  if (static_cast<int>(blockIdx.x) >= hash_blocks) {
+    selection_block(T, blockIdx.x - hash_blocks, n);
+    return;
+  }
+  const int lane = threadIdx.x & 31, path = blockIdx.x * kHashWarps + (threadIdx.x >> 5);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *arrived = 0;
+  if (path >= n) return;
+  const uint64_t h = hash_path(tok_ids, tok_offsets, ctx_key, path, weak, lane);
+  if (lane == 0) hash64[path] = h;
+}
+
 // Whole warp: paths i and j have the same context, length and ids.
 __device__ __forceinline__ bool same_path(const int32_t* __restrict__ tok_ids, const int64_t* __restrict__ tok_offsets,
                                           const int64_t* __restrict__ ctx_key, int i, int j, int lane) {
   const int64_t a0 = tok_offsets[i], b0 = tok_offsets[j], len = tok_offsets[i + 1] - a0;
   if (tok_offsets[j + 1] - b0 != len || (ctx_key && ctx_key[i] != ctx_key[j])) return false;
-  constexpr int kUnroll = 4;
+  constexpr int kUnroll = 8;
   for (int64_t p = lane; p - lane < len; p += 32 * kUnroll) {
     int32_t x[kUnroll], y[kUnroll];
 #pragma unroll
@@ -178,23 +216,69 @@ __device__ __forceinline__ void small_match(const int32_t* __restrict__ tok_ids,
   }
 }
 
-// One block, all of canon_out written: ranks, unique list, multiplicities, remap.  s_mem: 8 n bytes.
+// The descriptor rows of the unique paths (see gather_unique_kernel), made with the compaction where a whole step is one call.
+struct Gather {
+  const int32_t *path_leaf_node, *path_q_len;
+  const int64_t* q_offsets;
+  int32_t *u_leaf, *u_q_len;                                  // null: no gather
+  int64_t *u_q_offsets, *u_q_src;
+};
+constexpr int kOwn = kSmallMax / kThreads;                    // paths of a thread: tid, tid + kThreads, ...
+// A path's own descriptor row, loaded before it is known whether it is wanted (all blocks do, the last one needs them).
+struct GatherRows {
+  int leaf[kOwn], len[kOwn];
+  int64_t src[kOwn];
+};
+template <bool GATHER>
+__device__ __forceinline__ void load_rows(GatherRows& R, const Gather& G, int n) {
+  if (!GATHER) return;
+#pragma unroll
+  for (int e = 0; e < kOwn; ++e) {
+    const int i = threadIdx.x + e * kThreads;
+    R.leaf[e] = i < n ? G.path_leaf_node[i] : -1;
+    R.len[e] = i < n ? G.path_q_len[i] : 0;
+    R.src[e] = i < n ? G.q_offsets[i] : 0;
+  }
+}
+
+// One block, all of canon_out written: ranks, unique list, multiplicities, remap (and the gather).  s_mem: 8 n bytes.
+template <bool GATHER>
 __device__ __forceinline__ void small_compact(int n, const int32_t* __restrict__ slot_in, const int32_t* canon_out,
                                               int32_t* path_to_unique, int32_t* unique_paths, int32_t* multiplicity,
-                                              int32_t* slot_out, int32_t* num_unique, uint8_t* s_mem) {
+                                              int32_t* slot_out, int32_t* num_unique, uint8_t* s_mem, const Gather& G,
+                                              const GatherRows& R) {
   __shared__ int s_before[kSmallMax / 32];                    // unique paths in front of each group of 32
+  __shared__ long long s_rows[GATHER ? kSmallMax / 32 : 1], s_all_rows;   // and their query rows
   __shared__ int s_total;
   const int tid = threadIdx.x, lane = tid & 31, groups = (n + 31) >> 5;
   int* s_rank = reinterpret_cast<int*>(s_mem);
   int* s_mult = s_rank + n;
-  for (int i0 = tid & ~31; i0 < n; i0 += kThreads) {
-    const int i = i0 + lane;
-    const uint32_t u = __ballot_sync(0xffffffffu, i < n && __ldcg(canon_out + (i < n ? i : 0)) == i);
+  int canon[kOwn];
+  long long rows[kOwn];                                       // of the unique paths up to this one in its group
+#pragma unroll
+  for (int e = 0; e < kOwn; ++e) {
+    const int i = tid + e * kThreads;
+    canon[e] = i < n ? __ldcg(canon_out + i) : -1;
+  }
+#pragma unroll
+  for (int e = 0; e < kOwn; ++e) {
+    const int i = tid + e * kThreads;
+    if (i - lane >= n) break;
+    const uint32_t u = __ballot_sync(0xffffffffu, canon[e] == i);
     if (i < n) {
       s_rank[i] = __popc(u & ((1u << lane) - 1u));
       s_mult[i] = 0;
     }
-    if (lane == 0) s_before[i0 >> 5] = __popc(u);
+    if (lane == 0) s_before[i >> 5] = __popc(u);
+    if (GATHER) {
+      rows[e] = canon[e] == i ? R.len[e] : 0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const long long y = __shfl_up_sync(0xffffffffu, rows[e], o);
+        if (lane >= o) rows[e] += y;
+      }
+      if (lane == 31) s_rows[i >> 5] = rows[e];
+    }
   }
   __syncthreads();
   if (tid < 32) {                                             // 4 groups a lane
@@ -217,34 +301,76 @@ __device__ __forceinline__ void small_compact(int n, const int32_t* __restrict__
       run += v[k];
     }
     if (lane == 31) s_total = incl;
+  } else if (GATHER && tid < 64) {
+    long long v[4], sum = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      v[k] = 4 * lane + k < groups ? s_rows[4 * lane + k] : 0;
+      sum += v[k];
+    }
+    long long incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    long long run = incl - sum;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (4 * lane + k < groups) s_rows[4 * lane + k] = run;
+      run += v[k];
+    }
+    if (lane == 31) s_all_rows = incl;
   }
   __syncthreads();
-  for (int i = tid; i < n; i += kThreads) {
-    const int c = __ldcg(canon_out + i);
-    const int r = s_before[c >> 5] + s_rank[c];
+  const int total = s_total;
+#pragma unroll
+  for (int e = 0; e < kOwn; ++e) {
+    const int i = tid + e * kThreads;
+    if (i >= n) break;
+    const int c = canon[e], r = s_before[c >> 5] + s_rank[c];
     path_to_unique[i] = r;
     if (c == i) unique_paths[r] = i;
     atomicAdd(&s_mult[r], 1);
     if (slot_out) slot_out[i] = slot_in[c];
+    if (GATHER) {
+      if (c == i) {
+        G.u_leaf[r] = R.leaf[e];
+        G.u_q_len[r] = R.len[e];
+        G.u_q_src[r] = R.src[e];
+        G.u_q_offsets[r + 1] = s_rows[i >> 5] + rows[e];
+      }
+      if (i >= total) {                                       // inert entries
+        G.u_leaf[i] = -1;
+        G.u_q_len[i] = 0;
+        G.u_q_src[i] = 0;
+        G.u_q_offsets[i + 1] = s_all_rows;
+      }
+    }
   }
+  if (GATHER && tid == 0) G.u_q_offsets[0] = 0;
   __syncthreads();
-  for (int i = tid; i < s_total; i += kThreads) multiplicity[i] = s_mult[i];
-  for (int i = s_total + tid; i < n; i += kThreads) multiplicity[i] = 0;
-  if (tid == 0) *num_unique = s_total;
+  for (int i = tid; i < total; i += kThreads) multiplicity[i] = s_mult[i];
+  for (int i = total + tid; i < n; i += kThreads) multiplicity[i] = 0;
+  if (tid == 0) *num_unique = total;
 }
 
+template <bool GATHER>
 __global__ void __launch_bounds__(kThreads)
 small_match_kernel(const int32_t* __restrict__ tok_ids, const int64_t* __restrict__ tok_offsets,
                    const int64_t* __restrict__ ctx_key, int n, const uint64_t* __restrict__ hash64, uint32_t mask,
                    const int32_t* __restrict__ slot_in, int32_t* canon_out, int32_t* path_to_unique, int32_t* unique_paths,
-                   int32_t* multiplicity, int32_t* slot_out, int32_t* num_unique, unsigned int* arrived) {
+                   int32_t* multiplicity, int32_t* slot_out, int32_t* num_unique, unsigned int* arrived,
+                   const __grid_constant__ Gather G) {
   ss::grid_dependency_enter();
   extern __shared__ __align__(16) uint8_t s_mem[];
   uint64_t* s_hash = reinterpret_cast<uint64_t*>(s_mem);
+  GatherRows R;
+  load_rows<GATHER>(R, G, n);
   small_match(tok_ids, tok_offsets, ctx_key, n, hash64, canon_out, s_hash, reinterpret_cast<int*>(s_hash + n), mask, n);
   if (!last_block_arrives(arrived)) return;
   // compaction by the last block; the hashes' shared memory holds ranks and multiplicities
-  small_compact(n, slot_in, canon_out, path_to_unique, unique_paths, multiplicity, slot_out, num_unique, s_mem);
+  small_compact<GATHER>(n, slot_in, canon_out, path_to_unique, unique_paths, multiplicity, slot_out, num_unique, s_mem, G, R);
 }
 
 // ---- up to kClusterMax paths: one launch of one cluster, whose barrier separates hash, match and compaction -------------
@@ -255,15 +381,24 @@ constexpr int kClusterBlocks = 8;
 __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
+// STEP: with the gather, and the selection by the clusters behind the first.
+template <bool STEP>
 __global__ void __cluster_dims__(kClusterBlocks, 1, 1) __launch_bounds__(kThreads)
 cluster_dedup_kernel(const int32_t* __restrict__ tok_ids, const int64_t* __restrict__ tok_offsets,
                      const int64_t* __restrict__ ctx_key, int n, uint32_t weak, uint64_t* hash64, uint32_t mask,
                      const int32_t* __restrict__ slot_in, int32_t* canon_out, int32_t* path_to_unique, int32_t* unique_paths,
-                     int32_t* multiplicity, int32_t* slot_out, int32_t* num_unique) {
+                     int32_t* multiplicity, int32_t* slot_out, int32_t* num_unique, const __grid_constant__ Gather G,
+                     const __grid_constant__ Selection T) {
   ss::grid_dependency_enter();
+  if (STEP && blockIdx.x >= kClusterBlocks) {
+    if (static_cast<int>(blockIdx.x) - kClusterBlocks < T.n_segments) selection_block(T, blockIdx.x - kClusterBlocks, n);
+    return;
+  }
   __shared__ __align__(16) uint64_t s_hash[kClusterMax];
   __shared__ int s_tab[4 * kClusterMax];                        // (small_table_size: below 4 n, at least 64)
   const int lane = threadIdx.x & 31;
+  GatherRows R;
+  load_rows<STEP>(R, G, n);
   for (int i = blockIdx.x * kWarps + (threadIdx.x >> 5); i < n; i += kClusterBlocks * kWarps) {
     const uint64_t h = hash_path(tok_ids, tok_offsets, ctx_key, i, weak, lane);
     if (lane == 0) hash64[i] = h;
@@ -272,8 +407,8 @@ cluster_dedup_kernel(const int32_t* __restrict__ tok_ids, const int64_t* __restr
   small_match(tok_ids, tok_offsets, ctx_key, n, hash64, canon_out, s_hash, s_tab, mask, kClusterBlocks * kWarps);
   cluster_barrier();
   if (blockIdx.x == 0)
-    small_compact(n, slot_in, canon_out, path_to_unique, unique_paths, multiplicity, slot_out, num_unique,
-                  reinterpret_cast<uint8_t*>(s_hash));
+    small_compact<STEP>(n, slot_in, canon_out, path_to_unique, unique_paths, multiplicity, slot_out, num_unique,
+                        reinterpret_cast<uint8_t*>(s_hash), G, R);
 }
 
 // ---- more paths -----------------------------------------------------------------------------------------------------
@@ -463,7 +598,9 @@ static int32_t small_smem_ready() {
   static bool configured[kDeviceSlots] = {false};
   const int slot = current_device_slot();
   if (slot >= 0 && configured[slot]) return SS_OK;
-  if (cudaFuncSetAttribute(small_match_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (cudaFuncSetAttribute(small_match_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(small_match_smem(kSmallMax))) != cudaSuccess ||
+      cudaFuncSetAttribute(small_match_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            static_cast<int>(small_match_smem(kSmallMax))) != cudaSuccess) {
     (void)cudaGetLastError();
     return SS_ERR_CUDA;
@@ -529,9 +666,9 @@ extern "C" int32_t ss_dedup_paths(const int32_t* tok_ids, const int64_t* tok_off
   const uint32_t weak = (flags & SS_FLAG_WEAK_HASH) ? 1u : 0u;
   const int hash_blocks = (n + kHashWarps - 1) / kHashWarps, match_blocks = (n + kWarps - 1) / kWarps;
   if (n <= kClusterMax) {
-    SS_LAUNCH(cluster_dedup_kernel, kClusterBlocks, kThreads, 0, st, tok_ids, tok_offsets, ctx_key, n, weak, hash64,
+    SS_LAUNCH(cluster_dedup_kernel<false>, kClusterBlocks, kThreads, 0, st, tok_ids, tok_offsets, ctx_key, n, weak, hash64,
               static_cast<uint32_t>(small_table_size(n) - 1), slot_in, canon_out, path_to_unique_out, unique_paths_out,
-              multiplicity_out, slot_out, num_unique_out);
+              multiplicity_out, slot_out, num_unique_out, Gather{}, Selection{});
     return SS_OK;
   }
   if (n <= kSmallMax) {
@@ -540,9 +677,9 @@ extern "C" int32_t ss_dedup_paths(const int32_t* tok_ids, const int64_t* tok_off
     if (rc != SS_OK) return rc;
     SS_LAUNCH(hash_kernel, hash_blocks, kHashWarps * 32, 0, st, tok_ids, tok_offsets, ctx_key, n, weak, hash64,
               static_cast<unsigned long long*>(nullptr), 0u, static_cast<int*>(nullptr), static_cast<int32_t*>(nullptr), arrived);
-    SS_LAUNCH(small_match_kernel, match_blocks, kThreads, small_match_smem(n), st, tok_ids, tok_offsets, ctx_key, n, hash64,
+    SS_LAUNCH(small_match_kernel<false>, match_blocks, kThreads, small_match_smem(n), st, tok_ids, tok_offsets, ctx_key, n, hash64,
               static_cast<uint32_t>(small_table_size(n) - 1), slot_in, canon_out, path_to_unique_out, unique_paths_out,
-              multiplicity_out, slot_out, num_unique_out, arrived);
+              multiplicity_out, slot_out, num_unique_out, arrived, Gather{});
     return SS_OK;
   }
   unsigned long long* table = reinterpret_cast<unsigned long long*>(ws + L.table);
@@ -646,4 +783,82 @@ extern "C" int32_t ss_gather_unique_paths(const int32_t* unique_paths, const int
   SS_LAUNCH(gather_unique_kernel, 1, kGatherThreads, 0, st, unique_paths, num_unique, n_paths, path_leaf_node, path_q_len,
             q_offsets, u_leaf_out, u_q_len_out, u_q_offsets_out, u_q_src_out);
   return SS_OK;
+}
+
+// ---- ss_candidate_step ------------------------------------------------------------------------------------------------
+namespace ss {
+namespace dedup {
+
+// The front of a step of up to kSmallMax paths - deduplication, gather, selection - in one launch (a cluster, the selection's
+// blocks beside it) or two (the selection's blocks beside the hash, the gather by the block that compacts) where the four calls
+// take three or four.  Measured, the step: 8 paths 33.8 -> 29.3 us, 1024 paths 104.8 -> 94.7 (two levels 183.4 -> 174.2), 8
+// verification paths 40.2 -> 36.5.  Part of it (1024 paths) are the loads of the hash, eight a lane in flight instead of one.
+static int32_t launch_front(const ss_device_step_t& s, cudaStream_t st) {
+  const Layout L = layout(s.n_paths);
+  char* ws = static_cast<char*>(s.dedup_workspace);
+  uint64_t* hash64 = reinterpret_cast<uint64_t*>(ws + L.hash64);
+  const int n = s.n_paths;
+  const uint32_t weak = (s.dedup_flags & SS_FLAG_WEAK_HASH) ? 1u : 0u, mask = static_cast<uint32_t>(small_table_size(n) - 1);
+  const Gather G{s.path_leaf_node, s.path_q_len, s.q_offsets, s.u_leaf, s.u_q_len, s.u_q_offsets, s.u_q_src};
+  const Selection T{s.scores, s.seg_offsets, s.n_segments, s.top_k, s.survivors, s.keep,
+                    reinterpret_cast<uint64_t*>(static_cast<char*>(s.topk_workspace) + kAlign), static_cast<int32_t*>(s.topk_workspace)};
+  if (n <= kClusterMax) {
+    const int clusters = 1 + (s.n_segments + kClusterBlocks - 1) / kClusterBlocks;
+    SS_LAUNCH(cluster_dedup_kernel<true>, clusters * kClusterBlocks, kThreads, 0, st, s.tok_ids, s.tok_offsets, s.ctx_key, n, weak, hash64,
+              mask, s.slot_in, s.canon, s.path_to_unique, s.unique_paths, s.multiplicity, s.slot_out, s.num_unique, G, T);
+    return SS_OK;
+  }
+  const int32_t rc = small_smem_ready();
+  if (rc != SS_OK) return rc;
+  const int hash_blocks = (n + kHashWarps - 1) / kHashWarps, match_blocks = (n + kWarps - 1) / kWarps;
+  unsigned int* arrived = reinterpret_cast<unsigned int*>(ws + L.counters);
+  SS_LAUNCH(hash_select_kernel, hash_blocks + s.n_segments, kHashWarps * 32, 0, st, s.tok_ids, s.tok_offsets, s.ctx_key, n, weak, hash64,
+            arrived, hash_blocks, T);
+  SS_LAUNCH(small_match_kernel<true>, match_blocks, kThreads, small_match_smem(n), st, s.tok_ids, s.tok_offsets, s.ctx_key, n, hash64, mask,
+            s.slot_in, s.canon, s.path_to_unique, s.unique_paths, s.multiplicity, s.slot_out, s.num_unique, arrived, G);
+  return SS_OK;
+}
+
+// True if the four calls would accept their arguments, so that nothing has to be refused half-way.
+static bool front_args_ok(const ss_device_step_t& s) {
+  if ((s.slot_in == nullptr) != (s.slot_out == nullptr) || s.top_k < 1 || (s.dedup_flags & ~SS_FLAG_WEAK_HASH)) return false;
+  const void* const needed[] = {s.tok_ids, s.tok_offsets, s.canon, s.path_to_unique, s.unique_paths, s.multiplicity, s.num_unique,
+                                s.dedup_workspace, s.path_leaf_node, s.path_q_len, s.q_offsets, s.u_leaf, s.u_q_len, s.u_q_offsets,
+                                s.u_q_src, s.scores, s.seg_offsets, s.survivors, s.keep, s.topk_workspace};
+  for (const void* p : needed)
+    if (!p) return false;
+  size_t topk_bytes = 0;
+  if (ss_topk_workspace_bytes(s.n_paths, &topk_bytes) != SS_OK) return false;
+  return reinterpret_cast<uintptr_t>(s.dedup_workspace) % kAlign == 0 && reinterpret_cast<uintptr_t>(s.topk_workspace) % kAlign == 0 &&
+         s.dedup_workspace_bytes >= layout(s.n_paths).total && s.topk_workspace_bytes >= topk_bytes;
+}
+
+}  // namespace dedup
+}  // namespace ss
+
+extern "C" int32_t ss_candidate_step(const ss_device_step_t* step, void* stream) {
+  using namespace ss;
+  using namespace ss::dedup;
+  if (!step || step->struct_size != sizeof(ss_device_step_t) || !step->attn) return SS_ERR_INVALID_ARG;
+  const ss_device_step_t& s = *step;
+  const int n = s.n_paths;
+  // The selection shares the front's launches where 256 threads (1024 in the cluster form) are as many as its own launch would
+  // take, and its segments are not many times the other blocks.
+  const bool front = n > 0 && n <= kSmallMax && s.n_segments > 0 && s.n_segments <= 1024 && front_args_ok(s) &&
+                     (n <= kClusterMax || topk::block_threads(n, s.n_segments) <= kHashWarps * 32);
+  int32_t rc;
+  if (front) {
+    rc = launch_front(s, as_stream(stream));
+    return rc != SS_OK ? rc : ss_tree_attention(s.attn, s.attn_workspace, s.attn_workspace_bytes, stream);
+  }
+  rc = ss_dedup_paths(s.tok_ids, s.tok_offsets, s.ctx_key, s.slot_in, n, s.dedup_flags, s.canon, s.path_to_unique, s.unique_paths,
+                      s.multiplicity, s.slot_out, s.num_unique, s.dedup_workspace, s.dedup_workspace_bytes, stream);
+  if (rc != SS_OK) return rc;
+  rc = ss_gather_unique_paths(s.unique_paths, s.num_unique, n, s.path_leaf_node, s.path_q_len, s.q_offsets, s.u_leaf, s.u_q_len,
+                              s.u_q_offsets, s.u_q_src, stream);
+  if (rc != SS_OK) return rc;
+  rc = ss_tree_attention(s.attn, s.attn_workspace, s.attn_workspace_bytes, stream);
+  if (rc != SS_OK) return rc;
+  return ss_topk_prune(s.scores, s.seg_offsets, s.n_segments, n, s.top_k, s.survivors, s.keep, s.topk_workspace, s.topk_workspace_bytes,
+                       stream);
 }

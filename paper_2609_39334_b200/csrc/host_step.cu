@@ -1,7 +1,6 @@
 // ss_candidate_step_host: one pass of the whole candidate-path hot path for a caller whose per-step data lives in
 // HOST memory.  It only strings together what the library already exports - asynchronous copies of the step's
-// inputs into a caller-owned device arena, ss_dedup_paths, ss_gather_unique_paths, ss_tree_attention,
-// ss_topk_prune, asynchronous copies of every result back - all on the caller's stream, without a host
+// inputs into a caller-owned device arena, ss_candidate_step, asynchronous copies of every result back - all on the caller's stream, without a host
 // synchronisation, so that a caller that alternates between a few arenas and streams overlaps one step's copies
 // with another step's kernels.
 //
@@ -281,13 +280,6 @@ extern "C" int32_t ss_candidate_step_host(const ss_host_step_t* step, void* devi
   }
 
   // ---- the path ---------------------------------------------------------------------------------------------------
-  rc = ss_dedup_paths(a.tok_ids, a.tok_offsets, s.ctx_key ? a.ctx_key : nullptr, s.slot_in ? a.slot_in : nullptr,
-                      s.n_paths, s.dedup_flags, a.canon, a.path_to_unique, a.unique_paths, a.multiplicity,
-                      s.slot_in ? a.slot_out : nullptr, a.num_unique, a.dedup_ws, a.dedup_ws_bytes, stream);
-  if (rc != SS_OK) return rc;
-  rc = ss_gather_unique_paths(a.unique_paths, a.num_unique, s.n_paths, a.path_leaf_node, a.path_q_len, a.q_offsets,
-                              a.u_leaf, a.u_q_len, a.u_q_offsets, a.u_q_src, stream);
-  if (rc != SS_OK) return rc;
   ss_attn_desc_t d = step_desc(s, a);
   if (compact && d.max_sms == 0) {
     // the copy kernel of the step before this one (another stream) runs for as long as the bus takes and needs SMs
@@ -299,10 +291,22 @@ extern "C" int32_t ss_candidate_step_host(const ss_host_step_t* step, void* devi
     else
       (void)cudaGetLastError();
   }
-  rc = ss_tree_attention(&d, a.attn_ws, a.attn_ws_bytes, stream);
-  if (rc != SS_OK) return rc;
-  rc = ss_topk_prune(a.scores, a.seg_offsets, s.n_segments, s.n_paths, s.top_k, a.survivors, a.keep, a.topk_ws,
-                     a.topk_ws_bytes, stream);
+  ss_device_step_t p{};
+  p.struct_size = sizeof p;
+  p.dedup_flags = s.dedup_flags;
+  p.attn = &d;
+  p.n_paths = s.n_paths; p.n_segments = s.n_segments; p.top_k = s.top_k;
+  p.dedup_workspace_bytes = a.dedup_ws_bytes; p.attn_workspace_bytes = a.attn_ws_bytes; p.topk_workspace_bytes = a.topk_ws_bytes;
+  p.tok_ids = a.tok_ids; p.tok_offsets = a.tok_offsets; p.ctx_key = s.ctx_key ? a.ctx_key : nullptr;
+  p.slot_in = s.slot_in ? a.slot_in : nullptr;
+  p.path_leaf_node = a.path_leaf_node; p.path_q_len = a.path_q_len; p.q_offsets = a.q_offsets;
+  p.scores = a.scores; p.seg_offsets = a.seg_offsets;
+  p.canon = a.canon; p.path_to_unique = a.path_to_unique; p.unique_paths = a.unique_paths; p.multiplicity = a.multiplicity;
+  p.slot_out = s.slot_in ? a.slot_out : nullptr; p.num_unique = a.num_unique;
+  p.u_leaf = a.u_leaf; p.u_q_len = a.u_q_len; p.u_q_offsets = a.u_q_offsets; p.u_q_src = a.u_q_src;
+  p.survivors = a.survivors; p.keep = a.keep;
+  p.dedup_workspace = a.dedup_ws; p.attn_workspace = a.attn_ws; p.topk_workspace = a.topk_ws;
+  rc = ss_candidate_step(&p, stream);
   if (rc != SS_OK) return rc;
 
   // ---- device -> host: every result ------------------------------------------------------------------------------------

@@ -1,11 +1,12 @@
-"""Device-side plumbing around the three C-ABI calls: uploads a synthetic workload, owns the output and
-workspace tensors, and runs   ss_dedup_paths -> ss_gather_unique_paths -> ss_tree_attention -> ss_topk_prune.
+"""Device-side plumbing around the C-ABI calls: uploads a synthetic workload, owns the output and workspace tensors, and
+runs   ss_dedup_paths -> ss_gather_unique_paths -> ss_tree_attention -> ss_topk_prune   (a whole step: ss_candidate_step).
 
 Only memory management and argument marshalling happen here: every step is a library call.  The query rows are not
 moved by the gather: the attention call reads them in place through `q_src_offsets`.
 """
 from __future__ import annotations
 
+import ctypes
 from typing import Dict
 
 import numpy as np
@@ -83,6 +84,7 @@ class DevicePipeline:
         self.survivors = torch.empty((max(self.P, 1), w.top_k), **i32)
         self.keep = torch.empty(max(N, 1), dtype=torch.uint8, device=dev)
         self.topk_ws = B.alloc_workspace(B.ss_topk_workspace_bytes(N), dev)
+        self._step_desc, self._step_values = B.ss_device_step_t(), None
 
     @staticmethod
     def _max_depth(w: TreeWorkload) -> int:
@@ -113,11 +115,19 @@ class DevicePipeline:
                         self.topk_ws, stream=stream)
 
     def step(self):
-        """One pass of the whole hot path."""
-        self.dedup()
-        self.compact_unique()
-        self.attention()
-        self.topk()
+        """One pass of the whole hot path.  The call's struct is filled again whenever one of the tensors lies elsewhere."""
+        ptr = B._ptr
+        values = (self.dedup_flags, ctypes.addressof(self.desc), self.N, self.P, self.w.top_k, 0, self.dedup_ws.numel(),
+                  self.attn_ws.numel(), self.topk_ws.numel(), ptr(self.tok_ids), ptr(self.tok_offsets), ptr(self.ctx_key),
+                  ptr(self.slot_in), ptr(self.path_leaf_node), ptr(self.path_q_len), ptr(self.q_offsets), ptr(self.scores),
+                  ptr(self.seg_offsets), ptr(self.canon), ptr(self.path_to_unique), ptr(self.unique_paths),
+                  ptr(self.multiplicity), ptr(self.slot_out), ptr(self.num_unique), ptr(self.u_leaf), ptr(self.u_q_len),
+                  ptr(self.u_q_offsets), ptr(self.u_q_src), ptr(self.survivors), ptr(self.keep), ptr(self.dedup_ws),
+                  ptr(self.attn_ws), ptr(self.topk_ws))
+        if values != self._step_values:
+            self._step_desc = B.ss_device_step_t(ctypes.sizeof(B.ss_device_step_t), *values)
+            self._step_values = values
+        B.ss_candidate_step(self._step_desc)
 
     # ------------------------------------------------------------------------------------------------------------
     def results(self) -> Dict[str, np.ndarray]:
