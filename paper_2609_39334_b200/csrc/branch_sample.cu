@@ -2,18 +2,18 @@
 // sequence with potential size n draws n next tokens as independent trials from ONE logits row; equal draws are
 // grouped afterwards with ss_dedup_paths on (sequence, token) pairs.
 //
-// The token decision is taken in fp64 (so that it agrees with a plain fp64 CPU evaluation except for draws within
+// The token decision is that of fp64 (it agrees with a plain fp64 CPU evaluation except for draws within
 // ~1e-15 of a boundary), one exponential per logit.  A row is split over the 16 warps of a block, or of a CLUSTER of
 // 2, 4 or 8 blocks when there are too few rows to give every SM one: each warp has one contiguous slice, and the slice sums
 // meet in (distributed) shared memory.  Nothing is read twice but the 512 tokens around each draw.
 //   1. every warp sums 2^(logit_v * c), c = log2(e) / temperature, over its slice in segments of 512 tokens and keeps
 //      the running sum at every segment's end (shared memory)
 //   2. the slice sums are written to every block of the cluster
-//   3. each of the row's warps takes a share of its draws: it finds the slice that holds u * Z from the slice sums, the
+//   3. each draw is a warp's: it finds the slice that holds u * Z from the slice sums, the
 //      segment from the running sums of the slice's owner, evaluates the segment again with a warp scan, and writes the
 //      token
-// A block that handles several rows takes step 1 of the next row before step 3 of the current one, between the two halves
-// of a split barrier, so that neither the barrier nor a draw is waited for; the warps that draw change from row to row.
+// A cluster that handles several rows takes step 1 of the next row before step 3 of the current one, between the two halves
+// of a split barrier; a block that handles rows by itself has four warps for step 3 alone.
 // There is no pass for the maximum: fp64 holds 2^(logit * c) itself for rows whose largest exponent lies in
 // [kLowTop, kHighTop], which every ordinary row does; a row outside (or a temperature outside [1e-3, 1e6]) is summed again
 // relative to its maximum, and its draws are taken by the warps in whose slices they fall.
@@ -24,13 +24,19 @@
 // 2^(r/128) by a polynomial of degree 4 (interpolated at Chebyshev nodes; relative error below 1.6e-16 for |r| <= 0.505, 1.8e-16 for
 // 0.508, which the fp32 rounding of 128 * c allows at the largest exponents).
 // 8 fp64 instructions with the summation; the table is copied 16 times so that every lane reads its own bank pair.
-// Bound: issue slots.  An fp64 instruction holds two, so 32 logits take ~30 clocks of a sub-partition, 120 us for
-// 922 x 151936 logits (the loop alone, measured; 4 bytes a logit from HBM would take 85).  Measured, the call: 922 rows
-// 582 -> 182 us, 16 rows 91 -> 12.4 us, against one block of 1024 threads per row with a pass for the maximum, CUDA's exp
-// and a block-wide scan for every 4096 tokens.
+//
+// Those hold the issue slots: 32 logits take ~30 clocks of a sub-partition, 922 rows of 151936 120 us where the 560 MB take 85.  So
+// a block that takes rows by itself adds them up in fp32 (quick_sums: 7 packed instructions a logit, eight terms at a time before
+// fp64) where a row has few draws.  A quick sum is within 3.2e-7 of the exact one, proven; a draw whose target is not further than
+// that from the two ends of its token (1.5 % of them) is marked and made again by the table, its whole row, in the launch
+// that takes the rows that are left over.  No token is other than the table's.
+// Bound now: HBM latency and issue slots about equally (86 us with the arithmetic taken out).  Measured, the call: 922 rows, 1362
+// draws 184 us by the table -> 130 (rows 97, marked draws and left-over rows 33), of it 20 by adding up four segments' sums over
+// the warp at once; 16 rows 12.4.
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "umma.cuh"
 
 namespace ss {
 namespace sample {
@@ -43,7 +49,15 @@ constexpr int kSeg = 512;                                     // tokens per segm
 constexpr int kMaxSegs = 32;                                  // per slice
 constexpr int kMaxVocab = 2097152;
 constexpr int kTable = 128;
-constexpr int kLater = -1;                                    // not a token
+constexpr int kLater = -1, kUnsure = -2, kTaken = -3;         // not tokens
+// Blocks that take rows by themselves (branch_rows_kernel)
+constexpr int kDrawWarps = 4;                                 // behind the kWarps that add up
+constexpr int kRowThreads = kThreads + 32 * kDrawWarps;       // (96 registers a thread)
+constexpr int kStages = 4;                                    // segments of a warp in shared memory or on their way there
+constexpr int kRingBytes = kWarps * kStages * kSeg * 4;
+constexpr int kSums = 3;                                      // rows whose sums are held at a time
+constexpr int kQuickVocab = 16384;                            // see ss_branch_sample
+constexpr double kQuickError = 3.2e-7;                        // of the quick sums, see quick_sums
 constexpr float kLowTop = -200.f, kHighTop = 900.f;           // exponent range of a row's largest term
 constexpr float kLowest = -1020.f;                            // smaller exponents count as this one (2^-820 of the sum)
 constexpr double kTiny = 1e-300;                              // above 2^-1020: what a masked token counts for
@@ -60,6 +74,9 @@ struct Args {
   double inv_temperature;
   double ck;                   // kTable * log2(e) / temperature
   float ckf, lowest;           // lowest: the logit whose exponent is kLowest
+  float c_hi, c_lo, inv_c;     // log2(e) / temperature in two parts, and its reciprocal
+  int quick_draws;             // draws of a row up to which its sums are quick ones
+  int first_idle;              // clusters from here on have no row of their own and take marked draws
   double lowest_below;         // the same for l - dm
   bool fast;                   // the temperature allows sums that are not relative to the row's maximum
 };
@@ -75,6 +92,11 @@ struct Shared {
   double table[kTable * 16];
   Sums<CL> sums[3];                    // rows in turn (a warp may be two rows ahead of one that reads its running sums)
   int queue[kWarps][64];               // see row_below
+  int pick, taken;                     // see next_unsure
+};
+struct RowShared {                     // of branch_rows_kernel
+  uint64_t full[kSums], free[kSums];   // a row's sums are there; its draws are made
+  int abort_flag, later;
 };
 
 // 2^(K / 128) * 2^(r / 128) (see the head of the file); `bits`: K in the low bits, nothing in the ones above that the shift keeps;
@@ -171,6 +193,138 @@ __device__ __forceinline__ double slice_sums(const float* __restrict__ row, cons
   }
   return end;
 }
+// ---- rows that a block takes by itself -------------------------------------------------------------------------------
+// Every lane copies what it reads itself (16 logits a segment), so that nothing has to be synchronised: 3 segments of each
+// warp, 96 KB an SM, are in flight whatever the arithmetic does.
+template <bool VEC>
+__device__ __forceinline__ void request(uint32_t dst, const float* __restrict__ row, int base, int end, int lane) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int v = base + 128 * j + 4 * lane;
+    const uint32_t d = dst + 512 * j;
+    if (VEC) {
+      if (v < end)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(row + v) : "memory");
+      else
+        asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(d), "r"(0xff800000u) : "memory");   // -inf
+    } else {
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        if (v + x < end)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d + 4 * x), "l"(row + v + x) : "memory");
+        else
+          asm volatile("st.shared.b32 [%0], %1;" ::"r"(d + 4 * x), "r"(0xff800000u) : "memory");
+      }
+    }
+  }
+}
+// A whole segment, `src`: the lane's first logit of it.
+__device__ __forceinline__ void request_whole(uint32_t dst, const float* __restrict__ src) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 512 * j), "l"(src + 128 * j) : "memory");
+}
+__device__ __forceinline__ void read_segment(uint32_t src, float (&l)[16]) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(l[4 * j]), "=f"(l[4 * j + 1]), "=f"(l[4 * j + 2]), "=f"(l[4 * j + 3])
+                 : "r"(src + 512 * j) : "memory");
+}
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float d;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
+// A lane's sum of a segment by the table, and its largest logit so far.
+__device__ __forceinline__ double exact_sums(float (&l)[16], const Args& A, const double* bank, float& mx) {
+  double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+  for (int h = 0; h < 16; h += 8) {
+    float mn = l[h];
+#pragma unroll
+    for (int x = h; x < h + 8; ++x) { mx = fmaxf(mx, l[x]); mn = fminf(mn, l[x]); }
+    if (__any_sync(0xffffffffu, !(mn >= A.lowest))) {          // masked tokens, or past the end (a NaN stays one)
+#pragma unroll
+      for (int x = h; x < h + 8; ++x) l[x] = max_nan(l[x], A.lowest);
+    }
+#pragma unroll
+    for (int x = h; x < h + 8; x += 2) {
+      s0 += exp2_table(l[x], A, bank);
+      s1 += exp2_table(l[x + 1], A, bank);
+    }
+  }
+  return s0 + s1;
+}
+
+// The same in fp32, two logits at a time, relative to a power of two 2^e0 that the lane moves when a logit exceeds it by 2^60.
+// l * c = n + f with |f| <= 1/2: n from a sum whose low bits are the integer, f exactly by an FMA with the high part of c (one
+// rounding to 2^-26) and one with the low part; 2^f by a polynomial of degree 6 (minimax of the relative error on |f| <=
+// 0.5002, coefficients rounded: 1.6e-8); n into the exponent by an integer addition.  A term is within 1.21e-7: 1.6e-8, 2.1e-8
+// from f, 2.4e-8 from the polynomial's inner roundings and 6e-8 from its last one.  Eight terms are added pairwise (three
+// roundings, 1.79e-7) and go to fp64 from there: a sum of any of them is within kQuickError of the exact one.  Terms below
+// 2^(e0 - 124) count as that, 2^-124 of the lane's largest and less.
+// Sums of four values over the warp at once (18 instructions instead of 60): lane l gets that of v[l / 8].
+__device__ __forceinline__ double warp_sums_4(const double (&v)[4], int lane) {
+  const bool up = (lane & 16) != 0, right = (lane & 8) != 0;
+  const double a = (up ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, up ? v[0] : v[2], 16);
+  const double b = (up ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, up ? v[1] : v[3], 16);
+  double c = (right ? b : a) + __shfl_xor_sync(0xffffffffu, right ? a : b, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+  return c;
+}
+
+struct QuickState {
+  float mx, e0, low, shift;
+};
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) { f32x2 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b)); return r; }
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) { f32x2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) { f32x2 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ f32x2 both(float a) { return pack2(a, a); }
+__device__ __forceinline__ void quick_base(QuickState& q, const Args& A, float e0) {
+  q.e0 = e0;
+  q.low = (e0 - 124.f) * A.inv_c;
+  q.shift = 12582912.f - e0;                                   // 1.5 * 2^23
+}
+__device__ __forceinline__ f32x2 quick_terms(float l0, float l1, const QuickState& q, const Args& A) {
+  const f32x2 l = pack2(fmaxf(l0, q.low), fmaxf(l1, q.low)), c_hi = both(A.c_hi);
+  const f32x2 nb = fma2(l, c_hi, both(q.shift));               // bits: 0x4b400000 + (n - e0)
+  f32x2 f = fma2(l, c_hi, fma2(nb, both(-1.f), both(q.shift)));
+  f = fma2(l, both(A.c_lo), f);
+  f32x2 p = fma2(f, both(0.00015353319759014994f), both(0.0013398926239460707f));
+  p = fma2(p, f, both(0.009618437848985195f));
+  p = fma2(p, f, both(0.055503323674201965f));
+  p = fma2(p, f, both(0.24022647738456726f));
+  p = fma2(p, f, both(0.6931471824645996f));
+  p = fma2(p, f, both(1.f));
+  float p0, p1, n0, n1;
+  unpack2(p, p0, p1);
+  unpack2(nb, n0, n1);
+  return pack2(__int_as_float(__float_as_int(p0) + (__float_as_int(n0) << 23)), __int_as_float(__float_as_int(p1) + (__float_as_int(n1) << 23)));
+}
+__device__ __forceinline__ double quick_sums(const float (&l)[16], const Args& A, QuickState& q) {
+  float top = l[0];
+#pragma unroll
+  for (int x = 1; x < 16; ++x) top = max_nan(top, l[x]);
+  q.mx = max_nan(q.mx, top);
+  const float te = top * A.c_hi;
+  if (te > q.e0 + 60.f) quick_base(q, A, rintf(fminf(te, 2000.f)));   // (such a row is out of range anyway)
+  const int e0 = __float2int_rn(q.e0) << 20;
+  double s = 0.0;
+#pragma unroll
+  for (int h = 0; h < 16; h += 8) {
+    const f32x2 t = add2(add2(quick_terms(l[h], l[h + 1], q, A), quick_terms(l[h + 2], l[h + 3], q, A)),
+                         add2(quick_terms(l[h + 4], l[h + 5], q, A), quick_terms(l[h + 6], l[h + 7], q, A)));
+    float a, b;
+    unpack2(t, a, b);
+    const double d = static_cast<double>(a + b);
+    s += __hiloint2double(__double2hiint(d) + e0, __double2loint(d));
+  }
+  return s;
+}
+
 // The same relative to the row's maximum dm.
 template <bool VEC>
 __device__ __forceinline__ double slice_sums_below(const float* __restrict__ row, const Args& A, const double* bank,
@@ -253,8 +407,12 @@ __device__ __forceinline__ void segment_terms(Terms& T, const float* __restrict_
     }
   }
 }
-// The token of target t, which lies in the segment at `base`; `before`: the sum in front of it.
-__device__ __forceinline__ int pick(const Terms& T, const Args& A, int base, double before, double t) {
+// The token of target t, which lies in the segment at `base`; `before`: the sum in front of it.  With BOUNDS also the sums up to
+// the token and with it (from > to where t is above the segment's terms).
+template <bool BOUNDS = false>
+__device__ __forceinline__ int pick(const Terms& T, const Args& A, int base, double before, double t, double* from = nullptr,
+                                    double* to = nullptr) {
+  if (BOUNDS) { *from = INFINITY; *to = 0.0; }
   int token = -1;                                              // if rounding leaves t above everything: the last that counts
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
@@ -264,16 +422,28 @@ __device__ __forceinline__ int pick(const Terms& T, const Args& A, int base, dou
       const int f = over ? __ffs(over) - 1 : 31 - __clz(some);
       double c = before + (T.incl[j] - T.run[j]);
       int hit = -1, tail = 0;
+      double below = INFINITY, above = 0.0;
 #pragma unroll
       for (int x = 0; x < 4; ++x) {
+        const double start = c;
         c += T.e[j][x];
         if (T.e[j][x] > kTiny) {
           tail = x;
-          if (hit < 0 && c > t) hit = x;
+          if (hit < 0 && c > t) {
+            hit = x;
+            below = start;
+            above = c;
+          }
         }
       }
       token = base + 128 * j + 4 * f + __shfl_sync(0xffffffffu, hit < 0 ? tail : hit, f);
-      if (over) return token;
+      if (over) {
+        if (BOUNDS) {
+          *from = __shfl_sync(0xffffffffu, below, f);
+          *to = __shfl_sync(0xffffffffu, above, f);
+        }
+        return token;
+      }
     }
     before += __shfl_sync(0xffffffffu, T.incl[j], 31);
   }
@@ -469,19 +639,21 @@ __device__ __forceinline__ void row_below(const Args& A, Sums<CL>& S, int* queue
   }
 }
 
-// This warp's share of the draws of row `seq`; `at`: which of `sums` holds the row.  True, with nothing drawn, if the row is
-// outside the table's range or has many draws (the cluster agrees).
-template <int CL, bool VEC>
-__device__ __forceinline__ bool draws(const Args& A, Sums<CL>* sums, const double* bank, int at, int64_t seq, int slice, int lane) {
+// Draws d0 + turn, d0 + turn + turns, ... below d1 of row `seq`; `at`: which of `sums` holds the row.  True, with nothing drawn,
+// if the row is outside the table's range or has many draws (all that draw from it agree).
+// QUICK: the sums may be quick ones (`quick`), each within kQuickError of the exact one.  The terms of the segment that holds the
+// target are exact ones, so a token whose sums lie further from the target than the errors of both can add up to is the exact
+// sums' token too; a draw for which that cannot be said is marked, and taken by a launch that adds up its row by the table.
+template <int CL, bool VEC, bool QUICK>
+__device__ __forceinline__ bool draws(const Args& A, Sums<CL>* sums, const double* bank, int at, int64_t seq, int64_t d0, int64_t d1,
+                                      int turn, int turns, bool quick, int lane) {
   constexpr int kSlices = CL * kWarps;
-  const int64_t d0 = A.draw_offsets[seq], d1 = A.draw_offsets[seq + 1];
-  const int turn = static_cast<int>((slice + seq) % kSlices);
   float mx = -INFINITY;
   for (int i = lane; i < kSlices; i += 32) mx = fmaxf(mx, sums[at].slice_max[i]);
   mx = warp_max(mx);
   const float top = mx * A.ckf * (1.f / kTable);
   if (!(A.fast && top >= kLowTop && top <= kHighTop) || d1 - d0 > A.many) {   // its first draw's outputs say so meanwhile, and keep the maximum
-    if (slice == 0 && lane == 0) {
+    if (turn == 0 && lane == 0) {
       A.tokens_out[d0] = kLater;
       A.seq_out[d0] = __float_as_int(mx);
     }
@@ -492,11 +664,13 @@ __device__ __forceinline__ bool draws(const Args& A, Sums<CL>* sums, const doubl
   Sums<CL>& S = sums[at];
   double end_b, Z;
   block_ends<CL>(S, lane, end_b, Z);
-  for (int64_t d = d0 + turn; d < d1; d += kSlices) {
+  for (int64_t d = d0 + turn; d < d1; d += turns) {
     const double t = static_cast<double>(A.uniforms[d]) * Z;
     int token = A.vocab - 1;                                   // the answer if t is not below the total
+    bool sure = !(QUICK && quick) || Z != Z;
     if (t == 0.0) {                                            // the first term that is not 0 at all
       token = first_positive(row, A, S.slice_max, kSlices, static_cast<double>(mx), lane);
+      sure = true;
     } else if (t < Z) {
       const int b = __ffs(__ballot_sync(0xffffffffu, lane < CL && end_b > t)) - 1;
       const double start = b ? __shfl_sync(0xffffffffu, end_b, max(b - 1, 0)) : 0.0;
@@ -523,18 +697,244 @@ __device__ __forceinline__ bool draws(const Args& A, Sums<CL>* sums, const doubl
         const int base = L.v0 + s * kSeg;
         Terms T;
         segment_terms<false, VEC>(T, row, A, bank, 0.0, base, min(A.vocab, L.v0 + A.slice), lane);
-        token = pick(T, A, base, before + in_slice, t);
+        if (QUICK) {
+          double from, to;
+          token = pick<true>(T, A, base, before + in_slice, t, &from, &to);
+          const double slack = t * (2.05 * kQuickError);
+          sure = sure || (from <= t - slack && to > t + slack);
+        } else {
+          token = pick(T, A, base, before + in_slice, t);
+        }
       }
     }
     if (lane == 0) {
-      A.tokens_out[d] = token;
+      A.tokens_out[d] = sure ? token : kUnsure;
       A.seq_out[d] = seq;
     }
   }
   return false;
 }
 
-template <int CL, bool VEC>
+template <int THREADS>
+__device__ __forceinline__ void make_table(double* table) {
+  const int tid = threadIdx.x;
+  if (tid < kTable) {
+    const double e = exp2(static_cast<double>(tid) / kTable);
+    table[tid * 16] = __hiloint2double(__double2hiint(e) - (tid << 13), __double2loint(e));
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i0 = 0; i0 < kTable * 16; i0 += THREADS) {
+    const int i = i0 + tid;
+    if ((THREADS == kThreads || i < kTable * 16) && (i & 15)) table[i] = table[i & ~15];
+  }
+}
+
+// What is worked on in turn: draws d0 .. d1 - 1 of `row` (-1: nothing).
+struct Work {
+  int64_t row, d0, d1;
+};
+// The next row with something to draw.
+__device__ __forceinline__ Work next_row(const Args& A, int64_t r, int step) {
+  for (; r < A.n_seq; r += step) {
+    const int64_t d0 = A.draw_offsets[r], d1 = A.draw_offsets[r + 1];
+    if (d1 > d0) return Work{r, d0, d1};
+  }
+  return Work{-1, 0, 0};
+}
+
+// A row per block at a time.  kWarps warps add up the rows one after the other, quick where a row has few draws; kDrawWarps warps
+// make the draws of the rows whose sums are complete (a draw takes 2.9 us, and a warp that made it between two rows held up all
+// others at the end of the next).  The waits are between warps of a block and bounded.
+template <bool VEC>
+__global__ void __launch_bounds__(kRowThreads, 1) branch_rows_kernel(const __grid_constant__ Args A) {
+  ss::grid_dependency_enter();
+  extern __shared__ __align__(16) float ring[];
+  __shared__ Shared<1> S;
+  __shared__ RowShared C;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, step = gridDim.x;
+  const double* bank = S.table + (lane & 15);
+  volatile int* abort_flag = &C.abort_flag;
+  const int64_t row0 = A.row0 + static_cast<int64_t>(blockIdx.x);
+  if (tid == 0) {
+    for (int i = 0; i < kSums; ++i) {
+      umma::mbar_init(&C.full[i], kWarps);
+      umma::mbar_init(&C.free[i], kDrawWarps);
+    }
+    C.abort_flag = C.later = 0;
+    umma::fence_barrier_init();
+  }
+  const Slice L = slice_of(A, min(warp, kWarps - 1));
+  const int n_seg = (L.n_half + 1) >> 1, end = min(A.vocab, L.v0 + A.slice);
+  const int n_whole = end > L.v0 ? (end - L.v0) / kSeg : 0;    // segments without an end
+  const uint32_t my_ring = umma::smem_u32(ring) + (min(warp, kWarps - 1) * kStages * kSeg + 4 * lane) * 4;
+  Work now = next_row(A, row0, step), req = now;
+  int req_seg = 0, req_stage = 0, stage = 0;
+  // The requests run kStages - 1 segments ahead of the sums, into the rows that follow; a group is closed for every segment, asked
+  // for or not.
+  auto request_next = [&]() {
+    if (req.row >= 0 && n_seg > 0) {
+      const uint32_t dst = my_ring + req_stage * (kSeg * 4);
+      if (VEC && req_seg < n_whole)
+        request_whole(dst, A.logits + (req.row * A.vocab + L.v0 + req_seg * kSeg + 4 * lane));
+      else
+        request<VEC>(dst, A.logits + req.row * A.vocab, L.v0 + req_seg * kSeg, end, lane);
+      if (++req_seg == n_seg) {
+        req_seg = 0;
+        req = next_row(A, req.row + step, step);
+      }
+    }
+    req_stage = req_stage == kStages - 1 ? 0 : req_stage + 1;
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if (warp < kWarps) {
+#pragma unroll 1
+    for (int x = 0; x < kStages - 1; ++x) request_next();
+  }
+  make_table<kRowThreads>(S.table);
+  __syncthreads();
+
+  uint32_t count = 0;                                          // rows so far: their sums lie in turn in the kSums places
+  if (warp < kWarps) {
+    for (; now.row >= 0; ++count) {
+      const int at = count % kSums;
+      if (count >= kSums && !umma::mbar_wait(&C.free[at], (count / kSums - 1) & 1, abort_flag)) break;
+      const bool quick = A.fast && now.d1 - now.d0 <= A.quick_draws;
+      double sum = 0.0;
+      float mx = -INFINITY;
+      QuickState q;
+      q.mx = -INFINITY;
+      quick_base(q, A, -330.f);
+      auto next_segment = [&](float (&l)[16]) {
+        request_next();
+        asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 1) : "memory");
+        read_segment(my_ring + stage * (kSeg * 4), l);
+        stage = stage == kStages - 1 ? 0 : stage + 1;
+      };
+      if (quick) {
+        double mine = 0.0;                                     // of segment `lane`
+#pragma unroll 1
+        for (int s = 0; s < n_seg; s += 4) {
+          double v[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            v[k] = 0.0;
+            if (s + k < n_seg) {
+              float l[16];
+              next_segment(l);
+              v[k] = quick_sums(l, A, q);
+            }
+          }
+          const double four = __shfl_sync(0xffffffffu, warp_sums_4(v, lane), (lane & 3) * 8);
+          if ((lane & ~3) == s) mine = four;
+        }
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const double y = __shfl_up_sync(0xffffffffu, mine, o);
+          if (lane >= o) mine += y;
+        }
+        if (lane < n_seg) S.sums[at].seg_end[warp][lane] = mine;
+        sum = __shfl_sync(0xffffffffu, mine, 31);
+      } else {
+#pragma unroll 1
+        for (int s = 0; s < n_seg; ++s) {
+          float l[16];
+          next_segment(l);
+          if (A.fast) {
+            sum += warp_sum_d(exact_sums(l, A, bank, mx));
+            if (lane == 0) S.sums[at].seg_end[warp][s] = sum;
+          } else {
+#pragma unroll
+            for (int x = 0; x < 16; ++x) mx = fmaxf(mx, l[x]);
+          }
+        }
+      }
+      if (quick) {
+        if (__any_sync(0xffffffffu, q.mx != q.mx)) sum = __longlong_as_double(0x7ff8000000000000ll);   // (as the exact sums would be)
+        mx = q.mx;
+      }
+      mx = warp_max(mx);
+      if (lane == 0) {
+        S.sums[at].slice_sum[warp] = sum;
+        S.sums[at].slice_max[warp] = mx;
+      }
+      __syncwarp();                                            // (every lane has written a segment's end)
+      if (lane == 0) umma::mbar_arrive(&C.full[at]);
+      now = next_row(A, now.row + step, step);
+    }
+  } else {
+    bool later = false;                                        // a row outside the table's range: for when the others are done
+    for (; now.row >= 0; ++count) {
+      const int at = count % kSums;
+      if (!umma::mbar_wait(&C.full[at], (count / kSums) & 1, abort_flag)) break;
+      __syncwarp();
+      const int turn = (warp + static_cast<int>(now.row)) % kDrawWarps;
+      later |= draws<1, VEC, true>(A, S.sums, bank, at, now.row, now.d0, now.d1, turn, kDrawWarps,
+                                   A.fast && now.d1 - now.d0 <= A.quick_draws, lane);
+      __syncwarp();
+      if (lane == 0) umma::mbar_arrive(&C.free[at]);
+      now = next_row(A, now.row + step, step);
+    }
+    if (later && lane == 0) C.later = 1;
+  }
+  __syncthreads();                                             // (the marks; and nobody reads the running sums any more)
+  if (C.later && !C.abort_flag) {
+    for (Work r = next_row(A, row0, step); r.row >= 0; r = next_row(A, r.row + step, step)) {
+      if (__ldcg(A.tokens_out + r.d0) != kLater) continue;     // (read in front of row_below's barriers, written behind them)
+      if (warp < kWarps) {
+        row_below<1, VEC>(A, S.sums[0], S.queue[warp], bank, r.row, warp, lane, __int_as_float(static_cast<int>(__ldcg(A.seq_out + r.d0))));
+      } else {                                                 // (its two barriers)
+        cg::this_cluster().sync();
+        cg::this_cluster().sync();
+      }
+    }
+  }
+}
+
+// The cluster's next marked draw among those of the rows in front of this launch's: its first block looks at 4096 draws at a time
+// and takes the first mark behind a place of the cluster's own, until one is its.
+template <int CL>
+__device__ __forceinline__ Work next_unsure(cg::cluster_group& cl, const Args& A, Shared<CL>& S, int64_t& scanned, int cluster, int n_clusters) {
+  constexpr int kScan = 8 * kThreads;
+  const int tid = threadIdx.x;
+  const int64_t first = A.draw_offsets[0], count = A.draw_offsets[A.row0] - first;
+  if (cl.block_rank() == 0) {
+    int64_t found = -1;
+    while (found < 0 && scanned < count) {
+      const int left = static_cast<int>(count - scanned < kScan ? count - scanned : kScan);
+      const int start = static_cast<int>(static_cast<int64_t>(cluster - A.first_idle) * left / (n_clusters - A.first_idle));
+      if (tid == 0) S.pick = INT32_MAX;
+      __syncthreads();
+      int key = INT32_MAX;
+#pragma unroll
+      for (int k = 0; k < kScan / kThreads; ++k) {
+        const int i = k * kThreads + tid;
+        if (i < left && __ldcg(A.tokens_out + first + scanned + i) == kUnsure) key = min(key, (i - start) & (kScan - 1));
+      }
+      if (key != INT32_MAX) atomicMin(&S.pick, key);
+      __syncthreads();
+      const int pick = S.pick;
+      if (pick == INT32_MAX) {
+        scanned += kScan;
+      } else {
+        const int64_t d = first + scanned + ((pick + start) & (kScan - 1));
+        if (tid == 0) S.taken = atomicCAS(A.tokens_out + d, kUnsure, kTaken) == kUnsure ? 1 : 0;
+        __syncthreads();
+        if (S.taken) found = d - first;
+      }
+      __syncthreads();
+    }
+    if (tid < CL) cl.map_shared_rank(&S, tid)->taken = static_cast<int>(found);
+  }
+  cl.sync();
+  const int i = S.taken;
+  cl.sync();                                                   // (it is written to again)
+  if (i < 0) return Work{-1, 0, 0};
+  return Work{__ldcg(A.seq_out + first + i), first + i, first + i + 1};
+}
+
+// A row per cluster at a time; UNSURE: then the draws that the launch before this one has marked.
+template <int CL, bool VEC, bool UNSURE>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kThreads, 1)
 branch_sample_kernel(const __grid_constant__ Args A) {
   ss::grid_dependency_enter();
@@ -544,23 +944,18 @@ branch_sample_kernel(const __grid_constant__ Args A) {
   const int slice = static_cast<int>(cl.block_rank()) * kWarps + warp;
   const Slice L = slice_of(A, slice);
   const double* bank = S.table + (lane & 15);
+  const int cluster = blockIdx.x / CL, n_clusters = gridDim.x / CL;
+  const int64_t row0 = A.row0 + static_cast<int64_t>(cluster);
+  float first[8];
+  if (row0 < A.n_seq) load_half<VEC>(A.logits + row0 * A.vocab, L.v0, A.vocab, lane, first);   // in flight while the table is made
   // rows with something to draw, in turn (the cluster's blocks agree)
   auto next_row = [&](int64_t r) {
-    while (r < A.n_seq && A.draw_offsets[r + 1] <= A.draw_offsets[r]) r += gridDim.x / CL;
+    while (r < A.n_seq && A.draw_offsets[r + 1] <= A.draw_offsets[r]) r += n_clusters;
     return r;
   };
-  const int64_t row0 = A.row0 + static_cast<int64_t>(blockIdx.x / CL);   // (there are no more clusters than rows)
-  float first[8];
-  load_half<VEC>(A.logits + row0 * A.vocab, L.v0, A.vocab, lane, first);   // in flight while the table is made
   int64_t row = next_row(row0), prev = -1;
   if (row != row0 && row < A.n_seq) load_half<VEC>(A.logits + row * A.vocab, L.v0, A.vocab, lane, first);
-  if (tid < kTable) {
-    const double e = exp2(static_cast<double>(tid) / kTable);
-    S.table[tid * 16] = __hiloint2double(__double2hiint(e) - (tid << 13), __double2loint(e));
-  }
-  __syncthreads();
-  for (int i = tid; i < kTable * 16; i += kThreads)
-    if (i & 15) S.table[i] = S.table[i & ~15];
+  make_table<kThreads>(S.table);
   cl.sync();                                                   // (the table; and every block runs before it is written to)
 
   int at = 0, prev_at = 0;
@@ -582,12 +977,13 @@ branch_sample_kernel(const __grid_constant__ Args A) {
         }
       }
       mx = warp_max(mx);
-      after = next_row(row + gridDim.x / CL);
+      after = next_row(row + n_clusters);
       if (after < A.n_seq) load_half<VEC>(A.logits + after * A.vocab, L.v0, A.vocab, lane, first);
     }
     if (prev >= 0) {
       cluster_wait();
-      later |= draws<CL, VEC>(A, S.sums, bank, prev_at, prev, slice, lane);
+      later |= draws<CL, VEC, false>(A, S.sums, bank, prev_at, prev, A.draw_offsets[prev], A.draw_offsets[prev + 1],
+                                     static_cast<int>((slice + prev) % (CL * kWarps)), CL * kWarps, false, lane);
     }
     if (!more) break;
     publish<CL>(cl, S.sums[at], slice, lane, sum, mx);
@@ -599,13 +995,41 @@ branch_sample_kernel(const __grid_constant__ Args A) {
   }
   if (later) {                                                 // (the cluster agrees)
     cl.sync();                                                 // (the marks; and nobody reads the running sums any more)
-    for (int64_t r = next_row(row0); r < A.n_seq; r = next_row(r + gridDim.x / CL)) {
+    for (int64_t r = next_row(row0); r < A.n_seq; r = next_row(r + n_clusters)) {
       const int64_t d = A.draw_offsets[r];
       if (__ldcg(A.tokens_out + d) != kLater) continue;        // (read in front of row_below's barriers, written behind them)
       row_below<CL, VEC>(A, S.sums[0], S.queue[warp], bank, r, slice, lane, __int_as_float(static_cast<int>(__ldcg(A.seq_out + d))));
     }
   }
+  if (UNSURE && cluster >= A.first_idle) {
+    int64_t scanned = 0;
+    for (;;) {
+      const Work now = next_unsure<CL>(cl, A, S, scanned, cluster, n_clusters);
+      if (now.row < 0) break;
+      const float* p = A.logits + now.row * A.vocab;
+      float mx;
+      load_half<VEC>(p, L.v0, A.vocab, lane, first);
+      const double sum = slice_sums<VEC>(p, A, bank, S.sums[0].seg_end[warp], L.v0, L.n_half, lane, first, mx);
+      publish<CL>(cl, S.sums[0], slice, lane, sum, warp_max(mx));
+      cl.sync();
+      draws<CL, VEC, false>(A, S.sums, bank, 0, now.row, now.d0, now.d1, slice, CL * kWarps, false, lane);
+      cl.sync();
+    }
+  }
   if (CL > 1) cl.sync();                                       // (a block's running sums may still be read by another)
+}
+
+template <bool VEC>
+static bool ring_ready() {
+  static bool configured[kDeviceSlots] = {false};
+  const int slot = current_device_slot();
+  if (slot >= 0 && configured[slot]) return true;
+  if (cudaFuncSetAttribute(branch_rows_kernel<VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  if (slot >= 0) configured[slot] = true;
+  return true;
 }
 
 // Rows row0 .. n_seq-1, `clusters` at a time.
@@ -622,10 +1046,23 @@ static int32_t launch(Args A, bool vec, int row0, int n_seq, int clusters, cudaS
   A.many = CL <= 2 || idle ? CL * kWarps * (4 + A.slice / 384) : INT32_MAX;
   A.row0 = row0;
   A.n_seq = n_seq;
-  if (vec)
-    SS_LAUNCH((branch_sample_kernel<CL, true>), clusters * CL, kThreads, 0, st, A);
-  else
-    SS_LAUNCH((branch_sample_kernel<CL, false>), clusters * CL, kThreads, 0, st, A);
+  if constexpr (CL == 1) {
+    if (!(vec ? ring_ready<true>() : ring_ready<false>())) return SS_ERR_CUDA;
+    if (vec)
+      SS_LAUNCH(branch_rows_kernel<true>, clusters, kRowThreads, kRingBytes, st, A);
+    else
+      SS_LAUNCH(branch_rows_kernel<false>, clusters, kRowThreads, kRingBytes, st, A);
+  } else {
+    const bool unsure = A.first_idle != INT32_MAX;
+    if (vec && unsure)
+      SS_LAUNCH((branch_sample_kernel<CL, true, true>), clusters * CL, kThreads, 0, st, A);
+    else if (vec)
+      SS_LAUNCH((branch_sample_kernel<CL, true, false>), clusters * CL, kThreads, 0, st, A);
+    else if (unsure)
+      SS_LAUNCH((branch_sample_kernel<CL, false, true>), clusters * CL, kThreads, 0, st, A);
+    else
+      SS_LAUNCH((branch_sample_kernel<CL, false, false>), clusters * CL, kThreads, 0, st, A);
+  }
   return SS_OK;
 }
 
@@ -648,8 +1085,8 @@ static int resident_clusters(bool vec) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  const cudaError_t rc = vec ? cudaOccupancyMaxActiveClusters(&n, branch_sample_kernel<CL, true>, &cfg)
-                             : cudaOccupancyMaxActiveClusters(&n, branch_sample_kernel<CL, false>, &cfg);
+  const cudaError_t rc = vec ? cudaOccupancyMaxActiveClusters(&n, branch_sample_kernel<CL, true, true>, &cfg)
+                             : cudaOccupancyMaxActiveClusters(&n, branch_sample_kernel<CL, false, true>, &cfg);
   if (rc != cudaSuccess || n < 1) {
     (void)cudaGetLastError();
     n = 1;
@@ -683,6 +1120,11 @@ extern "C" int32_t ss_branch_sample(const float* logits, const int64_t* draw_off
   A.ckf = static_cast<float>(A.ck);
   A.lowest = static_cast<float>(kLowest / c);
   A.fast = T >= 1e-3 && T <= 1e6;
+  A.c_hi = static_cast<float>(c);
+  A.c_lo = static_cast<float>(c - static_cast<double>(A.c_hi));
+  A.inv_c = static_cast<float>(1.0 / c);
+  A.quick_draws = 0;
+  A.first_idle = INT32_MAX;
   A.lowest_below = kLowest / c;
   const bool vec = reinterpret_cast<uintptr_t>(logits) % 16 == 0 && vocab % 4 == 0;
   cudaStream_t st = as_stream(stream);
@@ -696,14 +1138,25 @@ extern "C" int32_t ss_branch_sample(const float* logits, const int64_t* draw_off
   auto cluster_size = [&](int rows) { return rows <= n8 ? 8 : rows <= n4 ? 4 : rows <= n2 ? 2 : 1; };
   int whole = blocks_min > 1 ? 0 : n_seq / sms * sms;
   if (blocks_min == 1 && cluster_size(n_seq - whole) == 1) whole = n_seq;
+  // Quick sums leave 1.5 % of the draws of a row of 151936 ordinary logits open (9 % if the logits are all equal), each of which
+  // costs another pass over its row, by the table: worth it up to 16 draws of such a row.
+  const bool quick = whole > 0 && A.fast && vocab >= kQuickVocab;
+  if (quick) A.quick_draws = 2500000 / vocab;
   if (whole > 0) {
     const int32_t rc = launch<1>(A, vec, 0, whole, whole < sms ? whole : sms, st);
     if (rc != SS_OK) return rc;
   }
   const int rest = n_seq - whole;
-  if (rest == 0) return SS_OK;
-  const int size = cluster_size(rest) > blocks_min ? cluster_size(rest) : blocks_min;
-  if (size > 4) return launch<8>(A, vec, whole, n_seq, rest < n8 ? rest : n8, st);
-  if (size > 2) return launch<4>(A, vec, whole, n_seq, rest < n4 ? rest : n4, st);
-  return launch<2>(A, vec, whole, n_seq, rest < n2 ? rest : n2, st);
+  if (rest == 0 && !quick) return SS_OK;
+  int size = rest ? cluster_size(rest) : 4;
+  if (size < blocks_min) size = blocks_min;
+  const int resident = size > 4 ? n8 : size > 2 ? n4 : n2;
+  int clusters = rest < resident ? rest : resident;
+  if (quick) {                                                  // marked draws: by the clusters without a row, unless they are few
+    clusters = resident;
+    A.first_idle = (resident - rest) * 4 >= resident ? rest : 0;
+  }
+  if (size > 4) return launch<8>(A, vec, whole, n_seq, clusters, st);
+  if (size > 2) return launch<4>(A, vec, whole, n_seq, clusters, st);
+  return launch<2>(A, vec, whole, n_seq, clusters, st);
 }

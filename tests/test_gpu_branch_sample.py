@@ -236,3 +236,34 @@ def test_many_draws_of_a_row(S, V, most, peak):
     got, sure = tok.cpu().numpy(), margin > 1e-12
     assert np.array_equal(seq.cpu().numpy(), want_seq)
     assert np.array_equal(got[sure], want_tok[sure]) and np.array_equal(got[u == 0.0], want_tok[u == 0.0])
+
+
+@pytest.mark.parametrize("S,V", [(148, 16384), (149, 40961), (222, 151936), (330, 128256)])
+@pytest.mark.parametrize("kind", ["flat", "peaked", "masked"])
+def test_draws_at_the_boundaries_between_tokens(S, V, kind):
+    """Rows that blocks take by themselves, whose sums are first made in fp32: uniforms that lie on a token's end (to fp32), between
+    two ends, at 0 and just below 1, so that many draws cannot be decided from those sums; flat rows, rows with all of their
+    probability on a few tokens, rows that begin and end with masked ones.  Few and many draws of a row."""
+    rng = np.random.default_rng(S + V)
+    logits = (rng.normal(size=(S, V)) * (0.0 if kind == "flat" else 3.0)).astype(np.float32)
+    if kind == "peaked":
+        logits[np.arange(S), rng.integers(0, V, size=S)] = 60.0
+    if kind == "masked":
+        logits[:, : V // 5] = -np.inf
+        logits[:, V - 700:] = -np.inf
+    pot = rng.integers(1, 12, size=S)
+    pot[::50] = 2500000 // V + 5
+    off = np.concatenate([[0], np.cumsum(pot)]).astype(np.int64)
+    u = rng.random(int(off[-1])).astype(np.float32)
+    for s in range(0, S, 3):
+        e = np.exp((logits[s].astype(np.float64) - logits[s].max()) / 0.8)
+        c = np.cumsum(e) / e.sum()
+        u[off[s]: off[s + 1]] = np.minimum(c[rng.integers(0, V, size=pot[s])], 1.0 - 2.0 ** -24).astype(np.float32)
+    u[5::31] = 0.0
+    u[7::37] = np.float32(1.0) - np.float32(2.0 ** -24)
+    tok, seq = run(logits, off, u, 0.8)
+    want_tok, want_seq, margin = oracle.branch_sample(logits, off, u, float(np.float32(0.8)))
+    got, sure = tok.cpu().numpy(), margin > 1e-12
+    assert np.array_equal(seq.cpu().numpy(), want_seq)
+    # (a third of the rows have their targets on the ends: exactly, where 16384 equal logits make those fp32 numbers)
+    assert np.array_equal(got[sure], want_tok[sure]) and sure.mean() > 0.5
