@@ -418,7 +418,9 @@ int32_t ss_candidate_step(const ss_device_step_t* step /* host */, void* stream)
  * u_q_offsets[num_unique]: a duplicate candidate gets no forward pass, hence no output of its own - written by a small
  * kernel straight into the host buffers; the rest of out / lse is left untouched.  (Buffers the device cannot address
  * are returned whole, as without the flag.)
- * Everything is enqueued on `stream`; the call does not synchronise, and it allocates nothing: staging buffers,
+ * Steps of one query row per path write out straight from the attention kernels then.
+ * Everything is enqueued on `stream` - in ss_candidate_step_host_2 with a `copy_stream` the copy of the query rows on that one, behind
+ * what `stream` holds and in front of the attention, so that it overlaps the deduplication; the call does not synchronise, and it allocates no memory: staging buffers,
  * results and the workspaces of the three calls are carved out of `device_arena` (caller-owned, 256-byte aligned,
  * >= ss_candidate_step_host_arena_bytes).  The KV pool and the tree stay resident on the device: they are the
  * cache state of the method, described by the resident fields of `attn` (flags, heads, sm_scale, pool, strides,
@@ -476,6 +478,8 @@ typedef struct ss_host_step {
 int32_t ss_candidate_step_host_arena_bytes(const ss_host_step_t* step /* host */, size_t* out_bytes /* host */);
 int32_t ss_candidate_step_host(const ss_host_step_t* step /* host */, void* device_arena, size_t arena_bytes,
                                void* stream);
+int32_t ss_candidate_step_host_2(const ss_host_step_t* step /* host */, void* device_arena, size_t arena_bytes,
+                                 void* stream, void* copy_stream /* may be NULL */);
 
 /* =========================================================================================================
  * Diagnostics

@@ -40,6 +40,7 @@ EXPORTS = [
     "ss_dedup_paths_static", "ss_debug_tile_kernel_occupancy", "ss_early_prune",
     "ss_branch_sample", "ss_gather_unique_paths", "ss_candidate_step_host_arena_bytes", "ss_candidate_step_host",
     "ss_prefix_tree_workspace_bytes", "ss_build_prefix_tree", "ss_candidate_step",
+    "ss_candidate_step_host_2",
 ]
 PHASES = ["plan", "tiles", "leaves", "generic", "merge"]
 
@@ -84,7 +85,7 @@ _SIGNATURES = {
     "ss_tree_attention_workspace_bytes": "pp", "ss_tree_attention": "ppzp", "ss_topk_workspace_bytes": "ip",
     "ss_topk_prune": "ppiiipppzp", "ss_early_prune": "pppiiippppzp", "ss_branch_sample": "pppiifppp",
     "ss_prefix_tree_workspace_bytes": "iqip", "ss_build_prefix_tree": "ppiqippppppppzp",
-    "ss_candidate_step": "pp", "ss_candidate_step_host_arena_bytes": "pp", "ss_candidate_step_host": "ppzp", "ss_profile_enable": "i",
+    "ss_candidate_step": "pp", "ss_candidate_step_host_arena_bytes": "pp", "ss_candidate_step_host": "ppzp", "ss_candidate_step_host_2": "ppzpp", "ss_profile_enable": "i",
     "ss_profile_read": "pp", "ss_debug_umma_tile": "pppiiipp", "ss_debug_bounded_wait": "pp",
 }
 
@@ -291,12 +292,13 @@ def ss_candidate_step_host_arena_bytes(step: ss_host_step_t) -> int:
     return int(out.value)
 
 
-def ss_candidate_step_host(step: ss_host_step_t, device_arena: torch.Tensor, stream=None, check=True) -> int:
+def ss_candidate_step_host(step: ss_host_step_t, device_arena: torch.Tensor, stream=None, check=True,
+                           copy_stream=None) -> int:
     """The whole path for host-resident per-step data: copies in, dedup, gather, attention, top-k, copies out; all
-    asynchronous on `stream`."""
-    rc = lib().ss_candidate_step_host(ctypes.byref(step), _ptr(device_arena),
-                                      device_arena.numel() * device_arena.element_size(),
-                                      _stream(stream))
+    asynchronous on `stream` (the copy of the query rows on `copy_stream`, if one is given)."""
+    rc = lib().ss_candidate_step_host_2(ctypes.byref(step), _ptr(device_arena),
+                                        device_arena.numel() * device_arena.element_size(),
+                                        _stream(stream), _stream(copy_stream) if copy_stream is not None else None)
     if check:
         _check(rc, "ss_candidate_step_host")
     return rc

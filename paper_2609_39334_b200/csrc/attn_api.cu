@@ -4,6 +4,7 @@
 #include <string.h>
 
 #include "attn_plan.cuh"
+#include "step.cuh"
 
 namespace ss {
 namespace attn {
@@ -140,9 +141,8 @@ extern "C" int32_t ss_tree_attention_workspace_bytes(const ss_attn_desc_t* desc,
   return SS_OK;
 }
 
-extern "C" int32_t ss_tree_attention(const ss_attn_desc_t* d, void* workspace, size_t workspace_bytes, void* stream) {
-  using namespace ss;
-  using namespace ss::attn;
+int32_t ss::attn::tree_attention(const ss_attn_desc_t* d, void* workspace, size_t workspace_bytes, void* stream, cudaEvent_t q_ready,
+                                 bool out_on_host) {
   int32_t rc = check_desc(d);
   if (rc != SS_OK) return rc;
   if (!workspace || reinterpret_cast<uintptr_t>(workspace) % kAlign) return SS_ERR_INVALID_ARG;
@@ -196,6 +196,7 @@ extern "C" int32_t ss_tree_attention(const ss_attn_desc_t* d, void* workspace, s
   int sms = sm_count_of_current_device();
   if (d->max_sms > 0 && d->max_sms < sms) sms = d->max_sms;
   P.sms = sms;
+  P.short_first = out_on_host ? 1 : 0;
   const bool timed = prof_begin_call();
   const int call = g_prof.used;
   // phase boundaries: event e is recorded before phase e, event SS_NUM_PHASES after the last one
@@ -206,6 +207,10 @@ extern "C" int32_t ss_tree_attention(const ss_attn_desc_t* d, void* workspace, s
   mark(SS_PHASE_PLAN);
   rc = launch_plan(P, st);
   ran(SS_PHASE_PLAN);
+  if (q_ready && cudaStreamWaitEvent(st, q_ready, 0) != cudaSuccess) {
+    (void)cudaGetLastError();
+    rc = rc == SS_OK ? SS_ERR_CUDA : rc;
+  }
   mark(SS_PHASE_TILES);
   if (rc == SS_OK && any && !generic_only) {
     const bool two_cta = (d->flags & SS_FLAG_TILES_2CTA) != 0;
@@ -234,6 +239,10 @@ extern "C" int32_t ss_tree_attention(const ss_attn_desc_t* d, void* workspace, s
   mark(SS_NUM_PHASES);
   if (timed) ++g_prof.used;
   return rc;
+}
+
+extern "C" int32_t ss_tree_attention(const ss_attn_desc_t* d, void* workspace, size_t workspace_bytes, void* stream) {
+  return ss::attn::tree_attention(d, workspace, workspace_bytes, stream, nullptr, false);
 }
 
 extern "C" int32_t ss_profile_enable(int32_t on) {

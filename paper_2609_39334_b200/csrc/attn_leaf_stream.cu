@@ -29,6 +29,8 @@ using namespace umma;
 
 constexpr int kBlockBytes = 4096;          // one (page, kv head) block of K or of V: 16 rows x 256 B
 constexpr int kStageBytes = 2 * kBlockBytes;
+constexpr int kOutRow = 272;               // bytes between two rows of a warp's 8 final rows in shared memory (no bank conflicts)
+constexpr int kOutBytes = 8 * kOutRow;
 constexpr int kClaimAhead = 5;             // pages before an item's end at which the next one is claimed (three dependent
                                            // loads, two pages requested ahead)
 constexpr float kLazyLog2 = 8.0f;          // the running maximum of a row moves only when exceeded by 2^8
@@ -39,7 +41,8 @@ struct Cfg {
   static constexpr int kWarps = WARPS;
   static constexpr int kStages = STAGES;
   static constexpr int kRingBytes = STAGES * kStageBytes;
-  static constexpr int kSmem = WARPS * kRingBytes + 1024;      // + slack for the 1024-byte alignment
+  static constexpr int kOffOut = WARPS * kRingBytes;           // a warp's final rows on their way out
+  static constexpr int kSmem = kOffOut + WARPS * kOutBytes + 1024;   // + slack for the 1024-byte alignment
 };
 
 __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
@@ -110,6 +113,7 @@ leaf_stream_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   uint8_t* ring_ptr = smem + warp * C::kRingBytes;
   const uint32_t ring = smem_u32(ring_ptr);
+  uint8_t* out_rows = smem + C::kOffOut + warp * kOutBytes;
   if (tid == 0) {
     abort_flag_s = 0;
     prefetch_tensormap(&tmap_k);
@@ -389,27 +393,36 @@ leaf_stream_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
           }
         }
       }
+      // bf16 rows, through shared memory: the rows of a group lie one after the other, 16 bytes a lane (a row at a time is what
+      // the bus takes well where `out` is host memory)
 #pragma unroll
-      for (int nt = 0; nt < NT; ++nt)
+      for (int nt = 0; nt < NT; ++nt) {
 #pragma unroll
         for (int x = 0; x < 2; ++x) {
           const int q = 8 * nt + 2 * tig + x;
-          const bool q_live = q < G;
-          const int h = cur.g * G + (q_live ? q : 0);
           const float inv = den[nt][x] > 0.f ? 1.f / den[nt][x] : 0.f;
-          // bf16 rows: lanes gid and gid ^ 1 hold neighbouring dims; the even one stores the pair of the lower 8 dims
-          // of each 16-dim tile, the odd one the pair of the upper 8
-          __nv_bfloat16* dst = P.out + (q_row * P.Hq + h) * kHeadDim + (gid & ~1) + ((gid & 1) ? 8 : 0);
+          // lanes gid and gid ^ 1 hold neighbouring dims; the even one stores the pair of the lower 8 dims of each 16-dim
+          // tile, the odd one the pair of the upper 8
+          uint8_t* dst = out_rows + (2 * tig + x) * kOutRow + ((gid & ~1) + ((gid & 1) ? 8 : 0)) * 2;
 #pragma unroll
           for (int mt = 0; mt < 8; ++mt) {
             const float lo = o[mt][nt][x] * inv, hi = o[mt][nt][2 + x] * inv;
             const float got = __shfl_xor_sync(0xffffffffu, (gid & 1) ? lo : hi, 4);
-            const uint32_t pk = (gid & 1) ? pack_bf16(got, hi) : pack_bf16(lo, got);
-            if (q_live && row_ok) *reinterpret_cast<uint32_t*>(dst + 16 * mt) = pk;
+            *reinterpret_cast<uint32_t*>(dst + 32 * mt) = (gid & 1) ? pack_bf16(got, hi) : pack_bf16(lo, got);
           }
-          if (q_live && row_ok && gid == 0 && P.lse)
-            P.lse[q_row * P.Hq + h] = den[nt][x] > 0.f ? big[nt][x] + __logf(den[nt][x]) : -INFINITY;
+          if (q < G && row_ok && gid == 0 && P.lse)
+            P.lse[q_row * P.Hq + cur.g * G + q] = den[nt][x] > 0.f ? big[nt][x] + __logf(den[nt][x]) : -INFINITY;
         }
+        __syncwarp();
+        __nv_bfloat16* rows = P.out + (q_row * P.Hq + cur.g * G + 8 * nt) * kHeadDim;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int r = 2 * k + (lane >> 4), part = lane & 15;
+          const uint4 v = *reinterpret_cast<const uint4*>(out_rows + r * kOutRow + part * 16);
+          if (8 * nt + r < G && row_ok) *reinterpret_cast<uint4*>(rows + r * kHeadDim + part * 8) = v;
+        }
+        __syncwarp();
+      }
     } else {
       bool slot_ok = true;
       SS_CHECK_OR(cur.slot >= 0 && cur.slot < P.caps.slots, &P.hdr->status, slot_ok = false);

@@ -325,6 +325,7 @@ __device__ __forceinline__ bool make_plan(const Params& P, const PlanArrays& A, 
           if (count(A.n_paths + leaf) == 1 && len > 0) {
             full = len / kLeafChunk;
             c = ceil_div(len - full * kLeafChunk, kPage);
+            if (!LARGE && P.short_first && c > 0) c = kLeafClasses - c;
           }
         } else if (A.p_class[i] == kClassChain) {
           chain = ceil_div(A.p_T[i], tpt) * Hkv;
@@ -412,6 +413,7 @@ __device__ __forceinline__ void emit_items(const Params& P, const PlanArrays& A,
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int N = P.num_nodes, Hkv = P.Hkv, tpt = P.tok_per_tile;
   const int live = hdr->live_paths, n_stacked = hdr->n_stacked_items, n_full = hdr->n_full_leaf_items;
+  const int full0 = !LARGE && P.short_first ? hdr->n_leaf_items - n_full : 0, last0 = P.short_first ? 0 : n_full;
   const int wid = blockIdx.x * (blockDim.x / 32) + warp, nw = gridDim.x * (blockDim.x / 32);
   auto page0_of = [&](int n) { return LARGE ? static_cast<int32_t>(P.node_page_offsets[n]) : A.n_page0[n]; };
   if (wid == 0 && lane == 0) P.dec_slot_base[hdr->n_dec] = hdr->n_slots;
@@ -438,7 +440,9 @@ __device__ __forceinline__ void emit_items(const Params& P, const PlanArrays& A,
       // The leaf kernel hands its items out in this order.  Small form: whole chunks first, then the last chunks of all leaves,
       // longest first, so that the short ones level out the warps' ends (922 leaves of 32 to 512 keys: 71.6 -> 68.9 us).  Large
       // form: leaf after leaf; with many items per warp the order by length only costs (6550 leaves of 128 to 1024 keys: 2.46 ms,
-      // whole chunks first 2.43, leaf after leaf 2.37)
+      // whole chunks first 2.43, leaf after leaf 2.37).  Where the rows go over the bus as the leaves are done, the small form
+      // turns its order round, so that the bus is not idle until the longest ones are (a step of 1024 paths from host buffers
+      // 227 -> 214 us)
       const int page0 = page0_of(leaf), full = len / kLeafChunk, n_items = ceil_div(len, kLeafChunk) * Hkv;
       const int last = LARGE ? 0 : A.p_last[p];
 #pragma unroll 1
@@ -453,7 +457,7 @@ __device__ __forceinline__ void emit_items(const Params& P, const PlanArrays& A,
         it.slot = slot + A.n_level[leaf] + c;
         it.q_src = src;
         it.dec = rank;
-        P.leaf_items[LARGE || c < full ? A.p_items[p] * Hkv + x : n_full + last * Hkv + g] = it;
+        P.leaf_items[LARGE || c < full ? full0 + A.p_items[p] * Hkv + x : last0 + last * Hkv + g] = it;
       }
     } else if (cls == kClassChain) {
       const int T = A.p_T[p], tiles = ceil_div(T, tpt);

@@ -145,6 +145,7 @@ struct Params {
   float* lse;
   int32_t target_tiles;      // the planner splits root nodes until about this many tile items exist
   int32_t sms;               // SMs the call may use
+  int32_t short_first;       // small planner: short leaves first (see emit_items)
   Caps caps;
   // ---- workspace regions ----
   PlanHeader* hdr;

@@ -17,6 +17,7 @@
 // third compacts with a block per 1024 paths.  Latency-bound: a few MB of ids, a handful of dependent trips to L2.
 // Measured, the call: 1024 paths 35 -> 14 us (a bitonic sort of the hashes and binary searches by one block before),
 // 8192 paths 78 -> 28 us (a sort by counting, a compaction by one block).
+#include "step.cuh"
 #include "topk.cuh"
 
 namespace ss {
@@ -836,11 +837,8 @@ static bool front_args_ok(const ss_device_step_t& s) {
 }  // namespace dedup
 }  // namespace ss
 
-extern "C" int32_t ss_candidate_step(const ss_device_step_t* step, void* stream) {
-  using namespace ss;
+int32_t ss::candidate_step(const ss_device_step_t& s, void* stream, cudaEvent_t q_ready, bool out_on_host) {
   using namespace ss::dedup;
-  if (!step || step->struct_size != sizeof(ss_device_step_t) || !step->attn) return SS_ERR_INVALID_ARG;
-  const ss_device_step_t& s = *step;
   const int n = s.n_paths;
   // The selection shares the front's launches where 256 threads (1024 in the cluster form) are as many as its own launch would
   // take, and its segments are not many times the other blocks.
@@ -849,7 +847,7 @@ extern "C" int32_t ss_candidate_step(const ss_device_step_t* step, void* stream)
   int32_t rc;
   if (front) {
     rc = launch_front(s, as_stream(stream));
-    return rc != SS_OK ? rc : ss_tree_attention(s.attn, s.attn_workspace, s.attn_workspace_bytes, stream);
+    return rc != SS_OK ? rc : attn::tree_attention(s.attn, s.attn_workspace, s.attn_workspace_bytes, stream, q_ready, out_on_host);
   }
   rc = ss_dedup_paths(s.tok_ids, s.tok_offsets, s.ctx_key, s.slot_in, n, s.dedup_flags, s.canon, s.path_to_unique, s.unique_paths,
                       s.multiplicity, s.slot_out, s.num_unique, s.dedup_workspace, s.dedup_workspace_bytes, stream);
@@ -857,8 +855,13 @@ extern "C" int32_t ss_candidate_step(const ss_device_step_t* step, void* stream)
   rc = ss_gather_unique_paths(s.unique_paths, s.num_unique, n, s.path_leaf_node, s.path_q_len, s.q_offsets, s.u_leaf, s.u_q_len,
                               s.u_q_offsets, s.u_q_src, stream);
   if (rc != SS_OK) return rc;
-  rc = ss_tree_attention(s.attn, s.attn_workspace, s.attn_workspace_bytes, stream);
+  rc = attn::tree_attention(s.attn, s.attn_workspace, s.attn_workspace_bytes, stream, q_ready, out_on_host);
   if (rc != SS_OK) return rc;
   return ss_topk_prune(s.scores, s.seg_offsets, s.n_segments, n, s.top_k, s.survivors, s.keep, s.topk_workspace, s.topk_workspace_bytes,
                        stream);
+}
+
+extern "C" int32_t ss_candidate_step(const ss_device_step_t* step, void* stream) {
+  if (!step || step->struct_size != sizeof(ss_device_step_t) || !step->attn) return SS_ERR_INVALID_ARG;
+  return ss::candidate_step(*step, stream, nullptr, false);
 }

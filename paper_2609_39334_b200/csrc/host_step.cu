@@ -17,10 +17,11 @@
 //
 // Small arrays (a copy of a few KB costs its place in the stream, 2 to 4 us, whatever its size; a decode step has 8 in and
 // 9 out) go through one kernel per direction that reads or writes the mapped host memory, if it is page-locked; arrays
-// above kSmallBytes keep their copy engine.  Measured, a step of 1024 decode paths: 330 -> 278 us.  Arrays that do not start on 16
+// above kSmallBytes keep their copy engine.  Measured, a step of 1024 decode paths: 330 -> 278 us; with the query rows on a stream of
+// their own, the arrays moved side by side and the rows written by the attention kernels 280 -> 214.  Arrays that do not start on 16
 // bytes are moved a byte per thread, which still beats the copies up to a few KB (8 paths 138 -> 67 us a step, 1024 265 -> 216; 4096
 // with three sets in flight 350 -> 457).
-#include "common.cuh"
+#include "step.cuh"
 
 namespace ss {
 namespace host_step {
@@ -29,11 +30,13 @@ constexpr size_t kSmallBytes = 64 << 10;      // three sets in flight, 4096 deco
                                               // 350; one at a time, 1024 paths: 227, 207, 206, 208; 16384: 2341, 2332, 2297, 2282
 constexpr int kMaxSegments = 12;
 
-// Arrays to move, one after the other.
+// Arrays to move, as one sequence of units of 16 bytes (the last of an array may be shorter): a thread has a unit, whichever array
+// it is of, so that a trip over the bus serves all of them (array after array, eight of them took 17 us of a decode step).
 struct Segments {
   const char* src[kMaxSegments];
   char* dst[kMaxSegments];
-  unsigned int bytes[kMaxSegments];
+  unsigned int bytes[kMaxSegments], first[kMaxSegments];   // first: unit
+  unsigned int units;
   int count;
 };
 
@@ -54,15 +57,46 @@ static char* mapped(const void* host, size_t bytes) {
 }
 
 __device__ __forceinline__ void move_segments(const Segments& S, int block, int n_blocks) {
-  for (int i = 0; i < S.count; ++i) {
-    const char* src = S.src[i];
-    char* dst = S.dst[i];
-    const unsigned int n = S.bytes[i], step = n_blocks * blockDim.x, t = block * blockDim.x + threadIdx.x;
-    if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0) {
-      for (unsigned int c = t; c < n / 16; c += step) reinterpret_cast<uint4*>(dst)[c] = reinterpret_cast<const uint4*>(src)[c];
-      for (unsigned int c = n / 16 * 16 + t; c < n; c += step) dst[c] = src[c];
-    } else {
-      for (unsigned int c = t; c < n; c += step) dst[c] = src[c];
+  constexpr int kAhead = 4;
+  const unsigned int step = n_blocks * blockDim.x;
+  for (unsigned int u0 = block * blockDim.x + threadIdx.x; u0 < S.units; u0 += kAhead * step) {
+    uint4 v[kAhead];
+    char* dst[kAhead];
+    unsigned int n[kAhead];                                // bytes; 16 in one piece: 17
+#pragma unroll
+    for (int a = 0; a < kAhead; ++a) {
+      const unsigned int u = u0 + a * step;
+      n[a] = 0;
+      dst[a] = nullptr;
+      v[a] = make_uint4(0, 0, 0, 0);
+      if (u >= S.units || u < u0) continue;
+      int i = 0;
+      while (i + 1 < S.count && S.first[i + 1] <= u) ++i;
+      const unsigned int at = (u - S.first[i]) * 16;
+      const char* src = S.src[i] + at;
+      dst[a] = S.dst[i] + at;
+      n[a] = min(16u, S.bytes[i] - at);
+      if (n[a] == 16 && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst[a])) & 15) == 0) {
+        v[a] = *reinterpret_cast<const uint4*>(src);
+        n[a] = 17;
+      } else {
+        uint32_t w[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int x = 0; x < 16; ++x)
+          if (x < n[a]) w[x >> 2] |= static_cast<uint32_t>(static_cast<unsigned char>(src[x])) << (8 * (x & 3));
+        v[a] = make_uint4(w[0], w[1], w[2], w[3]);
+      }
+    }
+#pragma unroll
+    for (int a = 0; a < kAhead; ++a) {
+      if (n[a] == 17) {
+        *reinterpret_cast<uint4*>(dst[a]) = v[a];
+      } else {
+        const uint32_t w[4] = {v[a].x, v[a].y, v[a].z, v[a].w};
+#pragma unroll
+        for (int x = 0; x < 16; ++x)
+          if (x < n[a]) dst[a][x] = static_cast<char>(w[x >> 2] >> (8 * (x & 3)));
+      }
     }
   }
 }
@@ -125,6 +159,31 @@ struct Arena {                       // device-side layout of one step
   void* attn_ws; size_t attn_ws_bytes;
   void* topk_ws; size_t topk_ws_bytes;
   size_t total;
+};
+
+// The copy of the query rows on a stream of its own: behind what `st` holds when it starts (the arena's last user), in front of
+// what waits for `ready`.  However the call ends, `st` waits for it.
+struct QueryCopy {
+  cudaStream_t st, other;
+  cudaEvent_t ready = nullptr;
+  bool start(void* dst, const void* src, size_t bytes) {
+    cudaEvent_t begin = nullptr;
+    bool ok = cudaEventCreateWithFlags(&begin, cudaEventDisableTiming) == cudaSuccess &&
+              cudaEventCreateWithFlags(&ready, cudaEventDisableTiming) == cudaSuccess && cudaEventRecord(begin, st) == cudaSuccess &&
+              cudaStreamWaitEvent(other, begin, 0) == cudaSuccess;
+    if (ok) {
+      const bool copied = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, other) == cudaSuccess;
+      ok = cudaEventRecord(ready, other) == cudaSuccess && copied;
+    }
+    if (begin) cudaEventDestroy(begin);                        // (an event in use goes when it is through)
+    if (!ok) (void)cudaGetLastError();
+    return ok;
+  }
+  ~QueryCopy() {
+    if (!ready) return;
+    if (cudaStreamWaitEvent(st, ready, 0) != cudaSuccess) (void)cudaGetLastError();
+    cudaEventDestroy(ready);
+  }
 };
 
 static size_t at_least_one(int64_t n) { return static_cast<size_t>(n > 0 ? n : 1); }
@@ -215,6 +274,11 @@ extern "C" int32_t ss_candidate_step_host_arena_bytes(const ss_host_step_t* step
 
 extern "C" int32_t ss_candidate_step_host(const ss_host_step_t* step, void* device_arena, size_t arena_bytes,
                                           void* stream) {
+  return ss_candidate_step_host_2(step, device_arena, arena_bytes, stream, nullptr);
+}
+
+extern "C" int32_t ss_candidate_step_host_2(const ss_host_step_t* step, void* device_arena, size_t arena_bytes,
+                                            void* stream, void* copy_stream) {
   using namespace ss;
   using namespace ss::host_step;
   int32_t rc = check(step);
@@ -252,15 +316,18 @@ extern "C" int32_t ss_candidate_step_host(const ss_host_step_t* step, void* devi
     }
     list.src[list.count] = to_host ? static_cast<const char*>(src) : map;
     list.dst[list.count] = to_host ? map : static_cast<char*>(dst);
+    list.first[list.count] = list.units;
+    list.units += static_cast<unsigned int>((bytes + 15) / 16);
     list.bytes[list.count++] = static_cast<unsigned int>(bytes);
     return true;
   };
+  const bool apart = copy_stream && as_stream(copy_stream) != st && q_bytes > kSmallBytes;   // the query rows on their own stream
   bool ok = move(in, a.tok_ids, s.tok_ids, static_cast<size_t>(s.total_tok) * 4, false) &&
             move(in, a.tok_offsets, s.tok_offsets, (N + 1) * 8, false) &&
             (!s.ctx_key || move(in, a.ctx_key, s.ctx_key, N * 8, false)) &&
             (!s.slot_in || move(in, a.slot_in, s.slot_in, N * 4, false)) &&
             move(in, a.path_leaf_node, s.path_leaf_node, N * 4, false) && move(in, a.path_q_len, s.path_q_len, N * 4, false) &&
-            move(in, a.q_offsets, s.q_offsets, (N + 1) * 8, false) && move(in, a.q, s.q, q_bytes, false) &&
+            move(in, a.q_offsets, s.q_offsets, (N + 1) * 8, false) && (apart || move(in, a.q, s.q, q_bytes, false)) &&
             move(in, a.scores, s.scores, N * 4, false) && move(in, a.seg_offsets, s.seg_offsets, (P + 1) * 4, false);
   if (!ok) return SS_ERR_CUDA;
   // compact return: needs out / lse mapped (the kernel writes them, 16 bytes at a time) and whole 16-byte chunks per row
@@ -273,15 +340,23 @@ extern "C" int32_t ss_candidate_step_host(const ss_host_step_t* step, void* devi
     compact = out_map && (!s.lse || lse_map) && ((reinterpret_cast<uintptr_t>(out_map) | reinterpret_cast<uintptr_t>(lse_map)) & 15) == 0;
   }
   if (in.count > 0) {
-    size_t bytes = 0;
-    for (int i = 0; i < in.count; ++i) bytes += in.bytes[i];
-    const int blocks = static_cast<int>((bytes + 16 * kCopyThreads - 1) / (16 * kCopyThreads));
+    const int blocks = static_cast<int>((in.units + kCopyThreads - 1) / kCopyThreads);
     SS_LAUNCH(small_inputs_kernel, blocks < kCopyBlocks ? blocks : kCopyBlocks, kCopyThreads, 0, st, in);
   }
 
+  // The query rows, which nothing in front of the attention kernels reads: with a second stream they are on their way (62 us for
+  // 1024 paths of 12 heads) while the candidates are deduplicated and the attention is planned.  (Behind the small arrays, which the
+  // deduplication waits for: side by side their kernel took 27 us instead of 8.)
+  QueryCopy queries{st, as_stream(copy_stream)};
+  if (apart && !queries.start(a.q, s.q, q_bytes)) return SS_ERR_CUDA;
+
   // ---- the path ---------------------------------------------------------------------------------------------------
   ss_attn_desc_t d = step_desc(s, a);
-  if (compact && d.max_sms == 0) {
+  // Decode rows (one a path) can be written to the caller's memory by the attention kernels themselves, as the leaves are done:
+  // their 16-byte stores keep the bus as busy as a copy kernel behind them does.
+  const bool direct = compact && s.total_q == s.n_paths && reinterpret_cast<uintptr_t>(out_map) % 32 == 0;
+  if (direct) d.out = out_map;
+  if (compact && !direct && d.max_sms == 0) {
     // the copy kernel of the step before this one (another stream) runs for as long as the bus takes and needs SMs
     // that this step's persistent attention blocks do not hold
     int dev = 0, n_sm = 0;
@@ -306,7 +381,7 @@ extern "C" int32_t ss_candidate_step_host(const ss_host_step_t* step, void* devi
   p.u_leaf = a.u_leaf; p.u_q_len = a.u_q_len; p.u_q_offsets = a.u_q_offsets; p.u_q_src = a.u_q_src;
   p.survivors = a.survivors; p.keep = a.keep;
   p.dedup_workspace = a.dedup_ws; p.attn_workspace = a.attn_ws; p.topk_workspace = a.topk_ws;
-  rc = ss_candidate_step(&p, stream);
+  rc = candidate_step(p, stream, queries.ready, direct);
   if (rc != SS_OK) return rc;
 
   // ---- device -> host: every result ------------------------------------------------------------------------------------
@@ -324,7 +399,7 @@ extern "C" int32_t ss_candidate_step_host(const ss_host_step_t* step, void* devi
     SS_LAUNCH(rows_to_host_kernel, kCopyBlocks, kCopyThreads, 0, st, static_cast<const uint4*>(a.out),
               reinterpret_cast<uint4*>(compact ? out_map : nullptr), reinterpret_cast<const uint4*>(a.lse),
               reinterpret_cast<uint4*>(lse_map), static_cast<const int32_t*>(a.num_unique), s.n_paths,
-              static_cast<const int64_t*>(a.u_q_offsets), static_cast<int64_t>(row * sizeof(__nv_bfloat16) / 16),
+              static_cast<const int64_t*>(a.u_q_offsets), direct ? 0 : static_cast<int64_t>(row * sizeof(__nv_bfloat16) / 16),
               static_cast<int64_t>(s.attn->num_q_heads) * 4, res);
   return SS_OK;
 }

@@ -190,7 +190,8 @@ class HostStepPipeline:
                                     dedup_flags=resident.dedup_flags,
                                     flags=B.SS_STEP_COMPACT_TRANSFERS if compact else 0)
             arena = B.alloc_workspace(B.ss_candidate_step_host_arena_bytes(step), dev)
-            self.sets.append(dict(h_in=h_in, h_out=h_out, step=step, arena=arena, stream=torch.cuda.Stream(dev)))
+            self.sets.append(dict(h_in=h_in, h_out=h_out, step=step, arena=arena, stream=torch.cuda.Stream(dev),
+                                  copy_stream=torch.cuda.Stream(dev)))
         self.h2d_bytes = sum(t.numel() * t.element_size() for t in self.sets[0]["h_in"].values())
         self.d2h_bytes = sum(t.numel() * t.element_size() for t in self.sets[0]["h_out"].values())
 
@@ -215,7 +216,7 @@ class HostStepPipeline:
 
     def submit(self, i: int):
         s = self.sets[i % len(self.sets)]
-        B.ss_candidate_step_host(s["step"], s["arena"], stream=s["stream"])
+        B.ss_candidate_step_host(s["step"], s["arena"], stream=s["stream"], copy_stream=s["copy_stream"])
 
     def synchronize(self):
         for s in self.sets:
