@@ -78,8 +78,8 @@ static Layout carve(const ss_attn_desc_t* d, char* base, Params* P) {
   const int64_t stacked = static_cast<int64_t>(Hkv) * (cap_dec * max_depth / tpt + d->num_nodes) + target + Hkv * kMaxRootSplits;
   const int64_t chain = static_cast<int64_t>(Hkv) * (d->total_q / tpt + d->num_paths);
   caps.tile_items = static_cast<int32_t>(stacked + chain);
-  caps.leaf_items = static_cast<int32_t>(static_cast<int64_t>(Hkv) * (d->total_node_pages * kPage / kLeafChunk + cap_dec));
-  caps.slots = cap_dec * (kMaxRootSplits + max_depth) + d->total_node_pages * kPage / kLeafChunk;
+  caps.leaf_items = static_cast<int32_t>(static_cast<int64_t>(Hkv) * ((d->total_node_pages * kPage >> kLeafChunkLog2) + cap_dec));
+  caps.slots = cap_dec * (kMaxRootSplits + max_depth) + (d->total_node_pages * kPage >> kLeafChunkLog2);
 
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes); return base ? base + o : nullptr; };
@@ -197,6 +197,9 @@ int32_t ss::attn::tree_attention(const ss_attn_desc_t* d, void* workspace, size_
   if (d->max_sms > 0 && d->max_sms < sms) sms = d->max_sms;
   P.sms = sms;
   P.short_first = out_on_host ? 1 : 0;
+  // (by the device's SMs, not by how many of them the call may use: that does not change a result's last bit)
+  P.leaf_log2 = static_cast<int64_t>(P.caps.dec) * P.Hkv >= static_cast<int64_t>(sm_count_of_current_device()) * kLeafStreamWarps
+                    ? kLeafChunkLog2Many : kLeafChunkLog2;
   const bool timed = prof_begin_call();
   const int call = g_prof.used;
   // phase boundaries: event e is recorded before phase e, event SS_NUM_PHASES after the last one

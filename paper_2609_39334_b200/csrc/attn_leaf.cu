@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(kLeafWarps * 32) leaf_items_kernel(const Param
     if (e >= n_items) break;
     const LeafItem it = P.leaf_items[e];
     const int n_keys = it.kv_end - it.kv_begin;
-    const int n_pages = (n_keys + kPage - 1) / kPage;                      // <= 16
+    const int n_pages = (n_keys + kPage - 1) / kPage;                      // <= 32
     const int64_t pg0 = P.node_page_offsets[it.node] + it.kv_begin / kPage;
     int my_page = lane < n_pages ? P.node_pages[pg0 + lane] : 0;
     SS_CHECK_OR(my_page >= 0 && my_page < P.num_pages, &P.hdr->status, my_page = 0);

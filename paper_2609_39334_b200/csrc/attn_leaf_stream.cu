@@ -153,7 +153,7 @@ leaf_stream_kernel(const __grid_constant__ CUtensorMap tmap_k, const __grid_cons
     it.valid = f_e < n_items ? 1 : 0;
     if (!it.valid) return;
     it.g = f_it.g; it.n_keys = f_it.kv_end - f_it.kv_begin; it.slot = f_it.slot; it.dec = f_it.dec;
-    it.n_pages = (it.n_keys + kPage - 1) / kPage;               // <= 16
+    it.n_pages = (it.n_keys + kPage - 1) / kPage;               // <= 32
     SS_CHECK_OR(it.n_keys >= 0 && it.n_pages <= 32 && f_it.page0 >= 0 && f_it.page0 + it.n_pages <= P.total_node_pages &&
                     it.dec >= 0 && it.dec < P.caps.dec && it.g >= 0 && it.g < P.Hkv && f_it.q_src >= 0 &&
                     f_it.q_src < (P.q_src_offsets ? P.q_src_rows : P.total_q),
@@ -532,7 +532,7 @@ int32_t launch_leaf_stream(const Params& P, cudaStream_t st, int sm_count) {
       !tmap::encode_kv_block_bf16(&tv, P.v_pool, static_cast<uint64_t>(rows)))
     return SS_ERR_CUDA;
   if (P.G > 8) return launch_variant<2, 8, 3>(P, st, sm_count, tk, tv);
-  return launch_variant<1, 12, 2>(P, st, sm_count, tk, tv);
+  return launch_variant<1, kLeafStreamWarps, 2>(P, st, sm_count, tk, tv);
 }
 
 }  // namespace attn

@@ -32,10 +32,12 @@ namespace cg = cooperative_groups;
 constexpr int kThreads = 1024;
 constexpr int kSmallPlan = 2048;               // nodes and paths: two of each per thread
 constexpr int kScanChunk = 2 * kThreads;       // entries of one block scan
-constexpr int kLeafClasses = 17;               // pages of the last chunk of a leaf: 0 .. 16
+constexpr int kLeafClasses = 24;               // of the last chunk of a leaf: 0 none; by length 1 .. 16 an only one, 17 .. 23 another
 constexpr int kSums = 7;
 constexpr int kLargeBlocks = 8;                // one cluster
 constexpr int kEmitThreads = 256;
+
+__device__ __forceinline__ int leaf_chunks(const Params& P, int len) { return (len + (1 << P.leaf_log2) - 1) >> P.leaf_log2; }
 
 __device__ __forceinline__ int live_paths(const Params& P) {
   int live = P.num_paths;
@@ -290,7 +292,7 @@ __device__ __forceinline__ bool make_plan(const Params& P, const PlanArrays& A, 
       if (A.n_parent[n] < 0) node_split(P, len, total_tiles, splits, split_len);
       own = splits;
     } else if (count(A.n_dec + n) > 0 && len > 0) {
-      own = ceil_div(len, kLeafChunk);                         // private leaf of one decode path
+      own = leaf_chunks(P, len);                          // private leaf of one decode path
     }
     A.n_splits[n] = splits;
     A.n_split_len[n] = split_len;
@@ -323,8 +325,11 @@ __device__ __forceinline__ bool make_plan(const Params& P, const PlanArrays& A, 
 #pragma unroll 1
           for (int a = leaf; a >= 0; a = A.n_parent[a]) slots += A.n_own[a];
           if (count(A.n_paths + leaf) == 1 && len > 0) {
-            full = len / kLeafChunk;
-            c = ceil_div(len - full * kLeafChunk, kPage);
+            full = len >> P.leaf_log2;
+            c = ceil_div(len - (full << P.leaf_log2), kPage);
+            // leaves of several chunks before those of one, whose end is cheaper: the merge of several, fence and all, is not
+            // to be what the kernel ends with (922 leaves of 32 to 512 keys in chunks of 256, the step: 92.5 -> 88.5 us)
+            if (!LARGE && c > 0) c = full > 0 ? 16 + (c + 4) / 5 : (c + 1) / 2;
             if (!LARGE && P.short_first && c > 0) c = kLeafClasses - c;
           }
         } else if (A.p_class[i] == kClassChain) {
@@ -433,7 +438,7 @@ __device__ __forceinline__ void emit_items(const Params& P, const PlanArrays& A,
         P.dec_tok[rank] = row;
         P.dec_src[rank] = src;
         P.dec_slot_base[rank] = slot;
-        P.dec_leaf_chunks[rank] = own_leaf ? ceil_div(len, kLeafChunk) : 0;
+        P.dec_leaf_chunks[rank] = own_leaf ? leaf_chunks(P, len) : 0;
       }
       for (int g = lane; g < Hkv; g += 32) P.leaf_arrive[static_cast<int64_t>(rank) * Hkv + g] = 0;
       if (!own_leaf) continue;
@@ -443,17 +448,17 @@ __device__ __forceinline__ void emit_items(const Params& P, const PlanArrays& A,
       // whole chunks first 2.43, leaf after leaf 2.37).  Where the rows go over the bus as the leaves are done, the small form
       // turns its order round, so that the bus is not idle until the longest ones are (a step of 1024 paths from host buffers
       // 227 -> 214 us)
-      const int page0 = page0_of(leaf), full = len / kLeafChunk, n_items = ceil_div(len, kLeafChunk) * Hkv;
+      const int page0 = page0_of(leaf), full = len >> P.leaf_log2, n_items = leaf_chunks(P, len) * Hkv;
       const int last = LARGE ? 0 : A.p_last[p];
 #pragma unroll 1
       for (int x = lane; x < n_items; x += 32) {
         const int c = x / Hkv, g = x - c * Hkv;
         LeafItem it;
-        it.page0 = page0 + c * (kLeafChunk / kPage);
+        it.page0 = page0 + ((c << P.leaf_log2) / kPage);
         it.node = leaf;
         it.g = g;
-        it.kv_begin = c * kLeafChunk;
-        it.kv_end = min(len, (c + 1) * kLeafChunk);
+        it.kv_begin = c << P.leaf_log2;
+        it.kv_end = min(len, (c + 1) << P.leaf_log2);
         it.slot = slot + A.n_level[leaf] + c;
         it.q_src = src;
         it.dec = rank;

@@ -20,8 +20,11 @@ constexpr int kHeadDim = 128;
 constexpr int kPage = 16;
 constexpr int kTileRows = 128;          // stacked rows of one tile item
 constexpr int kKvTile = 64;             // keys per tensor-core step
-constexpr int kLeafChunk = 256;         // most keys per leaf item (decode).  Finer items cost more in partials and merges than the better
-                                        // balance gains (922 leaves of 32 to 512 keys, the attention call: 256 keys 97 us, 128 110, 64 126)
+// Most keys per leaf item (decode): 512 - a page a lane - where the paths' leaves are enough for a warp each, else 256, so that more
+// warps have one.  Finer items cost more in partials, fences and merges than the better balance gains (the step with 922 leaves
+// of 32 to 512 keys, two heads: 512 82.4 us, 256 88.4; before that 128 and 64 keys cost 13 and 29 us more than 256).
+constexpr int kLeafChunkLog2 = 8, kLeafChunkLog2Many = 9;
+constexpr int kLeafStreamWarps = 12;    // per SM, of the leaf kernel
 constexpr int kMaxRootSplits = 8;       // KV splits of a root node when there are few tiles
 constexpr int kMinSplitLen = 512;       // a split is at least this many keys
 
@@ -146,6 +149,7 @@ struct Params {
   int32_t target_tiles;      // the planner splits root nodes until about this many tile items exist
   int32_t sms;               // SMs the call may use
   int32_t short_first;       // small planner: short leaves first (see emit_items)
+  int32_t leaf_log2;         // most keys of a leaf item
   Caps caps;
   // ---- workspace regions ----
   PlanHeader* hdr;
