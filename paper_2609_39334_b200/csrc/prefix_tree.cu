@@ -65,6 +65,7 @@ struct Args {
   int32_t *order, *path_leaf_node, *node_parent, *node_kv_len, *node_src_path, *node_src_offset, *num_nodes;
 };
 constexpr unsigned int kMore = 1, kBig = 2, kMixed = 4;
+constexpr int kCleared = 256;                     // bytes from the status word on: it, the barrier, the flags
 
 // ---- barrier over all blocks ----------------------------------------------------------------------------------------
 // False when the wait ran out (status SS_ERR_TIMEOUT; every block leaves).  A grid that is one cluster uses the hardware's
@@ -313,6 +314,10 @@ __device__ __forceinline__ void build(const Args& A) {
   const int n = A.n, n_warps = gridDim.x * kWarps, wid = blockIdx.x * kWarps + warp;
   unsigned int target = 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) *A.num_nodes = 0;
+  if (CLUSTER) {                                              // (in a grid it is cleared in front of the launch: a launch of its own costs 64
+    if (blockIdx.x == 0 && threadIdx.x < kCleared / 4) A.status[threadIdx.x] = 0;   // paths 2 us)
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  }
 
   // ---- sort: round 0 has one group of all positions, in index order ---------------------------------------------------
   int kc = 0, pc = 0;                                         // buffers of the sorted keys and the paths
@@ -390,6 +395,7 @@ __device__ __forceinline__ void build(const Args& A) {
       if (me != pivot) o = compare_paths(A, me, pivot, base, lane);
       if (lane == 0) A.key[kc ^ 1][p] = make_key(o);
     }
+    if (CLUSTER && round == 0) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");   // (the flags are clear)
     if (lane == 0 && need) atomicOr(&A.flags[round & 3], need);
     if (!grid_barrier<CLUSTER>(A, target)) return;
     const unsigned int flags = *reinterpret_cast<volatile unsigned int*>(&A.flags[round & 3]);
@@ -574,7 +580,7 @@ constexpr int kMaxBlocks = 1024;
 static Layout layout(int n) {
   Layout L;
   size_t off = 0;
-  L.status = off; off = align_up(off + 256);                  // status, barrier, flags: cleared by the host
+  L.status = off; off = align_up(off + kCleared);             // status, barrier, flags
   for (int i = 0; i < 2; ++i) { L.key[i] = off; off = align_up(off + static_cast<size_t>(n) * sizeof(uint64_t)); }
   L.ints = off; off = align_up(off + (static_cast<size_t>(11) * (n + 1) + kMaxBlocks) * 4);
   L.total = off;
@@ -640,7 +646,11 @@ extern "C" int32_t ss_build_prefix_tree(const int32_t* tok_ids, const int64_t* t
   if (workspace_bytes < L.total) return SS_ERR_WORKSPACE_TOO_SMALL;
   cudaStream_t st = as_stream(stream);
   char* ws = static_cast<char*>(workspace);
-  if (cudaMemsetAsync(ws + L.status, 0, 256, st) != cudaSuccess ||
+  // One block while it has a warp per position (its barrier is the cheapest).  A cluster of 8 blocks up to two positions per
+  // warp and 16 MB of ids, which its 8 SMs read in 20 us: what the grid's barriers (1.5 us against 0.3, a dozen of them)
+  // cost more.
+  const int cluster = n_paths == 0 ? 0 : n_paths <= kWarps ? 1 : n_paths <= 512 && total_tok <= (1 << 22) ? 8 : 0;
+  if ((cluster == 0 && cudaMemsetAsync(ws + L.status, 0, kCleared, st) != cudaSuccess) ||
       (n_paths == 0 && cudaMemsetAsync(num_nodes_out, 0, sizeof(int32_t), st) != cudaSuccess)) {
     (void)cudaGetLastError();
     return SS_ERR_CUDA;
@@ -671,11 +681,7 @@ extern "C" int32_t ss_build_prefix_tree(const int32_t* tok_ids, const int64_t* t
   A.node_src_offset = node_src_offset_out;
   A.num_nodes = num_nodes_out;
 
-  // One block while it has a warp per position (its barrier is the cheapest).  A cluster of 8 blocks up to two positions per
-  // warp and 16 MB of ids, which its 8 SMs read in 20 us: what the grid's barriers (1.5 us against 0.3, a dozen of them)
-  // cost more.
-  if (n <= kWarps) return launch(A, 1, true, st);
-  if (n <= 512 && total_tok <= (1 << 22)) return launch(A, 8, true, st);
+  if (cluster > 0) return launch(A, cluster, true, st);
   int sms = sm_count_of_current_device();
   if (sms > kMaxBlocks) sms = kMaxBlocks;
   const int wanted = (n + kWarps - 1) / kWarps;
