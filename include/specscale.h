@@ -316,6 +316,11 @@ int32_t ss_early_prune(const float* scores, const uint8_t* verified, const int32
  * ======================================================================================================= */
 int32_t ss_branch_sample(const float* logits, const int64_t* draw_offsets, const float* uniforms, int32_t n_seq,
                          int32_t vocab, float temperature, int32_t* tokens_out, int64_t* seq_out, void* stream);
+/* The same for a caller that knows a bound of draw_offsets[n_seq] - draw_offsets[0], such as the size of tokens_out: many
+ * sequences with few draws each are then sampled faster.  max_draws < 0: not known.  The results do not depend on it. */
+int32_t ss_branch_sample_upto(const float* logits, const int64_t* draw_offsets, const float* uniforms, int32_t n_seq,
+                              int32_t vocab, float temperature, int32_t* tokens_out, int64_t* seq_out, int64_t max_draws,
+                              void* stream);
 
 /* =========================================================================================================
  * ss_build_prefix_tree - radix tree of candidate paths over whole KV pages, from raw token ids.

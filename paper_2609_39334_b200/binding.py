@@ -40,7 +40,7 @@ EXPORTS = [
     "ss_dedup_paths_static", "ss_debug_tile_kernel_occupancy", "ss_early_prune",
     "ss_branch_sample", "ss_gather_unique_paths", "ss_candidate_step_host_arena_bytes", "ss_candidate_step_host",
     "ss_prefix_tree_workspace_bytes", "ss_build_prefix_tree", "ss_candidate_step",
-    "ss_candidate_step_host_2",
+    "ss_candidate_step_host_2", "ss_branch_sample_upto",
 ]
 PHASES = ["plan", "tiles", "leaves", "generic", "merge"]
 
@@ -84,6 +84,7 @@ _SIGNATURES = {
     "ss_dedup_paths_static": "ppppiIppppppp", "ss_gather_unique_paths": "ppipppppppp",
     "ss_tree_attention_workspace_bytes": "pp", "ss_tree_attention": "ppzp", "ss_topk_workspace_bytes": "ip",
     "ss_topk_prune": "ppiiipppzp", "ss_early_prune": "pppiiippppzp", "ss_branch_sample": "pppiifppp",
+    "ss_branch_sample_upto": "pppiifppqp",
     "ss_prefix_tree_workspace_bytes": "iqip", "ss_build_prefix_tree": "ppiqippppppppzp",
     "ss_candidate_step": "pp", "ss_candidate_step_host_arena_bytes": "pp", "ss_candidate_step_host": "ppzp", "ss_candidate_step_host_2": "ppzpp", "ss_profile_enable": "i",
     "ss_profile_read": "pp", "ss_debug_umma_tile": "pppiiipp", "ss_debug_bounded_wait": "pp",
@@ -390,9 +391,11 @@ def ss_early_prune(scores, verified, seg_offsets, n_segments, n_total, k, pruned
 
 def ss_branch_sample(logits, draw_offsets, uniforms, n_seq, vocab, temperature, tokens_out, seq_out, stream=None,
                      check=True) -> int:
-    rc = lib().ss_branch_sample(_ptr(logits), _ptr(draw_offsets), _ptr(uniforms), n_seq,
-                                vocab, temperature, _ptr(tokens_out), _ptr(seq_out),
-                                _stream(stream))
+    """`tokens_out` bounds the number of draws, which decides how many sequences with few of them are sampled."""
+    most = tokens_out.numel() if isinstance(tokens_out, torch.Tensor) else -1
+    rc = lib().ss_branch_sample_upto(_ptr(logits), _ptr(draw_offsets), _ptr(uniforms), n_seq,
+                                     vocab, temperature, _ptr(tokens_out), _ptr(seq_out), most,
+                                     _stream(stream))
     if check:
         _check(rc, "ss_branch_sample")
     return rc

@@ -26,8 +26,8 @@
 // 8 fp64 instructions with the summation; the table is copied 16 times so that every lane reads its own bank pair.
 //
 // Those hold the issue slots: 32 logits take ~30 clocks of a sub-partition, 922 rows of 151936 120 us where the 560 MB take 85.  So
-// a block that takes rows by itself adds them up in fp32 (quick_sums: 7 packed instructions a logit, eight terms at a time before
-// fp64) where a row has few draws.  A quick sum is within 3.2e-7 of the exact one, proven; a draw whose target is not further than
+// where there are many rows with few draws, blocks add them up in fp32 (quick_sums: 7 packed instructions a logit, eight terms at a
+// time before fp64).  A quick sum is within 3.2e-7 of the exact one, proven; a draw whose target is not further than
 // that from the two ends of its token (1.5 % of them) is marked and made again by the table, its whole row, in the launch
 // that takes the rows that are left over.  No token is other than the table's.
 // Bound now: HBM latency and issue slots about equally (86 us with the arithmetic taken out).  Measured, the call: 922 rows, 1362
@@ -56,7 +56,6 @@ constexpr int kRowThreads = kThreads + 32 * kDrawWarps;       // (96 registers a
 constexpr int kStages = 4;                                    // segments of a warp in shared memory or on their way there
 constexpr int kRingBytes = kWarps * kStages * kSeg * 4;
 constexpr int kSums = 3;                                      // rows whose sums are held at a time
-constexpr int kQuickVocab = 16384;                            // see ss_branch_sample
 constexpr double kQuickError = 3.2e-7;                        // of the quick sums, see quick_sums
 constexpr float kLowTop = -200.f, kHighTop = 900.f;           // exponent range of a row's largest term
 constexpr float kLowest = -1020.f;                            // smaller exponents count as this one (2^-820 of the sum)
@@ -76,6 +75,7 @@ struct Args {
   float ckf, lowest;           // lowest: the logit whose exponent is kLowest
   float c_hi, c_lo, inv_c;     // log2(e) / temperature in two parts, and its reciprocal
   int quick_draws;             // draws of a row up to which its sums are quick ones
+  int whole_draws;             // rows with more draws are left to the clusters as a whole
   int first_idle;              // clusters from here on have no row of their own and take marked draws
   double lowest_below;         // the same for l - dm
   bool fast;                   // the temperature allows sums that are not relative to the row's maximum
@@ -639,6 +639,14 @@ __device__ __forceinline__ void row_below(const Args& A, Sums<CL>& S, int* queue
   }
 }
 
+// A row that is left to the clusters: its first draw is marked, the others are none of theirs.
+__device__ __forceinline__ void mark_whole(const Args& A, int64_t seq, int64_t d0, int64_t d1, int lane) {
+  for (int64_t d = d0 + lane; d < d1; d += 32) {
+    A.tokens_out[d] = d == d0 ? kUnsure : kTaken;
+    A.seq_out[d] = seq;
+  }
+}
+
 // Draws d0 + turn, d0 + turn + turns, ... below d1 of row `seq`; `at`: which of `sums` holds the row.  True, with nothing drawn,
 // if the row is outside the table's range or has many draws (all that draw from it agree).
 // QUICK: the sums may be quick ones (`quick`), each within kQuickError of the exact one.  The terms of the segment that holds the
@@ -648,11 +656,15 @@ template <int CL, bool VEC, bool QUICK>
 __device__ __forceinline__ bool draws(const Args& A, Sums<CL>* sums, const double* bank, int at, int64_t seq, int64_t d0, int64_t d1,
                                       int turn, int turns, bool quick, int lane) {
   constexpr int kSlices = CL * kWarps;
+  if (QUICK && d1 - d0 > A.many) {
+    if (turn == 0) mark_whole(A, seq, d0, d1, lane);
+    return false;
+  }
   float mx = -INFINITY;
   for (int i = lane; i < kSlices; i += 32) mx = fmaxf(mx, sums[at].slice_max[i]);
   mx = warp_max(mx);
   const float top = mx * A.ckf * (1.f / kTable);
-  if (!(A.fast && top >= kLowTop && top <= kHighTop) || d1 - d0 > A.many) {   // its first draw's outputs say so meanwhile, and keep the maximum
+  if (!(A.fast && top >= kLowTop && top <= kHighTop) || (!QUICK && d1 - d0 > A.many)) {   // its first draw's outputs say so meanwhile, and keep the maximum
     if (turn == 0 && lane == 0) {
       A.tokens_out[d0] = kLater;
       A.seq_out[d0] = __float_as_int(mx);
@@ -745,7 +757,9 @@ __device__ __forceinline__ Work next_row(const Args& A, int64_t r, int step) {
 
 // A row per block at a time.  kWarps warps add up the rows one after the other, quick where a row has few draws; kDrawWarps warps
 // make the draws of the rows whose sums are complete (a draw takes 2.9 us, and a warp that made it between two rows held up all
-// others at the end of the next).  The waits are between warps of a block and bounded.
+// others at the end of the next).  Four warps make as many draws in the time of a row as it has thousands of tokens, about: a row
+// with more than a few times that is left to the clusters, which have 32 warps or more (592 rows of 151936, one draw each but 256
+// of one row: 209 us if its block makes them, 102 so).  The waits are between warps of a block and bounded.
 template <bool VEC>
 __global__ void __launch_bounds__(kRowThreads, 1) branch_rows_kernel(const __grid_constant__ Args A) {
   ss::grid_dependency_enter();
@@ -930,10 +944,11 @@ __device__ __forceinline__ Work next_unsure(cg::cluster_group& cl, const Args& A
   const int i = S.taken;
   cl.sync();                                                   // (it is written to again)
   if (i < 0) return Work{-1, 0, 0};
-  return Work{__ldcg(A.seq_out + first + i), first + i, first + i + 1};
+  const int64_t row = __ldcg(A.seq_out + first + i), d0 = A.draw_offsets[row], d1 = A.draw_offsets[row + 1];
+  return d1 - d0 > A.whole_draws ? Work{row, d0, d1} : Work{row, first + i, first + i + 1};
 }
 
-// A row per cluster at a time; UNSURE: then the draws that the launch before this one has marked.
+// A row per cluster at a time; UNSURE: then the draws and rows that the launch before this one has marked.
 template <int CL, bool VEC, bool UNSURE>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(kThreads, 1)
 branch_sample_kernel(const __grid_constant__ Args A) {
@@ -993,17 +1008,15 @@ branch_sample_kernel(const __grid_constant__ Args A) {
     at = at == 2 ? 0 : at + 1;
     row = after;
   }
-  if (later) {                                                 // (the cluster agrees)
-    cl.sync();                                                 // (the marks; and nobody reads the running sums any more)
-    for (int64_t r = next_row(row0); r < A.n_seq; r = next_row(r + n_clusters)) {
-      const int64_t d = A.draw_offsets[r];
-      if (__ldcg(A.tokens_out + d) != kLater) continue;        // (read in front of row_below's barriers, written behind them)
-      row_below<CL, VEC>(A, S.sums[0], S.queue[warp], bank, r, slice, lane, __int_as_float(static_cast<int>(__ldcg(A.seq_out + d))));
-    }
-  }
-  if (UNSURE && cluster >= A.first_idle) {
-    int64_t scanned = 0;
-    for (;;) {
+  if (later) cl.sync();                                        // (the marks; and nobody reads the running sums any more.  The cluster agrees)
+  int64_t r = later ? next_row(row0) : A.n_seq, scanned = 0;
+  for (;;) {                                                   // rows that wait for their maximum, then what the launch before has marked
+    int64_t below = -1, d0 = 0;
+    if (r < A.n_seq) {
+      d0 = A.draw_offsets[r];
+      if (__ldcg(A.tokens_out + d0) == kLater) below = r;      // (read in front of row_below's barriers, written behind them)
+      r = next_row(r + n_clusters);
+    } else if (UNSURE && cluster >= A.first_idle) {
       const Work now = next_unsure<CL>(cl, A, S, scanned, cluster, n_clusters);
       if (now.row < 0) break;
       const float* p = A.logits + now.row * A.vocab;
@@ -1012,9 +1025,14 @@ branch_sample_kernel(const __grid_constant__ Args A) {
       const double sum = slice_sums<VEC>(p, A, bank, S.sums[0].seg_end[warp], L.v0, L.n_half, lane, first, mx);
       publish<CL>(cl, S.sums[0], slice, lane, sum, warp_max(mx));
       cl.sync();
-      draws<CL, VEC, false>(A, S.sums, bank, 0, now.row, now.d0, now.d1, slice, CL * kWarps, false, lane);
+      if (draws<CL, VEC, false>(A, S.sums, bank, 0, now.row, now.d0, now.d1, slice, CL * kWarps, false, lane)) below = now.row;
+      d0 = now.d0;
       cl.sync();
+    } else {
+      break;
     }
+    if (below >= 0)
+      row_below<CL, VEC>(A, S.sums[0], S.queue[warp], bank, below, slice, lane, __int_as_float(static_cast<int>(__ldcg(A.seq_out + d0))));
   }
   if (CL > 1) cl.sync();                                       // (a block's running sums may still be read by another)
 }
@@ -1032,6 +1050,23 @@ static bool ring_ready() {
   return true;
 }
 
+// Rows 0 .. n_seq-1, one per block at a time; a launch of clusters has to follow.
+// Quick sums leave 1.5 % of the draws of a row of 151936 ordinary logits open (9 % if the logits are all equal), each of which
+// costs another pass over its row, by the table: worth it up to 16 draws of such a row.
+static int32_t launch_rows(Args A, bool vec, int n_seq, int blocks, cudaStream_t st) {
+  constexpr int kUnit = kSeg / 2;
+  A.slice = (A.vocab + kWarps * kUnit - 1) / (kWarps * kUnit) * kUnit;
+  A.many = A.whole_draws;
+  A.quick_draws = 2500000 / A.vocab;
+  A.n_seq = n_seq;
+  if (!(vec ? ring_ready<true>() : ring_ready<false>())) return SS_ERR_CUDA;
+  if (vec)
+    SS_LAUNCH(branch_rows_kernel<true>, blocks, kRowThreads, kRingBytes, st, A);
+  else
+    SS_LAUNCH(branch_rows_kernel<false>, blocks, kRowThreads, kRingBytes, st, A);
+  return SS_OK;
+}
+
 // Rows row0 .. n_seq-1, `clusters` at a time.
 template <int CL>
 static int32_t launch(Args A, bool vec, int row0, int n_seq, int clusters, cudaStream_t st) {
@@ -1046,23 +1081,15 @@ static int32_t launch(Args A, bool vec, int row0, int n_seq, int clusters, cudaS
   A.many = CL <= 2 || idle ? CL * kWarps * (4 + A.slice / 384) : INT32_MAX;
   A.row0 = row0;
   A.n_seq = n_seq;
-  if constexpr (CL == 1) {
-    if (!(vec ? ring_ready<true>() : ring_ready<false>())) return SS_ERR_CUDA;
-    if (vec)
-      SS_LAUNCH(branch_rows_kernel<true>, clusters, kRowThreads, kRingBytes, st, A);
-    else
-      SS_LAUNCH(branch_rows_kernel<false>, clusters, kRowThreads, kRingBytes, st, A);
-  } else {
-    const bool unsure = A.first_idle != INT32_MAX;
-    if (vec && unsure)
-      SS_LAUNCH((branch_sample_kernel<CL, true, true>), clusters * CL, kThreads, 0, st, A);
-    else if (vec)
-      SS_LAUNCH((branch_sample_kernel<CL, true, false>), clusters * CL, kThreads, 0, st, A);
-    else if (unsure)
-      SS_LAUNCH((branch_sample_kernel<CL, false, true>), clusters * CL, kThreads, 0, st, A);
-    else
-      SS_LAUNCH((branch_sample_kernel<CL, false, false>), clusters * CL, kThreads, 0, st, A);
-  }
+  const bool unsure = CL > 1 && A.first_idle != INT32_MAX;
+  if (vec && unsure)
+    SS_LAUNCH((branch_sample_kernel<CL, true, (CL > 1)>), clusters * CL, kThreads, 0, st, A);
+  else if (vec)
+    SS_LAUNCH((branch_sample_kernel<CL, true, false>), clusters * CL, kThreads, 0, st, A);
+  else if (unsure)
+    SS_LAUNCH((branch_sample_kernel<CL, false, (CL > 1)>), clusters * CL, kThreads, 0, st, A);
+  else
+    SS_LAUNCH((branch_sample_kernel<CL, false, false>), clusters * CL, kThreads, 0, st, A);
   return SS_OK;
 }
 
@@ -1101,6 +1128,12 @@ static int resident_clusters(bool vec) {
 extern "C" int32_t ss_branch_sample(const float* logits, const int64_t* draw_offsets, const float* uniforms,
                                     int32_t n_seq, int32_t vocab, float temperature, int32_t* tokens_out,
                                     int64_t* seq_out, void* stream) {
+  return ss_branch_sample_upto(logits, draw_offsets, uniforms, n_seq, vocab, temperature, tokens_out, seq_out, -1, stream);
+}
+
+extern "C" int32_t ss_branch_sample_upto(const float* logits, const int64_t* draw_offsets, const float* uniforms,
+                                         int32_t n_seq, int32_t vocab, float temperature, int32_t* tokens_out,
+                                         int64_t* seq_out, int64_t max_draws, void* stream) {
   using namespace ss;
   using namespace ss::sample;
   if (n_seq < 0 || vocab < 1 || !(temperature > 0.f)) return SS_ERR_INVALID_ARG;
@@ -1123,7 +1156,6 @@ extern "C" int32_t ss_branch_sample(const float* logits, const int64_t* draw_off
   A.c_hi = static_cast<float>(c);
   A.c_lo = static_cast<float>(c - static_cast<double>(A.c_hi));
   A.inv_c = static_cast<float>(1.0 / c);
-  A.quick_draws = 0;
   A.first_idle = INT32_MAX;
   A.lowest_below = kLowest / c;
   const bool vec = reinterpret_cast<uintptr_t>(logits) % 16 == 0 && vocab % 4 == 0;
@@ -1138,21 +1170,29 @@ extern "C" int32_t ss_branch_sample(const float* logits, const int64_t* draw_off
   auto cluster_size = [&](int rows) { return rows <= n8 ? 8 : rows <= n4 ? 4 : rows <= n2 ? 2 : 1; };
   int whole = blocks_min > 1 ? 0 : n_seq / sms * sms;
   if (blocks_min == 1 && cluster_size(n_seq - whole) == 1) whole = n_seq;
-  // Quick sums leave 1.5 % of the draws of a row of 151936 ordinary logits open (9 % if the logits are all equal), each of which
-  // costs another pass over its row, by the table: worth it up to 16 draws of such a row.
-  const bool quick = whole > 0 && A.fast && vocab >= kQuickVocab;
-  if (quick) A.quick_draws = 2500000 / vocab;
+  // fp32 sums save a block 0.06 us per 1000 tokens and cost a launch for the draws that they leave open, and four warps make a row's
+  // draws instead of sixteen: for calls with many tokens a block and, by the caller's bound, few draws a row.  Table -> fp32, us,
+  // rows x vocabulary, draws of a row: 922 x 151936, 1: 184 -> 121, 4: 185 -> 151; 740 x 128256, 4: 118 -> 105; 740 x 100352, 1: 95 ->
+  // 78; 592 x 100352, 1: 77 -> 68; 888 x 65536, 1: 80 -> 64; 2400 x 32000, 2: 131 -> 97.  On the other side 740 x 65536, 1: 66 -> 67;
+  // 592 x 65536, 1: 55 -> 61; 444 x 100352, 1: 60 -> 65; 740 x 100352, 4: 95 -> 106; 922 x 151936, 16: 196 -> 287; 148 x 151936, 1:
+  // 30 -> 40, 148 x 16384, 1: 8 -> 20.  Smaller vocabularies gain little at any number of rows (2400 x 16384, 1: 89 -> 85).
+  const int64_t tokens = static_cast<int64_t>(whole / sms) * vocab;   // of a block
+  const bool rows = max_draws >= 0 && A.fast && vocab >= 32000 && tokens >= 390000 &&
+                    max_draws <= static_cast<int64_t>(n_seq) * (tokens >= 1000000 ? 6 : tokens >= 605000 ? 4 : tokens >= 500000 ? 3 : 2);
+  if (rows) A.whole_draws = vocab >> 12 > 16 ? vocab >> 12 : 16;
   if (whole > 0) {
-    const int32_t rc = launch<1>(A, vec, 0, whole, whole < sms ? whole : sms, st);
+    const int blocks = whole < sms ? whole : sms;
+    const int32_t rc = rows ? launch_rows(A, vec, whole, blocks, st) : launch<1>(A, vec, 0, whole, blocks, st);
     if (rc != SS_OK) return rc;
   }
   const int rest = n_seq - whole;
-  if (rest == 0 && !quick) return SS_OK;
+  if (rest == 0 && !rows) return SS_OK;
   int size = rest ? cluster_size(rest) : 4;
+  if (rows && size > 4) size = 4;
   if (size < blocks_min) size = blocks_min;
   const int resident = size > 4 ? n8 : size > 2 ? n4 : n2;
   int clusters = rest < resident ? rest : resident;
-  if (quick) {                                                  // marked draws: by the clusters without a row, unless they are few
+  if (rows) {                                                   // marked draws: by the clusters without a row, unless they are few
     clusters = resident;
     A.first_idle = (resident - rest) * 4 >= resident ? rest : 0;
   }

@@ -267,3 +267,79 @@ def test_draws_at_the_boundaries_between_tokens(S, V, kind):
     assert np.array_equal(seq.cpu().numpy(), want_seq)
     # (a third of the rows have their targets on the ends: exactly, where 16384 equal logits make those fp32 numbers)
     assert np.array_equal(got[sure], want_tok[sure]) and sure.mean() > 0.5
+
+
+SMS = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 148
+
+
+@pytest.mark.parametrize("rounds,more,V", [(4, 0, 125000), (4, 9, 131072), (5, 40, 100001), (16, 1, 32000)])
+@pytest.mark.parametrize("kind,T", [("plain", 0.8), ("flat", 0.8), ("masked", 0.8), ("nan", 0.8), ("rising", 0.8), ("top", 1.1e-3), ("bottom", 9e5)])
+def test_few_draws_of_many_rows(rounds, more, V, kind, T):
+    """Whole rounds of rows on single blocks, whose sums are first made in fp32, and none, few and more rows left over: targets on
+    the ends of tokens, at 0 and just below 1; rows with none, one, 20 and 130 draws (beyond the quick sums, beyond what is drawn one
+    by one); flat rows, masked ones, rows with a NaN, rows whose logits rise by 2^60 and more within a warp's slice, rows whose
+    largest exponent is just inside and just outside the range of the sums, at temperatures near the ends of theirs."""
+    S = rounds * SMS + more
+    rng = np.random.default_rng(rounds + V)
+    logits = rng.standard_normal((S, V), dtype=np.float32)
+    nat = T / 1.4426950408889634                                # a logit of this is an exponent of 1
+    logits *= np.float32(0.0 if kind == "flat" else 2.0 * T)
+    if kind == "masked":
+        logits[:, : V // 5] = -np.inf
+        logits[1::2, V - 700:] = -np.inf
+    elif kind == "nan":
+        for s, at in ((1, 0), (5, V - 1), (S // 2, V // 2), (S - 1, 7), (9, slice(None))):
+            logits[s, at] = np.nan
+        logits[S // 2, V // 2 + 64] = 900.0 * nat               # (beside the NaN, in the same lane: the row's largest)
+    elif kind == "rising":
+        logits += (np.arange(V, dtype=np.float32) / V * 700.0 * nat)[None, :]
+    elif kind in ("top", "bottom"):
+        edge = {"top": 880.0, "bottom": -190.0}[kind] * nat
+        logits[::2] += np.float32(edge)
+        logits[::8] += np.float32(edge / 2)                     # (outside)
+    pot = np.ones(S, np.int64)
+    pot[3::40] = 0
+    pot[::50] = 20
+    pot[S // 3] = 130
+    off = np.concatenate([[0], np.cumsum(pot)]).astype(np.int64)
+    assert off[-1] <= 2 * S
+    u = rng.random(int(off[-1])).astype(np.float32)
+    for s in range(0, S, 9):
+        row = logits[s].astype(np.float64)
+        if np.isnan(row).any():
+            continue
+        e = np.exp((row - row.max()) / float(np.float32(T)))
+        c = np.cumsum(e) / e.sum()
+        u[off[s]: off[s + 1]] = np.minimum(c[rng.integers(0, V, size=pot[s])], 1.0 - 2.0 ** -24).astype(np.float32)
+    u[5::31] = 0.0
+    u[7::37] = np.float32(1.0) - np.float32(2.0 ** -24)
+    tok, seq = run(logits, off, u, T)
+    want_tok, want_seq, margin = oracle.branch_sample(logits, off, u, float(np.float32(T)))
+    got, bad = tok.cpu().numpy(), np.isnan(logits).any(axis=1)[want_seq]
+    sure = (margin > 1e-12) & ~bad
+    assert np.array_equal(seq.cpu().numpy(), want_seq)
+    assert np.array_equal(got[sure], want_tok[sure]) and sure.mean() > 0.5
+    assert np.array_equal(got[(u == 0.0) & ~bad], want_tok[(u == 0.0) & ~bad])
+    assert (got[bad] == V - 1).all()
+
+
+def test_calls_with_few_rows_or_many_draws_are_one_launch():
+    """Blocks add up in fp32, with a second launch for the draws that this leaves open, only where both are worth it: many rows of a
+    large vocabulary with few draws each (148 rows of 16384, one draw each: 8.2 us in one launch, 20 in two)."""
+    def launches(S, V, draws, bound=True):
+        lg = torch.zeros((S, V), device=DEV)
+        off = torch.arange(S + 1, dtype=torch.int64, device=DEV) * draws
+        u = torch.full((S * draws,), 0.5, device=DEV)
+        tok = torch.empty(S * draws, dtype=torch.int32, device=DEV)
+        seq = torch.empty(S * draws, dtype=torch.int64, device=DEV)
+        before = B.ss_launch_count()
+        if bound:
+            B.ss_branch_sample(lg, off, u, S, V, 0.8, tok, seq)
+        else:
+            args = [t.data_ptr() for t in (lg, off, u)] + [S, V, 0.8, tok.data_ptr(), seq.data_ptr(), None]
+            assert B.lib().ss_branch_sample(*args) == B.SS_OK
+        torch.cuda.synchronize()
+        return B.ss_launch_count() - before
+
+    assert [launches(SMS, 16384, 1), launches(SMS, 151936, 1), launches(4 * SMS, 131072, 8)] == [1, 1, 1]
+    assert launches(4 * SMS, 131072, 2) == 2 and launches(4 * SMS, 131072, 2, bound=False) == 1
