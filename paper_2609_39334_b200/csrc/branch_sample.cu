@@ -34,6 +34,7 @@
 // draws 184 us by the table -> 130 (rows 97, marked draws and left-over rows 33), of it 20 by adding up four segments' sums over
 // the warp at once; 16 rows 12.4.
 #include <cooperative_groups.h>
+#include <stdlib.h>
 
 #include "common.cuh"
 #include "umma.cuh"
@@ -79,6 +80,9 @@ struct Args {
   int first_idle;              // clusters from here on have no row of their own and take marked draws
   double lowest_below;         // the same for l - dm
   bool fast;                   // the temperature allows sums that are not relative to the row's maximum
+#ifdef SS_CHECKED
+  bool give_up;                // waits between warps are to be taken for run out
+#endif
 };
 
 template <int CL>
@@ -759,7 +763,8 @@ __device__ __forceinline__ Work next_row(const Args& A, int64_t r, int step) {
 // make the draws of the rows whose sums are complete (a draw takes 2.9 us, and a warp that made it between two rows held up all
 // others at the end of the next).  Four warps make as many draws in the time of a row as it has thousands of tokens, about: a row
 // with more than a few times that is left to the clusters, which have 32 warps or more (592 rows of 151936, one draw each but 256
-// of one row: 209 us if its block makes them, 102 so).  The waits are between warps of a block and bounded.
+// of one row: 209 us if its block makes them, 102 so).  The waits are between warps of a block and bounded; the call has no status to
+// say that one ran out, so the block then takes all of its rows again, by row_below with its hardware barriers.
 template <bool VEC>
 __global__ void __launch_bounds__(kRowThreads, 1) branch_rows_kernel(const __grid_constant__ Args A) {
   ss::grid_dependency_enter();
@@ -809,10 +814,17 @@ __global__ void __launch_bounds__(kRowThreads, 1) branch_rows_kernel(const __gri
   __syncthreads();
 
   uint32_t count = 0;                                          // rows so far: their sums lie in turn in the kSums places
+  auto wait = [&](uint64_t* bar, uint32_t turn) {
+#ifdef SS_CHECKED
+    if (A.give_up && warp >= kWarps && count == 1) *abort_flag = 1;
+    if (A.give_up && __any_sync(0xffffffffu, *abort_flag)) return false;
+#endif
+    return __all_sync(0xffffffffu, umma::mbar_wait(bar, turn & 1, abort_flag)) != 0;   // (a warp leaves as a whole)
+  };
   if (warp < kWarps) {
     for (; now.row >= 0; ++count) {
       const int at = count % kSums;
-      if (count >= kSums && !umma::mbar_wait(&C.free[at], (count / kSums - 1) & 1, abort_flag)) break;
+      if (count >= kSums && !wait(&C.free[at], count / kSums - 1)) break;
       const bool quick = A.fast && now.d1 - now.d0 <= A.quick_draws;
       double sum = 0.0;
       float mx = -INFINITY;
@@ -880,7 +892,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) branch_rows_kernel(const __gri
     bool later = false;                                        // a row outside the table's range: for when the others are done
     for (; now.row >= 0; ++count) {
       const int at = count % kSums;
-      if (!umma::mbar_wait(&C.full[at], (count / kSums) & 1, abort_flag)) break;
+      if (!wait(&C.full[at], count / kSums)) break;
       __syncwarp();
       const int turn = (warp + static_cast<int>(now.row)) % kDrawWarps;
       later |= draws<1, VEC, true>(A, S.sums, bank, at, now.row, now.d0, now.d1, turn, kDrawWarps,
@@ -892,7 +904,23 @@ __global__ void __launch_bounds__(kRowThreads, 1) branch_rows_kernel(const __gri
     if (later && lane == 0) C.later = 1;
   }
   __syncthreads();                                             // (the marks; and nobody reads the running sums any more)
-  if (C.later && !C.abort_flag) {
+  if (C.abort_flag) {                                          // a wait ran out
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    for (int64_t r = row0 + static_cast<int64_t>(step) * warp; r < A.n_seq; r += static_cast<int64_t>(step) * (kRowThreads / 32)) {
+      const int64_t d = A.draw_offsets[r];
+      if (A.draw_offsets[r + 1] <= d) continue;
+      float mx = -INFINITY;
+      for (int v = lane; v < A.vocab; v += 32) mx = fmaxf(mx, __ldg(A.logits + r * A.vocab + v));
+      mx = warp_max(mx);
+      if (lane == 0) {
+        A.tokens_out[d] = kLater;
+        A.seq_out[d] = __float_as_int(mx);
+      }
+    }
+    if (tid == 0) C.later = 1;
+    __syncthreads();
+  }
+  if (C.later) {
     for (Work r = next_row(A, row0, step); r.row >= 0; r = next_row(A, r.row + step, step)) {
       if (__ldcg(A.tokens_out + r.d0) != kLater) continue;     // (read in front of row_below's barriers, written behind them)
       if (warp < kWarps) {
@@ -1156,6 +1184,9 @@ extern "C" int32_t ss_branch_sample_upto(const float* logits, const int64_t* dra
   A.c_hi = static_cast<float>(c);
   A.c_lo = static_cast<float>(c - static_cast<double>(A.c_hi));
   A.inv_c = static_cast<float>(1.0 / c);
+#ifdef SS_CHECKED
+  A.give_up = getenv("SS_GIVE_UP") != nullptr;
+#endif
   A.first_idle = INT32_MAX;
   A.lowest_below = kLowest / c;
   const bool vec = reinterpret_cast<uintptr_t>(logits) % 16 == 0 && vocab % 4 == 0;

@@ -67,5 +67,49 @@ def test_checked_build_runs_the_benchmark_configurations_clean_and_refuses_a_bad
     assert "config 4 ok" in p.stdout and "out-of-range page id reported" in p.stdout
 
 
+def child_waits():
+    """Rows that blocks take by themselves, in a build whose waits between the warps of a block run out at the second row."""
+    import numpy as np
+    import torch
+
+    import oracle
+    from paper_2609_39334_b200 import binding as B
+
+    assert B.LIB_PATH.endswith("_checked.so") and "SS_GIVE_UP" in os.environ
+    S, V = 4 * torch.cuda.get_device_properties(0).multi_processor_count + 5, 131072
+    rng = np.random.default_rng(3)
+    logits = rng.standard_normal((S, V), dtype=np.float32) * np.float32(2.0)
+    logits[::7] += np.float32(900.0)                            # (outside the range of the sums)
+    logits[5::11, V // 2] = np.nan
+    pot = np.ones(S, np.int64)
+    pot[::3], pot[1::9], pot[S // 2] = 2, 0, 60
+    off = np.concatenate([[0], np.cumsum(pot)]).astype(np.int64)
+    u = rng.random(int(off[-1])).astype(np.float32)
+    u[::13] = 0.0
+    dev = [torch.from_numpy(a).cuda() for a in (logits, off, u)]
+    tok = torch.full((int(off[-1]),), -2, dtype=torch.int32, device="cuda:0")
+    seq = torch.full((int(off[-1]),), 1 << 60, dtype=torch.int64, device="cuda:0")
+    B.ss_branch_sample(*dev, S, V, 0.8, tok, seq)
+    torch.cuda.synchronize()
+    want, want_seq, margin = oracle.branch_sample(logits, off, u, float(np.float32(0.8)))
+    bad = np.isnan(logits).any(axis=1)[want_seq]
+    sure = (margin > 1e-12) & ~bad
+    got = tok.cpu().numpy()
+    assert np.array_equal(seq.cpu().numpy(), want_seq)
+    assert np.array_equal(got[sure], want[sure]) and (got[bad] == V - 1).all()
+    print(f"waits that run out: {len(got)} draws ok")
+
+
+def test_branch_sample_leaves_nothing_unwritten_when_a_wait_runs_out():
+    from paper_2609_39334_b200 import build as cuda_build
+    cuda_build.build(defines=["SS_CHECKED"], suffix="_checked")
+    env = dict(os.environ, SS_LIB_SUFFIX="_checked", SS_GIVE_UP="1", PYTHONPATH=ROOT + os.pathsep + os.environ.get("PYTHONPATH", ""))
+    p = subprocess.run([sys.executable, os.path.abspath(__file__), "--child-waits"], env=env, capture_output=True, text=True,
+                       timeout=600)
+    assert p.returncode == 0 and "draws ok" in p.stdout, p.stdout[-2000:] + p.stderr[-4000:]
+
+
 if __name__ == "__main__" and "--child" in sys.argv:
     child()
+if __name__ == "__main__" and "--child-waits" in sys.argv:
+    child_waits()
