@@ -197,9 +197,7 @@ int32_t ss::attn::tree_attention(const ss_attn_desc_t* d, void* workspace, size_
   if (d->max_sms > 0 && d->max_sms < sms) sms = d->max_sms;
   P.sms = sms;
   P.short_first = out_on_host ? 1 : 0;
-  // (by the device's SMs, not by how many of them the call may use: that does not change a result's last bit)
-  P.leaf_log2 = static_cast<int64_t>(P.caps.dec) * P.Hkv >= static_cast<int64_t>(sm_count_of_current_device()) * kLeafStreamWarps
-                    ? kLeafChunkLog2Many : kLeafChunkLog2;
+  P.leaf_warps = sm_count_of_current_device() * (P.G > 8 ? kLeafStreamWarps2 : kLeafStreamWarps);
   const bool timed = prof_begin_call();
   const int call = g_prof.used;
   // phase boundaries: event e is recorded before phase e, event SS_NUM_PHASES after the last one

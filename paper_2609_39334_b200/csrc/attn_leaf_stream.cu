@@ -531,7 +531,7 @@ int32_t launch_leaf_stream(const Params& P, cudaStream_t st, int sm_count) {
   if (!tmap::encode_kv_block_bf16(&tk, P.k_pool, static_cast<uint64_t>(rows)) ||
       !tmap::encode_kv_block_bf16(&tv, P.v_pool, static_cast<uint64_t>(rows)))
     return SS_ERR_CUDA;
-  if (P.G > 8) return launch_variant<2, 8, 3>(P, st, sm_count, tk, tv);
+  if (P.G > 8) return launch_variant<2, kLeafStreamWarps2, 3>(P, st, sm_count, tk, tv);
   return launch_variant<1, kLeafStreamWarps, 2>(P, st, sm_count, tk, tv);
 }
 

@@ -37,7 +37,7 @@ constexpr int kSums = 7;
 constexpr int kLargeBlocks = 8;                // one cluster
 constexpr int kEmitThreads = 256;
 
-__device__ __forceinline__ int leaf_chunks(const Params& P, int len) { return (len + (1 << P.leaf_log2) - 1) >> P.leaf_log2; }
+__device__ __forceinline__ int leaf_chunks(int len, int log2) { return (len + (1 << log2) - 1) >> log2; }
 
 __device__ __forceinline__ int live_paths(const Params& P) {
   int live = P.num_paths;
@@ -64,6 +64,7 @@ __device__ __forceinline__ void node_split(const Params& P, int len, int total_t
 // Seven exclusive scans at once over the block's entries 2 tid, 2 tid + 1 (v -> positions), and the totals; with RANK, in the
 // same two barriers, the rank of each entry among all of them, larger classes cls[] first (order[]: deterministic, but not
 // index order within a class).
+static_assert(8 + kLeafClasses <= 32, "a warp for each class, behind the first 8");
 struct BlockScan {
   int tot[kSums][32];          // per warp, then exclusive over the warps
   int total[kSums];
@@ -143,8 +144,8 @@ __device__ __forceinline__ void block_scan(BlockScan& S, int (&v)[kSums][2], con
 }
 
 // The plan up to the item lists.  `A`: its arrays, in shared memory (small) or in the workspace; `bad_phase`: a word per phase
-// in the block's shared memory; `totals` (tiles of the shared nodes, rows of GENERIC paths): in shared memory, of block 0 of
-// the cluster in the large form.  All start at zero.  False: it failed, the status says why.
+// in the block's shared memory; `totals` (tiles of the shared nodes, rows of GENERIC paths, shorter items of the private leaves of
+// a kv head): in shared memory, of block 0 of the cluster in the large form.  All start at zero.  False: it failed, the status says why.
 template <bool LARGE>
 __device__ __forceinline__ bool make_plan(const Params& P, const PlanArrays& A, PlanHeader* hdr, BlockScan& S, int* bad_phase,
                                           int* totals) {
@@ -268,22 +269,30 @@ __device__ __forceinline__ bool make_plan(const Params& P, const PlanArrays& A, 
   // ---- nodes: tiles (what other blocks' atomics counted is read from L2) ----------------------------------------------------
   auto count = [](const int32_t* c) { return LARGE ? __ldcg(c) : *c; };
   bad = false;
-  int mine = 0;
+  int mine = 0, my_leaves = 0;
 #pragma unroll 1
   for (int n = first; n < N; n += stride) {
     const int np = count(A.n_paths + n), nd = count(A.n_dec + n), p0 = count(A.n_first + n);
     bad = bad || (np > 0 && count(A.n_last + n) - p0 + 1 != np);
     int tiles = 0;
-    if (nd > 0 && A.n_len[n] > 0 && !(np == 1 && A.p_leaf[p0] == n)) tiles = ceil_div(nd, tpt);
+    if (nd > 0 && A.n_len[n] > 0) {
+      if (np == 1 && A.p_leaf[p0] == n)
+        my_leaves += leaf_chunks(A.n_len[n], kLeafChunkLog2);
+      else
+        tiles = ceil_div(nd, tpt);
+    }
     A.n_tiles[n] = tiles;
     mine += tiles;
   }
   mine = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned>(mine)));
   if (lane == 0 && mine) atomicAdd(&totals[0], mine);
+  my_leaves = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned>(my_leaves)));
+  if (lane == 0 && my_leaves) atomicAdd(&totals[2], my_leaves);
   if (phase_failed(bad, SS_ERR_BAD_INPUT)) return false;
 
   // ---- nodes: KV splits, partial slots ------------------------------------------------------------------------------------------
   const int total_tiles = totals[0] * Hkv;
+  const int leaf_log2 = static_cast<int64_t>(totals[2]) * Hkv >= P.leaf_warps ? kLeafChunkLog2Many : kLeafChunkLog2;
 #pragma unroll 1
   for (int n = first; n < N; n += stride) {
     const int len = A.n_len[n], tiles = A.n_tiles[n];
@@ -292,7 +301,7 @@ __device__ __forceinline__ bool make_plan(const Params& P, const PlanArrays& A, 
       if (A.n_parent[n] < 0) node_split(P, len, total_tiles, splits, split_len);
       own = splits;
     } else if (count(A.n_dec + n) > 0 && len > 0) {
-      own = leaf_chunks(P, len);                          // private leaf of one decode path
+      own = leaf_chunks(len, leaf_log2);                       // private leaf of one decode path
     }
     A.n_splits[n] = splits;
     A.n_split_len[n] = split_len;
@@ -325,8 +334,8 @@ __device__ __forceinline__ bool make_plan(const Params& P, const PlanArrays& A, 
 #pragma unroll 1
           for (int a = leaf; a >= 0; a = A.n_parent[a]) slots += A.n_own[a];
           if (count(A.n_paths + leaf) == 1 && len > 0) {
-            full = len >> P.leaf_log2;
-            c = ceil_div(len - (full << P.leaf_log2), kPage);
+            full = len >> leaf_log2;
+            c = ceil_div(len - (full << leaf_log2), kPage);
             // leaves of several chunks before those of one, whose end is cheaper: the merge of several, fence and all, is not
             // to be what the kernel ends with (922 leaves of 32 to 512 keys in chunks of 256, the step: 92.5 -> 88.5 us)
             if (!LARGE && c > 0) c = full > 0 ? 16 + (c + 4) / 5 : (c + 1) / 2;
@@ -406,6 +415,7 @@ __device__ __forceinline__ bool make_plan(const Params& P, const PlanArrays& A, 
     hdr->n_stacked_items = n_stacked;
     hdr->n_generic_rows = totals[1];
     hdr->n_full_leaf_items = n_full;
+    hdr->leaf_log2 = leaf_log2;
     hdr->n_leaf_items = small_ws ? 0 : n_leaf_items;
     hdr->n_tile_items = small_ws ? 0 : n_stacked + total[5];
   }
@@ -417,7 +427,7 @@ template <bool LARGE>
 __device__ __forceinline__ void emit_items(const Params& P, const PlanArrays& A, const PlanHeader* hdr) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int N = P.num_nodes, Hkv = P.Hkv, tpt = P.tok_per_tile;
-  const int live = hdr->live_paths, n_stacked = hdr->n_stacked_items, n_full = hdr->n_full_leaf_items;
+  const int live = hdr->live_paths, n_stacked = hdr->n_stacked_items, n_full = hdr->n_full_leaf_items, leaf_log2 = hdr->leaf_log2;
   const int full0 = !LARGE && P.short_first ? hdr->n_leaf_items - n_full : 0, last0 = P.short_first ? 0 : n_full;
   const int wid = blockIdx.x * (blockDim.x / 32) + warp, nw = gridDim.x * (blockDim.x / 32);
   auto page0_of = [&](int n) { return LARGE ? static_cast<int32_t>(P.node_page_offsets[n]) : A.n_page0[n]; };
@@ -438,7 +448,7 @@ __device__ __forceinline__ void emit_items(const Params& P, const PlanArrays& A,
         P.dec_tok[rank] = row;
         P.dec_src[rank] = src;
         P.dec_slot_base[rank] = slot;
-        P.dec_leaf_chunks[rank] = own_leaf ? leaf_chunks(P, len) : 0;
+        P.dec_leaf_chunks[rank] = own_leaf ? leaf_chunks(len, leaf_log2) : 0;
       }
       for (int g = lane; g < Hkv; g += 32) P.leaf_arrive[static_cast<int64_t>(rank) * Hkv + g] = 0;
       if (!own_leaf) continue;
@@ -448,17 +458,17 @@ __device__ __forceinline__ void emit_items(const Params& P, const PlanArrays& A,
       // whole chunks first 2.43, leaf after leaf 2.37).  Where the rows go over the bus as the leaves are done, the small form
       // turns its order round, so that the bus is not idle until the longest ones are (a step of 1024 paths from host buffers
       // 227 -> 214 us)
-      const int page0 = page0_of(leaf), full = len >> P.leaf_log2, n_items = leaf_chunks(P, len) * Hkv;
+      const int page0 = page0_of(leaf), full = len >> leaf_log2, n_items = leaf_chunks(len, leaf_log2) * Hkv;
       const int last = LARGE ? 0 : A.p_last[p];
 #pragma unroll 1
       for (int x = lane; x < n_items; x += 32) {
         const int c = x / Hkv, g = x - c * Hkv;
         LeafItem it;
-        it.page0 = page0 + ((c << P.leaf_log2) / kPage);
+        it.page0 = page0 + ((c << leaf_log2) / kPage);
         it.node = leaf;
         it.g = g;
-        it.kv_begin = c << P.leaf_log2;
-        it.kv_end = min(len, (c + 1) << P.leaf_log2);
+        it.kv_begin = c << leaf_log2;
+        it.kv_end = min(len, (c + 1) << leaf_log2);
         it.slot = slot + A.n_level[leaf] + c;
         it.q_src = src;
         it.dec = rank;
@@ -515,7 +525,7 @@ __global__ void __launch_bounds__(kThreads) plan_small_kernel(const __grid_const
   extern __shared__ __align__(16) int32_t plan_smem[];
   __shared__ PlanHeader s_hdr;
   __shared__ BlockScan s_scan;
-  __shared__ int s_totals[2];
+  __shared__ int s_totals[3];
   const int tid = threadIdx.x;
   PlanArrays A;
   int32_t* w = plan_smem;
@@ -524,7 +534,7 @@ __global__ void __launch_bounds__(kThreads) plan_small_kernel(const __grid_const
   A.sums = nullptr;
   for (int x = tid; x < kPlanHeaderWords; x += kThreads) reinterpret_cast<int32_t*>(&s_hdr)[x] = 0;
   for (int x = tid; x < kLeafClasses * 64; x += kThreads) (&s_scan.hist[0][0])[x] = 0;
-  if (tid < 2) s_totals[tid] = 0;
+  if (tid < 3) s_totals[tid] = 0;
   SS_STAMP_BEGIN(P.hdr, 0);
   make_plan<false>(P, A, &s_hdr, s_scan, nullptr, s_totals);
   __syncthreads();
@@ -542,10 +552,10 @@ __global__ void __launch_bounds__(kThreads) plan_small_kernel(const __grid_const
 __global__ void __cluster_dims__(kLargeBlocks, 1, 1) __launch_bounds__(kThreads) plan_large_kernel(const __grid_constant__ Params P) {
   ss::grid_dependency_enter();
   __shared__ BlockScan s_scan;
-  __shared__ int s_bad[8], s_totals[2];
+  __shared__ int s_bad[8], s_totals[3];
   const int tid = threadIdx.x;
   if (tid < 8) s_bad[tid] = 0;
-  if (tid < 2) s_totals[tid] = 0;
+  if (tid < 3) s_totals[tid] = 0;
   if (blockIdx.x == 0 && tid < kPlanHeaderWords) reinterpret_cast<int32_t*>(P.hdr)[tid] = 0;
   cg::this_cluster().sync();
   SS_STAMP_BEGIN(P.hdr, 0);

@@ -20,11 +20,14 @@ constexpr int kHeadDim = 128;
 constexpr int kPage = 16;
 constexpr int kTileRows = 128;          // stacked rows of one tile item
 constexpr int kKvTile = 64;             // keys per tensor-core step
-// Most keys per leaf item (decode): 512 - a page a lane - where the paths' leaves are enough for a warp each, else 256, so that more
-// warps have one.  Finer items cost more in partials, fences and merges than the better balance gains (the step with 922 leaves
-// of 32 to 512 keys, two heads: 512 82.4 us, 256 88.4; before that 128 and 64 keys cost 13 and 29 us more than 256).
+// Most keys per leaf item (decode): 512 - a page a lane - where the live paths' leaves make an item of 256 keys for every warp of the
+// leaf kernel (of the whole device's: how many SMs the call may use does not change a result's last bit), else 256, so that more
+// warps have one.  Fewer and longer items save partials, fences and merges.  The step with 256 -> 512, us: 922 leaves of 32 to 512
+// keys, two heads (2800 items of 256 for 1776 warps) 88.4 -> 82.4, 768 (2350) 73.7 -> 68.7, 512 (1570) 58.5 -> 60.9; 384 leaves of 512
+// keys (1536) 66.8 -> 62.5, 256 (1024) 55.4 -> 59.9; with 12 query heads a group 384 of 512 (1536 for 1184 warps) 87.4 -> 74.0, 256
+// (1024) 66.5 -> 66.0, 192 (768) 62.4 -> 63.7.  (Before that 128 and 64 keys cost 13 and 29 us more than 256.)
 constexpr int kLeafChunkLog2 = 8, kLeafChunkLog2Many = 9;
-constexpr int kLeafStreamWarps = 12;    // per SM, of the leaf kernel
+constexpr int kLeafStreamWarps = 12, kLeafStreamWarps2 = 8;   // per SM, of the leaf kernel: groups of up to 8 query heads, and of more
 constexpr int kMaxRootSplits = 8;       // KV splits of a root node when there are few tiles
 constexpr int kMinSplitLen = 512;       // a split is at least this many keys
 
@@ -70,7 +73,8 @@ struct PlanHeader {       // first bytes of the workspace; status MUST be the fi
   int32_t leaf_counter;
   int32_t n_stacked_items; // tile items [0, n_stacked_items) are stacked items, the rest chain items
   int32_t n_full_leaf_items;  // leaf items of whole chunks (they come first in the small planner's list; the large one's goes leaf by leaf)
-  int32_t pad[5];
+  int32_t leaf_log2;       // most keys of a leaf item
+  int32_t pad[4];
 #ifdef SS_STAMPS
   unsigned long long stamp[40];  // instrumented build: %globaltimer at kernel starts / ends (see SS_STAMP); 8..23:
                                  // clock sums of one softmax thread per tile-kernel block (where an item's time goes)
@@ -149,7 +153,7 @@ struct Params {
   int32_t target_tiles;      // the planner splits root nodes until about this many tile items exist
   int32_t sms;               // SMs the call may use
   int32_t short_first;       // small planner: short leaves first (see emit_items)
-  int32_t leaf_log2;         // most keys of a leaf item
+  int32_t leaf_warps;        // of the leaf kernel on the whole device: what the planner chooses the leaf items' length by
   Caps caps;
   // ---- workspace regions ----
   PlanHeader* hdr;

@@ -29,3 +29,27 @@ def test_leaf_items_at_their_ends(lo, hi, more):
     assert (np.abs(got - want) <= 2.0 ** -8 * np.abs(want) + 2.0 ** -9 * 4.6).all()
     assert np.abs(lse - want_lse).max() <= 2e-5
     assert np.isfinite(r["out"]).all()
+
+
+@pytest.mark.parametrize("heads", [(8, 2), (24, 2), (8, 4)])
+@pytest.mark.parametrize("dup", [0.0, 0.9])
+@pytest.mark.parametrize("fan", [64, 300])
+def test_leaf_items_follow_the_live_leaves(heads, dup, fan):
+    """The length of a leaf item depends on the leaves that are there, not on how many candidates there may be: 256 keys until those
+    make an item for every warp of the leaf kernel (12 an SM, 8 with groups of more than 8 query heads); both planners."""
+    w = synth.build_tree_workload("leaves", fan, heads[0], heads[1], [32], [fan], 8, (200, 700), lambda i, m, rng: 1, dup_frac=dup,
+                                  device=DEV)
+    pipe = DevicePipeline(w, DEV)
+    pipe.step()
+    r = pipe.results()
+    lens = w.node_kv_len[w.path_leaf_node[r["unique_paths"]]].astype(np.int64)
+    warps = torch.cuda.get_device_properties(0).multi_processor_count * (8 if heads[0] > 8 * heads[1] else 12)
+    short = int(np.ceil(lens / 256).sum()) * heads[1]
+    want_items = short if short < warps else int(np.ceil(lens / 512).sum()) * heads[1]
+    assert int(pipe.attn_ws[:64].view(torch.int32)[4]) == want_items
+    paths = r["unique_paths"]
+    sample = np.unique(np.concatenate([np.arange(0, len(paths), max(1, len(paths) // 40)), [len(paths) - 1]]))
+    want, want_lse = oracle.tree_attention_workload(w, paths=paths[sample])
+    got, lse = r["out"][sample], r["lse"][sample]
+    assert (np.abs(got - want) <= 2.0 ** -8 * np.abs(want) + 2.0 ** -9 * 4.6).all()      # (as above)
+    assert np.abs(lse - want_lse).max() <= 2e-5
