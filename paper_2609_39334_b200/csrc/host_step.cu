@@ -19,8 +19,8 @@
 // 9 out) go through one kernel per direction that reads or writes the mapped host memory, if it is page-locked; arrays
 // above kSmallBytes keep their copy engine.  Measured, a step of 1024 decode paths: 330 -> 278 us; with the query rows on a stream of
 // their own, the arrays moved side by side and the rows written by the attention kernels 280 -> 214.  Arrays that do not start on 16
-// bytes are moved a byte per thread, which still beats the copies up to a few KB (8 paths 138 -> 67 us a step, 1024 265 -> 216; 4096
-// with three sets in flight 350 -> 457).
+// bytes are read and written in the whole words of host memory that they cover, with single bytes at their two ends (all arrays an
+// element off: 8 paths a byte a thread 81 us a step, 16 bytes a thread one by one 73, so 52; 1024 335, 312, 248; 4096 943, 915, 802).
 #include "step.cuh"
 
 namespace ss {
@@ -30,12 +30,14 @@ constexpr size_t kSmallBytes = 64 << 10;      // three sets in flight, 4096 deco
                                               // 350; one at a time, 1024 paths: 227, 207, 206, 208; 16384: 2341, 2332, 2297, 2282
 constexpr int kMaxSegments = 12;
 
-// Arrays to move, as one sequence of units of 16 bytes (the last of an array may be shorter): a thread has a unit, whichever array
-// it is of, so that a trip over the bus serves all of them (array after array, eight of them took 17 us of a decode step).
+// Arrays to move, as one sequence of units of 16 bytes (the first and the last of an array may be shorter): a thread has a unit,
+// whichever array it is of, so that a trip over the bus serves all of them (array after array, eight of them took 17 us of a
+// decode step).  An array's units start on 16 bytes of HOST memory, behind a first one of `head` bytes if it does not: what goes
+// over the bus is whole 16-byte words side by side, and the device side, which may lie off them then, is in the L2.
 struct Segments {
   const char* src[kMaxSegments];
   char* dst[kMaxSegments];
-  unsigned int bytes[kMaxSegments], first[kMaxSegments];   // first: unit
+  unsigned int bytes[kMaxSegments], head[kMaxSegments], first[kMaxSegments];   // first: unit
   unsigned int units;
   int count;
 };
@@ -56,13 +58,39 @@ static char* mapped(const void* host, size_t bytes) {
   return one_page || static_cast<char*>(last) - static_cast<char*>(first) == end - at ? static_cast<char*>(first) : nullptr;
 }
 
+// Up to 16 bytes that start anywhere.  (Not inlined: a kernel that runs once and for 2 us is bound by its instruction fetches too;
+// with these in line a step of 8 paths takes 3 us more.)
+__device__ __noinline__ uint4 load_bytes(const char* p, unsigned int n) {
+  uint32_t w[4] = {0, 0, 0, 0};
+  if (n == 16 && (reinterpret_cast<uintptr_t>(p) & 3) == 0) {
+#pragma unroll
+    for (int x = 0; x < 4; ++x) w[x] = reinterpret_cast<const uint32_t*>(p)[x];
+  } else {
+#pragma unroll
+    for (int x = 0; x < 16; ++x)
+      if (x < n) w[x >> 2] |= static_cast<uint32_t>(static_cast<unsigned char>(p[x])) << (8 * (x & 3));
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+__device__ __noinline__ void store_bytes(char* p, uint4 v, unsigned int n) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+  if (n == 16 && (reinterpret_cast<uintptr_t>(p) & 3) == 0) {
+#pragma unroll
+    for (int x = 0; x < 4; ++x) reinterpret_cast<uint32_t*>(p)[x] = w[x];
+  } else {
+#pragma unroll
+    for (int x = 0; x < 16; ++x)
+      if (x < n) p[x] = static_cast<char>(w[x >> 2] >> (8 * (x & 3)));
+  }
+}
+
 __device__ __forceinline__ void move_segments(const Segments& S, int block, int n_blocks) {
   constexpr int kAhead = 4;
   const unsigned int step = n_blocks * blockDim.x;
   for (unsigned int u0 = block * blockDim.x + threadIdx.x; u0 < S.units; u0 += kAhead * step) {
     uint4 v[kAhead];
     char* dst[kAhead];
-    unsigned int n[kAhead];                                // bytes; 16 in one piece: 17
+    unsigned int n[kAhead];
 #pragma unroll
     for (int a = 0; a < kAhead; ++a) {
       const unsigned int u = u0 + a * step;
@@ -72,31 +100,21 @@ __device__ __forceinline__ void move_segments(const Segments& S, int block, int 
       if (u >= S.units || u < u0) continue;
       int i = 0;
       while (i + 1 < S.count && S.first[i + 1] <= u) ++i;
-      const unsigned int at = (u - S.first[i]) * 16;
+      const unsigned int k = u - S.first[i], head = S.head[i], at = head == 0 ? 16 * k : k == 0 ? 0 : head + 16 * (k - 1);
       const char* src = S.src[i] + at;
       dst[a] = S.dst[i] + at;
-      n[a] = min(16u, S.bytes[i] - at);
-      if (n[a] == 16 && ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst[a])) & 15) == 0) {
+      n[a] = min(head != 0 && k == 0 ? head : 16u, S.bytes[i] - at);
+      if (n[a] == 16 && (reinterpret_cast<uintptr_t>(src) & 15) == 0)
         v[a] = *reinterpret_cast<const uint4*>(src);
-        n[a] = 17;
-      } else {
-        uint32_t w[4] = {0, 0, 0, 0};
-#pragma unroll
-        for (int x = 0; x < 16; ++x)
-          if (x < n[a]) w[x >> 2] |= static_cast<uint32_t>(static_cast<unsigned char>(src[x])) << (8 * (x & 3));
-        v[a] = make_uint4(w[0], w[1], w[2], w[3]);
-      }
+      else
+        v[a] = load_bytes(src, n[a]);
     }
 #pragma unroll
     for (int a = 0; a < kAhead; ++a) {
-      if (n[a] == 17) {
+      if (n[a] == 16 && (reinterpret_cast<uintptr_t>(dst[a]) & 15) == 0)
         *reinterpret_cast<uint4*>(dst[a]) = v[a];
-      } else {
-        const uint32_t w[4] = {v[a].x, v[a].y, v[a].z, v[a].w};
-#pragma unroll
-        for (int x = 0; x < 16; ++x)
-          if (x < n[a]) dst[a][x] = static_cast<char>(w[x >> 2] >> (8 * (x & 3)));
-      }
+      else if (n[a] > 0)
+        store_bytes(dst[a], v[a], n[a]);
     }
   }
 }
@@ -316,8 +334,10 @@ extern "C" int32_t ss_candidate_step_host_2(const ss_host_step_t* step, void* de
     }
     list.src[list.count] = to_host ? static_cast<const char*>(src) : map;
     list.dst[list.count] = to_host ? map : static_cast<char*>(dst);
+    const size_t head = (0 - reinterpret_cast<uintptr_t>(map)) & 15;   // (bytes in front of the first whole word)
+    list.head[list.count] = static_cast<unsigned int>(head);
     list.first[list.count] = list.units;
-    list.units += static_cast<unsigned int>((bytes + 15) / 16);
+    list.units += static_cast<unsigned int>((head ? 1 : 0) + (bytes > head ? (bytes - head + 15) / 16 : 0));
     list.bytes[list.count++] = static_cast<unsigned int>(bytes);
     return true;
   };
