@@ -36,21 +36,40 @@ __device__ __forceinline__ uint64_t mix64(uint64_t x) {   // splitmix64 finalise
   return x;
 }
 
+// Ids of a path that a lane has on their way.  Up to kSmallMax paths wait for memory: with eight, paths of 300 tokens are two trips,
+// not ten (the step of 1024 paths 78.4 us, 83.5 with four; 4096 paths of up to 2000 tokens 29 us, 45 with one, 34 with a test for
+// each of eight).  More paths are bound by instructions and registers: 100000 of up to 300 tokens 96 us with four, 113 with eight.
+// Whole rounds go without a test for each id, and a warp leaves a round where nothing is left: 100000 of up to 8 tokens 57 us, 85
+// with a test for each of eight, 59 with one id at a time.
+constexpr int kAheadSmall = 8, kAheadLarge = 4;
+constexpr uint64_t kId = 0x9e3779b97f4a7c15ull, kAt = 0xd1b54a32d192ed03ull;
 // Whole warp: 64-bit hash of path `path` (returned to every lane).
+template <int kAhead>
 __device__ __forceinline__ uint64_t hash_path(const int32_t* __restrict__ tok_ids, const int64_t* __restrict__ tok_offsets,
                                               const int64_t* __restrict__ ctx_key, int path, uint32_t weak, int lane) {
   const int64_t lo = tok_offsets[path], hi = tok_offsets[path + 1];
-  uint64_t acc = 0;
-  constexpr int kUnroll = 8;                    // loads in flight: paths of 300 tokens are one or two trips to memory, not ten
-  for (int64_t j0 = lo + lane; j0 < hi; j0 += 32 * kUnroll) {
-    uint32_t t[kUnroll];
+  uint64_t acc = 0, at = static_cast<uint64_t>(lane + 1) * kAt;   // (position + 1) * kAt
+  const int32_t* p = tok_ids + lo + lane;
+  int64_t left = hi - lo;
+  for (; left >= 32 * kAhead; left -= 32 * kAhead, p += 32 * kAhead, at += 32 * kAhead * kAt) {
+    uint32_t t[kAhead];
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) t[u] = j0 + 32 * u < hi ? static_cast<uint32_t>(tok_ids[j0 + 32 * u]) : 0u;
+    for (int u = 0; u < kAhead; ++u) t[u] = static_cast<uint32_t>(p[32 * u]);
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      const int64_t j = j0 + 32 * u;
-      if (j < hi) acc += mix64(t[u] * 0x9e3779b97f4a7c15ull + static_cast<uint64_t>(j - lo + 1) * 0xd1b54a32d192ed03ull);
-    }
+    for (int u = 0; u < kAhead; ++u) acc += mix64(t[u] * kId + at + 32 * u * kAt);
+  }
+  const int rest = static_cast<int>(left);
+  uint32_t t[kAhead];
+#pragma unroll
+  for (int u = 0; u < kAhead; ++u) {                        // (the warp leaves where nothing is left: most paths have a few tokens)
+    if (kAhead == kAheadLarge && 32 * u >= rest) break;
+    t[u] = lane + 32 * u < rest ? static_cast<uint32_t>(p[32 * u]) : 0u;
+  }
+#pragma unroll
+  for (int u = 0; u < kAhead; ++u) {
+    if (32 * u >= rest) break;
+    const uint64_t m = mix64(t[u] * kId + at + 32 * u * kAt);
+    if (lane + 32 * u < rest) acc += m;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -66,6 +85,7 @@ __device__ __forceinline__ uint32_t tag_of(uint64_t h) { return static_cast<uint
 
 // Hash of every path.  `table` (mask + 1 entries, all ones): inserts; `chunk_count`, `multiplicity`: cleared for the kernels
 // that follow; `arrived`: the counter of small_match_kernel.
+template <int kAhead>
 __global__ void hash_kernel(const int32_t* __restrict__ tok_ids, const int64_t* __restrict__ tok_offsets,
                             const int64_t* __restrict__ ctx_key, int n, uint32_t weak, uint64_t* __restrict__ hash64,
                             unsigned long long* table, uint32_t mask, int* __restrict__ chunk_count,
@@ -80,7 +100,7 @@ __global__ void hash_kernel(const int32_t* __restrict__ tok_ids, const int64_t* 
   }
   if ((gtid >> 5) >= n) return;
   const int path = static_cast<int>(gtid >> 5);
-  const uint64_t h = hash_path(tok_ids, tok_offsets, ctx_key, path, weak, lane);
+  const uint64_t h = hash_path<kAhead>(tok_ids, tok_offsets, ctx_key, path, weak, lane);
   if (lane != 0) return;
   hash64[path] = h;
   if (!table) return;
@@ -125,44 +145,59 @@ hash_select_kernel(const int32_t* __restrict__ tok_ids, const int64_t* __restric
   const int lane = threadIdx.x & 31, path = blockIdx.x * kHashWarps + (threadIdx.x >> 5);
   if (blockIdx.x == 0 && threadIdx.x == 0) *arrived = 0;
   if (path >= n) return;
-  const uint64_t h = hash_path(tok_ids, tok_offsets, ctx_key, path, weak, lane);
+  const uint64_t h = hash_path<kAheadSmall>(tok_ids, tok_offsets, ctx_key, path, weak, lane);
   if (lane == 0) hash64[path] = h;
 }
 
 // Whole warp: paths i and j have the same context, length and ids.
+template <int kAhead>
 __device__ __forceinline__ bool same_path(const int32_t* __restrict__ tok_ids, const int64_t* __restrict__ tok_offsets,
                                           const int64_t* __restrict__ ctx_key, int i, int j, int lane) {
   const int64_t a0 = tok_offsets[i], b0 = tok_offsets[j], len = tok_offsets[i + 1] - a0;
   if (tok_offsets[j + 1] - b0 != len || (ctx_key && ctx_key[i] != ctx_key[j])) return false;
-  constexpr int kUnroll = 8;
-  for (int64_t p = lane; p - lane < len; p += 32 * kUnroll) {
-    int32_t x[kUnroll], y[kUnroll];
+  const int32_t *a = tok_ids + a0 + lane, *b = tok_ids + b0 + lane;
+  int64_t left = len;
+  for (; left >= 32 * kAhead; left -= 32 * kAhead, a += 32 * kAhead, b += 32 * kAhead) {
+    int32_t x[kAhead], y[kAhead];
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      const int64_t q = p + 32 * u;
-      x[u] = q < len ? tok_ids[a0 + q] : 0;
-      y[u] = q < len ? tok_ids[b0 + q] : 0;
+    for (int u = 0; u < kAhead; ++u) {
+      x[u] = a[32 * u];
+      y[u] = b[32 * u];
     }
-    bool eq = true;
+    int32_t diff = 0;
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) eq = eq && x[u] == y[u];
-    if (!__all_sync(0xffffffffu, eq)) return false;
+    for (int u = 0; u < kAhead; ++u) diff |= x[u] ^ y[u];
+    if (__any_sync(0xffffffffu, diff != 0)) return false;
   }
-  return true;
+  const int rest = static_cast<int>(left);
+  int32_t x[kAhead], y[kAhead];
+#pragma unroll
+  for (int u = 0; u < kAhead; ++u) {
+    x[u] = y[u] = 0;
+    if (lane + 32 * u < rest) {
+      x[u] = a[32 * u];
+      y[u] = b[32 * u];
+    }
+  }
+  int32_t diff = 0;
+#pragma unroll
+  for (int u = 0; u < kAhead; ++u) diff |= x[u] ^ y[u];
+  return !__any_sync(0xffffffffu, diff != 0);
 }
 
 // Whole warp: canonical representative of path i, given the smallest path j <= i in its table entry.
+template <int kAhead>
 __device__ __forceinline__ int canon_of(const int32_t* __restrict__ tok_ids, const int64_t* __restrict__ tok_offsets,
                                         const int64_t* __restrict__ ctx_key, const uint64_t* hash64, uint64_t h, int i, int j,
                                         int lane) {
-  if (j == i || (hash64[j] == h && same_path(tok_ids, tok_offsets, ctx_key, i, j, lane))) return j;
+  if (j == i || (hash64[j] == h && same_path<kAhead>(tok_ids, tok_offsets, ctx_key, i, j, lane))) return j;
   for (int b = 0; b < i; b += 32) {                           // a collision
     const int t = b + lane;
     uint32_t m = __ballot_sync(0xffffffffu, t < i && t != j && hash64[t < i ? t : 0] == h);
     while (m) {
       const int c = b + __ffs(m) - 1;
       m &= m - 1;
-      if (same_path(tok_ids, tok_offsets, ctx_key, i, c, lane)) return c;
+      if (same_path<kAhead>(tok_ids, tok_offsets, ctx_key, i, c, lane)) return c;
     }
   }
   return i;
@@ -212,7 +247,7 @@ __device__ __forceinline__ void small_match(const int32_t* __restrict__ tok_ids,
     const uint64_t h = s_hash[i];
     uint32_t s = static_cast<uint32_t>(h) & mask;
     while (s_hash[s_tab[s]] != h) s = (s + 1) & mask;
-    const int c = canon_of(tok_ids, tok_offsets, ctx_key, s_hash, h, i, s_tab[s], lane);
+    const int c = canon_of<kAheadSmall>(tok_ids, tok_offsets, ctx_key, s_hash, h, i, s_tab[s], lane);
     if (lane == 0) canon_out[i] = c;
   }
 }
@@ -401,7 +436,7 @@ cluster_dedup_kernel(const int32_t* __restrict__ tok_ids, const int64_t* __restr
   GatherRows R;
   load_rows<STEP>(R, G, n);
   for (int i = blockIdx.x * kWarps + (threadIdx.x >> 5); i < n; i += kClusterBlocks * kWarps) {
-    const uint64_t h = hash_path(tok_ids, tok_offsets, ctx_key, i, weak, lane);
+    const uint64_t h = hash_path<kAheadSmall>(tok_ids, tok_offsets, ctx_key, i, weak, lane);
     if (lane == 0) hash64[i] = h;
   }
   cluster_barrier();
@@ -431,7 +466,7 @@ match_kernel(const int32_t* __restrict__ tok_ids, const int64_t* __restrict__ to
       s = (s + 1) & mask;
       e = table[s];
     }
-    const int c = canon_of(tok_ids, tok_offsets, ctx_key, hash64, h, i, static_cast<int>(static_cast<uint32_t>(e)), lane);
+    const int c = canon_of<kAheadLarge>(tok_ids, tok_offsets, ctx_key, hash64, h, i, static_cast<int>(static_cast<uint32_t>(e)), lane);
     if (lane == 0) canon_out[i] = c;
     own = c == i ? 1 : 0;
   }
@@ -676,7 +711,7 @@ extern "C" int32_t ss_dedup_paths(const int32_t* tok_ids, const int64_t* tok_off
     unsigned int* arrived = reinterpret_cast<unsigned int*>(ws + L.counters);
     const int32_t rc = small_smem_ready();
     if (rc != SS_OK) return rc;
-    SS_LAUNCH(hash_kernel, hash_blocks, kHashWarps * 32, 0, st, tok_ids, tok_offsets, ctx_key, n, weak, hash64,
+    SS_LAUNCH(hash_kernel<kAheadSmall>, hash_blocks, kHashWarps * 32, 0, st, tok_ids, tok_offsets, ctx_key, n, weak, hash64,
               static_cast<unsigned long long*>(nullptr), 0u, static_cast<int*>(nullptr), static_cast<int32_t*>(nullptr), arrived);
     SS_LAUNCH(small_match_kernel<false>, match_blocks, kThreads, small_match_smem(n), st, tok_ids, tok_offsets, ctx_key, n, hash64,
               static_cast<uint32_t>(small_table_size(n) - 1), slot_in, canon_out, path_to_unique_out, unique_paths_out,
@@ -691,7 +726,7 @@ extern "C" int32_t ss_dedup_paths(const int32_t* tok_ids, const int64_t* tok_off
     (void)cudaGetLastError();
     return SS_ERR_CUDA;
   }
-  SS_LAUNCH(hash_kernel, hash_blocks, kHashWarps * 32, 0, st, tok_ids, tok_offsets, ctx_key, n, weak, hash64, table, L.mask,
+  SS_LAUNCH(hash_kernel<kAheadLarge>, hash_blocks, kHashWarps * 32, 0, st, tok_ids, tok_offsets, ctx_key, n, weak, hash64, table, L.mask,
             chunk_count, multiplicity_out, static_cast<unsigned int*>(nullptr));
   SS_LAUNCH(match_kernel, match_blocks, kThreads, 0, st, tok_ids, tok_offsets, ctx_key, n, hash64, table, L.mask, canon_out,
             unique, chunk_count);
