@@ -184,3 +184,54 @@ def test_arrays_off_16_bytes_cost_little():
         return float(np.median(times[10:]))
 
     assert min(best(hosts[1]) / best(hosts[0]) for _ in range(3)) < 1.2
+
+
+KINDS = {
+    # verification and mixed steps (rows copied behind the attention, which leaves SMs to that)
+    "verify": dict(heads=(28, 4), levels=[256], fanout=[9], problems=3, leaf=(20, 300), q=lambda i, n, r: int(r.integers(16, 40))),
+    "mixed": dict(heads=(12, 2), levels=[128, 32], fanout=[3, 7], problems=4, leaf=(0, 200), q=lambda i, n, r: 1 if i % 2 else 24),
+    # decode steps: rows written by the attention, leaves of several items of 256 keys and of 512, both planners, the four calls
+    "long_leaves_few": dict(heads=(12, 2), levels=[64], fanout=[20], problems=4, leaf=(200, 1100)),
+    "long_leaves_many": dict(heads=(12, 2), levels=[64], fanout=[100], problems=8, leaf=(200, 1100)),
+    "large_planner": dict(heads=(8, 4), levels=[32], fanout=[150], problems=15, leaf=(0, 600)),
+    "four_calls": dict(heads=(4, 2), levels=[32], fanout=[150], problems=30, leaf=(0, 300)),
+    "out_on_16_bytes": dict(heads=(12, 2), levels=[64], fanout=[20], problems=4, leaf=(0, 300)),
+    "uneven": dict(heads=(12, 2), levels=[64], fanout=[20], problems=4, leaf=(3, 300)),
+}
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_compact_steps_of_every_kind(kind):
+    """SS_STEP_COMPACT_TRANSFERS, bit for bit as on the device, rows past the live ones as the caller left them."""
+    k = KINDS[kind]
+    w = synth.build_tree_workload(kind, len(kind), k["heads"][0], k["heads"][1], k["levels"], k["fanout"], k["problems"], k["leaf"],
+                                  k.get("q", lambda i, n, r: 1), dup_frac=0.2, device=DEV)
+    if kind == "uneven":                                         # as many rows as paths, but not one each: a duplicate gives its to its first
+        canon = oracle.dedup(w.tok_ids, w.tok_offsets, w.ctx_key)["canon"]
+        for b in np.nonzero(canon != np.arange(len(canon)))[0][:6]:
+            if w.path_q_len[canon[b]] == 1:
+                w.path_q_len[canon[b]], w.path_q_len[b] = 2, 0
+        w.q_offsets[1:] = np.cumsum(w.path_q_len)
+        assert w.total_q == w.num_paths and w.path_q_len.max() == 2
+    pipe = DevicePipeline(w, DEV)
+    pipe.step()
+    r_dev = pipe.results()
+    host = HostStepPipeline(pipe, depth=2, compact=True)
+    for s in host.sets:
+        if kind == "out_on_16_bytes":
+            s["h_out"]["out"] = shifted(s["h_out"]["out"], 8)
+            s["step"] = B.make_host_step(pipe.desc, n_paths=pipe.N, n_segments=pipe.P, top_k=w.top_k, total_tok=int(w.tok_offsets[-1]),
+                                         total_q=w.total_q, host_in=s["h_in"], host_out=s["h_out"], dedup_flags=pipe.dedup_flags,
+                                         flags=B.SS_STEP_COMPACT_TRANSFERS)
+        s["h_out"]["out"].fill_(-7.0)
+        s["h_out"]["lse"].fill_(-7.0)
+    for i in range(4):
+        host.submit(i)
+    host.synchronize()
+    for i in range(2):
+        r = host.results(i)
+        assert np.array_equal(r["out"], r_dev["out"]) and np.array_equal(r["lse"], r_dev["lse"])
+        for key in ("canon", "path_to_unique", "unique_paths", "multiplicity", "slot_out", "survivors", "keep"):
+            assert np.array_equal(r[key], r_dev[key]), key
+        o = host.sets[i]["h_out"]
+        assert r_dev["total_q"] < w.total_q and (o["out"][r_dev["total_q"]:] == -7.0).all() and (o["lse"][r_dev["total_q"]:] == -7.0).all()

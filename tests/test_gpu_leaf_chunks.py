@@ -4,6 +4,7 @@ import pytest
 import torch
 
 import oracle
+from paper_2609_39334_b200 import binding as B
 from paper_2609_39334_b200 import synth
 from paper_2609_39334_b200.pipeline import DevicePipeline
 
@@ -53,3 +54,26 @@ def test_leaf_items_follow_the_live_leaves(heads, dup, fan):
     got, lse = r["out"][sample], r["lse"][sample]
     assert (np.abs(got - want) <= 2.0 ** -8 * np.abs(want) + 2.0 ** -9 * 4.6).all()      # (as above)
     assert np.abs(lse - want_lse).max() <= 2e-5
+
+
+@pytest.mark.parametrize("heads", [(8, 2), (24, 2)])
+def test_long_leaf_items_in_the_register_staged_kernel(heads):
+    """A pool whose blocks are 17 rows apart, which the streaming kernel does not take: items of 512 keys, groups of up to 8 query
+    heads and of more."""
+    w = synth.build_tree_workload("staged", sum(heads), heads[0], heads[1], [32], [150], 8, (200, 1100), lambda i, m, rng: 1, device=DEV)
+    pipe = DevicePipeline(w, DEV)
+    pool = pipe.kv_pool                                          # [page][2][Hkv][16][128]
+    padded = torch.full((pool.shape[0], 2, heads[1], 17, 128), float("nan"), dtype=torch.bfloat16, device=DEV)
+    padded[:, :, :, :16] = pool
+    d, blk = pipe.desc, heads[1] * 17 * 128
+    d.k_pool, d.v_pool = padded.data_ptr(), padded.data_ptr() + blk * 2
+    d.kv_page_stride, d.kv_head_stride, d.kv_token_stride = 2 * blk, 17 * 128, 128
+    pipe.attn_ws = B.alloc_workspace(B.ss_tree_attention_workspace_bytes(d), pool.device)
+    pipe.step()
+    r = pipe.results()
+    lens = w.node_kv_len[w.path_leaf_node].astype(np.int64)
+    assert int(pipe.attn_ws[:64].view(torch.int32)[4]) == int(np.ceil(lens / 512).sum()) * heads[1]
+    sample = np.arange(0, len(lens), 29)
+    want, want_lse = oracle.tree_attention_workload(w, paths=r["unique_paths"][sample])
+    assert (np.abs(r["out"][sample] - want) <= 2.0 ** -8 * np.abs(want) + 2.0 ** -9 * 4.6).all()   # (as above)
+    assert np.abs(r["lse"][sample] - want_lse).max() <= 2e-5

@@ -232,3 +232,28 @@ def test_prefix_tree_merges_of_sorted_runs(n, alphabet):
     rng = np.random.default_rng(n + alphabet)
     off = np.concatenate([[0], np.cumsum(rng.integers(0, 9, size=n))]).astype(np.int64)
     check(rng.integers(0, alphabet, size=int(off[-1])).astype(np.int32), off, 1)
+
+
+@pytest.mark.parametrize("n", [1, 30, 33, 400, 513])
+def test_the_workspace_may_hold_anything(n):
+    """One block, a cluster, a grid: the status, the barrier's counter and the flags are cleared by the call, which is made three
+    times on a workspace of all ones and on what the call before left."""
+    rng = np.random.default_rng(n)
+    ids, off = csr([rng.integers(0, 3, size=rng.integers(0, 90)).tolist() for _ in range(n)])
+    want = oracle.build_prefix_tree(ids, off, 16)
+    total, dev = int(off[-1]), torch.device(DEV)
+    i32 = dict(dtype=torch.int32, device=dev)
+    t_ids = torch.from_numpy(ids if total else np.zeros(1, np.int32)).to(dev)
+    t_off = torch.from_numpy(off).to(dev)
+    order, leaf, num = torch.empty(n, **i32), torch.empty(n, **i32), torch.empty(1, **i32)
+    four = [torch.empty(2 * n, **i32) for _ in range(4)]
+    ws = B.alloc_workspace(B.ss_prefix_tree_workspace_bytes(n, total, 16), dev)
+    ws.fill_(255)
+    for _ in range(3):
+        B.ss_build_prefix_tree(t_ids, t_off, n, total, 16, order, leaf, *four, num, ws)
+        torch.cuda.synchronize()
+        assert B.ss_last_device_status(ws) == B.SS_OK
+        m = int(num.item())
+        for t, key, size in zip([order, leaf] + four, ("order", "path_leaf_node", "node_parent", "node_kv_len", "node_src_path", "node_src_offset"),
+                                (n, n, m, m, m, m)):
+            assert np.array_equal(t[:size].cpu().numpy(), want[key]), key
