@@ -5,7 +5,8 @@
 // The token decision is that of fp64 (it agrees with a plain fp64 CPU evaluation except for draws within
 // ~1e-15 of a boundary), one exponential per logit.  A row is split over the 16 warps of a block, or of a CLUSTER of
 // 2, 4 or 8 blocks when there are too few rows to give every SM one: each warp has one contiguous slice, and the slice sums
-// meet in (distributed) shared memory.  Nothing is read twice but the 512 tokens around each draw.
+// meet in (distributed) shared memory.  Nothing is read twice but the 512 tokens around each draw, and the row of a draw that fp32
+// sums leave open (below).
 //   1. every warp sums 2^(logit_v * c), c = log2(e) / temperature, over its slice in segments of 512 tokens and keeps
 //      the running sum at every segment's end (shared memory)
 //   2. the slice sums are written to every block of the cluster
@@ -260,13 +261,6 @@ __device__ __forceinline__ double exact_sums(float (&l)[16], const Args& A, cons
   return s0 + s1;
 }
 
-// The same in fp32, two logits at a time, relative to a power of two 2^e0 that the lane moves when a logit exceeds it by 2^60.
-// l * c = n + f with |f| <= 1/2: n from a sum whose low bits are the integer, f exactly by an FMA with the high part of c (one
-// rounding to 2^-26) and one with the low part; 2^f by a polynomial of degree 6 (minimax of the relative error on |f| <=
-// 0.5002, coefficients rounded: 1.6e-8); n into the exponent by an integer addition.  A term is within 1.21e-7: 1.6e-8, 2.1e-8
-// from f, 2.4e-8 from the polynomial's inner roundings and 6e-8 from its last one.  Eight terms are added pairwise (three
-// roundings, 1.79e-7) and go to fp64 from there: a sum of any of them is within kQuickError of the exact one.  Terms below
-// 2^(e0 - 124) count as that, 2^-124 of the lane's largest and less.
 // Sums of four values over the warp at once (18 instructions instead of 60): lane l gets that of v[l / 8].
 __device__ __forceinline__ double warp_sums_4(const double (&v)[4], int lane) {
   const bool up = (lane & 16) != 0, right = (lane & 8) != 0;
@@ -278,6 +272,14 @@ __device__ __forceinline__ double warp_sums_4(const double (&v)[4], int lane) {
   return c;
 }
 
+// A lane's sum of a segment in fp32, two logits at a time, relative to a power of two 2^e0 that the lane moves when a logit exceeds
+// it by 2^60.
+// l * c = n + f with |f| <= 1/2: n from a sum whose low bits are the integer, f exactly by an FMA with the high part of c (one
+// rounding to 2^-26) and one with the low part; 2^f by a polynomial of degree 6 (minimax of the relative error on |f| <=
+// 0.5002, coefficients rounded: 1.6e-8); n into the exponent by an integer addition.  A term is within 1.21e-7: 1.6e-8, 2.1e-8
+// from f, 2.4e-8 from the polynomial's inner roundings and 6e-8 from its last one.  Eight terms are added pairwise (three
+// roundings, 1.79e-7) and go to fp64 from there: a sum of any of them is within kQuickError of the exact one.  Terms below
+// 2^(e0 - 124) count as that, 2^-124 of the lane's largest and less.
 struct QuickState {
   float mx, e0, low, shift;
 };
@@ -1208,8 +1210,11 @@ extern "C" int32_t ss_branch_sample_upto(const float* logits, const int64_t* dra
   // 592 x 65536, 1: 55 -> 61; 444 x 100352, 1: 60 -> 65; 740 x 100352, 4: 95 -> 106; 922 x 151936, 16: 196 -> 287; 148 x 151936, 1:
   // 30 -> 40, 148 x 16384, 1: 8 -> 20.  Smaller vocabularies gain little at any number of rows (2400 x 16384, 1: 89 -> 85).
   const int64_t tokens = static_cast<int64_t>(whole / sms) * vocab;   // of a block
-  const bool rows = max_draws >= 0 && A.fast && vocab >= 32000 && tokens >= 390000 &&
-                    max_draws <= static_cast<int64_t>(n_seq) * (tokens >= 1000000 ? 6 : tokens >= 605000 ? 4 : tokens >= 500000 ? 3 : 2);
+  // A few rows left over go to clusters of 8 otherwise, too few of them for the marked draws (1490 x 151936, 3: 286 -> 402 us with them,
+  // 260 with clusters of 4): with less than five rounds in front of them the table keeps them.
+  const bool few_left = n_seq > whole && n_seq - whole <= n8;
+  const bool rows = max_draws >= 0 && A.fast && vocab >= 32000 && tokens >= 390000 && (!few_left || whole / sms >= 5) &&
+                    max_draws <= static_cast<int64_t>(n_seq) * (tokens >= 1000000 ? 5 : tokens >= 605000 ? 4 : tokens >= 500000 ? 3 : 2);
   if (rows) A.whole_draws = vocab >> 12 > 16 ? vocab >> 12 : 16;
   if (whole > 0) {
     const int blocks = whole < sms ? whole : sms;

@@ -76,7 +76,7 @@ def child_waits():
     from paper_2609_39334_b200 import binding as B
 
     assert B.LIB_PATH.endswith("_checked.so") and "SS_GIVE_UP" in os.environ
-    S, V = 4 * torch.cuda.get_device_properties(0).multi_processor_count + 5, 131072
+    S, V = 4 * torch.cuda.get_device_properties(0).multi_processor_count + 20, 131072
     rng = np.random.default_rng(3)
     logits = rng.standard_normal((S, V), dtype=np.float32) * np.float32(2.0)
     logits[::7] += np.float32(900.0)                            # (outside the range of the sums)
