@@ -370,7 +370,7 @@ int32_t ss_build_prefix_tree(const int32_t* tok_ids, const int64_t* tok_offsets,
  * ss_topk_prune in this order, on the arguments of the same names; up to 4096 candidates the parts that do not need one another
  * share launches.  `attn` is passed to ss_tree_attention as it is: its per-path arrays are the u_* arrays and num_unique of this
  * struct where a step is wanted.  Nothing is allocated, and the call does not synchronise.
- * Errors: those of the four calls.
+ * Errors: those of the four calls; an error of the attention's own arguments is found behind the launches of the others.
  * ======================================================================================================= */
 typedef struct ss_device_step {
   uint32_t struct_size;              /* = sizeof(ss_device_step_t) */
@@ -425,7 +425,8 @@ int32_t ss_candidate_step(const ss_device_step_t* step /* host */, void* stream)
  * are returned whole, as without the flag.)
  * Steps of one query row per path write out straight from the attention kernels then.
  * Everything is enqueued on `stream` - in ss_candidate_step_host_2 with a `copy_stream` the copy of the query rows on that one, behind
- * what `stream` holds and in front of the attention, so that it overlaps the deduplication; the call does not synchronise, and it allocates no memory: staging buffers,
+ * what `stream` holds and in front of the attention, so that it overlaps the deduplication (two events are created and destroyed
+ * for it; with several steps in flight, query rows of more than about 16 MB are better copied on `stream`).  The call does not synchronise, and it allocates no memory: staging buffers,
  * results and the workspaces of the three calls are carved out of `device_arena` (caller-owned, 256-byte aligned,
  * >= ss_candidate_step_host_arena_bytes).  The KV pool and the tree stay resident on the device: they are the
  * cache state of the method, described by the resident fields of `attn` (flags, heads, sm_scale, pool, strides,

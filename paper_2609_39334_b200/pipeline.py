@@ -170,6 +170,11 @@ class HostStepPipeline:
             out.copy_(t)
             return out
 
+        # The query rows have a stream of their own beside the deduplication and the planning, but for large steps of several
+        # sets: there the copy of the next step, which would otherwise wait its turn, takes the bus from this one's results
+        # (two sets, 16384 decode paths 1370 us a step, 1911 with it; 256 verification paths 2.78 ms, 3.05; 4096 decode paths, 13
+        # MB, 514 with it and 517 without; one set, 16384 paths 2184 with it and 2268 without).
+        own_stream = depth == 1 or tq * Hq * D * 2 <= 16 << 20
         self.sets = []
         for _ in range(depth):
             h_in = dict(
@@ -191,7 +196,7 @@ class HostStepPipeline:
                                     flags=B.SS_STEP_COMPACT_TRANSFERS if compact else 0)
             arena = B.alloc_workspace(B.ss_candidate_step_host_arena_bytes(step), dev)
             self.sets.append(dict(h_in=h_in, h_out=h_out, step=step, arena=arena, stream=torch.cuda.Stream(dev),
-                                  copy_stream=torch.cuda.Stream(dev)))
+                                  copy_stream=torch.cuda.Stream(dev) if own_stream else None))
         self.h2d_bytes = sum(t.numel() * t.element_size() for t in self.sets[0]["h_in"].values())
         self.d2h_bytes = sum(t.numel() * t.element_size() for t in self.sets[0]["h_out"].values())
 
