@@ -855,7 +855,8 @@ static int32_t launch_front(const ss_device_step_t& s, cudaStream_t st) {
   return SS_OK;
 }
 
-// True if the four calls would accept their arguments, so that nothing has to be refused half-way.
+// True if the deduplication, the gather and the selection would accept their arguments.  (The attention looks at its own behind them,
+// as where the four calls are made one after the other; the selection's results are then there already.)
 static bool front_args_ok(const ss_device_step_t& s) {
   if ((s.slot_in == nullptr) != (s.slot_out == nullptr) || s.top_k < 1 || (s.dedup_flags & ~SS_FLAG_WEAK_HASH)) return false;
   const void* const needed[] = {s.tok_ids, s.tok_offsets, s.canon, s.path_to_unique, s.unique_paths, s.multiplicity, s.num_unique,

@@ -241,8 +241,8 @@ def test_many_draws_of_a_row(S, V, most, peak):
 @pytest.mark.parametrize("S,V", [(148, 16384), (149, 40961), (222, 151936), (330, 128256)])
 @pytest.mark.parametrize("kind", ["flat", "peaked", "masked"])
 def test_draws_at_the_boundaries_between_tokens(S, V, kind):
-    """Rows that blocks take by themselves, whose sums are first made in fp32: uniforms that lie on a token's end (to fp32), between
-    two ends, at 0 and just below 1, so that many draws cannot be decided from those sums; flat rows, rows with all of their
+    """Rows that blocks take by themselves (with fp32 sums: test_few_draws_of_many_rows): uniforms that lie on a token's end (to fp32),
+    between two ends, at 0 and just below 1; flat rows, rows with all of their
     probability on a few tokens, rows that begin and end with masked ones.  Few and many draws of a row."""
     rng = np.random.default_rng(S + V)
     logits = (rng.normal(size=(S, V)) * (0.0 if kind == "flat" else 3.0)).astype(np.float32)
